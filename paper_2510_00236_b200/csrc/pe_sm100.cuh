@@ -13,6 +13,16 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// True in exactly one lane of a converged warp.  Single-thread work (TMA issue, MMA issue, commits) sits behind this
+// in otherwise warp-uniform code: those instructions take their operands from the warp's uniform registers, and behind a
+// test of the lane number instead, where the compiler cannot know that one lane remains, an MMA took about 140 cycles
+// to issue and a TMA load 115.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r != 0;
+}
+
 // ---------------------------------------------------------------- thread-block cluster (CTA pair)
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
@@ -63,7 +73,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// The same test without the bounded suspension try_wait may add: for a thread that polls several barriers in turn.
+// The same test without the bounded suspension try_wait may add.
 __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -80,24 +90,21 @@ __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
 // exhausts it latches an error code and raises the block-wide abort flag so that every other role
 // leaves its loops as well.
 constexpr long long WAIT_CYCLE_LIMIT_DEFAULT = 1ll << 32;
+constexpr long long WAIT_CYCLE_LIMIT_STRICT = 1ll << 20;   // below this the budget is looked at on every poll
 __device__ long long g_wait_cycle_limit = WAIT_CYCLE_LIMIT_DEFAULT;
 __device__ __forceinline__ long long wait_cycle_limit() { return *(volatile long long*)&g_wait_cycle_limit; }
 
-// Returns false if the wait was abandoned (its own timeout, or another role's).  SLEEP_NS > 0 backs
-// off between polls: every poll is a shared-memory access, and shared-memory bandwidth is what the
-// MMA operand reads need, so roles that wait long (the epilogue warps) must not spin hot.
-template <int SLEEP_NS = 0>
+// Returns false if the wait was abandoned (its own timeout, or another role's).  strict: polls without suspending,
+// so that a budget of a few cycles (only a test sets one) is honoured to within one poll.
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                                  unsigned int* dev_status, int code) {
-  if (mbar_try_wait(bar, parity)) return true;
+                                                  unsigned int* dev_status, int code, bool strict = false) {
+  if (strict ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
   unsigned int spins = 0;
-  // the budget and the abort flag are looked at every 256 polls; with a budget below 2^20 cycles (only a
-  // test sets one) at every poll, so that such a budget is honoured to within one poll
-  const unsigned int check_mask = wait_cycle_limit() < (1ll << 20) ? 0u : 0xffu;
+  // the budget and the abort flag are looked at every 256 polls, with a small budget at every poll
+  const unsigned int check_mask = wait_cycle_limit() < WAIT_CYCLE_LIMIT_STRICT ? 0u : 0xffu;
   while (true) {
-    if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
-    if (mbar_try_wait(bar, parity)) return true;
+    if (!strict && mbar_try_wait(bar, parity)) return true;
     if ((++spins & check_mask) == 0) {
       if (*abort_flag) return false;
       if (clock64() - t0 > wait_cycle_limit()) {
@@ -106,7 +113,14 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
         return false;
       }
     }
+    if (strict && mbar_test_wait(bar, parity)) return true;
   }
+}
+// The same for a whole (converged) warp that acts on one answer: every lane polls, and no lane leaves alone when its
+// own wait is the one that gives up.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, unsigned int* dev_status, int code,
+                                               bool strict = false) {
+  return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, abort_flag, dev_status, code, strict)) != 0;
 }
 
 // ---------------------------------------------------------------- TMA

@@ -20,7 +20,7 @@
 //                        counts (48) and a third of sum_b G_b (32) in registers, the other two thirds of
 //                        sum_b G_b in the 128 tensor-memory columns the two accumulators leave free
 //   MEAN_TMEM, NT = 256: sum_b phi(G_b) in 128 registers per thread, sum_b G_b in
-//                        tensor memory beside ONE per-example accumulator, one issuer -- both outputs
+//                        tensor memory beside ONE per-example accumulator       -- both outputs
 //   MEAN_NONE, NT = 256: one running sum per thread (128 registers)               -- only sum_b phi(G_b) wanted
 //   MEAN_NORMS, NT = 256: no running sums; every example's sum of squares over the
 //                        tile is reduced and added to out_norms[b]                 -- per-example squared norms
@@ -29,14 +29,18 @@
 // update applied by the block that completes a tile's sums), F8 (e4m3 operands for the plain contraction).
 //
 // Warp roles per block (12 warps): 0 = TMA producer of the dY boxes, 2 = TMEM allocator, then TMA
-// producer of the X boxes, 1 and 3 = MMA issuers (leader block only), 4..11 = epilogue (warp w reads
-// TMEM lanes 32*(w%4)..+31, column half (w-4)/4).  One thread needs on the order of a hundred cycles
-// per TMA instruction, so the boxes are tall (BK tokens, 16 KiB for bf16) and split over two warps.
-// Two examples are in flight at once, one per issuer; the 512 TMEM columns hold 512/NT accumulators,
-// so the MMAs of later examples overlap the epilogue of earlier ones.  (MEAN_TMEM has one issuer and
-// one accumulator: while the epilogue drains it the producers keep filling the ring, and the issuer
-// then works the backlog off at full tensor rate, which absorbs the pause as long as the operand
-// supply, not the tensor pipe, is what bounds the example.)
+// producer of the X boxes, 1 = MMA issuer (leader block only), 3 idle, 4..11 = epilogue (warp w reads
+// TMEM lanes 32*(w%4)..+31, column half (w-4)/4).  The control warps run warp-uniform code in which
+// every lane waits and one elected lane issues: TMA, MMA and commit instructions take their operands
+// from uniform registers, and the same loops written for "lane 0 only" spent about 140 cycles per MMA,
+// 115 per TMA load and 550 per barrier probe behind queued MMAs, which bound every shape and needed two
+// issuers on alternate examples with half the operand ring each.  One issuer on the whole ring instead:
+// 128 x 512 tokens x 1024^2, both outputs 152 -> 127 us, three statistics 183 -> 134; 64 x 256 x 512 x 2048
+// 41.3 -> 36.3 us (cuBLAS' plain GEMM of the shape: 35.8); 1024 x 32 x 1024^2 170 -> 142.
+// The 512 TMEM columns hold 512/NT accumulators, so the MMAs of later examples overlap the epilogue of
+// earlier ones.  (MEAN_TMEM has one accumulator: while the epilogue drains it the producers keep filling
+// the ring, and the issuer then works the backlog off at full tensor rate, which absorbs the pause as long
+// as the operand supply, not the tensor pipe, is what bounds the example.)
 //
 // Barriers.  full[s] lives in the leader block: its producer posts the byte count of BOTH blocks'
 // loads, and the follower's TMA loads credit their bytes to it through the cluster window.
@@ -82,9 +86,7 @@ struct TcOperand {
   static_assert(!(TF32 && F8), "one operand type");
   static constexpr int ELEM_BYTES = TF32 ? 4 : (F8 ? 1 : 2);
   static constexpr int BOX_FEATS = 128 / ELEM_BYTES;            // features per 128-byte swizzle row: 64 | 32 | 128
-  // tokens per pipeline stage (one TMA box is BK tokens tall), chosen so that the ring has an EVEN
-  // number of stages: with two MMA issuers taking alternate stages every slot then always belongs
-  // to the same issuer (see the parity note at the issuer's wait).
+  // tokens per pipeline stage (one TMA box is BK tokens tall)
   static constexpr int BK = BK_;
   static constexpr int MMA_K = 32 / ELEM_BYTES;                 // tokens per MMA instruction: 16 | 8 | 32
   // Short sequences (the 32-token stages of the 256 x 128 tile): a stage holds TWO examples (the TMA box is
@@ -106,8 +108,7 @@ struct TcOperand {
   static constexpr int A_BYTES = A_BOXES * BOX_BYTES;           // 32 KiB (BK = 128) | 16 KiB
   static constexpr int B_BYTES = B_BOXES * B_BOX_BYTES;         // 16 KiB | 24 KiB (NT = 192)
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;         // per block: 48 KiB | 56 KiB | 32 KiB
-  static constexpr int STAGES = (tc_smem_budget(NT) / STAGE_BYTES) & ~1;   // 4 | 4 | 6 | 16 with 32-token stages
-  static_assert(STAGES % 2 == 0, "slots must alternate between the two issuers");
+  static constexpr int STAGES = tc_smem_budget(NT) / STAGE_BYTES;   // 4 | 4 | 6 | 8 with the grouped 32-token stages
   static constexpr int K_STEP_BYTES = MMA_K * 128;              // smem advance per MMA: 2048 | 1024
   static constexpr int B_K_STEP_BYTES = MMA_K * B_ROW_BYTES;
   static constexpr int ACC_BUFS = TC_TMEM_COLS / NT;            // 4 | 2 | 2 accumulators in tensor memory
@@ -224,19 +225,6 @@ __device__ __forceinline__ float phi_apply(float g) {
   }
   return g;
 }
-
-// The operand ring and the two issuers.  Issuer x owns the ring slots of parity x (a sub-ring of
-// STAGES / 2 slots with its own phase) and the examples x, x + 2, ... of the slice, so the two issuers
-// run independently of each other.  The producers fill the two sub-rings in alternation, one stage of
-// each in turn while both still have stages to fill: with equal sequence lengths that is stage kc of an
-// even example, stage kc of the next odd one, stage kc + 1 of the even one, ...; with unequal lengths
-// (packed batches) the issuer of a short example simply moves on to its next example earlier.  A parity
-// wait is only meaningful while the waiter is at most one phase away from the barrier; since a slot
-// only ever sees the stages of ONE sub-ring, in order, that always holds.
-struct RingCursor {
-  int e, kc, n;       // example (slice-local), stage within it, stages of this sub-ring filled so far
-  SeqGeom g;
-};
 
 // Zeroes the outputs of a split-batch launch.  The statistics kernel that follows is launched as a
 // programmatic dependent: it starts right away (it only touches the outputs in its very last step,
@@ -359,20 +347,18 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   constexpr bool NORMS = (MEAN == MEAN_NORMS);
   static_assert(!NORMS || (PHI == 1 && NT == 256), "per-example norms: squares on the 256 x 256 tile");
   static_assert(MEAN != MEAN_TMEM || (NT == 256 && PHI != 0), "the tensor-memory mean sits beside one 256-column accumulator");
-  static_assert(!RAGGED || (!TF32 && MEAN != MEAN_TMEM), "packed batches: 16-bit operands, two issuers");
+  static_assert(!RAGGED || (!TF32 && MEAN != MEAN_TMEM), "packed batches: 16-bit operands, several accumulators");
   static_assert(PHI != 3 || MEAN == MEAN_NONE, "the clipped sum is a statistic-only pass");
   static_assert(OPT != OPT_ADAM || (MEAN == MEAN_REGS && PHI == 1), "the Adam family consumes sum_b G_b and sum_b G_b^2");
   static_assert(OPT != OPT_SIGN || (MEAN == MEAN_NONE && PHI == 2), "MicroSignSGD consumes sum_b sign(G_b)");
   constexpr int STAGES = Op::STAGES, BK = Op::BK;
   constexpr int BOX_BYTES = Op::BOX_BYTES, A_BYTES = Op::A_BYTES, STAGE_BYTES = Op::STAGE_BYTES;
-  constexpr int ISSUERS = (MEAN == MEAN_TMEM) ? 1 : 2;
   constexpr int ACC_BUFS = (MEAN == MEAN_TMEM) ? 1 : Op::ACC_BUFS;
-  constexpr int BUFS_PER_ISSUER = ACC_BUFS / ISSUERS;     // 2 | 1
   // GROUP examples share a stage and a pair of accumulator barriers (short sequences): the unit of work of
-  // the producers, issuers and epilogue warps is then a group of GROUP consecutive examples
+  // the producers, the issuer and the epilogue warps is then a group of GROUP consecutive examples
   constexpr int GROUP = Op::GROUP;
-  constexpr int UNITS_PER_ISSUER = BUFS_PER_ISSUER / GROUP;      // accumulator units (of GROUP buffers) per issuer
-  static_assert(GROUP == 1 || ((MEAN == MEAN_REGS || MEAN == MEAN_REGS_SIGN) && !RAGGED && OPT == OPT_NONE && UNITS_PER_ISSUER == 1),
+  constexpr int UNITS = ACC_BUFS / GROUP;            // accumulator units (of GROUP buffers, one barrier pair each)
+  static_assert(GROUP == 1 || ((MEAN == MEAN_REGS || MEAN == MEAN_REGS_SIGN) && !RAGGED && OPT == OPT_NONE),
                 "grouped examples: the short-sequence variants of the two- and three-sum kernels");
   constexpr int MEAN_COL0 = 256;                    // first tensor-memory column of the MEAN_TMEM running sum
   constexpr int COLS = NT / 2;                      // accumulator columns per epilogue thread
@@ -389,7 +375,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(tail);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 8);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;      // the warp's number, uniform to the compiler too
   const uint32_t rank = cluster_ctarank();          // 0 = leader of the pair
   const int b_begin = (int)(((long long)p.B * blockIdx.z) / p.nsplit);
   const int b_end = (int)(((long long)p.B * (blockIdx.z + 1)) / p.nsplit);
@@ -413,109 +399,68 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   // branch of the role it applies to.
   if (warp < 4) {
     setmaxnreg_dec<Op::REGS_CONTROL>();
+    const bool strict = wait_cycle_limit() < WAIT_CYCLE_LIMIT_STRICT;
     if (warp == 0 || warp == 2) {
       // ---------------------------------------------------------- TMA producers (both blocks)
       // Warp 0 loads this block's rows of dY^T (and, in the leader, posts the stage's byte count);
-      // warp 2 loads this block's half of the X^T rows.  Both wait for the same "stage empty" phase and
-      // fill the two issuers' sub-rings in alternation (see RingCursor).
-      if (lane == 0) {
-        const bool is_a = (warp == 0);
-        int tile_m, tile_n;
-        tc_tile_of_block(p, rank, tile_m, tile_n);
-        const CUtensorMap* tmap = is_a ? &tmap_dy : &tmap_x;
-        const CUtensorMap* tmap_tail = is_a ? &tmap_dy_tail : &tmap_x_tail;
-        const int c0 = is_a ? tile_m * TC_TILE_M : tile_n * NT + (int)rank * Op::B_FEATS;   // first feature of this warp's boxes
-        const int n_boxes = is_a ? Op::A_BOXES : Op::B_BOXES;
-        const int box_feats = is_a ? Op::BOX_FEATS : Op::B_BOX_FEATS;
-        const int box_bytes = is_a ? BOX_BYTES : Op::B_BOX_BYTES;
+      // warp 2 loads this block's half of the X^T rows.  Both wait for the same "stage empty" phase.
+      const bool is_a = (warp == 0);
+      int tile_m, tile_n;
+      tc_tile_of_block(p, rank, tile_m, tile_n);
+      const CUtensorMap* tmap = is_a ? &tmap_dy : &tmap_x;
+      const CUtensorMap* tmap_tail = is_a ? &tmap_dy_tail : &tmap_x_tail;
+      const int c0 = is_a ? tile_m * TC_TILE_M : tile_n * NT + (int)rank * Op::B_FEATS;   // first feature of this warp's boxes
+      const int n_boxes = is_a ? Op::A_BOXES : Op::B_BOXES;
+      const int box_feats = is_a ? Op::BOX_FEATS : Op::B_BOX_FEATS;
+      const int box_bytes = is_a ? BOX_BYTES : Op::B_BOX_BYTES;
+      if (elect_one()) {
         prefetch_tensormap(tmap);
         if constexpr (RAGGED) prefetch_tensormap(tmap_tail);
-        constexpr int SUB = STAGES / ISSUERS;            // slots per sub-ring
-        auto start = [&](RingCursor& c, int x) {
-          c.e = x; c.kc = 0; c.n = 0;
-          if (c.e < nu) c.g = seq_geom<RAGGED>(p, b_begin + GROUP * c.e, BK);
-        };
-        // Fills the next stage of sub-ring x if it has one and its slot is free; never blocks, because a
-        // sub-ring may stay full for as long as the OTHER one has to be filled (its issuer waits for an
-        // accumulator that the epilogue frees only after the other issuer's example).
-        auto try_fill = [&](RingCursor& c, int x) -> bool {
-          if (c.e >= nu) return false;
-          const int s = ISSUERS * (c.n % SUB) + x;
-          const uint32_t ph = (uint32_t)(c.n / SUB) & 1u;
-          if (!mbar_test_wait(empty_bar(s), ph ^ 1u)) return false;
-          if (is_a && rank == 0) mbar_arrive_expect_tx(full_bar(s), 2 * STAGE_BYTES);     // both blocks' bytes
-          const uint32_t leader_full = map_to_cta(full_bar(s), 0);
-          const uint32_t dst = smem_base + s * STAGE_BYTES + (is_a ? 0 : A_BYTES);
-          if constexpr (RAGGED) {
-            const bool tail = c.kc >= c.g.nk_main;       // the zero-padded last partial group, from the side buffer
-            for (int g = 0; g < n_boxes; ++g)
-              tma_load_3d_pair(dst + g * box_bytes, tail ? tmap_tail : tmap, leader_full, c0 + g * box_feats,
-                               tail ? 0 : c.g.row0 + c.kc * BK, tail ? b_begin + c.e : 0);
-          } else {
+      }
+      int s = 0;
+      uint32_t ph = 1;
+      bool ok = true;
+      for (int e = 0; e < nu && ok; ++e) {
+        const SeqGeom g = seq_geom<RAGGED>(p, b_begin + GROUP * e, BK);
+        for (int kc = 0; kc < g.nk; ++kc) {
+          if (!mbar_wait_warp(empty_bar(s), ph, abort_flag, p.dev_status, TC_WAIT_EMPTY, strict)) { ok = false; break; }
+          if (elect_one()) {
+            if (is_a && rank == 0) mbar_arrive_expect_tx(full_bar(s), 2 * STAGE_BYTES);     // both blocks' bytes
+            const uint32_t leader_full = map_to_cta(full_bar(s), 0);
+            const uint32_t dst = smem_base + s * STAGE_BYTES + (is_a ? 0 : A_BYTES);
+            const bool tail = RAGGED && kc >= g.nk_main;       // the zero-padded last partial group, from the side buffer
+            const CUtensorMap* tm = tail ? tmap_tail : tmap;
+            const int c1 = tail ? 0 : g.row0 + kc * BK;
             // (grouped examples: the box is GROUP examples deep; past the batch's end it reads zeros)
-            for (int g = 0; g < n_boxes; ++g)
-              tma_load_3d_pair(dst + g * box_bytes, tmap, leader_full, c0 + g * box_feats, c.kc * BK, b_begin + GROUP * c.e);
+            const int c2 = RAGGED ? (tail ? b_begin + e : 0) : b_begin + GROUP * e;
+            for (int b = 0; b < n_boxes; ++b) tma_load_3d_pair(dst + b * box_bytes, tm, leader_full, c0 + b * box_feats, c1, c2);
           }
-          ++c.n;
-          if (++c.kc == c.g.nk) {
-            c.kc = 0;
-            c.e += ISSUERS;
-            if (c.e < nu) c.g = seq_geom<RAGGED>(p, b_begin + GROUP * c.e, BK);
-          }
-          return true;
-        };
-        RingCursor ca, cb;
-        start(ca, 0);
-        start(cb, ISSUERS == 2 ? 1 : nu);
-        long long t0 = -1;
-        unsigned int spins = 0;
-        while (ca.e < nu || cb.e < nu) {
-          bool progressed = try_fill(ca, 0);
-          if (ISSUERS == 2 && try_fill(cb, 1)) progressed = true;
-          if (progressed) { t0 = -1; spins = 0; continue; }
-          if ((++spins & (wait_cycle_limit() < (1ll << 20) ? 0u : 0xffu)) == 0) {      // bounded like every other wait
-            if (*abort_flag) break;
-            if (t0 < 0) t0 = clock64();
-            else if (clock64() - t0 > wait_cycle_limit()) {
-              *abort_flag = 1;
-              atomicCAS(p.dev_status, 0u, (unsigned int)TC_WAIT_EMPTY);
-              break;
-            }
-          }
+          __syncwarp();
+          if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
       }
-      __syncwarp();
-    } else if (rank == 0 && (warp == 1 || ISSUERS == 2)) {
-      // ---------------------------------------------------------- MMA issuers (leader block, warps 1 and 3)
-      // Two issuing threads (one per warp).  A barrier probe right after queuing MMAs costs the
-      // issuing thread a couple of hundred cycles; with two threads working on two different examples
-      // (own accumulators, alternate stages) one of them always has MMAs queued.  Issuer x owns
-      // examples x, x+2, ... of the slice and TMEM buffers x*BUFS_PER_ISSUER .. +BUFS_PER_ISSUER-1.
-      if (lane == 0) {
-        const int x = (warp == 1) ? 0 : 1;
-        // operand format code 0 is IEEE half under kind::f16 and e4m3 under kind::f8f6f4
-        const uint32_t idesc = (F8 || (!TF32 && p.half_operands)) ? make_idesc_half_mn_major(TC_PAIR_M, NT) : make_idesc_mn_major(TC_PAIR_M, NT, TF32);
-        bool ok = true;
-        uint32_t accumulate = 0;
-        constexpr int SUB = STAGES / ISSUERS;              // slots of this issuer's sub-ring
-        int i_local = 0;                                   // examples this issuer has started
-        int n_local = 0;                                   // stages this issuer has consumed
-        for (int e = x; e < nu && ok; e += ISSUERS, ++i_local) {
-          const SeqGeom sg = seq_geom<RAGGED>(p, b_begin + GROUP * e, BK);
-          const int grp = p.per_example ? i_local : 0;
-          const int buf = UNITS_PER_ISSUER * x + (grp % UNITS_PER_ISSUER);      // accumulator unit: GROUP buffers, one barrier pair
-          if (p.per_example || i_local == 0) {
-            const uint32_t acc_ph = (uint32_t)(grp / UNITS_PER_ISSUER) & 1u;
-            if (!mbar_wait_bounded(acc_empty_bar(buf), acc_ph ^ 1u, abort_flag, p.dev_status, TC_WAIT_ACC_EMPTY)) { ok = false; break; }
-            tc_fence_after();
-            accumulate = 0;
-          }
-          const uint32_t d_tmem = tmem_base + (uint32_t)(buf * GROUP * NT);
-          for (int kc = 0; kc < sg.nk; ++kc, ++n_local) {
-            const int s = ISSUERS * (n_local % SUB) + x;
-            const uint32_t ph = (uint32_t)(n_local / SUB) & 1u;
-            if (!mbar_wait_bounded(full_bar(s), ph, abort_flag, p.dev_status, TC_WAIT_FULL)) { ok = false; break; }
-            tc_fence_after();
+    } else if (rank == 0 && warp == 1) {
+      // ---------------------------------------------------------- MMA issuer (leader block)
+      // Unit e (an example, or GROUP of them) goes to accumulator unit e % UNITS.  A plain contraction (per_example == 0)
+      // alternates the same way but resets each accumulator only once, and the epilogue adds them up.
+      // operand format code 0 is IEEE half under kind::f16 and e4m3 under kind::f8f6f4
+      const uint32_t idesc = (F8 || (!TF32 && p.half_operands)) ? make_idesc_half_mn_major(TC_PAIR_M, NT) : make_idesc_mn_major(TC_PAIR_M, NT, TF32);
+      int s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int e = 0; e < nu && ok; ++e) {
+        const SeqGeom sg = seq_geom<RAGGED>(p, b_begin + GROUP * e, BK);
+        const int buf = e % UNITS;
+        if (p.per_example) {
+          if (!mbar_wait_warp(acc_empty_bar(buf), ((uint32_t)(e / UNITS) & 1u) ^ 1u, abort_flag, p.dev_status, TC_WAIT_ACC_EMPTY, strict)) break;
+          tc_fence_after();
+        }
+        const bool last_of_acc = p.per_example || e + UNITS >= nu;
+        const uint32_t d_tmem = tmem_base + (uint32_t)(buf * GROUP * NT);
+        for (int kc = 0; kc < sg.nk; ++kc) {
+          if (!mbar_wait_warp(full_bar(s), ph, abort_flag, p.dev_status, TC_WAIT_FULL, strict)) { ok = false; break; }
+          tc_fence_after();
+          if (elect_one()) {
             const uint32_t a_src = smem_base + s * STAGE_BYTES;
             const uint32_t b_src = a_src + A_BYTES;
             // tokens of this example in this stage: the rest of its whole 16-token groups, or the padded tail group
@@ -523,7 +468,8 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
 #pragma unroll
             for (int j = 0; j < GROUP; ++j) {
               // grouped examples: example j of the group sits BK tokens further in every box and has its own accumulator
-              if (GROUP > 1) { if (GROUP * e + j >= nb) break; accumulate = 0; }
+              if (GROUP > 1 && GROUP * e + j >= nb) break;
+              uint32_t accumulate = (kc > 0 || (!p.per_example && e >= UNITS)) ? 1u : 0u;
 #pragma unroll
               for (int k = 0; k < BK / Op::MMA_K; ++k) {
                 // rows past T are zero-filled by TMA; whole MMA steps past T are skipped
@@ -537,12 +483,12 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
               }
             }
             umma_commit_pair(empty_bar(s));                // stage reusable in both blocks once these MMAs retire
+            if (last_of_acc && kc == sg.nk - 1) umma_commit_pair(acc_full_bar(buf));   // accumulator complete, both blocks
           }
-          const bool last_of_group = p.per_example || (e + ISSUERS >= nu);
-          if (ok && last_of_group) umma_commit_pair(acc_full_bar(buf));   // accumulator complete, both blocks
+          __syncwarp();
+          if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
       }
-      __syncwarp();
     }
   } else {
     // ------------------------------------------------------------ epilogue (both blocks)
@@ -568,14 +514,12 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
 #pragma unroll
     for (int j = 0; j < N_MEAN; ++j) acc_mean[j] = 0.f;
     bool ok = true;
-    // per-example mode: one accumulator per example, in example order (example e -> issuer e&1).
-    // plain mode: one accumulator per issuer that had work.
-    const int n_acc = p.per_example ? nu : (nu >= ISSUERS ? ISSUERS : nu);
+    // per-example mode: one accumulator unit per example (or group), in order; plain mode: each accumulator once
+    const int n_acc = p.per_example ? nu : min(nu, UNITS);
     const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
     for (int a = 0; a < n_acc; ++a) {
-      const int x = a % ISSUERS, grp = p.per_example ? (a / ISSUERS) : 0;
-      const int buf = UNITS_PER_ISSUER * x + (grp % UNITS_PER_ISSUER);        // accumulator unit (GROUP buffers)
-      const uint32_t acc_ph = (uint32_t)(grp / UNITS_PER_ISSUER) & 1u;
+      const int buf = a % UNITS;
+      const uint32_t acc_ph = (uint32_t)(a / UNITS) & 1u;
       // PHI == 3: this example's clipping coefficient c_b = min(1, C / sqrt(N_b)); the load is issued before
       // the wait for the accumulator, which hides its latency.  N_b = 0 (a zero gradient) gives 1.
       uint64_t coef2 = 0;
@@ -587,7 +531,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       }
       // every lane polls, but the warp acts on one answer: the tensor-memory loads below are warp-wide
       // instructions, so no lane may leave the loop alone when its own wait is the one that gives up
-      if (!__all_sync(0xffffffffu, mbar_wait_bounded(acc_full_bar(buf), acc_ph, abort_flag, p.dev_status, TC_WAIT_ACC_FULL))) { ok = false; break; }
+      if (!mbar_wait_warp(acc_full_bar(buf), acc_ph, abort_flag, p.dev_status, TC_WAIT_ACC_FULL)) { ok = false; break; }
       tc_fence_after();
       const uint32_t taddr = lane_base + (uint32_t)(buf * GROUP * NT + h * COLS);
       if constexpr (MEAN == MEAN_TMEM) {
@@ -798,7 +742,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       auto send = [&](const CUtensorMap* tm, uint32_t first_panel) {
         fence_async_smem();
         __syncwarp();
-        if (lane == 0 && row0 < p.d_out) {
+        if (row0 < p.d_out && elect_one()) {
           if (p.nsplit > 1 && !p.accumulate) griddep_wait();       // the kernel that zeroes the outputs may still be running
           for (int c = 0; c < PANELS; ++c) {
             if (col0 + c * 32 < p.d_in) {
@@ -830,7 +774,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
           put_panel(first + (HYB_TMEM_COLS / 32) * 4096, &acc_mean[0]);
         } else if constexpr (MEAN == MEAN_TMEM) {
           // the panels are needed again: wait until TMA has read the first output out of them
-          if (lane == 0) bulk_wait_read_all();
+          if (elect_one()) bulk_wait_read_all();
           __syncwarp();
           first = stage_base;
           const uint32_t maddr = lane_base + (uint32_t)(MEAN_COL0 + h * COLS);
@@ -842,7 +786,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
           }
         } else if constexpr (KEEP_MEAN) {
           if constexpr (PANELS * 2 > WARP_PANELS) {           // PHI == 0 at NT = 256: one output only ever
-            if (lane == 0) bulk_wait_read_all();
+            if (elect_one()) bulk_wait_read_all();
             __syncwarp();
             first = stage_base;
           }
@@ -854,7 +798,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       if constexpr (TRIPLE) {
         // sum_b sign(G_b): the warp's staging area is in use, so wait until TMA has read it
         if (p.out_sign) {
-          if (lane == 0) bulk_wait_read_all();
+          if (elect_one()) bulk_wait_read_all();
           __syncwarp();
           const float nbf = (float)nb;
 #pragma unroll
@@ -867,7 +811,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
           send(&tmap_sign, stage_base);
         }
       }
-      if (lane == 0) bulk_wait_read_all();       // shared memory must outlive TMA's reads
+      if (elect_one()) bulk_wait_read_all();       // shared memory must outlive TMA's reads
     }
     __syncwarp();
     if constexpr (OPT != OPT_NONE) {
@@ -878,7 +822,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       // that gave up on a wait marks the counter so that nobody updates the parameters from incomplete sums.
       bool apply = ok && n_acc > 0;
       if (p.nsplit > 1) {
-        if (lane == 0) { bulk_wait_all(); __threadfence(); }
+        if (elect_one()) { bulk_wait_all(); __threadfence(); }
         __syncwarp();
         named_bar_sync(1, 256);                   // the eight epilogue warps; executed by all of them whatever `ok` says
         volatile int* last_flag = reinterpret_cast<volatile int*>(tail + 12);

@@ -95,7 +95,7 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 8);
   static_assert(8 * (2 * TOK_RAW_STAGES + 2 * TOK_COOKED_STAGES + 1) + 16 <= TC_BAR_BYTES, "barrier area too small");
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();          // 0 = leader of the pair
   int tile_m, tile_n;                               // 128-row tile of d_out, 256-column tile of d_in (banded tile order)
   {
@@ -123,49 +123,47 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp < 4) {
+    const bool strict = wait_cycle_limit() < WAIT_CYCLE_LIMIT_STRICT;
     if (warp == 0 || warp == 2) {
       // ---------------------------------------------------------- TMA producers (each block for itself)
-      if (lane == 0) {
-        const bool is_a = (warp == 0);
-        const CUtensorMap* tmap = is_a ? &tmap_dy : &tmap_x;
-        const int c0 = is_a ? tile_m * TC_TILE_M : tile_n * TOK_NT + (int)rank * (TOK_NT / 2);
-        prefetch_tensormap(tmap);
-        int s = 0; uint32_t ph = 0;
-        for (long long ch = c_begin; ch < c_end; ++ch) {
-          if (!mbar_wait_bounded(raw_empty(s), ph ^ 1u, abort_flag, p.dev_status, TOK_WAIT_RAW_EMPTY)) break;
+      const bool is_a = (warp == 0);
+      const CUtensorMap* tmap = is_a ? &tmap_dy : &tmap_x;
+      const int c0 = is_a ? tile_m * TC_TILE_M : tile_n * TOK_NT + (int)rank * (TOK_NT / 2);
+      if (elect_one()) prefetch_tensormap(tmap);
+      int s = 0; uint32_t ph = 1;
+      for (long long ch = c_begin; ch < c_end; ++ch) {
+        if (!mbar_wait_warp(raw_empty(s), ph, abort_flag, p.dev_status, TOK_WAIT_RAW_EMPTY, strict)) break;
+        if (elect_one()) {
           if (is_a) mbar_arrive_expect_tx(raw_full(s), TOK_RAW_STAGE);          // this block's four boxes
           const uint32_t dst = smem_base + s * TOK_RAW_STAGE + (is_a ? 0 : 2 * TOK_BOX_BYTES);
           tma_load_2d(dst, tmap, raw_full(s), c0, (int)(ch * TOK_BK));
           tma_load_2d(dst + TOK_BOX_BYTES, tmap, raw_full(s), c0 + 64, (int)(ch * TOK_BK));
-          if (++s == TOK_RAW_STAGES) { s = 0; ph ^= 1u; }
         }
+        __syncwarp();
+        if (++s == TOK_RAW_STAGES) { s = 0; ph ^= 1u; }
       }
-      __syncwarp();
     } else if (rank == 0 && warp == 1) {
       // ---------------------------------------------------------- MMA issuer (leader block)
-      if (lane == 0) {
-        constexpr uint32_t idesc = make_idesc_mn_major(TC_PAIR_M, TOK_NT, true);
-        int c = 0; uint32_t ph = 0;
-        uint32_t accumulate = 0;
-        bool ok = true;
-        for (long long ch = c_begin; ch < c_end; ++ch) {
-          if (!mbar_wait_bounded(cooked_full(c), ph, abort_flag, p.dev_status, TOK_WAIT_COOKED_FULL)) { ok = false; break; }
-          tc_fence_after();
+      constexpr uint32_t idesc = make_idesc_mn_major(TC_PAIR_M, TOK_NT, true);
+      int c = 0; uint32_t ph = 0;
+      for (long long ch = c_begin; ch < c_end; ++ch) {
+        if (!mbar_wait_warp(cooked_full(c), ph, abort_flag, p.dev_status, TOK_WAIT_COOKED_FULL, strict)) break;
+        tc_fence_after();
+        if (elect_one()) {
           const uint32_t a_src = cooked_base + c * TOK_COOKED_STAGE;
           const uint32_t b_src = a_src + TOK_COOKED_STAGE / 2;
 #pragma unroll
           for (int k = 0; k < TOK_BK / TOK_MMA_K; ++k) {       // rows past the end are zero: no need to skip them
             const uint64_t ad = make_smem_desc(a_src + k * TOK_MMA_K * 128, TOK_BOX_BYTES, 512u, 1u);
             const uint64_t bd = make_smem_desc(b_src + k * TOK_MMA_K * 128, TOK_BOX_BYTES, 512u, 1u);
-            umma_ss_pair<1>(tmem_base, ad, bd, idesc, accumulate);
-            accumulate = 1;
+            umma_ss_pair<1>(tmem_base, ad, bd, idesc, (k > 0 || ch > c_begin) ? 1u : 0u);
           }
           umma_commit_pair(cooked_empty(c));             // cooked stage reusable in both blocks once these MMAs retire
-          if (++c == TOK_COOKED_STAGES) { c = 0; ph ^= 1u; }
+          if (ch == c_end - 1) umma_commit_pair(acc_full);        // accumulator complete, both blocks
         }
-        if (ok) umma_commit_pair(acc_full);              // accumulator complete, both blocks
+        __syncwarp();
+        if (++c == TOK_COOKED_STAGES) { c = 0; ph ^= 1u; }
       }
-      __syncwarp();
     }
   } else {
     // ------------------------------------------------------------ converters, then write-out (both blocks)
@@ -180,8 +178,8 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         const int s = (int)(n % TOK_RAW_STAGES);          // raw and cooked rings advance together (same depth)
         const uint32_t ph = (uint32_t)(n / TOK_RAW_STAGES) & 1u;
         // every lane polls, the warp acts on one answer (what follows contains warp-wide instructions)
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded(raw_full(s), ph, abort_flag, p.dev_status, TOK_WAIT_RAW_FULL))) { ok = false; break; }
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded(cooked_empty(s), ph ^ 1u, abort_flag, p.dev_status, TOK_WAIT_COOKED_EMPTY))) { ok = false; break; }
+        if (!mbar_wait_warp(raw_full(s), ph, abort_flag, p.dev_status, TOK_WAIT_RAW_FULL)) { ok = false; break; }
+        if (!mbar_wait_warp(cooked_empty(s), ph ^ 1u, abort_flag, p.dev_status, TOK_WAIT_COOKED_EMPTY)) { ok = false; break; }
         const uint8_t* raw = smem_gen + s * TOK_RAW_STAGE;
         uint8_t* cooked = smem_gen + TOK_RAW_STAGES * TOK_RAW_STAGE + s * TOK_COOKED_STAGE;
         // A stage is 1024 16-byte chunks (4 boxes x 32 rows x 8 chunks of 8 features); chunk g of the
@@ -220,7 +218,7 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     }
     static_assert(TOK_RAW_STAGES == TOK_COOKED_STAGES && TOK_RAW_STAGES % 2 == 0, "the two rings advance together; each slot belongs to one converter group");
     ok = __all_sync(0xffffffffu, ok);
-    if (ok && w < 8) ok = __all_sync(0xffffffffu, mbar_wait_bounded(acc_full, 0, abort_flag, p.dev_status, TOK_WAIT_ACC));
+    if (ok && w < 8) ok = mbar_wait_warp(acc_full, 0, abort_flag, p.dev_status, TOK_WAIT_ACC);
     ok = __all_sync(0xffffffffu, ok);
     if (ok && w < 8) {
       // Write-out as in the statistics kernel: 32 rows x 128 columns per warp, staged in the idle ring
@@ -241,7 +239,7 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
       }
       fence_async_smem();
       __syncwarp();
-      if (lane == 0 && row0 < p.d_out) {
+      if (row0 < p.d_out && elect_one()) {
         if (p.nsplit > 1) griddep_wait();         // the kernel that zeroes the output may still be running
         for (int c = 0; c < 4; ++c) {
           if (col0 + c * 32 < p.d_in) {
