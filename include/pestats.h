@@ -71,9 +71,9 @@ typedef struct CUstream_st* pe_stream_t; /* a cudaStream_t */
  * either may be NULL to skip it (not both).  Products are exact in fp32 and accumulated in fp32.
  * B, T >= 0 (B == 0 or T == 0 writes zeros, and X, dY may then be NULL); d_in, d_out >= 1; B*T*max(d_in,d_out) < 2^40.
  * When the batch is split across thread blocks the outputs are zeroed first and every block adds its
- * partial tile with fp32 reduce-add bulk stores (the SIMT kernel: fp32 atomic adds), so the low bits
- * of out_mean / the square statistic may differ between runs; the sign statistic is always
- * exact-integer valued.
+ * partial tile with fp32 reduce-add bulk stores (the SIMT kernel adds up to eight slices in a fixed order
+ * and only the sums of more slices with fp32 atomics), so the low bits of out_mean / the square statistic
+ * may differ between runs; the sign statistic is always exact-integer valued.
  */
 pe_status_t pe_linear_stats(const void* X, const void* dY, int B, int T, int d_in, int d_out,
                             pe_phi_t phi, float* out_mean, float* out_stat, pe_stream_t stream);
@@ -315,7 +315,7 @@ pe_status_t microsignsgd_step(float* theta, void* theta_lp, float* m, const floa
  * of a tile applies the update.  If the workspace or an output is missing the batch is not split (one
  * block per tile walks all examples: correct, slower on layers with few tiles).  B >= 1, T >= 1; other
  * arguments as for pe_linear_stats and microadam_family_step.  The _f32 form takes fp32 inputs (SIMT
- * kernel, never splits the batch).  After PE_ERR_TIMEOUT the parameters of unfinished tiles are left as
+ * kernel; the slices of a split batch meet in shared memory, so it needs no outputs and no workspace for that).  After PE_ERR_TIMEOUT the parameters of unfinished tiles are left as
  * they were (the two-kernel sequence skips its update kernel while the device status word is set, i.e.
  * until pe_get_async_status has read and cleared it).
  * What the fusion buys is MEMORY, not time: with out_mean = out_stat = NULL no [d_out, d_in] statistic

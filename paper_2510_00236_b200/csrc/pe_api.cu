@@ -383,21 +383,97 @@ static pe_status_t launch_tc_norms(DeviceInfo* di, const void* X, const void* dY
   return launch_tc_inst<1, false, 256, MEAN_NORMS>(di, 11, mx, my, mx, mx, mx, p, dim3(2 * pairs_m * tiles_n, 1, ns), st);
 }
 
+// Tile and batch slices of a SIMT launch: the cheapest by an estimate in cycles of one block's walk, times the waves of
+// blocks.  A chunk of tokens costs the FMAs of the blocks that share an SM (128 lanes), at the rate the tile's shared-memory
+// reads leave, but not less than the latency of its barrier and loads.
+struct SimtPlan {
+  int tile, slices, cluster;      // tile: index into the four shapes, largest first
+};
+static SimtPlan plan_simt(DeviceInfo* di, int mode, int B, int T, int d_in, int d_out) {
+  static constexpr int rows[4] = {SimtTile84::ROWS, SimtTile44::ROWS, SimtTile22::ROWS, SimtTile11::ROWS};
+  static constexpr int cols[4] = {SimtTile84::COLS, SimtTile44::COLS, SimtTile22::COLS, SimtTile11::COLS};
+  static constexpr int kt[4] = {SimtTile84::KT, SimtTile44::KT, SimtTile22::KT, SimtTile11::KT};
+  static constexpr double fma_rate[4] = {0.8, 0.55, 0.25, 0.08};      // share of the FMA lanes kept busy
+  const long long units = mode == MODE_TOKEN ? (long long)B * T : B;  // what the slices divide: rows or examples
+  SimtPlan best = {0, 1, 1};
+  double best_cost = 1e300;
+  for (int k = 0; k < 4; ++k) {
+    const long long tiles = (long long)((d_in + cols[k] - 1) / cols[k]) * ((d_out + rows[k] - 1) / rows[k]);
+    for (int s = 1; s <= 64 && s <= units; s *= 2) {
+      const long long blocks = tiles * s, slots = 2ll * di->sm_count;
+      const long long waves = (blocks + slots - 1) / slots;
+      const double sharing = blocks > di->sm_count ? 2.0 : 1.0;
+      const long long per = (units + s - 1) / s;
+      const long long tokens = mode == MODE_TOKEN ? per : T;
+      const double chunks = (double)((tokens + kt[k] - 1) / kt[k]);
+      const double fma = (double)rows[k] * cols[k] * (double)((tokens + 7) / 8 * 8) / 128.0 / fma_rate[k] * sharing;
+      const double walk = (fma > 700.0 * chunks ? fma : 700.0 * chunks) + (mode == MODE_TOKEN ? 0.0 : rows[k] * cols[k] / 16.0);
+      const double cost = waves * (walk * (mode == MODE_TOKEN ? 1.0 : (double)per) + 3000.0 + 300.0 * s + (s > SIMT_MAX_CLUSTER ? 8000.0 : 0.0));
+      if (cost < best_cost * 0.98) { best_cost = cost; best = {k, s, s < SIMT_MAX_CLUSTER ? s : SIMT_MAX_CLUSTER}; }
+    }
+  }
+  if (mode == MODE_NORMS) best.cluster = 1;      // nothing is exchanged
+  return best;
+}
+
+template <typename TIn, int MODE, class Tile, int SUMS>
+static pe_status_t launch_simt_inst(const SimtPlan& plan, const TIn* X, const TIn* dY, int B, int T, int d_in, int d_out, int phi,
+                                    float* out_mean, float* out_stat, cudaStream_t st, bool accumulate, const SimtExtra& ex, const FusedOpt& opt) {
+  auto kernel = simt_stats_kernel<TIn, MODE, Tile, SUMS>;
+  constexpr int smem = (MODE == MODE_STATS ? Tile::smem_floats(SUMS) : (2 * Tile::CHUNK > Tile::ROWS * Tile::COLS ? 2 * Tile::CHUNK : Tile::ROWS * Tile::COLS)) * 4;
+  if constexpr (smem > 48 * 1024) {
+    int dev = 0;
+    static std::atomic<bool> attr_set[MAX_DEVICES];
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) { cudaGetLastError(); return PE_ERR_CUDA; }
+    if (!attr_set[dev].load(std::memory_order_acquire)) {       // (concurrent first calls set the same value)
+      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) { cudaGetLastError(); return PE_ERR_CUDA; }
+      attr_set[dev].store(true, std::memory_order_release);
+    }
+  }
+  // a group of four columns is one load when every row of the operand starts on such a boundary
+  const size_t group = 4 * sizeof(TIn);
+  const int vec_x = d_in % 4 == 0 && aligned(X, group) ? 1 : 0, vec_y = d_out % 4 == 0 && aligned(dY, group) ? 1 : 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((d_in + Tile::COLS - 1) / Tile::COLS, (d_out + Tile::ROWS - 1) / Tile::ROWS, plan.slices);
+  cfg.blockDim = dim3(SIMT_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  if (cfg.gridDim.y > 65535) return PE_ERR_DIM;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = 1; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = plan.cluster;
+  cfg.attrs = &attr; cfg.numAttrs = plan.cluster > 1 ? 1 : 0;
+  if (cudaLaunchKernelEx(&cfg, kernel, X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, accumulate ? 1 : 0, plan.cluster, vec_x, vec_y, ex, opt) != cudaSuccess) {
+    cudaGetLastError();
+    return PE_ERR_CUDA;
+  }
+  return check_launch();
+}
+
 template <typename TIn, int MODE>
 static pe_status_t launch_simt(DeviceInfo* di, const TIn* X, const TIn* dY, int B, int T, int d_in, int d_out, int phi,
                                float* out_mean, float* out_stat, cudaStream_t st, bool accumulate = false, SimtExtra ex = SimtExtra{},
                                const FusedOpt* opt = nullptr) {
-  const int tx = (d_in + SIMT_TILE - 1) / SIMT_TILE, ty = (d_out + SIMT_TILE - 1) / SIMT_TILE;
-  if (ty > 65535) return PE_ERR_DIM;
-  // a fused update needs the whole batch in one block (this kernel has no cross-block completion protocol)
-  const int ns = opt ? 1 : choose_nsplit((long long)tx * ty, B, T, di->sm_count * 3, 64);
-  if (ns > 1 && !accumulate) {
+  SimtPlan plan = plan_simt(di, MODE, B, T, d_in, d_out);
+  if (opt && plan.slices > SIMT_MAX_CLUSTER) plan.slices = SIMT_MAX_CLUSTER;      // a fused update needs the whole batch in one cluster
+  if ((d_out + SimtTile11::ROWS - 1) / SimtTile11::ROWS > 65535 && plan.tile > 0) plan.tile = 0;      // gridDim.y
+  if (MODE != MODE_NORMS && plan.slices > plan.cluster && !accumulate) {
     pe_status_t rc = zero_outputs(out_mean, out_stat, (size_t)d_in * d_out * sizeof(float), st);
     if (rc != PE_OK) return rc;
   }
-  simt_stats_kernel<TIn, MODE><<<dim3(tx, ty, ns), SIMT_THREADS, 0, st>>>(X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, accumulate ? 1 : 0, ex,
-                                                                            opt ? *opt : FusedOpt{});
-  return check_launch();
+  const FusedOpt o = opt ? *opt : FusedOpt{};
+  auto run = [&](auto tile) {
+    using Tile = decltype(tile);
+    if constexpr (MODE == MODE_STATS) {
+      if (out_mean || (opt && opt->kind == OPT_ADAM))
+        return launch_simt_inst<TIn, MODE, Tile, 2>(plan, X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, st, accumulate, ex, o);
+    }
+    return launch_simt_inst<TIn, MODE, Tile, 1>(plan, X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, st, accumulate, ex, o);
+  };
+  switch (plan.tile) {
+    case 0: return run(SimtTile84{});
+    case 1: return run(SimtTile44{});
+    case 2: return run(SimtTile22{});
+    default: return run(SimtTile11{});
+  }
 }
 
 // Side buffer of a packed batch: the zero-padded last partial 16-token group of every sequence, X's [B, 16, d_in]

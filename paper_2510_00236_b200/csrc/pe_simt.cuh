@@ -1,31 +1,52 @@
 // SIMT (CUDA-core) kernels for the per-example statistics: the fp32-input path and the path for
-// shapes the tensor-core kernel does not take.  One thread block owns a 64x64 tile of the
+// shapes the tensor-core kernel does not take.  A thread block owns a (16 TM) x (16 TN) tile of the
 // [d_out, d_in] output and walks over the examples of its slice of the batch; the per-example
 // gradient tile lives in registers and never reaches global memory.
+//
+// Bound: fp32 FMA (148 SMs x 128 lanes, 72 TFLOP/s) on layers that fill the chip, the latency of one load
+// and one reduction on those that do not.  Each thread forms TM x TN entries (two columns per packed FMA) from
+// 128-bit shared-memory reads; the next chunk of tokens is loaded into registers while the current one is
+// contracted, across example boundaries, and the two chunk buffers need one barrier per chunk.  The batch is
+// split over the blocks of a cluster, whose partial sums meet in shared memory: nothing is zeroed first, no
+// atomics, and the result does not depend on timing (more slices than a cluster holds fall back to atomics).
+// Measured, both outputs: 8 x 256 tokens x 1024 x 16384 46 TFLOP/s; 32 x 128 x 256 x 1024 157.8 -> 75 us, 8 x 16 x 64 x 64
+// 18.7 -> 11.4 us per call, against a 64 x 64 tile of 4 x 4 entries, one buffer and scalar reads.  Not faster: 8 x 8 entries
+// (one block per SM, 38 TFLOP/s), scalar FMAs (42), two tokens instead of two columns per packed FMA (spills, 30), 16-token
+// chunks (the barrier twice as often, 32 against 34 at 8 x 256 x 1024 x 2048).
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include "pe_optim.cuh"
+#include "pe_sm100.cuh"
 
 namespace pe {
 
-constexpr int SIMT_TILE = 64;   // output tile edge
-constexpr int SIMT_TK = 16;     // tokens staged per step
-constexpr int SIMT_THREADS = 256;
+constexpr int SIMT_THREADS = 256;       // 16 x 16 threads
+constexpr int SIMT_MAX_CLUSTER = 8;     // batch slices whose partial sums meet in shared memory
 
 enum : int { MODE_STATS = 0, MODE_TOKEN = 1, MODE_NORMS = 2 };
 
-__device__ __forceinline__ float to_f32(float v) { return v; }
-__device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
-
-// phi: 0 identity, 1 square, 2 sign, 3 the clipping scale coef * g
-__device__ __forceinline__ float apply_phi(float g, int phi, float coef) {
-  if (phi == 1) return g * g;
-  if (phi == 2) return (g > 0.f ? 1.f : 0.f) - (g < 0.f ? 1.f : 0.f);
-  if (phi == 3) return coef * g;
-  return g;
-}
+// Tile shapes.  TM x TN entries per thread; KT tokens per chunk.  The large tile has the most FMAs per shared-memory
+// read, the small ones spread a small layer over the chip.
+template <int TM_, int TN_, int KT_>
+struct SimtTile {
+  static constexpr int TM = TM_, TN = TN_, KT = KT_;
+  static constexpr int ROWS = 16 * TM, COLS = 16 * TN;
+  static constexpr int CHUNK = KT * (ROWS + COLS);               // floats of one chunk: dY part, then X part
+  static constexpr int YV = KT * ROWS / 4 / SIMT_THREADS, XV = KT * COLS / 4 / SIMT_THREADS;   // 4-column groups per thread
+  static_assert(YV * 4 * SIMT_THREADS == KT * ROWS && XV * 4 * SIMT_THREADS == KT * COLS, "whole groups per thread");
+  // the largest tile keeps its running sums in shared memory (64 registers of sums beside 32 of G_b would leave one block per SM)
+  static constexpr bool SUMS_IN_SMEM = TM * TN > 16;
+  // the chunk buffers; the sums' exchange at the end lies behind them where the sums live there, on top of them otherwise
+  static constexpr int smem_floats(int sums) {
+    return SUMS_IN_SMEM ? 2 * CHUNK + sums * ROWS * COLS : (2 * CHUNK > sums * ROWS * COLS ? 2 * CHUNK : sums * ROWS * COLS);
+  }
+};
+using SimtTile84 = SimtTile<8, 4, 32>;
+using SimtTile44 = SimtTile<4, 4, 16>;
+using SimtTile22 = SimtTile<2, 2, 32>;
+using SimtTile11 = SimtTile<1, 1, 64>;
 
 // What a packed batch or a clipped sum adds to the plain call; all NULL / 0 otherwise.
 struct SimtExtra {
@@ -35,132 +56,319 @@ struct SimtExtra {
   float clip_norm;
 };
 
+// phi: 0 identity, 1 square, 2 sign, 3 the clipping scale coef * g
+__device__ __forceinline__ float apply_phi(float g, int phi, float coef) {
+  if (phi == 1) return g * g;
+  if (phi == 2) return (g > 0.f ? 1.f : 0.f) - (g < 0.f ? 1.f : 0.f);
+  if (phi == 3) return coef * g;
+  return g;
+}
+
+// Columns c .. c+3 of a row of `width` elements.  vec: a group inside the row is one aligned load.
+__device__ __forceinline__ float4 load_group(const float* row, int c, int width, bool vec) {
+  if (vec && c + 3 < width) return __ldg(reinterpret_cast<const float4*>(row + c));
+  float v[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v[j] = c + j < width ? __ldg(row + c + j) : 0.f;
+  return make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ float4 load_group(const __nv_bfloat16* row, int c, int width, bool vec) {
+  uint32_t w[4];
+  if (vec && c + 3 < width) {
+    const uint2 u = __ldg(reinterpret_cast<const uint2*>(row + c));
+    w[0] = u.x << 16; w[1] = u.x & 0xFFFF0000u; w[2] = u.y << 16; w[3] = u.y & 0xFFFF0000u;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      w[j] = c + j < width ? (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(row + c + j)) << 16 : 0u;
+  }
+  return make_float4(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]), __uint_as_float(w[3]));
+}
+
+// A thread's N operands of one token: N = 1, 2 or 4 consecutive floats, 8 as two groups of four, 64 floats apart.
+template <int N>
+__device__ __forceinline__ void lds_vec(const float* p, float (&v)[N]) {
+  if constexpr (N == 1) {
+    v[0] = *p;
+  } else if constexpr (N == 2) {
+    const float2 t = *reinterpret_cast<const float2*>(p);
+    v[0] = t.x; v[1] = t.y;
+  } else {
+#pragma unroll
+    for (int h = 0; h < N / 4; ++h) {
+      const float4 t = *reinterpret_cast<const float4*>(p + 64 * h);
+      v[4 * h] = t.x; v[4 * h + 1] = t.y; v[4 * h + 2] = t.z; v[4 * h + 3] = t.w;
+    }
+  }
+}
+// Tile row (column) of entry j of a thread's N: the layout lds_vec reads.
+template <int N>
+__device__ __forceinline__ int micro_index(int thread, int j) { return N <= 4 ? thread * N + j : thread * 4 + (j & 3) + 64 * (j >> 2); }
+
 // MODE_STATS: out_mean = sum_b G_b, out_stat = sum_b phi(G_b)         (Section 2.3, Eq. (2))
 // MODE_TOKEN: out_stat = sum_{b,t} dY^2 X^2; operands are squared as they are staged and the
 //             accumulator is never reset between examples             (Section 2.3, per-token form)
 // MODE_NORMS: out_stat is a [B] array, zero on entry; every tile adds its share of ||G_b||_F^2 to
 //             out_stat[b] (Section 2.3, per-example squared norms); no [d_out, d_in] output
-// gridDim = (ceil(d_in/64), ceil(d_out/64), nsplit); block z handles examples [z*B/nsplit, (z+1)*B/nsplit).
-// With nsplit > 1 the outputs must be zero on entry and partial sums are added atomically; with
-// accumulate != 0 the results are added to whatever the outputs hold.  opt.kind != 0 (nsplit == 1 only):
-// the block also applies the parameter update to its tile (phi must then be square for the Adam family,
+// gridDim = (ceil(d_in/COLS), ceil(d_out/ROWS), slices) in clusters of (1, 1, cluster), cluster a power of two that divides
+// slices; slice z handles examples [z*B/slices, (z+1)*B/slices), or that share of the B*T rows (MODE_TOKEN).  With more
+// slices than one cluster the outputs must be zero on entry and the clusters' sums are added atomically; with
+// accumulate != 0 the results are added to whatever the outputs hold.  opt.kind != 0 (one cluster only): the block that
+// ends up with an entry's sums also applies the parameter update (phi must then be square for the Adam family,
 // sign for MicroSignSGD); out_mean / out_stat may then be NULL.
-template <typename TIn, int MODE>
-__global__ void __launch_bounds__(SIMT_THREADS)
+// SUMS: running sums per entry: 2 = sum_b phi(G_b) and sum_b G_b, 1 = the former alone (or the contraction of MODE_TOKEN).
+template <typename TIn, int MODE, class Tile, int SUMS>
+__global__ void __launch_bounds__(SIMT_THREADS, 2)
 simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, int T, int d_in, int d_out,
-                  int phi, float* __restrict__ out_mean, float* __restrict__ out_stat, int accumulate, SimtExtra ex, FusedOpt opt) {
-  __shared__ float sY[SIMT_TK][SIMT_TILE];
-  __shared__ float sX[SIMT_TK][SIMT_TILE];
+                  int phi, float* __restrict__ out_mean, float* __restrict__ out_stat, int accumulate, int cluster, int vec_x, int vec_y,
+                  SimtExtra ex, FusedOpt opt) {
+  constexpr int TM = Tile::TM, TN = Tile::TN, KT = Tile::KT, ROWS = Tile::ROWS, COLS = Tile::COLS;
+  constexpr bool IN_SMEM = Tile::SUMS_IN_SMEM && MODE == MODE_STATS;
+  extern __shared__ __align__(16) float simt_smem[];
+  // a warp is 4 x 8 threads of the 16 x 16: four distinct operands of dY and eight of X per shared-memory read
+  const int tx = (threadIdx.x & 7) | ((threadIdx.x >> 2) & 8), ty = ((threadIdx.x >> 3) & 3) | ((threadIdx.x >> 6) << 2);
+  const int i0 = blockIdx.x * COLS, o0 = blockIdx.y * ROWS;
+  const int slices = gridDim.z;
 
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int i0 = blockIdx.x * SIMT_TILE, o0 = blockIdx.y * SIMT_TILE;
-  const int nsplit = gridDim.z;
-  const int b_begin = (int)(((long long)B * blockIdx.z) / nsplit);
-  const int b_end = (int)(((long long)B * (blockIdx.z + 1)) / nsplit);
-
-  float g[4][4], acc_stat[4][4], acc_mean[4][4];
+  // g: this thread's entries of G_b.  Running sums ([0] = the statistic, [1] = sum_b G_b) in registers, or, IN_SMEM, in a
+  // thread-private arrangement of shared memory (one float4 per thread, 256 threads side by side: no bank conflicts).
+  float g[TM][TN];
+  float sum[IN_SMEM ? 1 : SUMS][TM][TN];
+  float* const smem_sums = simt_smem + 2 * Tile::CHUNK;
+  auto slot = [&](int s, int r, int c4) { return reinterpret_cast<float4*>(smem_sums) + ((s * TM + r) * (TN / 4) + c4) * SIMT_THREADS + threadIdx.x; };
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < TM; ++r) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) g[r][c] = acc_stat[r][c] = acc_mean[r][c] = 0.f;
-
-  for (int b = b_begin; b < b_end; ++b) {
-    if (MODE == MODE_STATS || MODE == MODE_NORMS) {
+    for (int c = 0; c < TN; ++c) g[r][c] = 0.f;
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+    for (int s = 0; s < SUMS; ++s) {
+      if constexpr (IN_SMEM) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) g[r][c] = 0.f;
+        for (int c4 = 0; c4 < TN / 4; ++c4) *slot(s, r, c4) = make_float4(0.f, 0.f, 0.f, 0.f);
+      } else {
+#pragma unroll
+        for (int c = 0; c < TN; ++c) sum[s][r][c] = 0.f;
+      }
     }
-    long long row0 = (long long)b * T;
-    int Tb = T;
+  }
+
+  // The walk: example b, tokens t .. t+KT-1 of it.  MODE_TOKEN: the slice's rows, in "examples" of 2^20 rows.
+  constexpr int TOKEN_RUN = 1 << 20;
+  int b = 0, b_end = 0, t = 0, Tb = 0;
+  long long row0 = 0, slice_row0 = 0, slice_rows = 0;
+  auto open_example = [&]() {
+    if (MODE == MODE_TOKEN) {
+      row0 = slice_row0 + (long long)b * TOKEN_RUN;
+      const long long rest = slice_rows - (long long)b * TOKEN_RUN;
+      Tb = rest < TOKEN_RUN ? (int)rest : TOKEN_RUN;
+      return;
+    }
+    row0 = (long long)b * T;
+    Tb = T;
     if (ex.seq_offsets) {            // packed batch: this example's own token range, clamped to the tensor
       const long long r0 = ex.seq_offsets[b], r1 = ex.seq_offsets[b + 1];
       row0 = r0 < 0 ? 0 : r0;
       const long long end = r1 > ex.total_rows ? ex.total_rows : r1;
       Tb = end > row0 ? (int)(end - row0) : 0;
     }
-    float coef = 1.f;
-    if (phi == 3) {
-      const float nrm = sqrtf(ex.sq_norms[b]);
-      coef = nrm > ex.clip_norm ? ex.clip_norm / nrm : 1.f;
+  };
+  if (MODE == MODE_TOKEN) {
+    const long long rows = (long long)B * T;
+    slice_row0 = rows * blockIdx.z / slices;
+    slice_rows = rows * (blockIdx.z + 1) / slices - slice_row0;
+    b_end = (int)((slice_rows + TOKEN_RUN - 1) / TOKEN_RUN);
+  } else {
+    b = (int)(((long long)B * blockIdx.z) / slices);
+    b_end = (int)(((long long)B * (blockIdx.z + 1)) / slices);
+  }
+  if (b < b_end) open_example();
+
+  float4 sy[Tile::YV], sx[Tile::XV];
+  auto load_chunk = [&]() {            // zero past the example's end and past the matrix edge
+#pragma unroll
+    for (int k = 0; k < Tile::YV; ++k) {
+      const int v = threadIdx.x + k * SIMT_THREADS, tt = t + v / (ROWS / 4), c = o0 + 4 * (v % (ROWS / 4));
+      sy[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (tt < Tb && c < d_out) sy[k] = load_group(dY + (size_t)(row0 + tt) * d_out, c, d_out, vec_y != 0);
     }
-    const TIn* Xb = X + (size_t)row0 * d_in;
-    const TIn* Yb = dY + (size_t)row0 * d_out;
-    for (int t0 = 0; t0 < Tb; t0 += SIMT_TK) {
-      // stage SIMT_TK tokens of both operands, zero-filling past T and past the matrix edge
 #pragma unroll
-      for (int k = 0; k < (SIMT_TK * SIMT_TILE) / SIMT_THREADS; ++k) {
-        int idx = threadIdx.x + k * SIMT_THREADS;
-        int tt = idx / SIMT_TILE, cc = idx % SIMT_TILE;
-        int t = t0 + tt;
-        float xv = 0.f, yv = 0.f;
-        if (t < Tb) {
-          if (i0 + cc < d_in) xv = to_f32(Xb[(size_t)t * d_in + i0 + cc]);
-          if (o0 + cc < d_out) yv = to_f32(Yb[(size_t)t * d_out + o0 + cc]);
-        }
-        if (MODE == MODE_TOKEN) { xv *= xv; yv *= yv; }
-        sX[tt][cc] = xv;
-        sY[tt][cc] = yv;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int k = 0; k < SIMT_TK; ++k) {
-        float y[4], x[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) y[r] = sY[k][ty + 16 * r];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) x[c] = sX[k][tx + 16 * c];
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) g[r][c] = fmaf(y[r], x[c], g[r][c]);
-      }
-      __syncthreads();
+    for (int k = 0; k < Tile::XV; ++k) {
+      const int v = threadIdx.x + k * SIMT_THREADS, tt = t + v / (COLS / 4), c = i0 + 4 * (v % (COLS / 4));
+      sx[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (tt < Tb && c < d_in) sx[k] = load_group(X + (size_t)(row0 + tt) * d_in, c, d_in, vec_x != 0);
     }
-    if (MODE == MODE_NORMS) {
+  };
+  auto put = [&](float* at, float4 v) {
+    *reinterpret_cast<float4*>(at) = MODE == MODE_TOKEN ? make_float4(v.x * v.x, v.y * v.y, v.z * v.z, v.w * v.w) : v;
+  };
+  // end of example eb: phi and the running sums
+  auto fold = [&](int eb) {
+    if constexpr (MODE == MODE_NORMS) {
       float s = 0.f;            // entries outside the matrix are exact zeros (their operands were zero-filled)
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < TM; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) s = fmaf(g[r][c], g[r][c], s);
+        for (int c = 0; c < TN; ++c) s = fmaf(g[r][c], g[r][c], s);
 #pragma unroll
       for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-      if ((threadIdx.x & 31) == 0) atomicAdd(out_stat + b, s);
-    }
-    if (MODE == MODE_STATS) {
+      if ((threadIdx.x & 31) == 0) atomicAdd(out_stat + eb, s);
+    } else if constexpr (MODE == MODE_STATS) {
+      float coef = 1.f;
+      if (phi == 3) {
+        const float nrm = sqrtf(ex.sq_norms[eb]);
+        coef = nrm > ex.clip_norm ? ex.clip_norm / nrm : 1.f;
+      }
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < TM; ++r) {
+        if constexpr (IN_SMEM) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          acc_mean[r][c] += g[r][c];
-          acc_stat[r][c] += apply_phi(g[r][c], phi, coef);
+          for (int c4 = 0; c4 < TN / 4; ++c4) {
+            float v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = g[r][4 * c4 + j];
+            float4 s = *slot(0, r, c4);
+            s.x += apply_phi(v[0], phi, coef); s.y += apply_phi(v[1], phi, coef);
+            s.z += apply_phi(v[2], phi, coef); s.w += apply_phi(v[3], phi, coef);
+            *slot(0, r, c4) = s;
+            if constexpr (SUMS == 2) {
+              float4 m = *slot(1, r, c4);
+              m.x += v[0]; m.y += v[1]; m.z += v[2]; m.w += v[3];
+              *slot(1, r, c4) = m;
+            }
+          }
+        } else {
+#pragma unroll
+          for (int c = 0; c < TN; ++c) {
+            const float v = g[r][c];
+            sum[0][r][c] += apply_phi(v, phi, coef);
+            if constexpr (SUMS == 2) sum[1][r][c] += v;
+          }
         }
+      }
     }
+    if constexpr (MODE != MODE_TOKEN) {
+#pragma unroll
+      for (int r = 0; r < TM; ++r)
+#pragma unroll
+        for (int c = 0; c < TN; ++c) g[r][c] = 0.f;
+    }
+  };
+
+  bool more = b < b_end;
+  if (more) load_chunk();
+  for (int buf = 0; more; buf ^= 1) {
+    const int left = Tb - t, cur_b = b;            // tokens of this example from this chunk on
+    float* const y = simt_smem + buf * Tile::CHUNK;
+    float* const x = y + KT * ROWS;
+#pragma unroll
+    for (int k = 0; k < Tile::YV; ++k) put(y + 4 * (threadIdx.x + k * SIMT_THREADS), sy[k]);
+#pragma unroll
+    for (int k = 0; k < Tile::XV; ++k) put(x + 4 * (threadIdx.x + k * SIMT_THREADS), sx[k]);
+    __syncthreads();           // a buffer is written again two chunks later, behind the barrier that follows its last reads
+    // the next chunk's loads are in flight during this one's arithmetic
+    t += KT;
+    const bool ends = t >= Tb;
+    if (ends) {
+      t = 0;
+      if (++b < b_end) open_example();
+    }
+    more = b < b_end;
+    if (more) load_chunk();
+    // tokens past the example's end are zero: whole groups of 8 of them are skipped
+#pragma unroll 1
+    for (int k0 = 0; k0 < KT && k0 < left; k0 += 8) {
+#pragma unroll
+      for (int kk = 0; kk < 8; ++kk) {
+        float yv[TM], xv[TN];
+        lds_vec<TM>(y + (k0 + kk) * ROWS + (TM < 4 ? TM : 4) * ty, yv);
+        lds_vec<TN>(x + (k0 + kk) * COLS + (TN < 4 ? TN : 4) * tx, xv);
+#pragma unroll
+        for (int r = 0; r < TM; ++r) {
+          if constexpr (TN >= 2) {
+            const uint64_t y2 = sm100::f32x2_pack(yv[r], yv[r]);
+#pragma unroll
+            for (int c = 0; c < TN; c += 2) {
+              const uint64_t a = sm100::f32x2_fma(y2, sm100::f32x2_pack(xv[c], xv[c + 1]), sm100::f32x2_pack(g[r][c], g[r][c + 1]));
+              sm100::f32x2_unpack(a, g[r][c], g[r][c + 1]);
+            }
+          } else {
+            g[r][0] = fmaf(yv[r], xv[0], g[r][0]);
+          }
+        }
+      }
+    }
+    if (ends) fold(cur_b);
   }
 
   if constexpr (MODE != MODE_NORMS) {       // MODE_NORMS has no [d_out, d_in] output
+    // Every block lays its partial sums out in its shared memory as [sum][row][column]; each block of the cluster
+    // then adds up its share of the rows over all of them, in slice order, and writes the result.
+    float* const xch = IN_SMEM ? smem_sums : simt_smem;
+    if constexpr (IN_SMEM) {
+      // the thread-private slots are overwritten by their own rearrangement: one sum at a time, through registers
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      int o = o0 + ty + 16 * r;
-      if (o >= d_out) continue;
+      for (int s = 0; s < SUMS; ++s) {
+        float4 v[TM][TN / 4];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        int i = i0 + tx + 16 * c;
-        if (i >= d_in) continue;
-        size_t at = (size_t)o * d_in + i;
-        float vs = (MODE == MODE_TOKEN) ? g[r][c] : acc_stat[r][c];
-        if (nsplit == 1 && !accumulate) {
-          if (out_stat) out_stat[at] = vs;
-          if (MODE == MODE_STATS && out_mean) out_mean[at] = acc_mean[r][c];
-          // the parameter update of Algorithm 1 / Section 3.1, applied where the sums over the whole batch are
-          if (MODE == MODE_STATS && opt.kind == OPT_ADAM) fused_update_one<OPT_ADAM>(opt, (long long)at, acc_mean[r][c], vs);
-          if (MODE == MODE_STATS && opt.kind == OPT_SIGN) fused_update_one<OPT_SIGN>(opt, (long long)at, vs, 0.f);
+        for (int r = 0; r < TM; ++r)
+#pragma unroll
+          for (int c4 = 0; c4 < TN / 4; ++c4) v[r][c4] = *slot(s, r, c4);
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < TM; ++r)
+#pragma unroll
+          for (int c4 = 0; c4 < TN / 4; ++c4)
+            *reinterpret_cast<float4*>(xch + (s * ROWS + micro_index<TM>(ty, r)) * COLS + micro_index<TN>(tx, 4 * c4)) = v[r][c4];
+      }
+    } else {
+      __syncthreads();         // the chunk buffers are idle from here on
+#pragma unroll
+      for (int s = 0; s < SUMS; ++s)
+#pragma unroll
+        for (int r = 0; r < TM; ++r)
+#pragma unroll
+          for (int c = 0; c < TN; ++c)
+            xch[(s * ROWS + micro_index<TM>(ty, r)) * COLS + micro_index<TN>(tx, c)] = MODE == MODE_TOKEN ? g[r][c] : sum[s][r][c];
+    }
+    if (cluster > 1) sm100::cluster_sync_all();
+    else __syncthreads();
+    const int rank = cluster > 1 ? (int)sm100::cluster_ctarank() : 0;
+    const bool add = slices > cluster || accumulate;
+    const uint32_t local = sm100::smem_u32(xch);
+    const int share = ROWS / cluster;         // rows this block finishes
+    for (int e = threadIdx.x; e < share * COLS; e += SIMT_THREADS) {
+      const int r = rank * share + e / COLS, c = e % COLS;
+      const int o = o0 + r, i = i0 + c;
+      if (o >= d_out || i >= d_in) continue;
+      float v[SUMS];
+#pragma unroll
+      for (int s = 0; s < SUMS; ++s) {
+        const int at = (s * ROWS + r) * COLS + c;
+        if (cluster == 1) {
+          v[s] = xch[at];
         } else {
-          if (out_stat) atomicAdd(out_stat + at, vs);
-          if (MODE == MODE_STATS && out_mean) atomicAdd(out_mean + at, acc_mean[r][c]);
+          float q[SIMT_MAX_CLUSTER];
+#pragma unroll
+          for (int k = 0; k < SIMT_MAX_CLUSTER; ++k) q[k] = k < cluster ? sm100::ld_shared_cluster(sm100::map_to_cta(local + 4u * (uint32_t)at, (uint32_t)k)) : 0.f;
+          float a = q[0];
+#pragma unroll
+          for (int k = 1; k < SIMT_MAX_CLUSTER; ++k) a += q[k];
+          v[s] = a;
         }
       }
+      const size_t at = (size_t)o * d_in + i;
+      if (!add) {
+        if (out_stat) out_stat[at] = v[0];
+        if (SUMS == 2 && out_mean) out_mean[at] = v[SUMS - 1];
+        // the parameter update of Algorithm 1 / Section 3.1, applied where the sums over the whole batch are
+        if (MODE == MODE_STATS && SUMS == 2 && opt.kind == OPT_ADAM) fused_update_one<OPT_ADAM>(opt, (long long)at, v[SUMS - 1], v[0]);
+        if (MODE == MODE_STATS && SUMS == 1 && opt.kind == OPT_SIGN) fused_update_one<OPT_SIGN>(opt, (long long)at, v[0], 0.f);
+      } else {
+        if (out_stat) atomicAdd(out_stat + at, v[0]);
+        if (SUMS == 2 && out_mean) atomicAdd(out_mean + at, v[SUMS - 1]);
+      }
     }
+    if (cluster > 1) sm100::cluster_sync_all();          // shared memory must outlive the peers' reads
   }
 }
 

@@ -49,6 +49,27 @@ def test_bf16_shape_not_multiple_of_8_takes_simt_automatically():
     assert e.value.status == 4        # PE_ERR_UNSUPPORTED_SHAPE
 
 
+# Every tile shape of the kernel (128 x 64 down to 16 x 16, chosen by size), edges one past and one short of a tile, rows
+# that are no 16-byte groups, tokens one past and one short of a chunk, batches split over 1, 2, 4 and 8 blocks of a cluster
+# and over more slices than a cluster holds, a single example, a single token.
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B,T,d_in,d_out", [(2, 33, 1028, 1028), (1, 31, 513, 1023), (3, 17, 257, 383), (8, 16, 64, 64), (5, 65, 63, 129),
+                                            (2, 129, 31, 33), (700, 3, 17, 15), (40, 1, 16, 16), (1, 200, 4, 2), (13, 64, 130, 66)])
+def test_simt_tiles_slices_and_edges(B, T, d_in, d_out, dtype):
+    pe.pe_set_path(pe.PATH_SIMT)
+    li = inputs.gaussian_layer(B, T, d_in, d_out, dtype=dtype, seed=300 + B + T, device=DEV)
+    # fp32 sums of at most B*T = 2600 products: a random walk of 2^-24 roundings, sqrt(2600) * 6e-8 = 3e-6 in the 2-norm
+    rep = check_all(li, phis=("identity", "square", "sign"), tol=3e-6)
+    assert rep["square_err"] <= 3e-6
+    mean, stat = gpu_stats(li, "square")
+    if B < 700:       # up to one cluster of slices the order of the sums is fixed
+        again = gpu_stats(li, "square")
+        assert np.array_equal(mean, again[0]) and np.array_equal(stat, again[1])
+    only = torch.full((d_out, d_in), float("nan"), device=DEV)
+    (pe.pe_linear_stats if dtype == torch.bfloat16 else pe.pe_linear_stats_f32)(li.X, li.dY, "square", None, only)
+    assert np.allclose(only.cpu().numpy(), stat, rtol=1e-5, atol=0)      # another order of at most 64 partial sums of positive terms
+
+
 def test_empty_batch_and_empty_sequence_give_zeros():
     for B, T in ((0, 5), (3, 0)):
         X = torch.zeros((B, T, 16), dtype=torch.float32, device=DEV)
