@@ -130,10 +130,6 @@ def _check(fn: str, status: int):
         raise PestatsError(fn, status, pe_status_string(status))
 
 
-def _stream(t: torch.Tensor) -> int:
-    return torch.cuda.current_stream(t.device).cuda_stream
-
-
 def _ptr(t):
     return None if t is None else t.data_ptr()
 
@@ -142,25 +138,42 @@ def _phi(phi) -> int:
     return _PHI_NAMES[phi] if isinstance(phi, str) else int(phi)
 
 
-def _dev_ctx(t: torch.Tensor):
+# The two lookups every call makes, in their cheapest form (0.1 us each): torch.cuda.current_stream builds a Stream object
+# (2.3 us) and torch.cuda.device switches and restores the device (1.6 us) even when it is the current one already, together
+# a third of a small call's host time.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
+def _launch(name, t, *args):
+    """Calls the library function `name` on `t`'s device with that device's current stream as the last argument."""
     if not t.is_cuda:
         raise PestatsError("binding", -1, "tensors must live on a CUDA device (there is no CPU path)")
-    return torch.cuda.device(t.device)
+    fn = getattr(_lib or load_library(), name)
+    dev = t.get_device()
+    if dev == _current_device():
+        status = fn(*args, _raw_stream(dev))
+    else:
+        with torch.cuda.device(dev):
+            status = fn(*args, _raw_stream(dev))
+    if status != 0:
+        raise PestatsError(name, status, pe_status_string(status))
 
 
 def _io_check(X, dY, dtype):
     if X.dtype != dtype or dY.dtype != dtype:
         raise TypeError(f"X and dY must be {dtype}")
-    if X.dim() != 3 or dY.dim() != 3 or X.shape[:2] != dY.shape[:2]:
+    xs, ys = X.shape, dY.shape
+    if len(xs) != 3 or len(ys) != 3 or xs[:2] != ys[:2]:
         raise ValueError("X must be [B,T,d_in] and dY [B,T,d_out] with equal B and T")
     if not (X.is_contiguous() and dY.is_contiguous()):
         raise ValueError("X and dY must be contiguous")
-    B, T, d_in = X.shape
-    return B, T, d_in, dY.shape[2]
+    B, T, d_in = xs
+    return B, T, d_in, ys[2]
 
 
 def _out_check(name, t, d_out, d_in):
-    if t is not None and (t.dtype != torch.float32 or tuple(t.shape) != (d_out, d_in) or not t.is_contiguous()):
+    if t is not None and (t.dtype != torch.float32 or t.shape != (d_out, d_in) or not t.is_contiguous()):
         raise ValueError(f"{name} must be a contiguous float32 [d_out, d_in] tensor")
 
 
@@ -169,13 +182,11 @@ def pe_linear_stats(X, dY, phi, out_mean=None, out_stat=None):
     Buffers are allocated when both are omitted; returns (out_mean, out_stat)."""
     B, T, d_in, d_out = _io_check(X, dY, torch.bfloat16)
     if out_mean is None and out_stat is None:
-        out_mean = torch.empty((d_out, d_in), dtype=torch.float32, device=X.device)
-        out_stat = torch.empty((d_out, d_in), dtype=torch.float32, device=X.device)
+        out_mean = X.new_empty((d_out, d_in), dtype=torch.float32)
+        out_stat = X.new_empty((d_out, d_in), dtype=torch.float32)
     _out_check("out_mean", out_mean, d_out, d_in)
     _out_check("out_stat", out_stat, d_out, d_in)
-    with _dev_ctx(X):
-        _check("pe_linear_stats", load_library().pe_linear_stats(
-            X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, _phi(phi), _ptr(out_mean), _ptr(out_stat), _stream(X)))
+    _launch("pe_linear_stats", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, _phi(phi), _ptr(out_mean), _ptr(out_stat))
     return out_mean, out_stat
 
 
@@ -183,12 +194,10 @@ def pe_example_sqnorms(X, dY, out_norms=None):
     """Per-example squared gradient norms ||dY_b^T X_b||_F^2 as a float32 [B] tensor (bf16 inputs)."""
     B, T, d_in, d_out = _io_check(X, dY, torch.bfloat16)
     if out_norms is None:
-        out_norms = torch.empty((B,), dtype=torch.float32, device=X.device)
+        out_norms = X.new_empty((B,), dtype=torch.float32)
     if out_norms.dtype != torch.float32 or tuple(out_norms.shape) != (B,) or not out_norms.is_contiguous():
         raise ValueError("out_norms must be a contiguous float32 [B] tensor")
-    with _dev_ctx(X):
-        _check("pe_example_sqnorms", load_library().pe_example_sqnorms(
-            X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, out_norms.data_ptr() if B > 0 else None, _stream(X)))
+    _launch("pe_example_sqnorms", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, out_norms.data_ptr() if B > 0 else None)
     return out_norms
 
 
@@ -221,15 +230,13 @@ def pe_linear_stats_ragged(X, dY, seq_offsets, phi, out_mean=None, out_stat=None
     seq_offsets[b] .. seq_offsets[b+1]-1 (int32 device tensor).  Returns (out_mean, out_stat)."""
     B, rows, d_in, d_out = _ragged_check(X, dY, seq_offsets)
     if out_mean is None and out_stat is None:
-        out_mean = torch.empty((d_out, d_in), dtype=torch.float32, device=X.device)
-        out_stat = torch.empty((d_out, d_in), dtype=torch.float32, device=X.device)
+        out_mean = X.new_empty((d_out, d_in), dtype=torch.float32)
+        out_stat = X.new_empty((d_out, d_in), dtype=torch.float32)
     _out_check("out_mean", out_mean, d_out, d_in)
     _out_check("out_stat", out_stat, d_out, d_in)
     workspace, wbytes = _ragged_workspace(workspace, B, d_in, d_out, X.device)
-    with _dev_ctx(X):
-        _check("pe_linear_stats_ragged", load_library().pe_linear_stats_ragged(
-            X.data_ptr(), dY.data_ptr(), seq_offsets.data_ptr(), B, rows, d_in, d_out, _phi(phi), _ptr(out_mean), _ptr(out_stat),
-            _ptr(workspace), wbytes, _stream(X)))
+    _launch("pe_linear_stats_ragged", X, X.data_ptr(), dY.data_ptr(), seq_offsets.data_ptr(), B, rows, d_in, d_out, _phi(phi), _ptr(out_mean), _ptr(out_stat),
+            _ptr(workspace), wbytes)
     return out_mean, out_stat
 
 
@@ -237,14 +244,12 @@ def pe_example_sqnorms_ragged(X, dY, seq_offsets, out_norms=None, workspace=None
     """Per-example squared gradient norms of a packed batch, float32 [B]."""
     B, rows, d_in, d_out = _ragged_check(X, dY, seq_offsets)
     if out_norms is None:
-        out_norms = torch.empty((B,), dtype=torch.float32, device=X.device)
+        out_norms = X.new_empty((B,), dtype=torch.float32)
     if out_norms.dtype != torch.float32 or tuple(out_norms.shape) != (B,) or not out_norms.is_contiguous():
         raise ValueError("out_norms must be a contiguous float32 [B] tensor")
     workspace, wbytes = _ragged_workspace(workspace, B, d_in, d_out, X.device)
-    with _dev_ctx(X):
-        _check("pe_example_sqnorms_ragged", load_library().pe_example_sqnorms_ragged(
-            X.data_ptr(), dY.data_ptr(), seq_offsets.data_ptr(), B, rows, d_in, d_out, out_norms.data_ptr() if B > 0 else None,
-            _ptr(workspace), wbytes, _stream(X)))
+    _launch("pe_example_sqnorms_ragged", X, X.data_ptr(), dY.data_ptr(), seq_offsets.data_ptr(), B, rows, d_in, d_out, out_norms.data_ptr() if B > 0 else None,
+            _ptr(workspace), wbytes)
     return out_norms
 
 
@@ -254,16 +259,14 @@ def pe_linear_clipped_sum(X, dY, clip_norm, sq_norms=None, out_sum=None):
     B, T, d_in, d_out = _io_check(X, dY, torch.bfloat16)
     given = sq_norms is not None
     if sq_norms is None:
-        sq_norms = torch.empty((B,), dtype=torch.float32, device=X.device)
+        sq_norms = X.new_empty((B,), dtype=torch.float32)
     if sq_norms.dtype != torch.float32 or tuple(sq_norms.shape) != (B,) or not sq_norms.is_contiguous():
         raise ValueError("sq_norms must be a contiguous float32 [B] tensor")
     if out_sum is None:
-        out_sum = torch.empty((d_out, d_in), dtype=torch.float32, device=X.device)
+        out_sum = X.new_empty((d_out, d_in), dtype=torch.float32)
     _out_check("out_sum", out_sum, d_out, d_in)
-    with _dev_ctx(X):
-        _check("pe_linear_clipped_sum", load_library().pe_linear_clipped_sum(
-            X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, float(clip_norm), sq_norms.data_ptr() if B > 0 else None, int(given),
-            out_sum.data_ptr(), _stream(X)))
+    _launch("pe_linear_clipped_sum", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, float(clip_norm), sq_norms.data_ptr() if B > 0 else None, int(given),
+            out_sum.data_ptr())
     return out_sum, sq_norms
 
 
@@ -272,7 +275,7 @@ def pe_linear_fused_workspace_bytes(d_in, d_out) -> int:
 
 
 def _param_check(name, t, d_out, d_in, dtype=torch.float32):
-    if t.dtype != dtype or tuple(t.shape) != (d_out, d_in) or not t.is_contiguous():
+    if t.dtype != dtype or t.shape != (d_out, d_in) or not t.is_contiguous():
         raise ValueError(f"{name} must be a contiguous {dtype} [d_out, d_in] tensor")
 
 
@@ -291,12 +294,11 @@ def pe_linear_microadam_step(X, dY, theta, m, v, *, lr, beta1, beta2, eps, step,
     common = (B, T, d_in, d_out, theta.data_ptr(), _ptr(theta_lp), m.data_ptr(), v.data_ptr(), _ptr(out_mean), _ptr(out_stat),
               ADAM_VARIANTS[variant] if isinstance(variant, str) else int(variant), float(grad_scale), float(lr), float(beta1),
               float(beta2), float(eps), int(bool(eps_inside_sqrt)), float(weight_decay), int(step))
-    with _dev_ctx(X):
-        if X.dtype == torch.float32:
-            _check("pe_linear_microadam_step_f32", load_library().pe_linear_microadam_step_f32(X.data_ptr(), dY.data_ptr(), *common, _stream(X)))
-        else:
-            wb = workspace.numel() * workspace.element_size() if workspace is not None else 0
-            _check("pe_linear_microadam_step", load_library().pe_linear_microadam_step(X.data_ptr(), dY.data_ptr(), *common, _ptr(workspace), wb, _stream(X)))
+    if X.dtype == torch.float32:
+        _launch("pe_linear_microadam_step_f32", X, X.data_ptr(), dY.data_ptr(), *common)
+    else:
+        wb = workspace.numel() * workspace.element_size() if workspace is not None else 0
+        _launch("pe_linear_microadam_step", X, X.data_ptr(), dY.data_ptr(), *common, _ptr(workspace), wb)
     return theta, m, v
 
 
@@ -316,10 +318,8 @@ def pe_linear_microsignsgd_step(X, dY, theta, m, *, lr, beta, weight_decay=0.0, 
         _param_check("theta_lp", theta_lp, d_out, d_in, torch.bfloat16)
     _out_check("out_sign", out_sign, d_out, d_in)
     wb = workspace.numel() * workspace.element_size() if workspace is not None else 0
-    with _dev_ctx(X):
-        _check("pe_linear_microsignsgd_step", load_library().pe_linear_microsignsgd_step(
-            X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, theta.data_ptr(), _ptr(theta_lp), m.data_ptr(), _ptr(out_sign), float(lr),
-            float(beta), float(weight_decay), _ptr(workspace), wb, _stream(X)))
+    _launch("pe_linear_microsignsgd_step", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, theta.data_ptr(), _ptr(theta_lp), m.data_ptr(), _ptr(out_sign), float(lr),
+            float(beta), float(weight_decay), _ptr(workspace), wb)
     return theta, m
 
 
@@ -328,9 +328,7 @@ def pe_linear_stats_accumulate(X, dY, phi, out_mean, out_stat):
     B, T, d_in, d_out = _io_check(X, dY, torch.bfloat16)
     _out_check("out_mean", out_mean, d_out, d_in)
     _out_check("out_stat", out_stat, d_out, d_in)
-    with _dev_ctx(X):
-        _check("pe_linear_stats_accumulate", load_library().pe_linear_stats_accumulate(
-            X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, _phi(phi), _ptr(out_mean), _ptr(out_stat), _stream(X)))
+    _launch("pe_linear_stats_accumulate", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, _phi(phi), _ptr(out_mean), _ptr(out_stat))
     return out_mean, out_stat
 
 
@@ -341,12 +339,10 @@ def pe_linear_stats_all(X, dY, out_mean=None, out_square=None, out_sign=None):
     outs = []
     for name, t in (("out_mean", out_mean), ("out_square", out_square), ("out_sign", out_sign)):
         if t is None:
-            t = torch.empty((d_out, d_in), dtype=torch.float32, device=X.device)
+            t = X.new_empty((d_out, d_in), dtype=torch.float32)
         _out_check(name, t, d_out, d_in)
         outs.append(t)
-    with _dev_ctx(X):
-        _check("pe_linear_stats_all", load_library().pe_linear_stats_all(
-            X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, outs[0].data_ptr(), outs[1].data_ptr(), outs[2].data_ptr(), _stream(X)))
+    _launch("pe_linear_stats_all", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, outs[0].data_ptr(), outs[1].data_ptr(), outs[2].data_ptr())
     return tuple(outs)
 
 
@@ -354,13 +350,11 @@ def pe_linear_stats_f32(X, dY, phi, out_mean=None, out_stat=None):
     """fp32-input variant of :func:`pe_linear_stats`."""
     B, T, d_in, d_out = _io_check(X, dY, torch.float32)
     if out_mean is None and out_stat is None:
-        out_mean = torch.empty((d_out, d_in), dtype=torch.float32, device=X.device)
-        out_stat = torch.empty((d_out, d_in), dtype=torch.float32, device=X.device)
+        out_mean = X.new_empty((d_out, d_in), dtype=torch.float32)
+        out_stat = X.new_empty((d_out, d_in), dtype=torch.float32)
     _out_check("out_mean", out_mean, d_out, d_in)
     _out_check("out_stat", out_stat, d_out, d_in)
-    with _dev_ctx(X):
-        _check("pe_linear_stats_f32", load_library().pe_linear_stats_f32(
-            X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, _phi(phi), _ptr(out_mean), _ptr(out_stat), _stream(X)))
+    _launch("pe_linear_stats_f32", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, _phi(phi), _ptr(out_mean), _ptr(out_stat))
     return out_mean, out_stat
 
 
@@ -368,11 +362,9 @@ def pe_token_sqstats(X, dY, out_stat=None):
     """Per-token second moment sum_{b,t} dY^2 X^2 (bf16 inputs), squared and contracted in one kernel."""
     B, T, d_in, d_out = _io_check(X, dY, torch.bfloat16)
     if out_stat is None:
-        out_stat = torch.empty((d_out, d_in), dtype=torch.float32, device=X.device)
+        out_stat = X.new_empty((d_out, d_in), dtype=torch.float32)
     _out_check("out_stat", out_stat, d_out, d_in)
-    with _dev_ctx(X):
-        _check("pe_token_sqstats", load_library().pe_token_sqstats(
-            X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, out_stat.data_ptr(), _stream(X)))
+    _launch("pe_token_sqstats", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, out_stat.data_ptr())
     return out_stat
 
 
@@ -386,15 +378,13 @@ def pe_token_sqstats_staged(X, dY, out_stat=None, workspace=None):
     of at least pe_token_sqstats_staged_workspace_bytes(...) bytes; allocated when omitted."""
     B, T, d_in, d_out = _io_check(X, dY, torch.bfloat16)
     if out_stat is None:
-        out_stat = torch.empty((d_out, d_in), dtype=torch.float32, device=X.device)
+        out_stat = X.new_empty((d_out, d_in), dtype=torch.float32)
     _out_check("out_stat", out_stat, d_out, d_in)
     need = pe_token_sqstats_staged_workspace_bytes(B, T, d_in, d_out)
     if workspace is None and need > 0:
         workspace = torch.empty(need, dtype=torch.uint8, device=X.device)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    with _dev_ctx(X):
-        _check("pe_token_sqstats_staged", load_library().pe_token_sqstats_staged(
-            X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, out_stat.data_ptr(), _ptr(workspace), ws_bytes, _stream(X)))
+    _launch("pe_token_sqstats_staged", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, out_stat.data_ptr(), _ptr(workspace), ws_bytes)
     return out_stat
 
 
@@ -416,15 +406,13 @@ def pe_token_sqstats_fp8(X, dY, out_stat=None, workspace=None):
     rate: an approximation with about 0.0375 * sqrt(sum w^2) / sum w relative error per entry (see pestats.h)."""
     B, T, d_in, d_out = _io_check(X, dY, torch.bfloat16)
     if out_stat is None:
-        out_stat = torch.empty((d_out, d_in), dtype=torch.float32, device=X.device)
+        out_stat = X.new_empty((d_out, d_in), dtype=torch.float32)
     _out_check("out_stat", out_stat, d_out, d_in)
     need = pe_token_sqstats_fp8_workspace_bytes(B, T, d_in, d_out)
     if workspace is None and need > 0:
         workspace = torch.empty(need, dtype=torch.uint8, device=X.device)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    with _dev_ctx(X):
-        _check("pe_token_sqstats_fp8", load_library().pe_token_sqstats_fp8(
-            X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, out_stat.data_ptr(), _ptr(workspace), ws_bytes, _stream(X)))
+    _launch("pe_token_sqstats_fp8", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, out_stat.data_ptr(), _ptr(workspace), ws_bytes)
     return out_stat
 
 
@@ -439,20 +427,16 @@ def pe_token_sqstats_static(X, dY, out_stat):
     if out_stat is None:
         raise ValueError("out_stat is required: this entry point allocates nothing")
     _out_check("out_stat", out_stat, d_out, d_in)
-    with _dev_ctx(X):
-        _check("pe_token_sqstats_static", load_library().pe_token_sqstats_static(
-            X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, out_stat.data_ptr(), _stream(X)))
+    _launch("pe_token_sqstats_static", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, out_stat.data_ptr())
     return out_stat
 
 
 def pe_token_sqstats_f32(X, dY, out_stat=None):
     B, T, d_in, d_out = _io_check(X, dY, torch.float32)
     if out_stat is None:
-        out_stat = torch.empty((d_out, d_in), dtype=torch.float32, device=X.device)
+        out_stat = X.new_empty((d_out, d_in), dtype=torch.float32)
     _out_check("out_stat", out_stat, d_out, d_in)
-    with _dev_ctx(X):
-        _check("pe_token_sqstats_f32", load_library().pe_token_sqstats_f32(
-            X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, out_stat.data_ptr(), _stream(X)))
+    _launch("pe_token_sqstats_f32", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, out_stat.data_ptr())
     return out_stat
 
 
@@ -472,11 +456,9 @@ def microadam_step(theta, m, v, sum_g, sum_g2, B, *, lr, beta1, beta2, eps, step
         _flat_f32(name, t, n)
     if theta_lp is not None and (theta_lp.dtype != torch.bfloat16 or theta_lp.numel() != n or not theta_lp.is_contiguous()):
         raise ValueError("theta_lp must be contiguous bfloat16 with theta's element count")
-    with _dev_ctx(theta):
-        _check("microadam_step", load_library().microadam_step(
-            theta.data_ptr(), _ptr(theta_lp), m.data_ptr(), v.data_ptr(), sum_g.data_ptr(), sum_g2.data_ptr(), n, int(B),
+    _launch("microadam_step", theta, theta.data_ptr(), _ptr(theta_lp), m.data_ptr(), v.data_ptr(), sum_g.data_ptr(), sum_g2.data_ptr(), n, int(B),
             float(grad_scale), float(lr), float(beta1), float(beta2), float(eps), int(bool(eps_inside_sqrt)),
-            float(weight_decay), int(step), _stream(theta)))
+            float(weight_decay), int(step))
 
 
 def microadam_family_step(theta, m, v, sum_g, sum_g2, B, variant, *, lr, beta1, beta2, eps, step, grad_scale=1.0,
@@ -489,11 +471,9 @@ def microadam_family_step(theta, m, v, sum_g, sum_g2, B, variant, *, lr, beta1, 
     if theta_lp is not None and (theta_lp.dtype != torch.bfloat16 or theta_lp.numel() != n or not theta_lp.is_contiguous()):
         raise ValueError("theta_lp must be contiguous bfloat16 with theta's element count")
     code = ADAM_VARIANTS[variant] if isinstance(variant, str) else int(variant)
-    with _dev_ctx(theta):
-        _check("microadam_family_step", load_library().microadam_family_step(
-            theta.data_ptr(), _ptr(theta_lp), m.data_ptr(), v.data_ptr(), sum_g.data_ptr(), sum_g2.data_ptr(), n, int(B), code,
+    _launch("microadam_family_step", theta, theta.data_ptr(), _ptr(theta_lp), m.data_ptr(), v.data_ptr(), sum_g.data_ptr(), sum_g2.data_ptr(), n, int(B), code,
             float(grad_scale), float(lr), float(beta1), float(beta2), float(eps), int(bool(eps_inside_sqrt)),
-            float(weight_decay), int(step), _stream(theta)))
+            float(weight_decay), int(step))
 
 
 def microsignsgd_step(theta, m, sum_sign, B, *, lr, beta, weight_decay=0.0, theta_lp=None):
@@ -503,10 +483,8 @@ def microsignsgd_step(theta, m, sum_sign, B, *, lr, beta, weight_decay=0.0, thet
     _flat_f32("sum_sign", sum_sign, n)
     if theta_lp is not None and (theta_lp.dtype != torch.bfloat16 or theta_lp.numel() != n or not theta_lp.is_contiguous()):
         raise ValueError("theta_lp must be contiguous bfloat16 with theta's element count")
-    with _dev_ctx(theta):
-        _check("microsignsgd_step", load_library().microsignsgd_step(
-            theta.data_ptr(), _ptr(theta_lp), m.data_ptr(), sum_sign.data_ptr(), n, int(B), float(lr), float(beta),
-            float(weight_decay), _stream(theta)))
+    _launch("microsignsgd_step", theta, theta.data_ptr(), _ptr(theta_lp), m.data_ptr(), sum_sign.data_ptr(), n, int(B), float(lr), float(beta),
+            float(weight_decay))
 
 
 def pe_get_async_status(device=None):
