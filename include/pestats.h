@@ -163,6 +163,36 @@ pe_status_t pe_linear_stats_all(const void* X, const void* dY, int B, int T, int
                                 float* out_mean, float* out_square, float* out_sign, pe_stream_t stream);
 
 /*
+ * The same statistics for widths that are no multiples of 8.  TMA, which feeds the tensor-core kernel, wants 16-byte row
+ * pitches; pe_linear_stats runs such layers on the SIMT kernel.  With a workspace this call first copies the
+ * operands concerned to a padded pitch and contracts the copies on the tensor cores.  accumulate != 0: as
+ * pe_linear_stats_accumulate; out_sign != NULL (phi square, accumulate 0): as pe_linear_stats_all.
+ * workspace: device memory, 256-byte aligned, pe_linear_stats_padded_workspace_bytes() bytes, contents undefined
+ * afterwards.  That function returns 0 where nothing is to be gained (widths that are multiples of 8, layers too small, a forced
+ * path): the call is then the ordinary one and ignores the workspace.  Other arguments, alignments and results as for
+ * pe_linear_stats.
+ */
+pe_status_t pe_linear_stats_padded(const void* X, const void* dY, int B, int T, int d_in, int d_out, pe_phi_t phi,
+                                   int accumulate, float* out_mean, float* out_stat, float* out_sign, void* workspace,
+                                   size_t workspace_bytes, pe_stream_t stream);
+size_t pe_linear_stats_padded_workspace_bytes(int B, int T, int d_in, int d_out);
+
+/*
+ * pe_linear_stats for the weight [F, C, Kh, Kw] of a 2-D convolution (Appendix B.4): every output position is a token, its
+ * receptive field the token's C*Kh*Kw features (channel-major, then kernel row, then kernel column).  x: bf16 [B, C, H, W],
+ * the layer's input; grad_out: bf16 [B, F, H_out, W_out], the cotangent of its output, H_out = (H + 2 pad_h - dil_h (Kh-1) - 1) /
+ * stride_h + 1 (W_out alike); both contiguous.  out_mean, out_stat: fp32 [F, C*Kh*Kw], as for pe_linear_stats.
+ * workspace: device memory, 256-byte aligned, pe_conv2d_stats_workspace_bytes() bytes: the unfolded input [B, H_out*W_out,
+ * C*Kh*Kw] and the transposed cotangents, rows padded to 16 bytes; contents undefined afterwards.  A return of 0 bytes means that
+ * the geometry is invalid, or its receptive field too large for the unfolding kernel (PE_ERR_DIM, PE_ERR_UNSUPPORTED_SHAPE here).
+ */
+pe_status_t pe_conv2d_stats(const void* x, const void* grad_out, int B, int C, int H, int W, int F, int Kh, int Kw,
+                            int stride_h, int stride_w, int pad_h, int pad_w, int dil_h, int dil_w, pe_phi_t phi,
+                            float* out_mean, float* out_stat, void* workspace, size_t workspace_bytes, pe_stream_t stream);
+size_t pe_conv2d_stats_workspace_bytes(int B, int C, int H, int W, int F, int Kh, int Kw, int stride_h, int stride_w,
+                                       int pad_h, int pad_w, int dil_h, int dil_w);
+
+/*
  * Per-token second moment (Section 2.3, the "per-token" alternative):
  *     out_stat[o,i] = sum_{b,t} dY[b,t,o]^2 * X[b,t,i]^2  =  ((dY o dY)^T (X o X))[o,i].
  * B and T only enter through the row count B*T.  bf16 inputs, 16-byte aligned; out_stat fp32

@@ -21,6 +21,7 @@ __all__ = [
     "pe_linear_stats_ragged", "pe_linear_stats_ragged_workspace_bytes", "pe_example_sqnorms_ragged", "pe_linear_clipped_sum",
     "pe_linear_microadam_step", "pe_linear_microadam_step_f32", "pe_linear_microsignsgd_step", "pe_linear_fused_workspace_bytes",
     "pe_token_sqstats_fp8", "pe_token_sqstats_fp8_workspace_bytes", "pe_set_wait_limit_cycles", "pe_tile_order_band",
+    "pe_linear_stats_padded", "pe_linear_stats_padded_workspace_bytes", "pe_conv2d_stats", "pe_conv2d_stats_workspace_bytes",
     "pe_set_fused_update", "FUSED_AUTO", "FUSED_ALWAYS", "FUSED_NEVER",
 ]
 
@@ -38,7 +39,8 @@ EXPORTED_SYMBOLS = [
     "pe_linear_stats_ragged", "pe_linear_stats_ragged_workspace_bytes", "pe_example_sqnorms_ragged", "pe_linear_clipped_sum",
     "pe_linear_microadam_step", "pe_linear_microadam_step_f32", "pe_linear_microsignsgd_step", "pe_linear_fused_workspace_bytes",
     "pe_token_sqstats_fp8", "pe_token_sqstats_fp8_workspace_bytes", "pe_set_wait_limit_cycles", "pe_tile_order_band",
-    "pe_set_fused_update",
+    "pe_set_fused_update", "pe_linear_stats_padded", "pe_linear_stats_padded_workspace_bytes", "pe_conv2d_stats",
+    "pe_conv2d_stats_workspace_bytes",
 ]
 ADAM_VARIANTS = {"adam": 0, "microadam": 1, "microadam_var": 2, "microadam_msq": 3}      # pe_adam_variant_t
 STATIC_SCRATCH_BYTES = 32 * 1024 * 1024      # PE_STATIC_SCRATCH_BYTES of pestats.h
@@ -71,6 +73,12 @@ def load_library() -> ctypes.CDLL:
     vp, i, f, ll, sz = ctypes.c_void_p, ctypes.c_int, ctypes.c_float, ctypes.c_longlong, ctypes.c_size_t
     lib.pe_linear_stats.argtypes = [vp, vp, i, i, i, i, i, vp, vp, vp]
     lib.pe_linear_stats_f32.argtypes = [vp, vp, i, i, i, i, i, vp, vp, vp]
+    lib.pe_linear_stats_padded.argtypes = [vp, vp, i, i, i, i, i, i, vp, vp, vp, vp, sz, vp]
+    lib.pe_linear_stats_padded_workspace_bytes.argtypes = [i] * 4
+    lib.pe_linear_stats_padded_workspace_bytes.restype = sz
+    lib.pe_conv2d_stats.argtypes = [vp, vp] + [i] * 14 + [vp, vp, vp, sz, vp]
+    lib.pe_conv2d_stats_workspace_bytes.argtypes = [i] * 13
+    lib.pe_conv2d_stats_workspace_bytes.restype = sz
     lib.pe_linear_stats_all.argtypes = [vp, vp, i, i, i, i, vp, vp, vp, vp]
     lib.pe_linear_stats_accumulate.argtypes = [vp, vp, i, i, i, i, i, vp, vp, vp]
     lib.pe_example_sqnorms.argtypes = [vp, vp, i, i, i, i, vp, vp]
@@ -111,7 +119,7 @@ def load_library() -> ctypes.CDLL:
     lib.pe_launch_count.restype = ll
     lib.pe_reset_launch_count.argtypes = []
     lib.pe_reset_launch_count.restype = None
-    for name in ("pe_linear_stats", "pe_linear_stats_f32", "pe_linear_stats_all", "pe_linear_stats_accumulate", "pe_example_sqnorms", "pe_token_sqstats", "pe_token_sqstats_f32", "pe_token_sqstats_static",
+    for name in ("pe_linear_stats", "pe_linear_stats_padded", "pe_conv2d_stats", "pe_linear_stats_f32", "pe_linear_stats_all", "pe_linear_stats_accumulate", "pe_example_sqnorms", "pe_token_sqstats", "pe_token_sqstats_f32", "pe_token_sqstats_static",
                  "pe_token_sqstats_staged", "pe_token_sqstats_fp8",
                  "pe_linear_stats_ragged", "pe_example_sqnorms_ragged", "pe_linear_clipped_sum",
                  "pe_linear_microadam_step", "pe_linear_microadam_step_f32", "pe_linear_microsignsgd_step",
@@ -177,6 +185,59 @@ def _out_check(name, t, d_out, d_in):
         raise ValueError(f"{name} must be a contiguous float32 [d_out, d_in] tensor")
 
 
+def pe_linear_stats_padded_workspace_bytes(B, T, d_in, d_out) -> int:
+    return int(load_library().pe_linear_stats_padded_workspace_bytes(int(B), int(T), int(d_in), int(d_out)))
+
+
+def _padded(X, dY, B, T, d_in, d_out, phi, accumulate, out_mean, out_stat, out_sign) -> bool:
+    """Runs pe_linear_stats_padded with a workspace from torch's allocator if the widths are no multiples of 8 and the
+    library says that it pays; False if the ordinary call is the one to make."""
+    if not (d_in & 7 or d_out & 7):
+        return False
+    need = pe_linear_stats_padded_workspace_bytes(B, T, d_in, d_out)
+    if need == 0:
+        return False
+    pe_linear_stats_padded(X, dY, phi, accumulate, out_mean, out_stat, out_sign, X.new_empty((need,), dtype=torch.uint8))
+    return True
+
+
+def pe_linear_stats_padded(X, dY, phi, accumulate, out_mean, out_stat, out_sign, workspace):
+    """The C entry point: statistics of a layer whose widths are no multiples of 8 by way of padded copies in `workspace`
+    (uint8, pe_linear_stats_padded_workspace_bytes(...) bytes; None where that is 0).  pe_linear_stats, _accumulate and
+    _all call it where it pays."""
+    B, T, d_in, d_out = _io_check(X, dY, torch.bfloat16)
+    for name, t in (("out_mean", out_mean), ("out_stat", out_stat), ("out_sign", out_sign)):
+        _out_check(name, t, d_out, d_in)
+    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
+    _launch("pe_linear_stats_padded", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, _phi(phi), int(bool(accumulate)), _ptr(out_mean),
+            _ptr(out_stat), _ptr(out_sign), _ptr(workspace), ws_bytes)
+
+
+def pe_conv2d_stats_workspace_bytes(B, C, H, W, F, Kh, Kw, stride, padding, dilation) -> int:
+    """stride, padding, dilation: (vertical, horizontal).  0: the unfolding kernel does not take this geometry."""
+    return int(load_library().pe_conv2d_stats_workspace_bytes(B, C, H, W, F, Kh, Kw, *stride, *padding, *dilation))
+
+
+def pe_conv2d_stats(x, grad_out, kernel_size, phi, stride, padding, dilation, out_mean, out_stat):
+    """The C entry point pe_conv2d_stats: x bf16 [B, C, H, W], grad_out bf16 [B, F, H_out, W_out], both contiguous;
+    kernel_size, stride, padding, dilation: (vertical, horizontal); outputs float32 [F, C*Kh*Kw].  False if the
+    geometry is not one the unfolding kernel takes (nothing is launched)."""
+    for name, t in (("x", x), ("grad_out", grad_out)):
+        if t.dtype != torch.bfloat16 or t.dim() != 4 or not t.is_contiguous():
+            raise ValueError(f"{name} must be a contiguous 4-D bfloat16 tensor")
+    B, C, H, W = x.shape
+    F = grad_out.shape[1]
+    _out_check("out_mean", out_mean, F, C * kernel_size[0] * kernel_size[1])
+    _out_check("out_stat", out_stat, F, C * kernel_size[0] * kernel_size[1])
+    need = pe_conv2d_stats_workspace_bytes(B, C, H, W, F, *kernel_size, stride, padding, dilation)
+    if need == 0:
+        return False
+    workspace = x.new_empty((need,), dtype=torch.uint8)
+    _launch("pe_conv2d_stats", x, x.data_ptr(), grad_out.data_ptr(), B, C, H, W, F, *kernel_size, *stride, *padding, *dilation, _phi(phi),
+            _ptr(out_mean), _ptr(out_stat), workspace.data_ptr(), need)
+    return True
+
+
 def pe_linear_stats(X, dY, phi, out_mean=None, out_stat=None):
     """out_mean = sum_b G_b, out_stat = sum_b phi(G_b) with G_b = dY_b^T X_b (bf16 inputs).
     Buffers are allocated when both are omitted; returns (out_mean, out_stat)."""
@@ -186,7 +247,8 @@ def pe_linear_stats(X, dY, phi, out_mean=None, out_stat=None):
         out_stat = X.new_empty((d_out, d_in), dtype=torch.float32)
     _out_check("out_mean", out_mean, d_out, d_in)
     _out_check("out_stat", out_stat, d_out, d_in)
-    _launch("pe_linear_stats", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, _phi(phi), _ptr(out_mean), _ptr(out_stat))
+    if not _padded(X, dY, B, T, d_in, d_out, _phi(phi), 0, out_mean, out_stat, None):
+        _launch("pe_linear_stats", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, _phi(phi), _ptr(out_mean), _ptr(out_stat))
     return out_mean, out_stat
 
 
@@ -328,7 +390,8 @@ def pe_linear_stats_accumulate(X, dY, phi, out_mean, out_stat):
     B, T, d_in, d_out = _io_check(X, dY, torch.bfloat16)
     _out_check("out_mean", out_mean, d_out, d_in)
     _out_check("out_stat", out_stat, d_out, d_in)
-    _launch("pe_linear_stats_accumulate", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, _phi(phi), _ptr(out_mean), _ptr(out_stat))
+    if not _padded(X, dY, B, T, d_in, d_out, _phi(phi), 1, out_mean, out_stat, None):
+        _launch("pe_linear_stats_accumulate", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, _phi(phi), _ptr(out_mean), _ptr(out_stat))
     return out_mean, out_stat
 
 
@@ -342,7 +405,8 @@ def pe_linear_stats_all(X, dY, out_mean=None, out_square=None, out_sign=None):
             t = X.new_empty((d_out, d_in), dtype=torch.float32)
         _out_check(name, t, d_out, d_in)
         outs.append(t)
-    _launch("pe_linear_stats_all", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, outs[0].data_ptr(), outs[1].data_ptr(), outs[2].data_ptr())
+    if not _padded(X, dY, B, T, d_in, d_out, PHI_SQUARE, 0, *outs):
+        _launch("pe_linear_stats_all", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, outs[0].data_ptr(), outs[1].data_ptr(), outs[2].data_ptr())
     return tuple(outs)
 
 

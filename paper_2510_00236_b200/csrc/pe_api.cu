@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/pestats.h"
+#include "pe_layout.cuh"
 #include "pe_optim.cuh"
 #include "pe_stage.cuh"
 #include "pe_simt.cuh"
@@ -114,13 +115,15 @@ static pe_status_t check_launch() {
 // bytes of features x one pipeline stage of tokens of one example, 128-byte swizzled (16-byte chunks for bf16, 32-byte
 // chunks for fp32: the MN-major tf32 MMA accepts no other layout).  rows64: 64 bytes of features per box row with
 // the 64-byte swizzle (X of the 256 x 192 tile).  Tokens past T and features past d read as zero.
+// pitch: elements from one token's row to the next (a multiple of 8 for bf16), 0 = d.
 static pe_status_t make_operand_map(CUtensorMap* m, const void* base, int B, int T, int d, bool f32, int box_feats, int box_tokens,
-                                    bool rows64 = false, int box_examples = 1) {
+                                    bool rows64 = false, int box_examples = 1, int pitch = 0) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return PE_ERR_CUDA;
   const cuuint64_t es = f32 ? 4ull : 2ull;
   cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)T, (cuuint64_t)B};
-  cuuint64_t strides[2] = {(cuuint64_t)d * es, (cuuint64_t)T * (cuuint64_t)d * es};
+  const cuuint64_t row = (cuuint64_t)(pitch ? pitch : d) * es;
+  cuuint64_t strides[2] = {row, (cuuint64_t)T * row};
   cuuint32_t box[3] = {(cuuint32_t)box_feats, (cuuint32_t)box_tokens, (cuuint32_t)box_examples};
   cuuint32_t estr[3] = {1u, 1u, 1u};
   CUresult r = enc(m, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
@@ -238,11 +241,10 @@ static pe_status_t zero_for_split(DeviceInfo* di, float* a, float* b, size_t n, 
   float* first = a ? a : b;
   float* second = a ? b : nullptr;
   if (!first) return PE_OK;
-  const long long n4 = (long long)(n / 4);          // d_in % 8 == 0 on this path
-  long long blocks = (n4 + 255) / 256;
+  long long blocks = ((long long)(n / 4) + 255) / 256;
   if (blocks > di->sm_count) blocks = di->sm_count;   // few blocks: the dependent kernel needs the SMs
   zero_outputs_kernel<<<(int)(blocks < 1 ? 1 : blocks), 256, 0, st>>>(reinterpret_cast<float4*>(first), reinterpret_cast<float4*>(second),
-                                                                            reinterpret_cast<float4*>(c), n4, counters, n_counters);
+                                                                            reinterpret_cast<float4*>(c), (long long)n, counters, n_counters);
   return check_launch();
 }
 
@@ -264,7 +266,7 @@ static pe_status_t launch_pair_kernel(Kernel kernel, dim3 grid, int smem, cudaSt
 }
 
 // mxt, myt: the maps of the zero-padded tail groups of a packed batch (RAGGED); any valid map otherwise.
-template <int PHI, bool TF32, int NT, int MEAN, int BKT = tc_default_bk(TF32, NT), bool RAGGED = false, int OPT = OPT_NONE, bool F8 = false>
+template <int PHI, bool TF32, int NT, int MEAN, int BKT = tc_default_bk(TF32, NT), bool RAGGED = false, int OPT = OPT_NONE, bool F8 = false, bool CHUNKED = false>
 static pe_status_t launch_tc_inst(DeviceInfo* di, int slot, const CUtensorMap& mx, const CUtensorMap& my, const CUtensorMap& mm,
                                   const CUtensorMap& ms, const CUtensorMap& msgn, const TcParams& p, dim3 grid, cudaStream_t st,
                                   const CUtensorMap* mxt = nullptr, const CUtensorMap* myt = nullptr, const FusedOpt* opt = nullptr) {
@@ -273,14 +275,14 @@ static pe_status_t launch_tc_inst(DeviceInfo* di, int slot, const CUtensorMap& m
   {
     std::lock_guard<std::mutex> lock(g_dev_mutex);
     if (!di->tc_attr_set[slot]) {
-      if (cudaFuncSetAttribute(tc_stats_kernel<PHI, TF32, NT, MEAN, BKT, RAGGED, OPT, F8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+      if (cudaFuncSetAttribute(tc_stats_kernel<PHI, TF32, NT, MEAN, BKT, RAGGED, OPT, F8, CHUNKED>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
         cudaGetLastError();
         return PE_ERR_CUDA;
       }
       di->tc_attr_set[slot] = true;
     }
   }
-  return launch_pair_kernel(tc_stats_kernel<PHI, TF32, NT, MEAN, BKT, RAGGED, OPT, F8>, grid, smem, st, after_zeroing, mx, my, mm, ms, msgn,
+  return launch_pair_kernel(tc_stats_kernel<PHI, TF32, NT, MEAN, BKT, RAGGED, OPT, F8, CHUNKED>, grid, smem, st, after_zeroing, mx, my, mm, ms, msgn,
                             mxt ? *mxt : mx, myt ? *myt : my, p, opt ? *opt : FusedOpt{});
 }
 
@@ -289,18 +291,20 @@ static pe_status_t launch_tc_inst(DeviceInfo* di, int slot, const CUtensorMap& m
 // pair tile is 256 x 128 (two running sums per thread); with only out_stat it is 256 x 256.
 static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int B, int T, int d_in, int d_out, int phi,
                              int per_example, float* out_mean, float* out_stat, cudaStream_t st, bool half_ops = false,
-                             float* out_sign = nullptr, bool accumulate = false, const float* sq_norms = nullptr, float clip_norm = 0.f) {
+                             float* out_sign = nullptr, bool accumulate = false, const float* sq_norms = nullptr, float clip_norm = 0.f,
+                             int pitch_x = 0, int pitch_y = 0, bool chunked = false) {
   const bool triple = out_sign != nullptr;       // mean + square + sign in one pass (phi = square, all three outputs given)
-  const bool both = per_example && out_mean && out_stat;
+  const bool both = per_example && ((out_mean && out_stat) || chunked);
+  const bool runs = chunked && T > TC_CHUNK_TOKENS;     // several accumulators per example
   // Both outputs: sum_b G_b in tensor memory beside a 256-wide accumulator, unless the sequences are
   // so short that the per-example drain of that single accumulator would dominate.
   const int forced = g_path.load();
   // 256 x 192 tile: 22 % less operand traffic per flop than 256 x 128
   const long long pad192 = (long long)((d_in + 191) / 192) * 192, pad128 = (long long)((d_in + 127) / 128) * 128;
-  const bool wide = both && forced != PE_PATH_TENSOR_NARROW &&
+  const bool wide = both && !runs && forced != PE_PATH_TENSOR_NARROW &&
                     (forced == PE_PATH_TENSOR_WIDE || (T >= (triple ? TC_WIDE_TRIPLE_MIN_T : TC_WIDE_MIN_T) &&
                                                        pad192 * 100 <= pad128 * (100 + TC_WIDE_MAX_PAD_PERCENT)));
-  const bool mean_regs = both && (triple || wide || T < TC_MEAN_TMEM_MIN_T || forced == PE_PATH_TENSOR_NARROW);
+  const bool mean_regs = both && (triple || wide || runs || T < TC_MEAN_TMEM_MIN_T || forced == PE_PATH_TENSOR_NARROW);
   const int nt = mean_regs ? (wide ? 192 : 128) : 256;
   const int box_feats = TcOperand<false, 256>::BOX_FEATS;
   const bool short_seq = mean_regs && !wide && T <= TC_SHORT_T;      // many short examples, both sums in registers: small stages
@@ -308,34 +312,42 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
   CUtensorMap mx, my;
   // short sequences: a box is two examples deep (a stage holds two examples of 32 tokens each)
   const int box_examples = short_seq ? TcOperand<false, 128, TC_SHORT_BK>::GROUP : 1;
-  pe_status_t rc = wide ? make_operand_map(&mx, X, B, T, d_in, false, TcOperand<false, 192>::B_BOX_FEATS, box_tokens, true)
-                        : make_operand_map(&mx, X, B, T, d_in, false, box_feats, box_tokens, false, box_examples);
+  pe_status_t rc = wide ? make_operand_map(&mx, X, B, T, d_in, false, TcOperand<false, 192>::B_BOX_FEATS, box_tokens, true, 1, pitch_x)
+                        : make_operand_map(&mx, X, B, T, d_in, false, box_feats, box_tokens, false, box_examples, pitch_x);
   if (rc != PE_OK) return rc;
-  rc = make_operand_map(&my, dY, B, T, d_out, false, box_feats, box_tokens, false, box_examples);
+  rc = make_operand_map(&my, dY, B, T, d_out, false, box_feats, box_tokens, false, box_examples, pitch_y);
   if (rc != PE_OK) return rc;
-  CUtensorMap mm, ms;       // an output that is not wanted gets the other one's map and is never used
-  rc = make_output_map(&mm, out_mean ? out_mean : out_stat, d_in, d_out);
-  if (rc != PE_OK) return rc;
-  rc = make_output_map(&ms, out_stat ? out_stat : out_mean, d_in, d_out);
-  if (rc != PE_OK) return rc;
-  CUtensorMap msgn = ms;
-  if (triple && (rc = make_output_map(&msgn, out_sign, d_in, d_out)) != PE_OK) return rc;
+  // an output that is not wanted gets the other one's map and is never used; rows that are no 16-byte multiples cannot be
+  // described by a map at all and are written without one (scalar_out)
+  const bool scalar_out = d_in % 4 != 0;
+  CUtensorMap mm = mx, ms = mx, msgn = mx;
+  if (!scalar_out) {
+    rc = make_output_map(&mm, out_mean ? out_mean : out_stat, d_in, d_out);
+    if (rc == PE_OK) rc = make_output_map(&ms, out_stat ? out_stat : out_mean, d_in, d_out);
+    if (rc == PE_OK && triple) rc = make_output_map(&msgn, out_sign, d_in, d_out);
+    if (rc != PE_OK) return rc;
+  }
   const int tiles_n = (d_in + nt - 1) / nt, pairs_m = (d_out + TC_PAIR_M - 1) / TC_PAIR_M;
   if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
-  int ns = choose_nsplit((long long)tiles_n * pairs_m, B, T, di->sm_count / 2 > 0 ? di->sm_count / 2 : 1, 16);
+  const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
+  int ns = choose_nsplit((long long)tiles_n * pairs_m, B, T, slots, std::max(16, slots));
   if (triple && (B + ns - 1) / ns > TC_SIGN_COUNT_MAX) ns = (B + TC_SIGN_COUNT_MAX - 1) / TC_SIGN_COUNT_MAX;   // 16-bit sign counters
   if (ns > 1 && !accumulate) {
     rc = zero_for_split(di, out_mean, out_stat, (size_t)d_in * d_out, st, out_sign);
     if (rc != PE_OK) return rc;
   }
-  TcParams p;
+  TcParams p{};
   p.B = B; p.T = T; p.d_in = d_in; p.d_out = d_out; p.nsplit = ns; p.per_example = per_example; p.half_operands = half_ops ? 1 : 0;
-  p.accumulate = accumulate ? 1 : 0;
+  p.accumulate = accumulate ? 1 : 0; p.scalar_out = scalar_out ? 1 : 0;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, nt, ns, di->sm_count / 2);
   p.out_mean = out_mean; p.out_stat = out_stat; p.out_sign = out_sign; p.out_norms = nullptr; p.dev_status = di->status_ptr;
   p.seq_offsets = nullptr; p.sq_norms = sq_norms; p.clip_norm = clip_norm;
   dim3 grid(2 * pairs_m * tiles_n, 1, ns);
   if (phi == PHI_CLIP_SCALE) return launch_tc_inst<3, false, 256, MEAN_NONE>(di, 14, mx, my, mm, ms, msgn, p, grid, st);
+  if (runs) {
+    if (phi == PE_PHI_SQUARE) return launch_tc_inst<1, false, 128, MEAN_REGS, 128, false, OPT_NONE, false, true>(di, 28, mx, my, mm, ms, msgn, p, grid, st);
+    return launch_tc_inst<2, false, 128, MEAN_REGS, 128, false, OPT_NONE, false, true>(di, 29, mx, my, mm, ms, msgn, p, grid, st);
+  }
   if (triple && wide) return launch_tc_inst<1, false, 192, MEAN_HYBRID_SIGN>(di, 26, mx, my, mm, ms, msgn, p, grid, st);
   if (triple && short_seq) return launch_tc_inst<1, false, 128, MEAN_REGS_SIGN, TC_SHORT_BK>(di, 27, mx, my, mm, ms, msgn, p, grid, st);
   if (triple) return launch_tc_inst<1, false, 128, MEAN_REGS_SIGN>(di, 10, mx, my, mm, ms, msgn, p, grid, st);
@@ -373,7 +385,7 @@ static pe_status_t launch_tc_norms(DeviceInfo* di, const void* X, const void* dY
   const int tiles_n = (d_in + 255) / 256, pairs_m = (d_out + TC_PAIR_M - 1) / TC_PAIR_M;
   if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
   const int ns = choose_nsplit((long long)tiles_n * pairs_m, B, T, di->sm_count / 2 > 0 ? di->sm_count / 2 : 1, 16);
-  TcParams p;
+  TcParams p{};
   p.B = B; p.T = T; p.d_in = d_in; p.d_out = d_out; p.nsplit = ns; p.per_example = 1; p.half_operands = 0;
   p.accumulate = 1;       // nothing is zeroed by a preceding kernel and no matrix is written
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, 256, ns, di->sm_count / 2);
@@ -418,7 +430,8 @@ static SimtPlan plan_simt(DeviceInfo* di, int mode, int B, int T, int d_in, int 
 
 template <typename TIn, int MODE, class Tile, int SUMS>
 static pe_status_t launch_simt_inst(const SimtPlan& plan, const TIn* X, const TIn* dY, int B, int T, int d_in, int d_out, int phi,
-                                    float* out_mean, float* out_stat, cudaStream_t st, bool accumulate, const SimtExtra& ex, const FusedOpt& opt) {
+                                    float* out_mean, float* out_stat, cudaStream_t st, bool accumulate, int ldx, int ldy, const SimtExtra& ex,
+                                    const FusedOpt& opt) {
   auto kernel = simt_stats_kernel<TIn, MODE, Tile, SUMS>;
   constexpr int smem = (MODE == MODE_STATS ? Tile::smem_floats(SUMS) : (2 * Tile::CHUNK > Tile::ROWS * Tile::COLS ? 2 * Tile::CHUNK : Tile::ROWS * Tile::COLS)) * 4;
   if constexpr (smem > 48 * 1024) {
@@ -432,7 +445,7 @@ static pe_status_t launch_simt_inst(const SimtPlan& plan, const TIn* X, const TI
   }
   // a group of four columns is one load when every row of the operand starts on such a boundary
   const size_t group = 4 * sizeof(TIn);
-  const int vec_x = d_in % 4 == 0 && aligned(X, group) ? 1 : 0, vec_y = d_out % 4 == 0 && aligned(dY, group) ? 1 : 0;
+  const int vec_x = ldx % 4 == 0 && aligned(X, group) ? 1 : 0, vec_y = ldy % 4 == 0 && aligned(dY, group) ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((d_in + Tile::COLS - 1) / Tile::COLS, (d_out + Tile::ROWS - 1) / Tile::ROWS, plan.slices);
   cfg.blockDim = dim3(SIMT_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
@@ -441,7 +454,7 @@ static pe_status_t launch_simt_inst(const SimtPlan& plan, const TIn* X, const TI
   attr.id = cudaLaunchAttributeClusterDimension;
   attr.val.clusterDim.x = 1; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = plan.cluster;
   cfg.attrs = &attr; cfg.numAttrs = plan.cluster > 1 ? 1 : 0;
-  if (cudaLaunchKernelEx(&cfg, kernel, X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, accumulate ? 1 : 0, plan.cluster, vec_x, vec_y, ex, opt) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, kernel, X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, accumulate ? 1 : 0, plan.cluster, ldx, ldy, vec_x, vec_y, ex, opt) != cudaSuccess) {
     cudaGetLastError();
     return PE_ERR_CUDA;
   }
@@ -451,7 +464,8 @@ static pe_status_t launch_simt_inst(const SimtPlan& plan, const TIn* X, const TI
 template <typename TIn, int MODE>
 static pe_status_t launch_simt(DeviceInfo* di, const TIn* X, const TIn* dY, int B, int T, int d_in, int d_out, int phi,
                                float* out_mean, float* out_stat, cudaStream_t st, bool accumulate = false, SimtExtra ex = SimtExtra{},
-                               const FusedOpt* opt = nullptr) {
+                               const FusedOpt* opt = nullptr, int pitch_x = 0, int pitch_y = 0) {
+  const int ldx = pitch_x ? pitch_x : d_in, ldy = pitch_y ? pitch_y : d_out;
   SimtPlan plan = plan_simt(di, MODE, B, T, d_in, d_out);
   if (opt && plan.slices > SIMT_MAX_CLUSTER) plan.slices = SIMT_MAX_CLUSTER;      // a fused update needs the whole batch in one cluster
   if ((d_out + SimtTile11::ROWS - 1) / SimtTile11::ROWS > 65535 && plan.tile > 0) plan.tile = 0;      // gridDim.y
@@ -464,9 +478,9 @@ static pe_status_t launch_simt(DeviceInfo* di, const TIn* X, const TIn* dY, int 
     using Tile = decltype(tile);
     if constexpr (MODE == MODE_STATS) {
       if (out_mean || (opt && opt->kind == OPT_ADAM))
-        return launch_simt_inst<TIn, MODE, Tile, 2>(plan, X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, st, accumulate, ex, o);
+        return launch_simt_inst<TIn, MODE, Tile, 2>(plan, X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, st, accumulate, ldx, ldy, ex, o);
     }
-    return launch_simt_inst<TIn, MODE, Tile, 1>(plan, X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, st, accumulate, ex, o);
+    return launch_simt_inst<TIn, MODE, Tile, 1>(plan, X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, st, accumulate, ldx, ldy, ex, o);
   };
   switch (plan.tile) {
     case 0: return run(SimtTile84{});
@@ -534,7 +548,7 @@ static pe_status_t launch_tc_ragged(DeviceInfo* di, const void* X, const void* d
     rc = zero_for_split(di, both ? out_mean : nullptr, first, (size_t)d_in * d_out, st);
     if (rc != PE_OK) return rc;
   }
-  TcParams p;
+  TcParams p{};
   p.B = B; p.T = 0; p.d_in = d_in; p.d_out = d_out; p.nsplit = ns; p.per_example = 1; p.half_operands = 0;
   p.accumulate = norms ? 1 : 0;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, nt, ns, di->sm_count / 2);
@@ -579,6 +593,55 @@ static void regroup_rows(int& B, int& T) {
   if (T < REGROUP && rows % REGROUP == 0) { B = (int)(rows / REGROUP); T = REGROUP; }
 }
 
+// pe_linear_stats on the tensor cores.
+static pe_status_t tc_linear_stats(DeviceInfo* di, const void* X, const void* dY, int B, int T, int d_in, int d_out, int phi, float* out_mean,
+                                   float* out_stat, bool accumulate, cudaStream_t st) {
+  g_last_path.store(PE_PATH_TENSOR);
+  auto plain = [&](float* out) { return launch_tc(di, X, dY, B, T, d_in, d_out, phi, 0, out, nullptr, st, false, nullptr, accumulate); };
+  if (phi == PE_PHI_IDENTITY || !out_stat) {
+    // phi = identity, or only sum_b G_b wanted: the plain contraction over all B*T rows, where B and T only enter
+    // through B*T: regroup short sequences into full two-stage "examples" when the rows divide evenly.
+    regroup_rows(B, T);
+    pe_status_t rc = plain(out_mean ? out_mean : out_stat);
+    if (rc != PE_OK || !out_mean || !out_stat) return rc;
+    if (accumulate) return plain(out_stat);          // a copy would overwrite: contract once more into the second
+    if (cudaMemcpyAsync(out_stat, out_mean, (size_t)d_in * d_out * sizeof(float), cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
+      cudaGetLastError();
+      return PE_ERR_CUDA;
+    }
+    return PE_OK;
+  }
+  return launch_tc(di, X, dY, B, T, d_in, d_out, phi, 1, out_mean, out_stat, st, false, nullptr, accumulate);
+}
+
+// The same for layers that the SIMT kernel would otherwise serve, from copies whose rows are pitch_x, pitch_y elements
+// apart (multiples of 8; 0: back to back), held to that kernel's accuracy: at most TC_CHUNK_TOKENS tokens per accumulator, and sum_b G_b
+// from the examples' sums rather than from one accumulation over all rows.  out_sign != NULL: the three statistics of
+// pe_linear_stats_all (phi = square).
+static pe_status_t tc_linear_stats_pitched(DeviceInfo* di, const void* X, const void* dY, int B, int T, int d_in, int d_out, int phi,
+                                           float* out_mean, float* out_stat, float* out_sign, bool accumulate, int pitch_x, int pitch_y,
+                                           cudaStream_t st) {
+  g_last_path.store(PE_PATH_TENSOR);
+  auto run = [&](int f, float* mean, float* stat, float* sign) {
+    return launch_tc(di, X, dY, B, T, d_in, d_out, f, 1, mean, stat, st, false, sign, accumulate, nullptr, 0.f, pitch_x, pitch_y, true);
+  };
+  if (phi == PE_PHI_IDENTITY) {
+    pe_status_t rc = run(PE_PHI_SQUARE, out_mean ? out_mean : out_stat, nullptr, nullptr);
+    if (rc != PE_OK || !out_mean || !out_stat) return rc;
+    if (accumulate) return run(PE_PHI_SQUARE, out_stat, nullptr, nullptr);
+    if (cudaMemcpyAsync(out_stat, out_mean, (size_t)d_in * d_out * sizeof(float), cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
+      cudaGetLastError();
+      return PE_ERR_CUDA;
+    }
+    return PE_OK;
+  }
+  if (out_sign && T > TC_CHUNK_TOKENS) {
+    pe_status_t rc = run(PE_PHI_SQUARE, out_mean, out_stat, nullptr);
+    return rc == PE_OK ? run(PE_PHI_SIGN, nullptr, out_sign, nullptr) : rc;
+  }
+  return run(phi, out_mean, out_stat, out_sign);
+}
+
 template <typename TIn>
 static pe_status_t linear_stats_impl(const TIn* X, const TIn* dY, int B, int T, int d_in, int d_out, pe_phi_t phi,
                                      float* out_mean, float* out_stat, cudaStream_t st, bool allow_tc, bool accumulate = false) {
@@ -593,30 +656,7 @@ static pe_status_t linear_stats_impl(const TIn* X, const TIn* dY, int B, int T, 
   const bool tc_ok = allow_tc && tc_shape_ok(B, T, d_in, d_out);
   if (forced >= PE_PATH_TENSOR && !tc_ok) return PE_ERR_UNSUPPORTED_SHAPE;
   if (tc_ok && forced != PE_PATH_SIMT) {
-    if constexpr (sizeof(TIn) == 2) {
-      g_last_path.store(PE_PATH_TENSOR);
-      if (phi == PE_PHI_IDENTITY) {
-        // phi = identity: both outputs are the plain contraction over all B*T rows, and B and T only enter
-        // through B*T: regroup short sequences into full two-stage "examples" when the rows divide evenly.
-        regroup_rows(B, T);
-        float* first = out_mean ? out_mean : out_stat;
-        rc = launch_tc(di, X, dY, B, T, d_in, d_out, phi, 0, first, nullptr, st, false, nullptr, accumulate);
-        if (rc == PE_OK && out_mean && out_stat && accumulate)      // a copy would overwrite: contract once more into the second
-          return launch_tc(di, X, dY, B, T, d_in, d_out, phi, 0, out_stat, nullptr, st, false, nullptr, true);
-        if (rc == PE_OK && out_mean && out_stat) {
-          if (cudaMemcpyAsync(out_stat, out_mean, (size_t)d_in * d_out * sizeof(float), cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
-            cudaGetLastError();
-            return PE_ERR_CUDA;
-          }
-        }
-        return rc;
-      }
-      if (!out_stat) {    // only sum_b G_b wanted: the plain contraction
-        regroup_rows(B, T);
-        return launch_tc(di, X, dY, B, T, d_in, d_out, phi, 0, out_mean, nullptr, st, false, nullptr, accumulate);
-      }
-      return launch_tc(di, X, dY, B, T, d_in, d_out, phi, 1, out_mean, out_stat, st, false, nullptr, accumulate);
-    }
+    if constexpr (sizeof(TIn) == 2) return tc_linear_stats(di, X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, accumulate, st);
   }
   g_last_path.store(PE_PATH_SIMT);
   return launch_simt<TIn, MODE_STATS>(di, X, dY, B, T, d_in, d_out, (int)phi, out_mean, out_stat, st, accumulate);
@@ -677,7 +717,7 @@ static pe_status_t launch_tc_fused(DeviceInfo* di, const void* X, const void* dY
     rc = zero_for_split(di, adam ? out_a : nullptr, out_b, (size_t)d_in * d_out, st, nullptr, counters, (int)blocks);
     if (rc != PE_OK) return rc;
   }
-  TcParams p;
+  TcParams p{};
   p.B = B; p.T = T; p.d_in = d_in; p.d_out = d_out; p.nsplit = ns; p.per_example = 1; p.half_operands = 0; p.accumulate = 0;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, nt, ns, di->sm_count / 2);
   p.out_mean = adam ? out_a : nullptr; p.out_stat = out_b; p.out_sign = nullptr; p.out_norms = nullptr; p.dev_status = di->status_ptr;
@@ -804,6 +844,147 @@ pe_status_t pe_linear_stats_all(const void* X, const void* dY, int B, int T, int
   rc = linear_stats_impl<__nv_bfloat16>(Xb, Yb, B, T, d_in, d_out, PE_PHI_SQUARE, out_mean, out_square, st, true);
   if (rc != PE_OK) return rc;
   return linear_stats_impl<__nv_bfloat16>(Xb, Yb, B, T, d_in, d_out, PE_PHI_SIGN, nullptr, out_sign, st, true);
+}
+
+// Copies of the operands at 16-byte row pitches: X's, then dY's, each 256-byte aligned; a tensor whose width is a multiple of 8
+// needs none.
+struct PaddedLayout {
+  int pitch_x, pitch_y;
+  size_t x_bytes, y_bytes;
+};
+static PaddedLayout padded_layout(int B, int T, int d_in, int d_out, bool always) {
+  PaddedLayout l;
+  l.pitch_x = (d_in + 7) & ~7;
+  l.pitch_y = (d_out + 7) & ~7;
+  l.x_bytes = (always || d_in % 8) ? align_up((size_t)B * T * l.pitch_x * 2, 256) : 0;
+  l.y_bytes = (always || d_out % 8) ? align_up((size_t)B * T * l.pitch_y * 2, 256) : 0;
+  return l;
+}
+// Widths that are no multiples of 8: from this many multiply-adds on, copying the operands to a padded pitch and
+// contracting them on the tensor cores beats the SIMT kernel.  Three launches against one, 20.8 us of host time per call:
+// 4 x 64 x 129 x 255 (2^23) 10.4 us SIMT, 8 x 64 x 257 x 511 (2^26) 24.0, 8 x 256 x 129 x 257 (2^26) 22.7,
+// 16 x 64 x 513 x 511 (2^28) 49.4, 16 x 128 x 513 x 511 (2^29) 87.2.
+constexpr long long PAD_MIN_MACS = 1ll << 26;
+static bool padding_pays(int B, int T, int d_in, int d_out) {
+  return B > 0 && T > 0 && (d_in % 8 || d_out % 8) && tc_shape_ok(B, T, (d_in + 7) & ~7, (d_out + 7) & ~7) &&
+         (double)B * T * d_in * d_out >= (double)PAD_MIN_MACS && (long long)B * T < (1ll << 31);
+}
+
+size_t pe_linear_stats_padded_workspace_bytes(int B, int T, int d_in, int d_out) {
+  if (B < 1 || T < 1 || d_in < 1 || d_out < 1 || g_path.load() != PE_PATH_AUTO || !padding_pays(B, T, d_in, d_out)) return 0;
+  const PaddedLayout l = padded_layout(B, T, d_in, d_out, false);
+  return l.x_bytes + l.y_bytes;
+}
+
+pe_status_t pe_linear_stats_padded(const void* X, const void* dY, int B, int T, int d_in, int d_out, pe_phi_t phi, int accumulate,
+                                   float* out_mean, float* out_stat, float* out_sign, void* workspace, size_t workspace_bytes,
+                                   pe_stream_t stream) {
+  const size_t need = pe_linear_stats_padded_workspace_bytes(B, T, d_in, d_out);
+  if (out_sign && (accumulate || phi != PE_PHI_SQUARE)) return PE_ERR_PHI;
+  if (need == 0) {
+    if (out_sign) return pe_linear_stats_all(X, dY, B, T, d_in, d_out, out_mean, out_stat, out_sign, stream);
+    return accumulate ? pe_linear_stats_accumulate(X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, stream)
+                      : pe_linear_stats(X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, stream);
+  }
+  if (out_sign && (!out_mean || !out_stat)) return PE_ERR_NULL;
+  pe_status_t rc = validate_stats(X, dY, B, T, d_in, d_out, out_mean, out_stat, true, 16);
+  if (rc != PE_OK) return rc;
+  if (phi != PE_PHI_IDENTITY && phi != PE_PHI_SQUARE && phi != PE_PHI_SIGN) return PE_ERR_PHI;
+  if (out_sign && !aligned(out_sign, 16)) return PE_ERR_ALIGN;
+  if (!workspace || workspace_bytes < need) return PE_ERR_WORKSPACE;
+  if (!aligned(workspace, 256)) return PE_ERR_ALIGN;
+  DeviceInfo* di = nullptr;
+  rc = device_info(&di);
+  if (rc != PE_OK) return rc;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  const PaddedLayout l = padded_layout(B, T, d_in, d_out, false);
+  const long long rows = (long long)B * T;
+  PadTensor px = {static_cast<const uint16_t*>(X), static_cast<uint16_t*>(workspace), d_in, l.pitch_x};
+  PadTensor py = {static_cast<const uint16_t*>(dY), reinterpret_cast<uint16_t*>(static_cast<char*>(workspace) + l.x_bytes), d_out, l.pitch_y};
+  const bool pad_x = l.x_bytes > 0, pad_y = l.y_bytes > 0;
+  const long long groups = rows * ((pad_x && pad_y ? std::max(l.pitch_x, l.pitch_y) : pad_x ? l.pitch_x : l.pitch_y) / 8);
+  long long blocks = (groups + 4 * LAYOUT_THREADS - 1) / (4 * LAYOUT_THREADS);
+  if (blocks > 16ll * di->sm_count) blocks = 16ll * di->sm_count;
+  pad_rows_kernel<<<dim3((unsigned)blocks, pad_x && pad_y ? 2 : 1), LAYOUT_THREADS, 0, st>>>(pad_x ? px : py, py, rows);
+  rc = check_launch();
+  if (rc != PE_OK) return rc;
+  return tc_linear_stats_pitched(di, pad_x ? (const void*)px.dst : X, pad_y ? (const void*)py.dst : dY, B, T, d_in, d_out, phi, out_mean, out_stat, out_sign,
+                         accumulate != 0, l.pitch_x, l.pitch_y, st);
+}
+
+// Tile of the unfolding kernel: output positions of one row and channels per round, so that a block's shared memory (input rows
+// and feature table) stays within its budget.  False: a receptive field too large for that.
+struct UnfoldTile {
+  int tile_w, chan, cols, smem;
+};
+static bool unfold_tile(const ConvGeom& g, UnfoldTile* t) {
+  const int kk = g.Kh * g.Kw;
+  auto smem = [&](int chan, int cols) { return (long long)((chan * kk + 7) / 8 * 8) * 4 + ((long long)chan * g.Kh * cols + 8) * 2; };
+  auto cols_of = [&](int w) { return (long long)(w - 1) * g.sw + (long long)(g.Kw - 1) * g.dw + 1; };
+  for (int w = g.Wo < 128 ? g.Wo : 128;; w = (w + 1) / 2) {
+    const long long cols = cols_of(w);
+    for (int chan = g.C; chan > 0; chan = chan > 8 ? (chan - 1) / 8 * 8 : 0) {
+      if ((long long)chan * kk < (1 << 14) && cols < (1 << 16) && smem(chan, (int)cols) <= UNFOLD_SMEM_BYTES) {
+        *t = {w, chan, (int)cols, (int)smem(chan, (int)cols)};
+        return true;
+      }
+    }
+    if (w == 1) return false;
+  }
+}
+static bool conv_geom(int B, int C, int H, int W, int F, int Kh, int Kw, int sh, int sw, int ph, int pw, int dh, int dw, ConvGeom* g) {
+  if (B < 1 || C < 1 || H < 1 || W < 1 || F < 1 || Kh < 1 || Kw < 1 || sh < 1 || sw < 1 || ph < 0 || pw < 0 || dh < 1 || dw < 1) return false;
+  const long long ho = ((long long)H + 2ll * ph - (long long)dh * (Kh - 1) - 1) / sh + 1, wo = ((long long)W + 2ll * pw - (long long)dw * (Kw - 1) - 1) / sw + 1;
+  if ((long long)H + 2ll * ph < (long long)dh * (Kh - 1) + 1 || (long long)W + 2ll * pw < (long long)dw * (Kw - 1) + 1) return false;
+  if (ho > 65535 || wo > (1 << 24) || B > 65535 || (double)C * Kh * Kw >= (double)(1 << 28) || (double)ho * wo * B >= (double)(1ll << 31)) return false;
+  *g = {B, C, H, W, F, Kh, Kw, sh, sw, ph, pw, dh, dw, (int)ho, (int)wo};
+  return true;
+}
+
+size_t pe_conv2d_stats_workspace_bytes(int B, int C, int H, int W, int F, int Kh, int Kw, int stride_h, int stride_w, int pad_h, int pad_w,
+                                       int dil_h, int dil_w) {
+  ConvGeom g;
+  UnfoldTile t;
+  if (!conv_geom(B, C, H, W, F, Kh, Kw, stride_h, stride_w, pad_h, pad_w, dil_h, dil_w, &g) || !unfold_tile(g, &t)) return 0;
+  const PaddedLayout l = padded_layout(B, g.Ho * g.Wo, C * Kh * Kw, F, true);
+  return l.x_bytes + l.y_bytes;
+}
+
+pe_status_t pe_conv2d_stats(const void* x, const void* grad_out, int B, int C, int H, int W, int F, int Kh, int Kw, int stride_h, int stride_w,
+                            int pad_h, int pad_w, int dil_h, int dil_w, pe_phi_t phi, float* out_mean, float* out_stat, void* workspace,
+                            size_t workspace_bytes, pe_stream_t stream) {
+  ConvGeom g;
+  UnfoldTile t;
+  if (!conv_geom(B, C, H, W, F, Kh, Kw, stride_h, stride_w, pad_h, pad_w, dil_h, dil_w, &g)) return PE_ERR_DIM;
+  if (!unfold_tile(g, &t)) return PE_ERR_UNSUPPORTED_SHAPE;
+  if (!x || !grad_out) return PE_ERR_NULL;
+  const int T = g.Ho * g.Wo, d_in = C * Kh * Kw;
+  const PaddedLayout l = padded_layout(B, T, d_in, F, true);
+  if (!workspace || workspace_bytes < l.x_bytes + l.y_bytes) return PE_ERR_WORKSPACE;
+  if (!aligned(workspace, 256) || !aligned(x, 2) || !aligned(grad_out, 2)) return PE_ERR_ALIGN;
+  uint16_t* const X = static_cast<uint16_t*>(workspace);
+  uint16_t* const dY = reinterpret_cast<uint16_t*>(static_cast<char*>(workspace) + l.x_bytes);
+  pe_status_t rc = validate_stats(X, dY, B, T, d_in, F, out_mean, out_stat, true, 16);
+  if (rc != PE_OK) return rc;
+  if (phi != PE_PHI_IDENTITY && phi != PE_PHI_SQUARE && phi != PE_PHI_SIGN) return PE_ERR_PHI;
+  const int forced = g_path.load();
+  const bool whole = tc_shape_ok(B, T, d_in, F);
+  if (forced >= PE_PATH_TENSOR && !whole) return PE_ERR_UNSUPPORTED_SHAPE;
+  DeviceInfo* di = nullptr;
+  rc = device_info(&di);
+  if (rc != PE_OK) return rc;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  unfold_kernel<<<dim3((g.Wo + t.tile_w - 1) / t.tile_w, g.Ho, B), LAYOUT_THREADS, t.smem, st>>>(static_cast<const uint16_t*>(x), X, g, l.pitch_x, t.tile_w,
+                                                                                                   t.chan, t.cols);
+  if ((rc = check_launch()) != PE_OK) return rc;
+  transpose_rows_kernel<<<dim3((T + 63) / 64, (l.pitch_y + 63) / 64, B), LAYOUT_THREADS, 0, st>>>(static_cast<const uint16_t*>(grad_out), dY, F, T, l.pitch_y);
+  if ((rc = check_launch()) != PE_OK) return rc;
+  if (forced != PE_PATH_SIMT && whole) return tc_linear_stats(di, X, dY, B, T, d_in, F, phi, out_mean, out_stat, false, st);
+  if (forced != PE_PATH_SIMT && padding_pays(B, T, d_in, F))
+    return tc_linear_stats_pitched(di, X, dY, B, T, d_in, F, phi, out_mean, out_stat, nullptr, false, l.pitch_x, l.pitch_y, st);
+  g_last_path.store(PE_PATH_SIMT);
+  return launch_simt<__nv_bfloat16, MODE_STATS>(di, reinterpret_cast<const __nv_bfloat16*>(X), reinterpret_cast<const __nv_bfloat16*>(dY), B, T, d_in, F,
+                                                (int)phi, out_mean, out_stat, st, false, SimtExtra{}, nullptr, l.pitch_x, l.pitch_y);
 }
 
 size_t pe_linear_stats_ragged_workspace_bytes(int B, int d_in, int d_out) {
@@ -1094,7 +1275,7 @@ static pe_status_t launch_tc_fp8(DeviceInfo* di, const void* x8, const void* y8,
     rc = zero_for_split(di, out, nullptr, (size_t)d_in * d_out, st);
     if (rc != PE_OK) return rc;
   }
-  TcParams p;
+  TcParams p{};
   p.B = B; p.T = T; p.d_in = d_in; p.d_out = d_out; p.nsplit = ns; p.per_example = 0; p.half_operands = 0; p.accumulate = 0;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, 256, ns, di->sm_count / 2);
   p.out_mean = nullptr; p.out_stat = out; p.out_sign = nullptr; p.out_norms = nullptr; p.dev_status = di->status_ptr;

@@ -116,11 +116,12 @@ __device__ __forceinline__ int micro_index(int thread, int j) { return N <= 4 ? 
 // accumulate != 0 the results are added to whatever the outputs hold.  opt.kind != 0 (one cluster only): the block that
 // ends up with an entry's sums also applies the parameter update (phi must then be square for the Adam family,
 // sign for MicroSignSGD); out_mean / out_stat may then be NULL.
+// ldx, ldy: elements from one token's row of X, dY to the next.
 // SUMS: running sums per entry: 2 = sum_b phi(G_b) and sum_b G_b, 1 = the former alone (or the contraction of MODE_TOKEN).
 template <typename TIn, int MODE, class Tile, int SUMS>
 __global__ void __launch_bounds__(SIMT_THREADS, 2)
 simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, int T, int d_in, int d_out,
-                  int phi, float* __restrict__ out_mean, float* __restrict__ out_stat, int accumulate, int cluster, int vec_x, int vec_y,
+                  int phi, float* __restrict__ out_mean, float* __restrict__ out_stat, int accumulate, int cluster, int ldx, int ldy, int vec_x, int vec_y,
                   SimtExtra ex, FusedOpt opt) {
   constexpr int TM = Tile::TM, TN = Tile::TN, KT = Tile::KT, ROWS = Tile::ROWS, COLS = Tile::COLS;
   constexpr bool IN_SMEM = Tile::SUMS_IN_SMEM && MODE == MODE_STATS;
@@ -189,13 +190,13 @@ simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, 
     for (int k = 0; k < Tile::YV; ++k) {
       const int v = threadIdx.x + k * SIMT_THREADS, tt = t + v / (ROWS / 4), c = o0 + 4 * (v % (ROWS / 4));
       sy[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (tt < Tb && c < d_out) sy[k] = load_group(dY + (size_t)(row0 + tt) * d_out, c, d_out, vec_y != 0);
+      if (tt < Tb && c < d_out) sy[k] = load_group(dY + (size_t)(row0 + tt) * ldy, c, d_out, vec_y != 0);
     }
 #pragma unroll
     for (int k = 0; k < Tile::XV; ++k) {
       const int v = threadIdx.x + k * SIMT_THREADS, tt = t + v / (COLS / 4), c = i0 + 4 * (v % (COLS / 4));
       sx[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (tt < Tb && c < d_in) sx[k] = load_group(X + (size_t)(row0 + tt) * d_in, c, d_in, vec_x != 0);
+      if (tt < Tb && c < d_in) sx[k] = load_group(X + (size_t)(row0 + tt) * ldx, c, d_in, vec_x != 0);
     }
   };
   auto put = [&](float* at, float4 v) {

@@ -79,6 +79,7 @@ __host__ __device__ constexpr int tc_smem_budget(int nt) { return (nt == 192 ? 2
 __host__ __device__ constexpr int tc_default_bk(bool tf32, int nt) { return tf32 ? 32 : (nt == 256 ? 64 : 128); }
 constexpr int TC_SHORT_BK = 32;
 constexpr int TC_SHORT_T = 32;
+constexpr int TC_CHUNK_TOKENS = 512;    // CHUNKED: tokens per accumulator
 // F8: 8-bit operands (kind::f8f6f4, e4m3, 32 tokens per instruction): the scaled squares of the two-pass
 // per-token statistic's fp8 form.
 template <bool TF32, int NT, int BK_ = tc_default_bk(TF32, NT), bool F8 = false>
@@ -125,7 +126,6 @@ struct TcOperand {
   // 96 floats each need the larger epilogue share.
   static constexpr int REGS_CONTROL = (NT == 192) ? 40 : TC_REGS_CONTROL;
   static constexpr int REGS_EPILOGUE = (NT == 192) ? 232 : TC_REGS_EPILOGUE;
-  static_assert(128 * REGS_CONTROL + 256 * REGS_EPILOGUE <= TC_THREADS * TC_REGS_AT_LAUNCH, "setmaxnreg: the epilogue's increase must fit what the control warps give up");
 };
 
 // error codes latched in the device status word (which wait gave up)
@@ -139,6 +139,7 @@ struct TcParams {
                        // 0: one accumulation over the whole slice (plain contraction, phi = identity)
   int half_operands;   // 16-bit operands are IEEE half instead of bf16 (the staged per-token statistic)
   int accumulate;      // add the results to what the outputs hold (no zeroing kernel runs before this one)
+  int scalar_out;      // d_in % 4 != 0: the outputs' rows are no 16-byte multiples, so the warps write them themselves
   float* out_mean;     // may be NULL; written through tmap_mean
   float* out_stat;     // may be NULL; written through tmap_stat
   float* out_sign;     // MEAN_REGS_SIGN only: sum_b sign(G_b), written through tmap_sign
@@ -228,19 +229,26 @@ __device__ __forceinline__ float phi_apply(float g) {
 
 // Zeroes the outputs of a split-batch launch.  The statistics kernel that follows is launched as a
 // programmatic dependent: it starts right away (it only touches the outputs in its very last step,
-// behind griddepcontrol.wait), so the zeroing costs no time on the stream.  a, b, c: n4 float4 each; b and
+// behind griddepcontrol.wait), so the zeroing costs no time on the stream.  a, b, c: n floats each, 16-byte aligned; b and
 // c may be NULL.  counters: the tile counters of a fused update (n_counters words; may be NULL).
 __global__ void __launch_bounds__(256) zero_outputs_kernel(float4* __restrict__ a, float4* __restrict__ b, float4* __restrict__ c,
-                                                           long long n4, unsigned int* __restrict__ counters, int n_counters) {
+                                                           long long n, unsigned int* __restrict__ counters, int n_counters) {
   sm100::griddep_launch_dependents();
   const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
   const long long stride = (long long)gridDim.x * blockDim.x;
   if (counters)
     for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n_counters; k += stride) counters[k] = 0u;
+  const long long n4 = n >> 2;
   for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n4; k += stride) {
     a[k] = z;
     if (b) b[k] = z;
     if (c) c[k] = z;
+  }
+  const long long k = (n4 << 2) + threadIdx.x;             // the last n % 4
+  if (blockIdx.x == 0 && k < n) {
+    reinterpret_cast<float*>(a)[k] = 0.f;
+    if (b) reinterpret_cast<float*>(b)[k] = 0.f;
+    if (c) reinterpret_cast<float*>(c)[k] = 0.f;
   }
 }
 
@@ -327,9 +335,13 @@ __device__ __forceinline__ void fused_update_piece(const FusedOpt& o, const TcPa
 // RAGGED: packed batch with per-example token ranges (tmap_x / tmap_dy are then (d, rows, 1), tmap_x_tail /
 // tmap_dy_tail (d, 16, B) over the zero-padded last partial token groups); otherwise the tail maps are unused.
 // PHI: 0 identity, 1 square, 2 sign, 3 the clipping scale c_b * g with c_b = min(1, C / sqrt(N_b)).
+// CHUNKED: an example's tokens are contracted TC_CHUNK_TOKENS at a time, each run into an accumulator of its own, and the
+// runs are added in registers (round to nearest).  The tensor core truncates when it adds to an accumulator, which shrinks a sum of
+// n instructions by about n * 2^-25: 6e-6 (G_b) and 1.2e-5 (G_b^2) at 6000 tokens, against 5e-7 and 1e-6 with runs of 512, what
+// fp32 FMAs in order give too.  64 more registers per epilogue thread, hence the 256 x 128 tile.
 // OPT: the parameter update applied by the block that completes a tile's sums (OPT_ADAM needs both running
 // sums, OPT_SIGN the sign statistic alone); `o` is ignored when OPT == OPT_NONE.
-template <int PHI, bool TF32, int NT, int MEAN, int BKT = tc_default_bk(TF32, NT), bool RAGGED = false, int OPT = OPT_NONE, bool F8 = false>
+template <int PHI, bool TF32, int NT, int MEAN, int BKT = tc_default_bk(TF32, NT), bool RAGGED = false, int OPT = OPT_NONE, bool F8 = false, bool CHUNKED = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
 tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_dy,
                 const __grid_constant__ CUtensorMap tmap_mean, const __grid_constant__ CUtensorMap tmap_stat,
@@ -349,6 +361,10 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   static_assert(MEAN != MEAN_TMEM || (NT == 256 && PHI != 0), "the tensor-memory mean sits beside one 256-column accumulator");
   static_assert(!RAGGED || (!TF32 && MEAN != MEAN_TMEM), "packed batches: 16-bit operands, several accumulators");
   static_assert(PHI != 3 || MEAN == MEAN_NONE, "the clipped sum is a statistic-only pass");
+  static_assert(!CHUNKED || (MEAN == MEAN_REGS && NT == 128 && !RAGGED && OPT == OPT_NONE && Op::GROUP == 1), "runs of an example: the two-sum kernel on the 256 x 128 tile");
+  constexpr int CHUNK_STAGES = CHUNKED ? TC_CHUNK_TOKENS / BKT : 1;
+  constexpr int REGS_CONTROL = CHUNKED ? 40 : Op::REGS_CONTROL, REGS_EPILOGUE = CHUNKED ? 232 : Op::REGS_EPILOGUE;
+  static_assert(128 * REGS_CONTROL + 256 * REGS_EPILOGUE <= TC_THREADS * TC_REGS_AT_LAUNCH, "setmaxnreg: the epilogue's increase must fit what the control warps give up");
   static_assert(OPT != OPT_ADAM || (MEAN == MEAN_REGS && PHI == 1), "the Adam family consumes sum_b G_b and sum_b G_b^2");
   static_assert(OPT != OPT_SIGN || (MEAN == MEAN_NONE && PHI == 2), "MicroSignSGD consumes sum_b sign(G_b)");
   constexpr int STAGES = Op::STAGES, BK = Op::BK;
@@ -398,7 +414,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   // read per thread; the producer / MMA warpgroup needs little.  Each setmaxnreg sits inside the
   // branch of the role it applies to.
   if (warp < 4) {
-    setmaxnreg_dec<Op::REGS_CONTROL>();
+    setmaxnreg_dec<REGS_CONTROL>();
     const bool strict = wait_cycle_limit() < WAIT_CYCLE_LIMIT_STRICT;
     if (warp == 0 || warp == 2) {
       // ---------------------------------------------------------- TMA producers (both blocks)
@@ -447,17 +463,26 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       const uint32_t idesc = (F8 || (!TF32 && p.half_operands)) ? make_idesc_half_mn_major(TC_PAIR_M, NT) : make_idesc_mn_major(TC_PAIR_M, NT, TF32);
       int s = 0;
       uint32_t ph = 0;
+      int run = 0;                    // CHUNKED: accumulators filled so far
       bool ok = true;
       for (int e = 0; e < nu && ok; ++e) {
         const SeqGeom sg = seq_geom<RAGGED>(p, b_begin + GROUP * e, BK);
-        const int buf = e % UNITS;
-        if (p.per_example) {
+        int buf = e % UNITS;
+        if (p.per_example && !CHUNKED) {
           if (!mbar_wait_warp(acc_empty_bar(buf), ((uint32_t)(e / UNITS) & 1u) ^ 1u, abort_flag, p.dev_status, TC_WAIT_ACC_EMPTY, strict)) break;
           tc_fence_after();
         }
         const bool last_of_acc = p.per_example || e + UNITS >= nu;
-        const uint32_t d_tmem = tmem_base + (uint32_t)(buf * GROUP * NT);
         for (int kc = 0; kc < sg.nk; ++kc) {
+          const int kin = CHUNKED ? kc % CHUNK_STAGES : kc;           // stage within its accumulator
+          const bool acc_done = kc == sg.nk - 1 || (CHUNKED && kin == CHUNK_STAGES - 1);
+          if (CHUNKED && kin == 0) {
+            buf = run % UNITS;
+            if (!mbar_wait_warp(acc_empty_bar(buf), ((uint32_t)(run / UNITS) & 1u) ^ 1u, abort_flag, p.dev_status, TC_WAIT_ACC_EMPTY, strict)) { ok = false; break; }
+            tc_fence_after();
+            ++run;
+          }
+          const uint32_t d_tmem = tmem_base + (uint32_t)(buf * GROUP * NT);
           if (!mbar_wait_warp(full_bar(s), ph, abort_flag, p.dev_status, TC_WAIT_FULL, strict)) { ok = false; break; }
           tc_fence_after();
           if (elect_one()) {
@@ -469,7 +494,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
             for (int j = 0; j < GROUP; ++j) {
               // grouped examples: example j of the group sits BK tokens further in every box and has its own accumulator
               if (GROUP > 1 && GROUP * e + j >= nb) break;
-              uint32_t accumulate = (kc > 0 || (!p.per_example && e >= UNITS)) ? 1u : 0u;
+              uint32_t accumulate = (kin > 0 || (!p.per_example && e >= UNITS)) ? 1u : 0u;
 #pragma unroll
               for (int k = 0; k < BK / Op::MMA_K; ++k) {
                 // rows past T are zero-filled by TMA; whole MMA steps past T are skipped
@@ -483,7 +508,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
               }
             }
             umma_commit_pair(empty_bar(s));                // stage reusable in both blocks once these MMAs retire
-            if (last_of_acc && kc == sg.nk - 1) umma_commit_pair(acc_full_bar(buf));   // accumulator complete, both blocks
+            if (last_of_acc && acc_done) umma_commit_pair(acc_full_bar(buf));   // accumulator complete, both blocks
           }
           __syncwarp();
           if (++s == STAGES) { s = 0; ph ^= 1u; }
@@ -492,7 +517,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     }
   } else {
     // ------------------------------------------------------------ epilogue (both blocks)
-    setmaxnreg_inc<Op::REGS_EPILOGUE>();
+    setmaxnreg_inc<REGS_EPILOGUE>();
     const int q = warp & 3;                 // TMEM lane quadrant this warp may access
     const int h = (warp - 4) >> 2;          // column half of the tile
     constexpr bool KEEP_MEAN = MEAN == MEAN_REGS || MEAN == MEAN_REGS_SIGN || PHI == 0;     // running sum of G_b in registers
@@ -515,7 +540,12 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     for (int j = 0; j < N_MEAN; ++j) acc_mean[j] = 0.f;
     bool ok = true;
     // per-example mode: one accumulator unit per example (or group), in order; plain mode: each accumulator once
-    const int n_acc = p.per_example ? nu : min(nu, UNITS);
+    const int n_runs = CHUNKED ? (p.T + TC_CHUNK_TOKENS - 1) / TC_CHUNK_TOKENS : 1;      // accumulators per example
+    const int n_acc = p.per_example ? nu * n_runs : min(nu, UNITS);
+    constexpr int N_RUN = CHUNKED ? COLS : 1;
+    float acc_run[N_RUN];           // CHUNKED: the sum of the example's runs so far
+#pragma unroll
+    for (int j = 0; j < N_RUN; ++j) acc_run[j] = 0.f;
     const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
     for (int a = 0; a < n_acc; ++a) {
       const int buf = a % UNITS;
@@ -624,7 +654,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       } else {
         // CH columns per tensor-memory read: 32, or 16 where the running sums leave few registers (NT = 192; the three
         // statistics on the 256 x 128 tile, whose 160 registers of sums leave room for two reads of 16 in flight, not 32)
-        constexpr int CH = (NT == 192 || TRIPLE) ? 16 : 32;
+        constexpr int CH = (NT == 192 || TRIPLE || CHUNKED) ? 16 : 32;
         constexpr int NCH = COLS / CH;                // reads per example
         // grouped examples: the unit's accumulators one after the other; the unit is released after the last read
         const int in_unit = (GROUP > 1) ? min(GROUP, nb - GROUP * a) : 1;
@@ -701,7 +731,20 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
               if constexpr (CH == 32) tmem_ld_32x32b_x32_wait(taddr_j + c * CH, r);
               else tmem_ld_32x32b_x16_wait(taddr_j + c * CH, r);
               if (c == NCH - 1 && ju == in_unit - 1) release_unit();
-              fold(r, c);
+              if constexpr (CHUNKED) {
+                const bool last_run = a % n_runs == n_runs - 1;
+#pragma unroll
+                for (int j = 0; j < CH; j += 2) {
+                  float lo, hi;
+                  f32x2_unpack(f32x2_add(f32x2_pack(acc_run[c * CH + j], acc_run[c * CH + j + 1]), f32x2_pack(__uint_as_float(r[j]), __uint_as_float(r[j + 1]))), lo, hi);
+                  r[j] = __float_as_uint(lo); r[j + 1] = __float_as_uint(hi);
+                  acc_run[c * CH + j] = last_run ? 0.f : lo;
+                  acc_run[c * CH + j + 1] = last_run ? 0.f : hi;
+                }
+                if (last_run) fold(r, c);
+              } else {
+                fold(r, c);
+              }
             }
           }
         }
@@ -739,7 +782,25 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         for (int k = 0; k < 8; ++k)
           *reinterpret_cast<float4*>(dst + ((k ^ (lane & 7)) << 4)) = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
       };
-      auto send = [&](const CUtensorMap* tm, uint32_t first_panel) {
+      auto send = [&](const CUtensorMap* tm, float* out, uint32_t first_panel) {
+        if (p.scalar_out) {
+          if (p.nsplit > 1 && !p.accumulate) griddep_wait();
+          __syncwarp();
+          for (int c = 0; c < PANELS; ++c) {
+            const int col = col0 + c * 32 + lane;
+            const uint8_t* src = smem_gen + (first_panel + c * 4096 - smem_base) + (lane & 3) * 4;
+            for (int r = 0; r < 32 && row0 + r < p.d_out; ++r) {
+              const float v = *reinterpret_cast<const float*>(src + r * 128 + (((lane >> 2) ^ (r & 7)) << 4));
+              if (col < p.d_in) {
+                float* const at = out + (size_t)(row0 + r) * p.d_in + col;
+                if (p.nsplit == 1 && !p.accumulate) *at = v;
+                else atomicAdd(at, v);
+              }
+            }
+          }
+          __syncwarp();           // the panels may be refilled for the next output
+          return;
+        }
         fence_async_smem();
         __syncwarp();
         if (row0 < p.d_out && elect_one()) {
@@ -757,7 +818,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       if (p.out_stat || stage_for_update) {
 #pragma unroll
         for (int c = 0; c < PANELS; ++c) put_panel(stage_base + c * 4096, (PHI != 0) ? &acc_stat[c * 32] : &acc_mean[c * 32]);
-        if (p.out_stat) send(&tmap_stat, stage_base);
+        if (p.out_stat) send(&tmap_stat, p.out_stat, stage_base);
       }
       // sum_b G_b
       if ((p.out_mean || (stage_for_update && OPT == OPT_ADAM)) && (KEEP_MEAN || MEAN == MEAN_TMEM || HYBRID)) {
@@ -793,7 +854,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
 #pragma unroll
           for (int c = 0; c < PANELS; ++c) put_panel(first + c * 4096, &acc_mean[c * 32]);
         }
-        if (p.out_mean) send(&tmap_mean, first);
+        if (p.out_mean) send(&tmap_mean, p.out_mean, first);
       }
       if constexpr (TRIPLE) {
         // sum_b sign(G_b): the warp's staging area is in use, so wait until TMA has read it
@@ -808,7 +869,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
             for (int j = 0; j < 32; ++j) v[j] = (float)((acc_cnt[(c * 32 + j) >> 1] >> (16 * (j & 1))) & 0xFFFFu) - nbf;
             put_panel(stage_base + c * 4096, v);
           }
-          send(&tmap_sign, stage_base);
+          send(&tmap_sign, p.out_sign, stage_base);
         }
       }
       if (elect_one()) bulk_wait_read_all();       // shared memory must outlive TMA's reads
