@@ -29,19 +29,10 @@ static std::atomic<int> g_path{PE_PATH_AUTO};
 static std::atomic<int> g_last_path{PE_PATH_AUTO};
 static std::atomic<long long> g_launches{0};
 static std::atomic<int> g_fused_mode{PE_FUSED_AUTO};
-// Both outputs: from this sequence length on the running sum of G_b lives in tensor memory beside a
-// 256-column accumulator (measured: wins or ties at T = 4096, loses 16 % at T = 2048, 17 % at T = 1024).
+// Both outputs of a layer whose d_in fills neither 192- nor 128-column tiles well: from this sequence length on the running sum
+// of G_b may live in tensor memory beside a 256-column accumulator.
 constexpr int TC_MEAN_TMEM_MIN_T = 4096;
-// Both outputs, phi = square or sign: from this sequence length on the pair tile is 256 x 192 instead of
-// 256 x 128 (measured: ties at T = 64 and 128, 3-21 % faster from T = 256 on, 17-25 % faster than the
-// tensor-memory mean at T = 4096; 18-22 % slower at T = 32), unless d_in is so narrow that the wider
-// tile's padding (columns up to the next multiple of 192) eats the gain.
-constexpr int TC_WIDE_MIN_T = 64;
 constexpr int TC_WIDE_MAX_PAD_PERCENT = 13;
-// The three-statistic pass on the 256 x 192 tile keeps two thirds of sum_b G_b in tensor memory (a read, an add
-// and a write per example): it needs longer sequences than the two-sum kernel to hide that epilogue (measured: 6-8 % faster
-// than the 256 x 128 one-pass kernel at T = 512 and 1024, 10 % slower at T = 256).
-constexpr int TC_WIDE_TRIPLE_MIN_T = 512;
 constexpr int PHI_CLIP_SCALE = 3;   // internal phi of the clipped sum: c_b * G_b (not part of pe_phi_t)
 constexpr int TC_BAND = 8;          // pair rows per band of the tile order (8 x 256 rows of d_out)
 
@@ -166,16 +157,56 @@ static bool tc_shape_ok(int B, int T, int d_in, int d_out) {
   return true;
 }
 
-// Batch slices per tile: minimise (waves of thread blocks) x (examples per slice) plus a flush term.
-static int choose_nsplit(long long tiles, int B, int T, int slots, int max_split) {
-  int best = 1;
+// What a unit of work (one tile, one slice of the batch) costs a CTA pair on a given kernel, in microseconds, for choosing the tile
+// and the number of slices.  Fitted to sweeps of both over layers from 512 x 512 to 1024 x 32104 with T = 1 to 1000.
+struct UnitCost {
+  int nt;                     // d_in columns per tile
+  double token_lo, token_hi;  // per token of an example, with few pairs running and with all of them (operand supply from L2)
+  double example;             // added per example
+  double example_min;         // at least this much per example (what the epilogue takes)
+  double fixed;               // per unit: prologue, first stage, write-out, teardown
+};
+constexpr double FUSED_UPDATE_FIXED = 20.0;       // the parameter update of a 256 x 192 tile inside the statistics kernel
+constexpr double SPLIT_FIXED = 2.0;               // adding to the outputs instead of storing, per unit
+constexpr double ZERO_BYTES_PER_US = 6.4e6;       // zeroing the outputs of a split launch
+constexpr UnitCost COST_STAT = {256, 0.51 / 128, 0.68 / 128, 0.0, 0.34, 8.5};            // one statistic (square, clipping) on 256 x 256
+constexpr UnitCost COST_SIGN = {256, 0.51 / 128, 0.68 / 128, 0.0, 0.66, 8.5};
+constexpr UnitCost COST_NORMS = {256, 0.51 / 128, 0.68 / 128, 0.0, 0.30, 7.0};
+constexpr UnitCost COST_PLAIN = {256, 0.51 / 128, 0.68 / 128, 0.0, 0.0, 8.5};
+constexpr UnitCost COST_TOKEN = {TOK_NT, 0.42 / TOK_BK, 0.45 / TOK_BK, 0.0, 0.0, 8.5};     // an "example" is one 32-row stage
+constexpr UnitCost COST_PLAIN_FP8 = {256, 0.28 / 128, 0.40 / 128, 0.0, 0.0, 8.5};
+constexpr UnitCost COST_BOTH_192 = {192, 0.375 / 128, 0.55 / 128, 0.02, 0.35, 10.0};     // two sums
+constexpr UnitCost COST_BOTH_128 = {128, 0.35 / 128, 0.44 / 128, 0.12, 0.20, 8.3};
+constexpr UnitCost COST_BOTH_SHORT = {128, 0.05 / 32, 0.10 / 32, 0.0, 0.245, 8.3};       // two examples per stage (T <= 32)
+constexpr UnitCost COST_ALL_192 = {192, 0.375 / 128, 0.60 / 128, 0.05, 0.95, 11.0};      // three statistics
+constexpr UnitCost COST_ALL_128 = {128, 0.35 / 128, 0.44 / 128, 0.16, 0.55, 9.5};
+constexpr UnitCost COST_ALL_SHORT = {128, 0.05 / 32, 0.10 / 32, 0.0, 0.54, 9.5};
+
+// Time of a launch of `tiles` tiles in ns slices of the batch: waves of `slots` pairs, the last one with fewer pairs.
+static double launch_cost(const UnitCost& c, long long tiles, int B, double T, int slots, int ns, double out_bytes) {
+  const long long units = tiles * ns, full = units / slots, rest = units % slots;
+  const double per = (double)(((long long)B + ns - 1) / ns);
+  auto unit = [&](double busy) {
+    const double ex = T * (c.token_lo + (c.token_hi - c.token_lo) * busy) + c.example;
+    return per * (ex > c.example_min ? ex : c.example_min) + c.fixed + (ns > 1 ? SPLIT_FIXED : 0.0);
+  };
+  return full * unit(1.0) + (rest ? unit((double)rest / slots) : 0.0) + (ns > 1 ? out_bytes / ZERO_BYTES_PER_US : 0.0);
+}
+struct TilePlan {
+  int choice, ns;             // index into the candidates, batch slices
+};
+// The cheapest of the candidate kernels and slice counts.
+static TilePlan plan_tiles(const UnitCost* cand, int n_cand, int B, double T, int d_in, int d_out, int slots, int max_split, int outputs) {
+  TilePlan best = {0, 1};
   double best_cost = 1e300;
-  int tt = T < 32 ? 32 : T;
-  for (int ns = 1; ns <= max_split && ns <= B; ++ns) {
-    long long waves = (tiles * ns + slots - 1) / slots;
-    long long per = ((long long)B + ns - 1) / ns;
-    double cost = (double)waves * ((double)per * tt + (ns > 1 ? 512.0 : 128.0));
-    if (cost < best_cost * 0.999) { best_cost = cost; best = ns; }
+  const long long pairs_m = ((long long)d_out + TC_PAIR_M - 1) / TC_PAIR_M;
+  const double out_bytes = 4.0 * outputs * d_in * d_out;
+  for (int k = 0; k < n_cand; ++k) {
+    const long long tiles = pairs_m * ((d_in + cand[k].nt - 1) / cand[k].nt);
+    for (int ns = 1; ns <= max_split && ns <= B && (ns == 1 || tiles * (ns - 1) < 16ll * slots); ++ns) {
+      const double cost = launch_cost(cand[k], tiles, B, T, slots, ns, out_bytes);
+      if (cost < best_cost * 0.995) { best_cost = cost; best = {k, ns}; }
+    }
   }
   return best;
 }
@@ -296,15 +327,27 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
   const bool triple = out_sign != nullptr;       // mean + square + sign in one pass (phi = square, all three outputs given)
   const bool both = per_example && ((out_mean && out_stat) || chunked);
   const bool runs = chunked && T > TC_CHUNK_TOKENS;     // several accumulators per example
-  // Both outputs: sum_b G_b in tensor memory beside a 256-wide accumulator, unless the sequences are
-  // so short that the per-example drain of that single accumulator would dominate.
   const int forced = g_path.load();
-  // 256 x 192 tile: 22 % less operand traffic per flop than 256 x 128
+  const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1, max_split = std::max(16, slots);
+  // Tile and batch slices by estimated time.  Both outputs: 256 x 192 or 256 x 128 (22 % more operand traffic per flop, but
+  // less padding and more even waves on some layers: 64 x 256 x 512 x 32768 528 us against 497); T <= 32: 256 x 128 with two
+  // examples per stage.
+  UnitCost cand[2];
+  int n_cand = 0;
+  bool cand_wide[2] = {false, false};
+  if (both) {
+    const bool short_t = T <= TC_SHORT_T;
+    if (forced != PE_PATH_TENSOR_NARROW && !runs && (!short_t || forced == PE_PATH_TENSOR_WIDE)) { cand_wide[n_cand] = true; cand[n_cand++] = triple ? COST_ALL_192 : COST_BOTH_192; }
+    if (forced != PE_PATH_TENSOR_WIDE || n_cand == 0) cand[n_cand++] = short_t ? (triple ? COST_ALL_SHORT : COST_BOTH_SHORT) : (triple ? COST_ALL_128 : COST_BOTH_128);
+  } else {
+    cand[n_cand++] = !per_example ? COST_PLAIN : phi == PE_PHI_SIGN ? COST_SIGN : COST_STAT;
+  }
+  const TilePlan plan = plan_tiles(cand, n_cand, B, T, d_in, d_out, slots, max_split, (out_mean ? 1 : 0) + (out_stat ? 1 : 0) + (out_sign ? 1 : 0));
   const long long pad192 = (long long)((d_in + 191) / 192) * 192, pad128 = (long long)((d_in + 127) / 128) * 128;
-  const bool wide = both && !runs && forced != PE_PATH_TENSOR_NARROW &&
-                    (forced == PE_PATH_TENSOR_WIDE || (T >= (triple ? TC_WIDE_TRIPLE_MIN_T : TC_WIDE_MIN_T) &&
-                                                       pad192 * 100 <= pad128 * (100 + TC_WIDE_MAX_PAD_PERCENT)));
-  const bool mean_regs = both && (triple || wide || runs || T < TC_MEAN_TMEM_MIN_T || forced == PE_PATH_TENSOR_NARROW);
+  const bool mean_tmem = both && !triple && !runs && forced != PE_PATH_TENSOR_NARROW && forced != PE_PATH_TENSOR_WIDE && T >= TC_MEAN_TMEM_MIN_T &&
+                         pad192 * 100 > pad128 * (100 + TC_WIDE_MAX_PAD_PERCENT);
+  const bool wide = both && !mean_tmem && cand_wide[plan.choice];
+  const bool mean_regs = both && !mean_tmem;
   const int nt = mean_regs ? (wide ? 192 : 128) : 256;
   const int box_feats = TcOperand<false, 256>::BOX_FEATS;
   const bool short_seq = mean_regs && !wide && T <= TC_SHORT_T;      // many short examples, both sums in registers: small stages
@@ -329,8 +372,7 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
   }
   const int tiles_n = (d_in + nt - 1) / nt, pairs_m = (d_out + TC_PAIR_M - 1) / TC_PAIR_M;
   if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
-  const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
-  int ns = choose_nsplit((long long)tiles_n * pairs_m, B, T, slots, std::max(16, slots));
+  int ns = mean_tmem ? plan_tiles(&COST_STAT, 1, B, T, d_in, d_out, slots, max_split, 2).ns : plan.ns;
   if (triple && (B + ns - 1) / ns > TC_SIGN_COUNT_MAX) ns = (B + TC_SIGN_COUNT_MAX - 1) / TC_SIGN_COUNT_MAX;   // 16-bit sign counters
   if (ns > 1 && !accumulate) {
     rc = zero_for_split(di, out_mean, out_stat, (size_t)d_in * d_out, st, out_sign);
@@ -384,7 +426,8 @@ static pe_status_t launch_tc_norms(DeviceInfo* di, const void* X, const void* dY
   if (rc != PE_OK) return rc;
   const int tiles_n = (d_in + 255) / 256, pairs_m = (d_out + TC_PAIR_M - 1) / TC_PAIR_M;
   if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
-  const int ns = choose_nsplit((long long)tiles_n * pairs_m, B, T, di->sm_count / 2 > 0 ? di->sm_count / 2 : 1, 16);
+  const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
+  const int ns = plan_tiles(&COST_NORMS, 1, B, T, d_in, d_out, slots, std::max(16, slots), 0).ns;
   TcParams p{};
   p.B = B; p.T = T; p.d_in = d_in; p.d_out = d_out; p.nsplit = ns; p.per_example = 1; p.half_operands = 0;
   p.accumulate = 1;       // nothing is zeroed by a preceding kernel and no matrix is written
@@ -542,8 +585,9 @@ static pe_status_t launch_tc_ragged(DeviceInfo* di, const void* X, const void* d
   const int tiles_n = (d_in + nt - 1) / nt, pairs_m = (d_out + TC_PAIR_M - 1) / TC_PAIR_M;
   if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
   const long long t_avg = rows / B > 0 ? rows / B : 1;
-  const int ns = choose_nsplit((long long)tiles_n * pairs_m, B, (int)(t_avg > (1 << 20) ? (1 << 20) : t_avg),
-                               di->sm_count / 2 > 0 ? di->sm_count / 2 : 1, 16);
+  const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
+  const UnitCost& unit = norms ? COST_NORMS : both ? COST_BOTH_192 : plain ? COST_STAT : phi == PE_PHI_SIGN ? COST_SIGN : COST_STAT;
+  const int ns = plan_tiles(&unit, 1, B, (double)t_avg, d_in, d_out, slots, std::max(16, slots), norms ? 0 : both ? 2 : 1).ns;
   if (ns > 1 && !norms) {
     rc = zero_for_split(di, both ? out_mean : nullptr, first, (size_t)d_in * d_out, st);
     if (rc != PE_OK) return rc;
@@ -694,10 +738,18 @@ static pe_status_t launch_tc_fused(DeviceInfo* di, const void* X, const void* dY
                                    float* out_a, float* out_b, FusedOpt opt, unsigned int* counters, size_t counter_words,
                                    cudaStream_t st) {
   const bool adam = kind == OPT_ADAM;
-  const long long pad192 = (long long)((d_in + 191) / 192) * 192, pad128 = (long long)((d_in + 127) / 128) * 128;
   const int forced = g_path.load();
-  const bool wide = adam && forced != PE_PATH_TENSOR_NARROW &&
-                    (forced == PE_PATH_TENSOR_WIDE || (T >= TC_WIDE_MIN_T && pad192 * 100 <= pad128 * (100 + TC_WIDE_MAX_PAD_PERCENT)));
+  const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
+  // the batch is only split if somebody can complete a tile: outputs to add to and a counter per block
+  const bool can_split = out_b && (!adam || out_a) && counters && counter_words >= fused_counter_words(d_in, d_out);
+  UnitCost cand[2];
+  int n_cand = 0;
+  if (adam && forced != PE_PATH_TENSOR_NARROW) cand[n_cand++] = COST_BOTH_192;
+  if (adam && (forced != PE_PATH_TENSOR_WIDE || n_cand == 0)) cand[n_cand++] = COST_BOTH_128;
+  if (!adam) cand[n_cand++] = COST_SIGN;
+  for (int k = 0; k < n_cand; ++k) cand[k].fixed += FUSED_UPDATE_FIXED * cand[k].nt / 192.0;
+  const TilePlan plan = plan_tiles(cand, n_cand, B, T, d_in, d_out, slots, can_split ? std::max(16, slots) : 1, adam ? 2 : 1);
+  const bool wide = adam && cand[plan.choice].nt == 192;
   const int nt = adam ? (wide ? 192 : 128) : 256;
   const int box_feats = TcOperand<false, 256>::BOX_FEATS, box_tokens = tc_default_bk(false, nt);
   CUtensorMap mx, my, mm, ms;
@@ -710,9 +762,8 @@ static pe_status_t launch_tc_fused(DeviceInfo* di, const void* X, const void* dY
   if (rc != PE_OK) return rc;
   const int tiles_n = (d_in + nt - 1) / nt, pairs_m = (d_out + TC_PAIR_M - 1) / TC_PAIR_M;
   if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
-  int ns = choose_nsplit((long long)tiles_n * pairs_m, B, T, di->sm_count / 2 > 0 ? di->sm_count / 2 : 1, 16);
+  const int ns = plan.ns;
   const size_t blocks = 2 * (size_t)tiles_n * pairs_m;
-  if (ns > 1 && (!out_b || (adam && !out_a) || !counters || counter_words < blocks)) ns = 1;
   if (ns > 1) {
     rc = zero_for_split(di, adam ? out_a : nullptr, out_b, (size_t)d_in * d_out, st, nullptr, counters, (int)blocks);
     if (rc != PE_OK) return rc;
@@ -758,7 +809,8 @@ static pe_status_t launch_tok(DeviceInfo* di, const void* X, const void* dY, lon
   if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
   const long long n_chunks = (rows + TOK_BK - 1) / TOK_BK;
   const int units = n_chunks > (1 << 30) ? (1 << 30) : (int)n_chunks;
-  const int ns = choose_nsplit((long long)tiles_n * pairs_m, units, TOK_BK, di->sm_count / 2 > 0 ? di->sm_count / 2 : 1, 32);
+  const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
+  const int ns = plan_tiles(&COST_TOKEN, 1, units, TOK_BK, d_in, d_out, slots, std::max(32, slots), 1).ns;
   if (ns > 1) {
     rc = zero_for_split(di, out, nullptr, (size_t)d_in * d_out, st);
     if (rc != PE_OK) return rc;
@@ -1270,7 +1322,8 @@ static pe_status_t launch_tc_fp8(DeviceInfo* di, const void* x8, const void* y8,
   if (rc != PE_OK) return rc;
   const int tiles_n = (d_in + 255) / 256, pairs_m = (d_out + TC_PAIR_M - 1) / TC_PAIR_M;
   if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
-  const int ns = choose_nsplit((long long)tiles_n * pairs_m, B, T, di->sm_count / 2 > 0 ? di->sm_count / 2 : 1, 16);
+  const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
+  const int ns = plan_tiles(&COST_PLAIN_FP8, 1, B, T, d_in, d_out, slots, std::max(16, slots), 1).ns;
   if (ns > 1) {
     rc = zero_for_split(di, out, nullptr, (size_t)d_in * d_out, st);
     if (rc != PE_OK) return rc;
