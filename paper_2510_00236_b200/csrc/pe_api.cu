@@ -279,29 +279,24 @@ static pe_status_t zero_for_split(DeviceInfo* di, float* a, float* b, size_t n, 
   return check_launch();
 }
 
-// Launches `kernel`; as a programmatic dependent of the zeroing kernel when the batch is split.
+// Launches `kernel` as a programmatic dependent of the kernel before it in the stream (every kernel launched this way waits for
+// that one to complete before it touches what others may have written: griddep_wait).
 template <typename Kernel, typename... Args>
-static pe_status_t launch_pair_kernel_t(Kernel kernel, dim3 grid, int threads, int smem, cudaStream_t st, bool after_zeroing, Args... args) {
+static pe_status_t launch_dependent(Kernel kernel, dim3 grid, int threads, int smem, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = st;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr; cfg.numAttrs = after_zeroing ? 1 : 0;
+  cfg.attrs = &attr; cfg.numAttrs = 1;
   if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess) { cudaGetLastError(); return PE_ERR_CUDA; }
   return check_launch();
 }
-template <typename Kernel, typename... Args>
-static pe_status_t launch_pair_kernel(Kernel kernel, dim3 grid, int smem, cudaStream_t st, bool after_zeroing, Args... args) {
-  return launch_pair_kernel_t(kernel, grid, TC_THREADS, smem, st, after_zeroing, args...);
-}
-
 // mxt, myt: the maps of the zero-padded tail groups of a packed batch (RAGGED); any valid map otherwise.
 template <int PHI, bool TF32, int NT, int MEAN, int BKT = tc_default_bk(TF32, NT), bool RAGGED = false, int OPT = OPT_NONE, bool F8 = false, bool CHUNKED = false>
 static pe_status_t launch_tc_inst(DeviceInfo* di, int slot, const CUtensorMap& mx, const CUtensorMap& my, const CUtensorMap& mm,
                                   const CUtensorMap& ms, const CUtensorMap& msgn, const TcParams& p, dim3 grid, cudaStream_t st,
                                   const CUtensorMap* mxt = nullptr, const CUtensorMap* myt = nullptr, const FusedOpt* opt = nullptr) {
-  const bool after_zeroing = p.nsplit > 1 && !p.accumulate;
   constexpr int smem = TcOperand<TF32, NT, BKT, F8>::SMEM_BYTES;
   {
     std::lock_guard<std::mutex> lock(g_dev_mutex);
@@ -313,7 +308,7 @@ static pe_status_t launch_tc_inst(DeviceInfo* di, int slot, const CUtensorMap& m
       di->tc_attr_set[slot] = true;
     }
   }
-  return launch_pair_kernel(tc_stats_kernel<PHI, TF32, NT, MEAN, BKT, RAGGED, OPT, F8, CHUNKED>, grid, smem, st, after_zeroing, mx, my, mm, ms, msgn,
+  return launch_dependent(tc_stats_kernel<PHI, TF32, NT, MEAN, BKT, RAGGED, OPT, F8, CHUNKED>, grid, TC_THREADS, smem, st, mx, my, mm, ms, msgn,
                             mxt ? *mxt : mx, myt ? *myt : my, p, opt ? *opt : FusedOpt{});
 }
 
@@ -533,6 +528,29 @@ static pe_status_t launch_simt(DeviceInfo* di, const TIn* X, const TIn* dY, int 
   }
 }
 
+static int grid_for(long long work_items, int sm_count) {
+  long long blocks = (work_items + OPT_THREADS - 1) / OPT_THREADS;
+  long long cap = (long long)sm_count * 8;
+  if (blocks < 1) blocks = 1;
+  return (int)(blocks < cap ? blocks : cap);
+}
+
+// The update kernels.  skip_if_set: NULL, or the device status word that makes the step leave the parameters alone.
+static pe_status_t launch_microadam(DeviceInfo* di, int variant, float* theta, __nv_bfloat16* lp, float* m, float* v, const float* sum_g,
+                                    const float* sum_g2, long long n, const AdamParams& p, const unsigned int* skip_if_set, cudaStream_t st) {
+  const dim3 grid(grid_for(n / 4 + 4, di->sm_count));
+  switch (variant) {
+    case ADAM_ORIGINAL: return launch_dependent(microadam_kernel<ADAM_ORIGINAL>, grid, OPT_THREADS, 0, st, theta, lp, m, v, sum_g, sum_g2, n, p, skip_if_set);
+    case ADAM_MICRO: return launch_dependent(microadam_kernel<ADAM_MICRO>, grid, OPT_THREADS, 0, st, theta, lp, m, v, sum_g, sum_g2, n, p, skip_if_set);
+    case ADAM_MICRO_VAR: return launch_dependent(microadam_kernel<ADAM_MICRO_VAR>, grid, OPT_THREADS, 0, st, theta, lp, m, v, sum_g, sum_g2, n, p, skip_if_set);
+    default: return launch_dependent(microadam_kernel<ADAM_MICRO_MSQ>, grid, OPT_THREADS, 0, st, theta, lp, m, v, sum_g, sum_g2, n, p, skip_if_set);
+  }
+}
+static pe_status_t launch_microsignsgd(DeviceInfo* di, float* theta, __nv_bfloat16* lp, float* m, const float* sum_sign, long long n,
+                                       const SignParams& p, const unsigned int* skip_if_set, cudaStream_t st) {
+  return launch_dependent(microsignsgd_kernel, dim3(grid_for(n / 4 + 4, di->sm_count)), OPT_THREADS, 0, st, theta, lp, m, sum_sign, n, p, skip_if_set);
+}
+
 // Side buffer of a packed batch: the zero-padded last partial 16-token group of every sequence, X's [B, 16, d_in]
 // then dY's [B, 16, d_out] (bf16), each part 256-byte aligned.
 struct RaggedLayout {
@@ -555,9 +573,7 @@ static pe_status_t launch_tc_ragged(DeviceInfo* di, const void* X, const void* d
   uint16_t* xt = static_cast<uint16_t*>(ws);
   uint16_t* yt = reinterpret_cast<uint16_t*>(static_cast<char*>(ws) + l.x_bytes);
   const TailTensor tx = {static_cast<const uint16_t*>(X), xt, d_in}, ty = {static_cast<const uint16_t*>(dY), yt, d_out};
-  pack_tails_kernel<<<dim3((unsigned)B, 2, 1), STAGE_THREADS, 0, st>>>(tx, ty, offsets, rows);
-  pe_status_t rc = check_launch();
-  if (rc != PE_OK) return rc;
+  pe_status_t rc = PE_OK;
   const bool both = !norms && out_mean && out_stat && phi != PE_PHI_IDENTITY;
   const bool plain = !norms && (phi == PE_PHI_IDENTITY || !out_stat);      // only sum_b G_b
   const int nt = both ? 192 : 256;
@@ -567,13 +583,13 @@ static pe_status_t launch_tc_ragged(DeviceInfo* di, const void* X, const void* d
   const int bf = TcOperand<false, 256>::BOX_FEATS;
   if (both) {
     rc = make_operand_map(&mx, X, 1, rows_i, d_in, false, TcOperand<false, 192>::B_BOX_FEATS, box_tokens, true);
-    if (rc == PE_OK) rc = make_operand_map(&mxt, xt, B, 16, d_in, false, TcOperand<false, 192>::B_BOX_FEATS, box_tokens, true);
+    if (rc == PE_OK) rc = make_operand_map(&mxt, xt, B, 16, d_in, false, TcOperand<false, 192>::B_BOX_FEATS, 16, true);
   } else {
     rc = make_operand_map(&mx, X, 1, rows_i, d_in, false, bf, box_tokens);
-    if (rc == PE_OK) rc = make_operand_map(&mxt, xt, B, 16, d_in, false, bf, box_tokens);
+    if (rc == PE_OK) rc = make_operand_map(&mxt, xt, B, 16, d_in, false, bf, 16);
   }
   if (rc == PE_OK) rc = make_operand_map(&my, dY, 1, rows_i, d_out, false, bf, box_tokens);
-  if (rc == PE_OK) rc = make_operand_map(&myt, yt, B, 16, d_out, false, bf, box_tokens);
+  if (rc == PE_OK) rc = make_operand_map(&myt, yt, B, 16, d_out, false, bf, 16);
   if (rc != PE_OK) return rc;
   float* first = plain ? (out_mean ? out_mean : out_stat) : out_stat;
   CUtensorMap mm = mx, ms = mx;       // never used by the norms variant
@@ -588,15 +604,18 @@ static pe_status_t launch_tc_ragged(DeviceInfo* di, const void* X, const void* d
   const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
   const UnitCost& unit = norms ? COST_NORMS : both ? COST_BOTH_192 : plain ? COST_STAT : phi == PE_PHI_SIGN ? COST_SIGN : COST_STAT;
   const int ns = plan_tiles(&unit, 1, B, (double)t_avg, d_in, d_out, slots, std::max(16, slots), norms ? 0 : both ? 2 : 1).ns;
-  if (ns > 1 && !norms) {
-    rc = zero_for_split(di, both ? out_mean : nullptr, first, (size_t)d_in * d_out, st);
-    if (rc != PE_OK) return rc;
-  }
+  // the pre-pass: the partial 16-token groups to the side buffer, and the outputs of a split batch to zero
+  const bool zero = ns > 1 && !norms;
+  const int chunks = (int)std::min<long long>(8, std::max<long long>(1, 8ll * di->sm_count / (2ll * B)));
+  pack_tails_kernel<<<dim3((unsigned)B, 2, (unsigned)chunks), STAGE_THREADS, 0, st>>>(tx, ty, offsets, rows, zero ? first : nullptr,
+                                                                                         zero && both ? out_mean : nullptr, (long long)d_in * d_out);
+  if ((rc = check_launch()) != PE_OK) return rc;
   TcParams p{};
   p.B = B; p.T = 0; p.d_in = d_in; p.d_out = d_out; p.nsplit = ns; p.per_example = 1; p.half_operands = 0;
   p.accumulate = norms ? 1 : 0;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, nt, ns, di->sm_count / 2);
   p.out_mean = both ? out_mean : nullptr; p.out_stat = norms ? nullptr : first; p.out_sign = nullptr; p.out_norms = norms;
+  p.by_tokens = ns > 1 && (phi != PE_PHI_SIGN || B <= TC_SIGN_COUNT_MAX) ? 1 : 0;
   p.seq_offsets = offsets; p.sq_norms = nullptr; p.clip_norm = 0.f; p.dev_status = di->status_ptr;
   const dim3 grid(2 * pairs_m * tiles_n, 1, ns);
   if (norms) return launch_tc_inst<1, false, 256, MEAN_NORMS, 64, true>(di, 15, mx, my, mm, ms, ms, p, grid, st, &mxt, &myt);
@@ -781,12 +800,6 @@ static pe_status_t launch_tc_fused(DeviceInfo* di, const void* X, const void* dY
   return launch_tc_inst<1, false, 128, MEAN_REGS, 128, false, OPT_ADAM>(di, 22, mx, my, mm, ms, ms, p, grid, st, nullptr, nullptr, &opt);
 }
 
-static int grid_for(long long work_items, int sm_count) {
-  long long blocks = (work_items + OPT_THREADS - 1) / OPT_THREADS;
-  long long cap = (long long)sm_count * 8;
-  if (blocks < 1) blocks = 1;
-  return (int)(blocks < cap ? blocks : cap);
-}
 
 // Fused per-token statistic: squares, rounds to tf32 and contracts inside one kernel.
 static pe_status_t launch_tok(DeviceInfo* di, const void* X, const void* dY, long long rows, int d_in, int d_out, float* out,
@@ -828,7 +841,7 @@ static pe_status_t launch_tok(DeviceInfo* di, const void* X, const void* dY, lon
   TokParams p;
   p.rows = rows; p.d_in = d_in; p.d_out = d_out; p.pairs_m = pairs_m; p.tiles_n = tiles_n;
   p.band = choose_band(pairs_m, tiles_n, TOK_NT, ns, di->sm_count / 2); p.nsplit = ns; p.dev_status = di->status_ptr;
-  return launch_pair_kernel_t(tok_sqstats_kernel, dim3(2 * pairs_m * tiles_n, 1, ns), TOK_THREADS, TOK_SMEM_BYTES, st, ns > 1, mx, my, mo, p);
+  return launch_dependent(tok_sqstats_kernel, dim3(2 * pairs_m * tiles_n, 1, ns), TOK_THREADS, TOK_SMEM_BYTES, st, mx, my, mo, p);
 }
 
 }  // namespace pe
@@ -1168,19 +1181,9 @@ pe_status_t fused_impl(const TIn* X, const TIn* dY, int B, int T, int d_in, int 
                        kind == OPT_ADAM ? out_a : nullptr, out_b, st);
         if (rc != PE_OK) return rc;
         const long long n = (long long)d_in * d_out;
-        const int grid = grid_for(n / 4 + 4, di->sm_count);
         __nv_bfloat16* lp = static_cast<__nv_bfloat16*>(theta_lp);
-        if (kind == OPT_ADAM) {
-          switch (opt.variant) {
-            case ADAM_ORIGINAL: microadam_kernel<ADAM_ORIGINAL><<<grid, OPT_THREADS, 0, st>>>(theta, lp, m, v, out_a, out_b, n, opt.adam, di->status_ptr); break;
-            case ADAM_MICRO: microadam_kernel<ADAM_MICRO><<<grid, OPT_THREADS, 0, st>>>(theta, lp, m, v, out_a, out_b, n, opt.adam, di->status_ptr); break;
-            case ADAM_MICRO_VAR: microadam_kernel<ADAM_MICRO_VAR><<<grid, OPT_THREADS, 0, st>>>(theta, lp, m, v, out_a, out_b, n, opt.adam, di->status_ptr); break;
-            default: microadam_kernel<ADAM_MICRO_MSQ><<<grid, OPT_THREADS, 0, st>>>(theta, lp, m, v, out_a, out_b, n, opt.adam, di->status_ptr); break;
-          }
-        } else {
-          microsignsgd_kernel<<<grid, OPT_THREADS, 0, st>>>(theta, lp, m, out_b, n, opt.sign, di->status_ptr);
-        }
-        return check_launch();
+        if (kind == OPT_ADAM) return launch_microadam(di, opt.variant, theta, lp, m, v, out_a, out_b, n, opt.adam, di->status_ptr, st);
+        return launch_microsignsgd(di, theta, lp, m, out_b, n, opt.sign, di->status_ptr, st);
       }
       return launch_tc_fused(di, X, dY, B, T, d_in, d_out, kind, out_a, out_b, opt, static_cast<unsigned int*>(workspace),
                              workspace_bytes / sizeof(unsigned int), st);
@@ -1476,16 +1479,8 @@ pe_status_t microadam_family_step(float* theta, void* theta_lp, float* m, float*
   if (rc != PE_OK) return rc;
   if (n == 0) return PE_OK;
   const AdamParams p = make_adam_params(B, grad_scale, lr, beta1, beta2, eps, eps_inside_sqrt, weight_decay, step);
-  const int grid = grid_for(n / 4 + 4, di->sm_count);
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  __nv_bfloat16* lp = static_cast<__nv_bfloat16*>(theta_lp);
-  switch ((int)variant) {
-    case ADAM_ORIGINAL: microadam_kernel<ADAM_ORIGINAL><<<grid, OPT_THREADS, 0, st>>>(theta, lp, m, v, sum_g, sum_g2, n, p); break;
-    case ADAM_MICRO: microadam_kernel<ADAM_MICRO><<<grid, OPT_THREADS, 0, st>>>(theta, lp, m, v, sum_g, sum_g2, n, p); break;
-    case ADAM_MICRO_VAR: microadam_kernel<ADAM_MICRO_VAR><<<grid, OPT_THREADS, 0, st>>>(theta, lp, m, v, sum_g, sum_g2, n, p); break;
-    default: microadam_kernel<ADAM_MICRO_MSQ><<<grid, OPT_THREADS, 0, st>>>(theta, lp, m, v, sum_g, sum_g2, n, p); break;
-  }
-  return check_launch();
+  return launch_microadam(di, (int)variant, theta, static_cast<__nv_bfloat16*>(theta_lp), m, v, sum_g, sum_g2, n, p, nullptr,
+                          reinterpret_cast<cudaStream_t>(stream));
 }
 
 pe_status_t microadam_step(float* theta, void* theta_lp, float* m, float* v, const float* sum_g, const float* sum_g2,
@@ -1506,9 +1501,7 @@ pe_status_t microsignsgd_step(float* theta, void* theta_lp, float* m, const floa
   if (n == 0) return PE_OK;
   SignParams p;
   p.inv_B = (float)(1.0 / (double)B); p.beta = beta; p.lr = lr; p.wd = weight_decay;
-  microsignsgd_kernel<<<grid_for(n / 4 + 4, di->sm_count), OPT_THREADS, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-      theta, static_cast<__nv_bfloat16*>(theta_lp), m, sum_sign, n, p);
-  return check_launch();
+  return launch_microsignsgd(di, theta, static_cast<__nv_bfloat16*>(theta_lp), m, sum_sign, n, p, nullptr, reinterpret_cast<cudaStream_t>(stream));
 }
 
 const char* pe_status_string(pe_status_t s) {

@@ -6,6 +6,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "pe_sm100.cuh"
+
 namespace pe {
 
 struct AdamParams {
@@ -62,6 +64,9 @@ __global__ void __launch_bounds__(OPT_THREADS)
 microadam_kernel(float* __restrict__ theta, __nv_bfloat16* __restrict__ theta_lp, float* __restrict__ m,
                  float* __restrict__ v, const float* __restrict__ sum_g, const float* __restrict__ sum_g2,
                  long long n, AdamParams p, const unsigned int* __restrict__ skip_if_set = nullptr) {
+  // Launched as a programmatic dependent: the blocks move in as the predecessor's leave, and start when it has completed.
+  sm100::griddep_launch_dependents();
+  sm100::griddep_wait();
   // when this step follows a statistics kernel in the same call: leave the parameters alone if that kernel gave up
   if (skip_if_set && *reinterpret_cast<const volatile unsigned int*>(skip_if_set) != 0u) return;
   const long long n4 = n >> 2;
@@ -113,6 +118,8 @@ __global__ void __launch_bounds__(OPT_THREADS)
 microsignsgd_kernel(float* __restrict__ theta, __nv_bfloat16* __restrict__ theta_lp, float* __restrict__ m,
                     const float* __restrict__ sum_sign, long long n, SignParams p,
                     const unsigned int* __restrict__ skip_if_set = nullptr) {
+  sm100::griddep_launch_dependents();
+  sm100::griddep_wait();
   if (skip_if_set && *reinterpret_cast<const volatile unsigned int*>(skip_if_set) != 0u) return;
   const long long n4 = n >> 2;
   const long long stride = (long long)gridDim.x * blockDim.x;

@@ -145,6 +145,7 @@ struct TcParams {
   float* out_sign;     // MEAN_REGS_SIGN only: sum_b sign(G_b), written through tmap_sign
   float* out_norms;    // MEAN_NORMS only: [B], zero on entry; every tile adds its share of ||G_b||_F^2
   const int* seq_offsets;   // RAGGED only: [B + 1] token-row offsets; example b owns rows offsets[b] .. offsets[b+1]-1
+  int by_tokens;            // RAGGED only: the batch is sliced by tokens instead of by examples
   const float* sq_norms;    // PHI == 3 only: [B] per-example squared norms the clipping coefficient is taken from
   float clip_norm;          // PHI == 3 only: C of c_b = min(1, C / sqrt(N_b))
   unsigned int* dev_status;
@@ -176,6 +177,26 @@ __device__ __forceinline__ SeqGeom seq_geom(const TcParams& p, int b, int bk) {
     g.nk_main = g.nk = (p.T + bk - 1) / bk;
   }
   return g;
+}
+
+// Slices of a packed batch: equal shares of tokens (plus 64 per example for its hand-offs), not of examples, whose lengths
+// differ: first example of the slice that starts at `target`, the smallest b with offsets[b] + 64 b >= target.  A warp
+// searches 32 ways at a time (two rounds up to 1024 examples).
+__device__ __forceinline__ long long ragged_key(const int* offsets, int b) { return (long long)__ldg(offsets + b) + 64ll * b; }
+__device__ __forceinline__ int ragged_slice_begin(const int* offsets, int B, int slice, int nsplit, int lane) {
+  if (slice <= 0) return 0;
+  if (slice >= nsplit) return B;
+  const long long first = ragged_key(offsets, 0), target = first + (ragged_key(offsets, B) - first) * slice / nsplit;
+  int lo = 0, hi = B;
+  while (lo < hi) {
+    const int step = (hi - lo + 31) / 32, idx = lo + lane * step;
+    const unsigned below = __ballot_sync(0xffffffffu, idx < hi && ragged_key(offsets, idx) < target);
+    if (below == 0u) break;
+    const int last = lo + (__popc(below) - 1) * step;
+    lo = last + 1;
+    hi = min(hi, last + step);
+  }
+  return lo < B ? lo : B;
 }
 
 // Tile order.  Pairs that run at the same time should share operand panels in L2, so consecutive
@@ -393,8 +414,14 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;      // the warp's number, uniform to the compiler too
   const uint32_t rank = cluster_ctarank();          // 0 = leader of the pair
-  const int b_begin = (int)(((long long)p.B * blockIdx.z) / p.nsplit);
-  const int b_end = (int)(((long long)p.B * (blockIdx.z + 1)) / p.nsplit);
+  int b_begin = (int)(((long long)p.B * blockIdx.z) / p.nsplit);
+  int b_end = (int)(((long long)p.B * (blockIdx.z + 1)) / p.nsplit);
+  if constexpr (RAGGED) {
+    if (p.by_tokens) {
+      b_begin = ragged_slice_begin(p.seq_offsets, p.B, blockIdx.z, p.nsplit, lane);
+      b_end = max(b_begin, ragged_slice_begin(p.seq_offsets, p.B, blockIdx.z + 1, p.nsplit, lane));
+    }
+  }
   const int nb = b_end - b_begin;
   const int nu = (nb + GROUP - 1) / GROUP;          // units of work: groups of GROUP examples (GROUP = 1: the examples)
 
@@ -409,6 +436,14 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   cluster_sync_all();          // barriers of both blocks initialised before any remote arrival
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // The next kernel of the stream may be launched from here on (it finds no room before blocks of this one leave).  With an unsplit
+  // batch this kernel is itself a programmatic dependent of whatever precedes it: everything above overlapped that
+  // kernel's end, and nothing below may start before it has completed.  (With a split batch its predecessor is the kernel
+  // that zeroes the outputs, itself an ordinary launch, and only the write-out waits for it.)
+  // A packed batch's predecessor is the kernel that fills the side buffer (and zeroes the outputs), an ordinary launch too: the
+  // producers wait for it before the first load from there.
+  griddep_launch_dependents();
+  if (!RAGGED && (p.nsplit == 1 || p.accumulate)) griddep_wait();
 
   // Register budget: the epilogue warpgroups hold 128 floats of running sums plus a 32-register TMEM
   // read per thread; the producer / MMA warpgroup needs little.  Each setmaxnreg sits inside the
@@ -436,15 +471,17 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       int s = 0;
       uint32_t ph = 1;
       bool ok = true;
+      bool side_ready = false;        // RAGGED: the side buffer is complete
       for (int e = 0; e < nu && ok; ++e) {
         const SeqGeom g = seq_geom<RAGGED>(p, b_begin + GROUP * e, BK);
         for (int kc = 0; kc < g.nk; ++kc) {
           if (!mbar_wait_warp(empty_bar(s), ph, abort_flag, p.dev_status, TC_WAIT_EMPTY, strict)) { ok = false; break; }
           if (elect_one()) {
-            if (is_a && rank == 0) mbar_arrive_expect_tx(full_bar(s), 2 * STAGE_BYTES);     // both blocks' bytes
+            const bool tail = RAGGED && kc >= g.nk_main;       // the zero-padded last partial group, from the side buffer (boxes 16 tokens tall)
+            if (is_a && rank == 0) mbar_arrive_expect_tx(full_bar(s), tail ? 2 * STAGE_BYTES / (BK / 16) : 2 * STAGE_BYTES);     // both blocks' bytes
             const uint32_t leader_full = map_to_cta(full_bar(s), 0);
             const uint32_t dst = smem_base + s * STAGE_BYTES + (is_a ? 0 : A_BYTES);
-            const bool tail = RAGGED && kc >= g.nk_main;       // the zero-padded last partial group, from the side buffer
+            if (tail && !side_ready) griddep_wait();
             const CUtensorMap* tm = tail ? tmap_tail : tmap;
             const int c1 = tail ? 0 : g.row0 + kc * BK;
             // (grouped examples: the box is GROUP examples deep; past the batch's end it reads zeros)
@@ -452,6 +489,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
             for (int b = 0; b < n_boxes; ++b) tma_load_3d_pair(dst + b * box_bytes, tm, leader_full, c0 + b * box_feats, c1, c2);
           }
           __syncwarp();
+          if (RAGGED && kc >= g.nk_main) side_ready = true;
           if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
       }

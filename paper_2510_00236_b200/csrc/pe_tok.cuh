@@ -121,6 +121,8 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
   cluster_sync_all();          // barriers of both blocks initialised before any remote arrival
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  griddep_launch_dependents();            // as in the statistics kernel
+  if (p.nsplit == 1) griddep_wait();
 
   if (warp < 4) {
     const bool strict = wait_cycle_limit() < WAIT_CYCLE_LIMIT_STRICT;
