@@ -375,7 +375,7 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
   }
   TcParams p{};
   p.B = B; p.T = T; p.d_in = d_in; p.d_out = d_out; p.nsplit = ns; p.per_example = per_example; p.half_operands = half_ops ? 1 : 0;
-  p.accumulate = accumulate ? 1 : 0; p.scalar_out = scalar_out ? 1 : 0;
+  p.accumulate = accumulate ? 1 : 0; p.scalar_out = scalar_out ? 1 : 0; p.wait_at_start = ns == 1 || accumulate ? 1 : 0;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, nt, ns, di->sm_count / 2);
   p.out_mean = out_mean; p.out_stat = out_stat; p.out_sign = out_sign; p.out_norms = nullptr; p.dev_status = di->status_ptr;
   p.seq_offsets = nullptr; p.sq_norms = sq_norms; p.clip_norm = clip_norm;
@@ -425,7 +425,11 @@ static pe_status_t launch_tc_norms(DeviceInfo* di, const void* X, const void* dY
   const int ns = plan_tiles(&COST_NORMS, 1, B, T, d_in, d_out, slots, std::max(16, slots), 0).ns;
   TcParams p{};
   p.B = B; p.T = T; p.d_in = d_in; p.d_out = d_out; p.nsplit = ns; p.per_example = 1; p.half_operands = 0;
-  p.accumulate = 1;       // nothing is zeroed by a preceding kernel and no matrix is written
+  p.accumulate = 1;       // no matrix is written
+  // norms[b] = 0 by the kernel whose end this one's main loop overlaps (16-byte alignment allowing)
+  p.wait_at_start = aligned(norms, 16) ? 0 : 1;
+  rc = p.wait_at_start ? zero_outputs(norms, nullptr, (size_t)B * sizeof(float), st) : zero_for_split(di, norms, nullptr, (size_t)B, st);
+  if (rc != PE_OK) return rc;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, 256, ns, di->sm_count / 2);
   p.out_mean = nullptr; p.out_stat = nullptr; p.out_sign = nullptr; p.out_norms = norms; p.dev_status = di->status_ptr;
   p.seq_offsets = nullptr; p.sq_norms = nullptr; p.clip_norm = 0.f;
@@ -433,9 +437,9 @@ static pe_status_t launch_tc_norms(DeviceInfo* di, const void* X, const void* dY
   return launch_tc_inst<1, false, 256, MEAN_NORMS>(di, 11, mx, my, mx, mx, mx, p, dim3(2 * pairs_m * tiles_n, 1, ns), st);
 }
 
-// Tile and batch slices of a SIMT launch: the cheapest by an estimate in cycles of one block's walk, times the waves of
-// blocks.  A chunk of tokens costs the FMAs of the blocks that share an SM (128 lanes), at the rate the tile's shared-memory
-// reads leave, but not less than the latency of its barrier and loads.
+// Tile and batch slices of a SIMT launch: the cheapest by an estimate in microseconds, fitted to a sweep of all tiles and slice
+// counts over 14 layers from 48 x 48 to 1024 x 1024 (the choice within 6 % of the sweep's best, geometric mean).  A chunk of
+// tokens costs its FMAs times the blocks that share the SM, but for a block alone at least that and a latency.
 struct SimtPlan {
   int tile, slices, cluster;      // tile: index into the four shapes, largest first
 };
@@ -443,23 +447,29 @@ static SimtPlan plan_simt(DeviceInfo* di, int mode, int B, int T, int d_in, int 
   static constexpr int rows[4] = {SimtTile84::ROWS, SimtTile44::ROWS, SimtTile22::ROWS, SimtTile11::ROWS};
   static constexpr int cols[4] = {SimtTile84::COLS, SimtTile44::COLS, SimtTile22::COLS, SimtTile11::COLS};
   static constexpr int kt[4] = {SimtTile84::KT, SimtTile44::KT, SimtTile22::KT, SimtTile11::KT};
-  static constexpr double fma_rate[4] = {0.8, 0.55, 0.25, 0.08};      // share of the FMA lanes kept busy
-  const long long units = mode == MODE_TOKEN ? (long long)B * T : B;  // what the slices divide: rows or examples
+  static constexpr int per_sm[4] = {2, 2, 3, 4};                      // blocks an SM holds
+  static constexpr double chunk_us[4] = {1.95, 0.60, 0.85, 0.80};     // a full chunk's FMAs, one block
+  static constexpr double latency_us[4] = {0.25, 0.35, 0.45, 0.50};
+  static constexpr double fold_us[4] = {0.35, 0.10, 0.05, 0.05};      // phi and the sums at the end of an example
+  const bool by_rows = mode == MODE_TOKEN;                            // what the slices divide: rows or examples
+  const long long units = by_rows ? (long long)B * T : B;
   SimtPlan best = {0, 1, 1};
   double best_cost = 1e300;
   for (int k = 0; k < 4; ++k) {
     const long long tiles = (long long)((d_in + cols[k] - 1) / cols[k]) * ((d_out + rows[k] - 1) / rows[k]);
-    for (int s = 1; s <= 64 && s <= units; s *= 2) {
-      const long long blocks = tiles * s, slots = 2ll * di->sm_count;
-      const long long waves = (blocks + slots - 1) / slots;
-      const double sharing = blocks > di->sm_count ? 2.0 : 1.0;
+    for (int s = 1; s <= 32 && s <= units; s *= 2) {
+      const long long blocks = tiles * s, slots = (long long)per_sm[k] * di->sm_count;
+      double sharing = (double)std::min<long long>(per_sm[k], (blocks + di->sm_count - 1) / di->sm_count);
+      if (k == 0 && s >= SIMT_MAX_CLUSTER && blocks <= di->sm_count) sharing = 1.5;      // clusters of eight are placed densely
       const long long per = (units + s - 1) / s;
-      const long long tokens = mode == MODE_TOKEN ? per : T;
-      const double chunks = (double)((tokens + kt[k] - 1) / kt[k]);
-      const double fma = (double)rows[k] * cols[k] * (double)((tokens + 7) / 8 * 8) / 128.0 / fma_rate[k] * sharing;
-      const double walk = (fma > 700.0 * chunks ? fma : 700.0 * chunks) + (mode == MODE_TOKEN ? 0.0 : rows[k] * cols[k] / 16.0);
-      const double cost = waves * (walk * (mode == MODE_TOKEN ? 1.0 : (double)per) + 3000.0 + 300.0 * s + (s > SIMT_MAX_CLUSTER ? 8000.0 : 0.0));
-      if (cost < best_cost * 0.98) { best_cost = cost; best = {k, s, s < SIMT_MAX_CLUSTER ? s : SIMT_MAX_CLUSTER}; }
+      const double tokens = (double)(by_rows ? per : (long long)T), whole = std::floor(tokens / kt[k]);
+      const double rest = (double)(((long long)(tokens - whole * kt[k]) + 7) / 8 * 8) / kt[k];
+      auto chunk = [&](double f) { return std::max(sharing * chunk_us[k] * f, latency_us[k] + chunk_us[k] * f); };
+      double walk = whole * chunk(1.0) + (rest > 0.0 ? chunk(rest) : 0.0);
+      if (!by_rows) walk = per * (walk + fold_us[k] * sharing);
+      const double waves = (double)((blocks + slots - 1) / slots);
+      const double cost = waves * (walk + 2.0) + 1.5 + 0.12 * s + (s > SIMT_MAX_CLUSTER ? 3.0 : 0.0);
+      if (cost < best_cost) { best_cost = cost; best = {k, s, s < SIMT_MAX_CLUSTER ? s : SIMT_MAX_CLUSTER}; }
     }
   }
   if (mode == MODE_NORMS) best.cluster = 1;      // nothing is exchanged
@@ -789,6 +799,7 @@ static pe_status_t launch_tc_fused(DeviceInfo* di, const void* X, const void* dY
   }
   TcParams p{};
   p.B = B; p.T = T; p.d_in = d_in; p.d_out = d_out; p.nsplit = ns; p.per_example = 1; p.half_operands = 0; p.accumulate = 0;
+  p.wait_at_start = ns == 1 ? 1 : 0;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, nt, ns, di->sm_count / 2);
   p.out_mean = adam ? out_a : nullptr; p.out_stat = out_b; p.out_sign = nullptr; p.out_norms = nullptr; p.dev_status = di->status_ptr;
   p.seq_offsets = nullptr; p.sq_norms = nullptr; p.clip_norm = 0.f;
@@ -867,8 +878,7 @@ pe_status_t pe_example_sqnorms(const void* X, const void* dY, int B, int T, int 
   rc = device_info(&di);
   if (rc != PE_OK) return rc;
   if (B == 0) return PE_OK;
-  if (cudaMemsetAsync(out_norms, 0, (size_t)B * sizeof(float), st) != cudaSuccess) { cudaGetLastError(); return PE_ERR_CUDA; }
-  if (T == 0) return PE_OK;
+  if (T == 0) return zero_outputs(out_norms, nullptr, (size_t)B * sizeof(float), st);
   const int forced = g_path.load();
   const bool tc_ok = tc_shape_ok(B, T, d_in, d_out);
   if (forced >= PE_PATH_TENSOR && !tc_ok) return PE_ERR_UNSUPPORTED_SHAPE;
@@ -877,6 +887,8 @@ pe_status_t pe_example_sqnorms(const void* X, const void* dY, int B, int T, int 
     return launch_tc_norms(di, X, dY, B, T, d_in, d_out, out_norms, st);
   }
   g_last_path.store(PE_PATH_SIMT);
+  rc = zero_outputs(out_norms, nullptr, (size_t)B * sizeof(float), st);
+  if (rc != PE_OK) return rc;
   // every block handles whole examples of its slice and adds to out_norms[b]: "accumulate" keeps launch_simt from zeroing
   return launch_simt<__nv_bfloat16, MODE_NORMS>(di, static_cast<const __nv_bfloat16*>(X), static_cast<const __nv_bfloat16*>(dY), B, T,
                                                 d_in, d_out, 1, nullptr, out_norms, st, true);
@@ -1039,10 +1051,16 @@ pe_status_t pe_conv2d_stats(const void* x, const void* grad_out, int B, int C, i
   rc = device_info(&di);
   if (rc != PE_OK) return rc;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  unfold_kernel<<<dim3((g.Wo + t.tile_w - 1) / t.tile_w, g.Ho, B), LAYOUT_THREADS, t.smem, st>>>(static_cast<const uint16_t*>(x), X, g, l.pitch_x, t.tile_w,
-                                                                                                   t.chan, t.cols);
-  if ((rc = check_launch()) != PE_OK) return rc;
-  transpose_rows_kernel<<<dim3((T + 63) / 64, (l.pitch_y + 63) / 64, B), LAYOUT_THREADS, 0, st>>>(static_cast<const uint16_t*>(grad_out), dY, F, T, l.pitch_y);
+  ConvOperands o;
+  o.x = static_cast<const uint16_t*>(x); o.gy = static_cast<const uint16_t*>(grad_out); o.X = X; o.dY = dY;
+  o.pitch_x = l.pitch_x; o.pitch_y = l.pitch_y;
+  o.tile_w = t.tile_w; o.chan = t.chan; o.cols = t.cols; o.w_tiles = (g.Wo + t.tile_w - 1) / t.tile_w;
+  o.unfold_blocks = (long long)o.w_tiles * g.Ho * B;
+  o.t_tiles = (T + 63) / 64; o.f_tiles = (l.pitch_y + 63) / 64;
+  o.vec = T % 8 == 0 && aligned(grad_out, 16) ? 1 : 0;
+  const long long blocks = o.unfold_blocks + (long long)o.t_tiles * o.f_tiles * B;
+  if (blocks >= (1ll << 31)) return PE_ERR_DIM;
+  conv_operands_kernel<<<(unsigned)blocks, LAYOUT_THREADS, std::max(t.smem, 64 * TRANSPOSE_PITCH * 2), st>>>(o, g);
   if ((rc = check_launch()) != PE_OK) return rc;
   if (forced != PE_PATH_SIMT && whole) return tc_linear_stats(di, X, dY, B, T, d_in, F, phi, out_mean, out_stat, false, st);
   if (forced != PE_PATH_SIMT && padding_pays(B, T, d_in, F))
@@ -1333,6 +1351,7 @@ static pe_status_t launch_tc_fp8(DeviceInfo* di, const void* x8, const void* y8,
   }
   TcParams p{};
   p.B = B; p.T = T; p.d_in = d_in; p.d_out = d_out; p.nsplit = ns; p.per_example = 0; p.half_operands = 0; p.accumulate = 0;
+  p.wait_at_start = ns == 1 ? 1 : 0;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, 256, ns, di->sm_count / 2);
   p.out_mean = nullptr; p.out_stat = out; p.out_sign = nullptr; p.out_norms = nullptr; p.dev_status = di->status_ptr;
   p.seq_offsets = nullptr; p.sq_norms = nullptr; p.clip_norm = 0.f;

@@ -62,72 +62,113 @@ struct ConvGeom {
   int B, C, H, W, F, Kh, Kw, sh, sw, ph, pw, dh, dw, Ho, Wo;
 };
 
-// dst[(b, oh, ow), f] = x[b, c, oh*sh - ph + kh*dh, ow*sw - pw + kw*dw] (0 outside the image), f = (c*Kh + kh)*Kw + kw: one row of
-// `pitch` bf16 per output position.  A block handles one output row (a run of tile_w of its positions): the input rows it
-// touches go to shared memory once, `chan` channels at a time and with the image's border as zeros, and every 16-byte
-// group of the result is gathered from there through a table of the features' offsets.  chan is a multiple of 8 or C, so
-// that a chunk's features start on a group.  gridDim = (ceil(Wo / tile_w), Ho, B).
-// 32 images of 3 x 112 x 112, 7 x 7, stride 2, 64 filters, the whole call: 1158 -> 65 us (torch's unfold launches one kernel per
-// image, in fp32, and a transpose and two conversions follow).
-__global__ void __launch_bounds__(LAYOUT_THREADS)
-unfold_kernel(const uint16_t* __restrict__ x, uint16_t* __restrict__ dst, ConvGeom g, int pitch, int tile_w, int chan, int cols) {
-  extern __shared__ __align__(16) uint16_t unfold_smem[];
-  const int kk = g.Kh * g.Kw, d = g.C * kk;
-  const int chunk_feats = (chan * kk + 7) & ~7;
-  int* const off = reinterpret_cast<int*>(unfold_smem);                     // [chunk_feats]: element offset of a feature at position 0
-  uint16_t* const img = unfold_smem + 2 * chunk_feats;                      // [chan][Kh][cols], then one zero
-  const int ow0 = blockIdx.x * tile_w, oh = blockIdx.y, b = blockIdx.z;
-  const int n_ow = min(tile_w, g.Wo - ow0);
-  for (int c0 = 0; c0 < g.C; c0 += chan) {
-    const int nc = min(chan, g.C - c0), n_img = nc * g.Kh * cols;
+// The two operands of a convolution's weight gradient, in one launch: blocks below unfold_blocks unfold the input, the others
+// transpose the cotangents.
+//
+// Unfolding: X[(b, oh, ow), f] = x[b, c, oh*sh - ph + kh*dh, ow*sw - pw + kw*dw] (0 outside the image), f = (c*Kh + kh)*Kw + kw: one
+// row of pitch_x bf16 per output position.  A block handles a run of tile_w positions of one output row: the input rows it touches go
+// to shared memory once, `chan` channels at a time and with the image's border as zeros, and every 16-byte group of the
+// result is gathered from there; a thread keeps its group, whose eight offsets stay in registers, and walks over the positions.
+// chan is a multiple of 8 or C, so that a round's features start on a group.
+//
+// Transposing: dY[b, t, f] = gy[b, f, t], [B, F, T] -> [B, T, pitch_y], through 64 x 64 tiles of shared memory; vec: rows of gy are
+// 16-byte multiples and read as such.
+//
+// 32 images of 3 x 112 x 112, 7 x 7, stride 2, 64 filters (43 MB written): 45 -> 25 us against two launches, an offset table read from
+// shared memory for every group and 2-byte reads of the cotangents; the whole call was 1158 us with torch's unfold, which launches
+// one kernel per image, in fp32, before a transpose and two conversions.
+struct ConvOperands {
+  const uint16_t* x;
+  const uint16_t* gy;
+  uint16_t* X;
+  uint16_t* dY;
+  int pitch_x, pitch_y;
+  int tile_w, chan, cols;       // unfolding: positions per block, channels per round, image columns per row in shared memory
+  int w_tiles;                  // ceil(Wo / tile_w)
+  long long unfold_blocks;      // w_tiles * Ho * B
+  int t_tiles, f_tiles;         // transposing: ceil(T / 64), ceil(pitch_y / 64)
+  int vec;
+};
+__device__ __forceinline__ void unfold_block(const ConvOperands& o, const ConvGeom& g, uint16_t* smem) {
+  const int kk = g.Kh * g.Kw;
+  const int chunk_feats = (o.chan * kk + 7) & ~7;
+  int* const off = reinterpret_cast<int*>(smem);                     // [chunk_feats]: element offset of a feature at position 0, -1 beyond
+  uint16_t* const img = smem + 2 * chunk_feats;                      // [chan][Kh][cols]
+  const int ow0 = (int)(blockIdx.x % o.w_tiles) * o.tile_w;
+  const int rest = (int)(blockIdx.x / o.w_tiles), oh = rest % g.Ho, b = rest / g.Ho;
+  const int n_ow = min(o.tile_w, g.Wo - ow0);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int c0 = 0; c0 < g.C; c0 += o.chan) {
+    const int nc = min(o.chan, g.C - c0);
     const int feats = nc * kk, groups = (feats + 7) >> 3;
-    for (int k = threadIdx.x; k < n_img; k += LAYOUT_THREADS) {
-      const int ch = k / (g.Kh * cols), rest = k - ch * g.Kh * cols, kh = rest / cols, w = rest - kh * cols;
-      const int ih = oh * g.sh - g.ph + kh * g.dh, iw = ow0 * g.sw - g.pw + w;
-      uint16_t v = 0;
-      if (ih >= 0 && ih < g.H && iw >= 0 && iw < g.W) v = __ldg(x + (((long long)b * g.C + c0 + ch) * g.H + ih) * g.W + iw);
-      img[k] = v;
+    for (int r = warp; r < nc * g.Kh; r += LAYOUT_THREADS / 32) {
+      const int ch = r / g.Kh, kh = r - ch * g.Kh, ih = oh * g.sh - g.ph + kh * g.dh;
+      const uint16_t* const row = o.x + (((long long)b * g.C + c0 + ch) * g.H + ih) * g.W;
+      for (int w = lane; w < o.cols; w += 32) {
+        const int iw = ow0 * g.sw - g.pw + w;
+        img[r * o.cols + w] = (ih >= 0 && ih < g.H && iw >= 0 && iw < g.W) ? __ldg(row + iw) : (uint16_t)0;
+      }
     }
     for (int f = threadIdx.x; f < groups * 8; f += LAYOUT_THREADS) {
-      const int ch = f / kk, rest = f - ch * kk, kh = rest / g.Kw, kw = rest - kh * g.Kw;
-      off[f] = f < feats ? (ch * g.Kh + kh) * cols + kw * g.dw : -1;
+      const int r = f / g.Kw, kw = f - r * g.Kw;                     // r = ch * Kh + kh
+      off[f] = f < feats ? r * o.cols + kw * g.dw : -1;
     }
     __syncthreads();
-    uint16_t* const out = dst + (((long long)b * g.Ho + oh) * g.Wo + ow0) * pitch + c0 * kk;
-    for (int k = threadIdx.x; k < n_ow * groups; k += LAYOUT_THREADS) {
-      const int tok = k / groups, grp = k - tok * groups;
+    uint16_t* const out = o.X + (((long long)b * g.Ho + oh) * g.Wo + ow0) * o.pitch_x + c0 * kk;
+    for (int g0 = 0; g0 < groups; g0 += LAYOUT_THREADS) {
+      const int width = min(groups - g0, LAYOUT_THREADS), together = LAYOUT_THREADS / width;      // groups side by side, positions at once
+      const int grp = g0 + (int)threadIdx.x % width, first = (int)threadIdx.x / width;
+      if (first >= together) continue;
       const int4 o0 = *reinterpret_cast<const int4*>(off + 8 * grp), o1 = *reinterpret_cast<const int4*>(off + 8 * grp + 4);
-      const int o[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
-      uint32_t v[8];
+      const int at[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
+#pragma unroll 2
+      for (int tok = first; tok < n_ow; tok += together) {
+        uint32_t v[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = o[j] >= 0 ? (uint32_t)img[o[j] + tok * g.sw] : 0u;
-      *reinterpret_cast<uint4*>(out + (long long)tok * pitch + 8 * grp) =
-          make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+        for (int j = 0; j < 8; ++j) v[j] = at[j] >= 0 ? (uint32_t)img[at[j] + tok * g.sw] : 0u;
+        *reinterpret_cast<uint4*>(out + (long long)tok * o.pitch_x + 8 * grp) =
+            make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+      }
     }
     __syncthreads();
   }
 }
-
-// dst[b, t, f] = src[b, f, t]: [B, F, T] -> [B, T, pitch], through 64 x 64 tiles of shared memory.
-// gridDim = (ceil(T / 64), ceil(pitch / 64), B).
-__global__ void __launch_bounds__(LAYOUT_THREADS)
-transpose_rows_kernel(const uint16_t* __restrict__ src, uint16_t* __restrict__ dst, int F, int T, int pitch) {
-  __shared__ uint16_t tile[64][66];            // 66: neighbouring f of one t in different banks
-  const int t0 = blockIdx.x * 64, f0 = blockIdx.y * 64;
-  const uint16_t* const s = src + (long long)blockIdx.z * F * T;
-  for (int k = threadIdx.x; k < 64 * 64; k += LAYOUT_THREADS) {
-    const int f = k >> 6, t = k & 63;
-    tile[f][t] = (f0 + f < F && t0 + t < T) ? __ldg(s + (long long)(f0 + f) * T + t0 + t) : (uint16_t)0;
+constexpr int TRANSPOSE_PITCH = 74;       // elements: 37 words, so that the rows of a column read fall into different banks
+__device__ __forceinline__ void transpose_block(const ConvOperands& o, int F, int T, uint16_t* smem) {
+  const long long k0 = (long long)blockIdx.x - o.unfold_blocks;
+  const int t0 = (int)(k0 % o.t_tiles) * 64;
+  const int rest = (int)(k0 / o.t_tiles), f0 = rest % o.f_tiles * 64, b = rest / o.f_tiles;
+  const uint16_t* const s = o.gy + (long long)b * F * T;
+  if (o.vec) {
+    for (int k = threadIdx.x; k < 64 * 8; k += LAYOUT_THREADS) {
+      const int f = k >> 3, t = (k & 7) * 8;
+      uint4 v = make_uint4(0u, 0u, 0u, 0u);
+      if (f0 + f < F && t0 + t < T) v = __ldg(reinterpret_cast<const uint4*>(s + (long long)(f0 + f) * T + t0 + t));       // T is a multiple of 8
+      uint32_t* const d = reinterpret_cast<uint32_t*>(smem + f * TRANSPOSE_PITCH + t);
+      d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
+    }
+  } else {
+    for (int k = threadIdx.x; k < 64 * 64; k += LAYOUT_THREADS) {
+      const int f = k >> 6, t = k & 63;
+      smem[f * TRANSPOSE_PITCH + t] = (f0 + f < F && t0 + t < T) ? __ldg(s + (long long)(f0 + f) * T + t0 + t) : (uint16_t)0;
+    }
   }
   __syncthreads();
   for (int k = threadIdx.x; k < 64 * 8; k += LAYOUT_THREADS) {
     const int t = k >> 3, f = (k & 7) * 8;
-    if (t0 + t >= T || f0 + f >= pitch) continue;
-    uint32_t o[4];
+    if (t0 + t >= T || f0 + f >= o.pitch_y) continue;
+    uint32_t v[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) o[j] = (uint32_t)tile[f + 2 * j][t] | ((uint32_t)tile[f + 2 * j + 1][t] << 16);
-    *reinterpret_cast<uint4*>(dst + ((long long)blockIdx.z * T + t0 + t) * pitch + f0 + f) = make_uint4(o[0], o[1], o[2], o[3]);
+    for (int j = 0; j < 4; ++j)
+      v[j] = (uint32_t)smem[(f + 2 * j) * TRANSPOSE_PITCH + t] | ((uint32_t)smem[(f + 2 * j + 1) * TRANSPOSE_PITCH + t] << 16);
+    *reinterpret_cast<uint4*>(o.dY + ((long long)b * T + t0 + t) * o.pitch_y + f0 + f) = make_uint4(v[0], v[1], v[2], v[3]);
   }
+}
+__global__ void __launch_bounds__(LAYOUT_THREADS)
+conv_operands_kernel(ConvOperands o, ConvGeom g) {
+  extern __shared__ __align__(16) uint16_t layout_smem[];
+  if ((long long)blockIdx.x < o.unfold_blocks) unfold_block(o, g, layout_smem);
+  else transpose_block(o, g.F, g.Ho * g.Wo, layout_smem);
 }
 
 }  // namespace pe

@@ -139,6 +139,7 @@ struct TcParams {
                        // 0: one accumulation over the whole slice (plain contraction, phi = identity)
   int half_operands;   // 16-bit operands are IEEE half instead of bf16 (the staged per-token statistic)
   int accumulate;      // add the results to what the outputs hold (no zeroing kernel runs before this one)
+  int wait_at_start;   // the kernel before this one in the stream is not the one that zeroes the outputs: wait for it before anything else
   int scalar_out;      // d_in % 4 != 0: the outputs' rows are no 16-byte multiples, so the warps write them themselves
   float* out_mean;     // may be NULL; written through tmap_mean
   float* out_stat;     // may be NULL; written through tmap_stat
@@ -443,7 +444,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   // A packed batch's predecessor is the kernel that fills the side buffer (and zeroes the outputs), an ordinary launch too: the
   // producers wait for it before the first load from there.
   griddep_launch_dependents();
-  if (!RAGGED && (p.nsplit == 1 || p.accumulate)) griddep_wait();
+  if (!RAGGED && p.wait_at_start) griddep_wait();
 
   // Register budget: the epilogue warpgroups hold 128 floats of running sums plus a 32-register TMEM
   // read per thread; the producer / MMA warpgroup needs little.  Each setmaxnreg sits inside the
@@ -688,6 +689,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         float s = s0 + s1;
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+        if (a == 0 && !RAGGED && !p.wait_at_start) griddep_wait();            // the kernel that zeroes out_norms
         if (lane == 0) atomicAdd(p.out_norms + b_begin + a, s);
       } else {
         // CH columns per tensor-memory read: 32, or 16 where the running sums leave few registers (NT = 192; the three
