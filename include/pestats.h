@@ -219,6 +219,10 @@ pe_status_t pe_token_sqstats_f32(const float* X, const float* dY, int B, int T, 
  * than pe_token_sqstats once B*T*(d_in + d_out) reaches about 10^8 elements, slower below (several
  * launches instead of one).  Also the kernel sequence behind pe_token_sqstats_static.  The SIMT path
  * ignores the workspace (it may then be NULL).
+ * From 10^8 elements on the staging is one pass: every chunk of 512 rows has column scales of its own, found and applied while the
+ * rows are in registers, and the contraction undoes them chunk by chunk as it adds the chunks up.  The workspace bytes
+ * reported then include the scales and the padding to whole chunks; a workspace with room for the two-pass form only still gets
+ * that form.
  */
 pe_status_t pe_token_sqstats_staged(const void* X, const void* dY, int B, int T, int d_in, int d_out,
                                     float* out_stat, void* workspace, size_t workspace_bytes,

@@ -33,6 +33,7 @@ static std::atomic<int> g_fused_mode{PE_FUSED_AUTO};
 // of G_b may live in tensor memory beside a 256-column accumulator.
 constexpr int TC_MEAN_TMEM_MIN_T = 4096;
 constexpr int TC_WIDE_MAX_PAD_PERCENT = 13;
+constexpr int PHI_UNSCALE = 4;      // internal phi of the staged per-token statistic: a chunk's scales undone
 constexpr int PHI_CLIP_SCALE = 3;   // internal phi of the clipped sum: c_b * G_b (not part of pe_phi_t)
 constexpr int TC_BAND = 8;          // pair rows per band of the tile order (8 x 256 rows of d_out)
 
@@ -318,7 +319,8 @@ static pe_status_t launch_tc_inst(DeviceInfo* di, int slot, const CUtensorMap& m
 static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int B, int T, int d_in, int d_out, int phi,
                              int per_example, float* out_mean, float* out_stat, cudaStream_t st, bool half_ops = false,
                              float* out_sign = nullptr, bool accumulate = false, const float* sq_norms = nullptr, float clip_norm = 0.f,
-                             int pitch_x = 0, int pitch_y = 0, bool chunked = false) {
+                             int pitch_x = 0, int pitch_y = 0, bool chunked = false, const float* scale_x = nullptr,
+                             const float* scale_y = nullptr) {
   const bool triple = out_sign != nullptr;       // mean + square + sign in one pass (phi = square, all three outputs given)
   const bool both = per_example && ((out_mean && out_stat) || chunked);
   const bool runs = chunked && T > TC_CHUNK_TOKENS;     // several accumulators per example
@@ -378,8 +380,9 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
   p.accumulate = accumulate ? 1 : 0; p.scalar_out = scalar_out ? 1 : 0; p.wait_at_start = ns == 1 || accumulate ? 1 : 0;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, nt, ns, di->sm_count / 2);
   p.out_mean = out_mean; p.out_stat = out_stat; p.out_sign = out_sign; p.out_norms = nullptr; p.dev_status = di->status_ptr;
-  p.seq_offsets = nullptr; p.sq_norms = sq_norms; p.clip_norm = clip_norm;
+  p.seq_offsets = nullptr; p.sq_norms = sq_norms; p.clip_norm = clip_norm; p.scale_x = scale_x; p.scale_y = scale_y;
   dim3 grid(2 * pairs_m * tiles_n, 1, ns);
+  if (phi == PHI_UNSCALE) return launch_tc_inst<4, false, 256, MEAN_NONE>(di, 30, mx, my, mm, ms, msgn, p, grid, st);
   if (phi == PHI_CLIP_SCALE) return launch_tc_inst<3, false, 256, MEAN_NONE>(di, 14, mx, my, mm, ms, msgn, p, grid, st);
   if (runs) {
     if (phi == PE_PHI_SQUARE) return launch_tc_inst<1, false, 128, MEAN_REGS, 128, false, OPT_NONE, false, true>(di, 28, mx, my, mm, ms, msgn, p, grid, st);
@@ -1287,13 +1290,30 @@ pe_status_t pe_token_sqstats(const void* X, const void* dY, int B, int T, int d_
 
 // Workspace of the staged per-token statistic: the column maxima of X and dY (one 32-bit word per
 // column), then the scaled squares of X and of dY (IEEE half, or e4m3 in the fp8 form), each part 256-byte aligned.
+// On large layers (half form) the squares are staged chunk by chunk in one pass instead: the scales of every chunk, then the
+// squares, padded to whole chunks.
 struct StagedLayout {
   size_t max_bytes, x_bytes, y_bytes;
+  long long chunks;           // 0: two passes over the inputs
   size_t total() const { return max_bytes + x_bytes + y_bytes; }
 };
+// From this many input elements on (1.2e8: 419 -> 352 us, 1.7e8: 646 -> 557); below it callers take the one-kernel form.
+constexpr double STAGE_CHUNKS_MIN_ELEMS = 1e8;
+static StagedLayout chunked_layout(int B, int T, int d_in, int d_out) {
+  StagedLayout l;
+  l.chunks = ((long long)B * T + STAGE_CHUNK - 1) / STAGE_CHUNK;
+  l.max_bytes = align_up((size_t)l.chunks * ((size_t)d_in + (size_t)d_out) * sizeof(float), 256);
+  l.x_bytes = align_up((size_t)l.chunks * STAGE_CHUNK * d_in * 2, 256);
+  l.y_bytes = align_up((size_t)l.chunks * STAGE_CHUNK * d_out * 2, 256);
+  return l;
+}
+static bool chunks_pay(int B, int T, int d_in, int d_out) {
+  return (double)B * T * ((double)d_in + d_out) >= STAGE_CHUNKS_MIN_ELEMS && ((long long)B * T + STAGE_CHUNK - 1) / STAGE_CHUNK <= 65535;
+}
 static StagedLayout staged_layout(int B, int T, int d_in, int d_out, bool fp8 = false) {
   const size_t rows = (size_t)B * (size_t)T, es = fp8 ? 1 : 2;
   StagedLayout l;
+  l.chunks = 0;
   l.max_bytes = align_up(((size_t)d_in + (size_t)d_out) * 4, 256);
   l.x_bytes = align_up(rows * d_in * es, 256);
   l.y_bytes = align_up(rows * d_out * es, 256);
@@ -1304,7 +1324,7 @@ static bool token_fp8_ok(int B, int T, int d_in, int d_out) { return token_tc_ok
 
 size_t pe_token_sqstats_staged_workspace_bytes(int B, int T, int d_in, int d_out) {
   if (g_path.load() == PE_PATH_SIMT || !token_tc_ok(B, T, d_in, d_out)) return 0;
-  return staged_layout(B, T, d_in, d_out).total();
+  return (chunks_pay(B, T, d_in, d_out) ? chunked_layout(B, T, d_in, d_out) : staged_layout(B, T, d_in, d_out)).total();
 }
 size_t pe_token_sqstats_fp8_workspace_bytes(int B, int T, int d_in, int d_out) {
   if (g_path.load() == PE_PATH_SIMT || !token_tc_ok(B, T, d_in, d_out)) return 0;
@@ -1377,6 +1397,20 @@ static pe_status_t token_staged_impl(const void* X, const void* dY, int B, int T
     const StagedLayout l = staged_layout(B, T, d_in, d_out, fp8);
     if (!workspace || workspace_bytes < l.total()) return PE_ERR_WORKSPACE;
     if (!aligned(workspace, 256)) return PE_ERR_ALIGN;
+    if (!fp8 && chunks_pay(B, T, d_in, d_out) && workspace_bytes >= chunked_layout(B, T, d_in, d_out).total()) {
+      const StagedLayout c = chunked_layout(B, T, d_in, d_out);
+      float* const scale_x = static_cast<float*>(workspace);
+      float* const scale_y = scale_x + c.chunks * d_in;
+      __half* const hx = reinterpret_cast<__half*>(static_cast<char*>(workspace) + c.max_bytes);
+      __half* const hy = reinterpret_cast<__half*>(static_cast<char*>(workspace) + c.max_bytes + c.x_bytes);
+      const ChunkTensor cx = {static_cast<const uint16_t*>(X), hx, scale_x, d_in}, cy = {static_cast<const uint16_t*>(dY), hy, scale_y, d_out};
+      const int gx = (d_in + 63) / 64, gy = (d_out + 63) / 64;
+      square_chunks_kernel<<<dim3((unsigned)(gx + gy), (unsigned)c.chunks), STAGE_THREADS, 0, st>>>(cx, cy, gx, rows);
+      if ((rc = check_launch()) != PE_OK) return rc;
+      g_last_path.store(PE_PATH_TENSOR);
+      return launch_tc(di, hx, hy, (int)c.chunks, STAGE_CHUNK, d_in, d_out, PHI_UNSCALE, 1, nullptr, out_stat, st, true, nullptr, false, nullptr, 0.f, 0, 0,
+                       false, scale_x, scale_y);
+    }
     uint32_t* max_x = static_cast<uint32_t*>(workspace);
     uint32_t* max_y = max_x + d_in;
     void* x2 = static_cast<char*>(workspace) + l.max_bytes;

@@ -157,6 +157,82 @@ unscale_kernel(float* __restrict__ out, int d_out, int d_in, const uint32_t* __r
   }
 }
 
+// The first two steps in one pass, for large layers: the scale of a column is taken from its largest magnitude among
+// STAGE_CHUNK rows (a chunk) instead of among all, which a block can find and apply with the rows in its registers: the
+// inputs are read once (twice above) and the products of one chunk are unscaled as they are added to the sum, so that
+// unscale_kernel is not needed either.  A chunk's own maximum is never larger than the column's: no value keeps fewer bits.
+// Block: 64 columns x one chunk, 16 rows of 8 columns per thread.  gridDim = (column groups of X, then of dY; chunks).
+// dst is padded to whole chunks (zeros).  inv_scale: [chunks, d], 2^(2e - 13).
+// HBM-bound.  The whole statistic, 16384 rows: 2048 x 8192 646 -> 557 us, 4096 x 4096 (32768 rows) 1159 -> 1054, 1024 x 3000 (40000)
+// 419 -> 352; under the power limit (2048 x 8192, 262144 rows) the contraction's clock drops by what the staging saves.
+constexpr int STAGE_CHUNK = 512;
+struct ChunkTensor {
+  const uint16_t* src;     // [rows, d] bf16 bit patterns
+  __half* dst;             // [chunks * STAGE_CHUNK, d]
+  float* inv_scale;
+  int d;
+};
+__global__ void __launch_bounds__(STAGE_THREADS, 2)
+square_chunks_kernel(ChunkTensor tx_, ChunkTensor ty_, int groups_x, long long rows) {
+  constexpr int PER = STAGE_CHUNK / 32;
+  const bool is_x = (int)blockIdx.x < groups_x;
+  const ChunkTensor& tn = is_x ? tx_ : ty_;
+  __shared__ uint32_t part[8][8][4];
+  const int cg = threadIdx.x & 7, rl = threadIdx.x >> 3, warp = threadIdx.x >> 5;
+  const int col = ((int)blockIdx.x - (is_x ? 0 : groups_x)) * 64 + cg * 8;
+  const bool col_ok = col < tn.d;                    // d is a multiple of 8
+  const long long r0 = (long long)blockIdx.y * STAGE_CHUNK + rl;
+  uint4 v[PER];
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    const long long r = r0 + 32 * i;
+    v[i] = (col_ok && r < rows) ? __ldcs(reinterpret_cast<const uint4*>(tn.src + r * tn.d + col)) : make_uint4(0u, 0u, 0u, 0u);
+  }
+  uint32_t m[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    m[0] = __vmaxu2(m[0], v[i].x & 0x7FFF7FFFu);
+    m[1] = __vmaxu2(m[1], v[i].y & 0x7FFF7FFFu);
+    m[2] = __vmaxu2(m[2], v[i].z & 0x7FFF7FFFu);
+    m[3] = __vmaxu2(m[3], v[i].w & 0x7FFF7FFFu);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    m[k] = __vmaxu2(m[k], __shfl_xor_sync(0xffffffffu, m[k], 8));
+    m[k] = __vmaxu2(m[k], __shfl_xor_sync(0xffffffffu, m[k], 16));
+    if ((threadIdx.x & 31) < 8) part[warp][cg][k] = m[k];
+  }
+  __syncthreads();
+  float sc[8], inv[8];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    uint32_t w = part[0][cg][k];
+#pragma unroll
+    for (int y = 1; y < 8; ++y) w = __vmaxu2(w, part[y][cg][k]);
+    const int e0 = stage_exponent(w & 0xFFFFu), e1 = stage_exponent(w >> 16);
+    sc[2 * k] = stage_scale<false>(e0); sc[2 * k + 1] = stage_scale<false>(e1);
+    inv[2 * k] = stage_inv_scale<false>(e0); inv[2 * k + 1] = stage_inv_scale<false>(e1);
+  }
+  if (!col_ok) return;
+  if (rl == 0) {
+    float4* const at = reinterpret_cast<float4*>(tn.inv_scale + (long long)blockIdx.y * tn.d + col);
+    at[0] = make_float4(inv[0], inv[1], inv[2], inv[3]);
+    at[1] = make_float4(inv[4], inv[5], inv[6], inv[7]);
+  }
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+    uint32_t o[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float a = __uint_as_float(w[k] << 16), b = __uint_as_float(w[k] & 0xFFFF0000u);
+      const __half2 h = __floats2half2_rn(a * a * sc[2 * k], b * b * sc[2 * k + 1]);
+      o[k] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    *reinterpret_cast<uint4*>(tn.dst + (r0 + 32 * i) * tn.d + col) = make_uint4(o[0], o[1], o[2], o[3]);
+  }
+}
+
 // Packed (ragged) batches, Section 2.3: example b owns token rows offsets[b] .. offsets[b+1]-1.  The tensor-core
 // kernel contracts 16 tokens per instruction, so a sequence's last len % 16 tokens are copied here, followed
 // by zero rows up to 16, into tails [B, 16, d] (an empty sequence gets 16 zero rows): that group is then

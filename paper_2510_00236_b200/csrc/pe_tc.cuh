@@ -148,6 +148,8 @@ struct TcParams {
   const int* seq_offsets;   // RAGGED only: [B + 1] token-row offsets; example b owns rows offsets[b] .. offsets[b+1]-1
   int by_tokens;            // RAGGED only: the batch is sliced by tokens instead of by examples
   const float* sq_norms;    // PHI == 3 only: [B] per-example squared norms the clipping coefficient is taken from
+  const float* scale_x;     // PHI == 4 only: [B, d_in] and [B, d_out] factors of example b's columns and rows of G_b
+  const float* scale_y;
   float clip_norm;          // PHI == 3 only: C of c_b = min(1, C / sqrt(N_b))
   unsigned int* dev_status;
 };
@@ -356,7 +358,8 @@ __device__ __forceinline__ void fused_update_piece(const FusedOpt& o, const TcPa
 
 // RAGGED: packed batch with per-example token ranges (tmap_x / tmap_dy are then (d, rows, 1), tmap_x_tail /
 // tmap_dy_tail (d, 16, B) over the zero-padded last partial token groups); otherwise the tail maps are unused.
-// PHI: 0 identity, 1 square, 2 sign, 3 the clipping scale c_b * g with c_b = min(1, C / sqrt(N_b)).
+// PHI: 0 identity, 1 square, 2 sign, 3 the clipping scale c_b * g with c_b = min(1, C / sqrt(N_b)), 4 the factors
+// scale_y[b, o] * scale_x[b, i] * g[o, i] (powers of two: the staged per-token statistic, whose examples are chunks of rows).
 // CHUNKED: an example's tokens are contracted TC_CHUNK_TOKENS at a time, each run into an accumulator of its own, and the
 // runs are added in registers (round to nearest).  The tensor core truncates when it adds to an accumulator, which shrinks a sum of
 // n instructions by about n * 2^-25: 6e-6 (G_b) and 1.2e-5 (G_b^2) at 6000 tokens, against 5e-7 and 1e-6 with runs of 512, what
@@ -382,7 +385,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   static_assert(!NORMS || (PHI == 1 && NT == 256), "per-example norms: squares on the 256 x 256 tile");
   static_assert(MEAN != MEAN_TMEM || (NT == 256 && PHI != 0), "the tensor-memory mean sits beside one 256-column accumulator");
   static_assert(!RAGGED || (!TF32 && MEAN != MEAN_TMEM), "packed batches: 16-bit operands, several accumulators");
-  static_assert(PHI != 3 || MEAN == MEAN_NONE, "the clipped sum is a statistic-only pass");
+  static_assert((PHI != 3 && PHI != 4) || MEAN == MEAN_NONE, "the clipped sum and the scaled contraction are statistic-only passes");
   static_assert(!CHUNKED || (MEAN == MEAN_REGS && NT == 128 && !RAGGED && OPT == OPT_NONE && Op::GROUP == 1), "runs of an example: the two-sum kernel on the 256 x 128 tile");
   constexpr int CHUNK_STAGES = CHUNKED ? TC_CHUNK_TOKENS / BKT : 1;
   constexpr int REGS_CONTROL = CHUNKED ? 40 : Op::REGS_CONTROL, REGS_EPILOGUE = CHUNKED ? 232 : Op::REGS_EPILOGUE;
@@ -578,6 +581,8 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
 #pragma unroll
     for (int j = 0; j < N_MEAN; ++j) acc_mean[j] = 0.f;
     bool ok = true;
+    int tile_m, tile_n;
+    tc_tile_of_block(p, rank, tile_m, tile_n);
     // per-example mode: one accumulator unit per example (or group), in order; plain mode: each accumulator once
     const int n_runs = CHUNKED ? (p.T + TC_CHUNK_TOKENS - 1) / TC_CHUNK_TOKENS : 1;      // accumulators per example
     const int n_acc = p.per_example ? nu * n_runs : min(nu, UNITS);
@@ -596,6 +601,12 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         const float nb2 = __ldg(p.sq_norms + b_begin + a);
         const float nrm = sqrtf(nb2);
         const float c = nrm > p.clip_norm ? p.clip_norm / nrm : 1.f;
+        coef2 = f32x2_pack(c, c);
+      }
+      // PHI == 4: this row's factor; the columns' are loaded beside each tensor-memory read
+      if constexpr (PHI == 4) {
+        const int row = tile_m * TC_TILE_M + q * 32 + lane;
+        const float c = row < p.d_out ? __ldg(p.scale_y + (long long)(b_begin + a) * p.d_out + row) : 0.f;
         coef2 = f32x2_pack(c, c);
       }
       // every lane polls, but the warp acts on one answer: the tensor-memory loads below are warp-wide
@@ -699,6 +710,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         // grouped examples: the unit's accumulators one after the other; the unit is released after the last read
         const int in_unit = (GROUP > 1) ? min(GROUP, nb - GROUP * a) : 1;
         // phi and the running sums for one read of CH columns (chunk c of this thread's COLS columns)
+        float4 col_scale[PHI == 4 ? CH / 4 : 1];
         auto fold = [&](const uint32_t (&r)[CH], int c) {
           if constexpr (PHI == 2) {
             // the running sum holds sum_b (sign(G_b) + 1) / 2 until the write-out turns it into sum_b sign(G_b)
@@ -721,6 +733,12 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
                 const uint64_t m2 = f32x2_add(f32x2_pack(acc_mean[c * CH + j], acc_mean[c * CH + j + 1]), g2);
                 f32x2_unpack(m2, acc_mean[c * CH + j], acc_mean[c * CH + j + 1]);
               }
+              if constexpr (PHI == 4) {
+                const float4 f = col_scale[j >> 2];
+                const uint64_t f2 = (j & 2) ? f32x2_pack(f.z, f.w) : f32x2_pack(f.x, f.y);
+                const uint64_t s2 = f32x2_fma(f32x2_mul(g2, f2), coef2, f32x2_pack(acc_stat[c * CH + j], acc_stat[c * CH + j + 1]));
+                f32x2_unpack(s2, acc_stat[c * CH + j], acc_stat[c * CH + j + 1]);
+              }
               if (PHI == 1 || PHI == 3) {
                 const uint64_t s2 = f32x2_fma(g2, PHI == 1 ? g2 : coef2, f32x2_pack(acc_stat[c * CH + j], acc_stat[c * CH + j + 1]));
                 f32x2_unpack(s2, acc_stat[c * CH + j], acc_stat[c * CH + j + 1]);
@@ -742,7 +760,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         // tensor-memory latency.  That latency, paid twice per example, was a third of the two-sum epilogue's time
         // per example, which is what bounds short sequences (the three-statistic epilogue, bound by its instruction
         // count, gains 2-3 %).
-        constexpr bool PIPELINED = (CH == 32 && PHI != 3) || (TRIPLE && NT == 128);
+        constexpr bool PIPELINED = (CH == 32 && PHI != 3 && PHI != 4) || (TRIPLE && NT == 128);
         if constexpr (PIPELINED) {
           constexpr int TOTAL = GROUP * NCH;          // reads per unit when every example of the group exists
           const int n_reads = in_unit * NCH;
@@ -768,6 +786,13 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
 #pragma unroll
             for (int c = 0; c < NCH; ++c) {
               uint32_t r[CH];
+              if constexpr (PHI == 4) {
+                const int col = tile_n * NT + h * COLS + c * CH;
+#pragma unroll
+                for (int j = 0; j < CH / 4; ++j)
+                  col_scale[j] = col + 4 * j < p.d_in ? __ldg(reinterpret_cast<const float4*>(p.scale_x + (long long)(b_begin + a) * p.d_in + col) + j)
+                                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+              }
               if constexpr (CH == 32) tmem_ld_32x32b_x32_wait(taddr_j + c * CH, r);
               else tmem_ld_32x32b_x16_wait(taddr_j + c * CH, r);
               if (c == NCH - 1 && ju == in_unit - 1) release_unit();
@@ -804,8 +829,6 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       for (int j = 0; j < N_STAT; ++j) acc_stat[j] = fmaf(2.f, acc_stat[j], -nbf);
     }
     constexpr int PANELS = COLS / 32;
-    int tile_m, tile_n;
-    tc_tile_of_block(p, rank, tile_m, tile_n);
     // each epilogue warp stages in its own eighth of the operand ring: 6 panels of 4 KiB (7 at NT = 192)
     constexpr int WARP_PANELS = (STAGES * STAGE_BYTES / 8) / 4096;
     static_assert(WARP_PANELS >= PANELS, "an epilogue warp stages one output at a time");
