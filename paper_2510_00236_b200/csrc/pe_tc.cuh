@@ -258,6 +258,7 @@ __device__ __forceinline__ float phi_apply(float g) {
 __global__ void __launch_bounds__(256) zero_outputs_kernel(float4* __restrict__ a, float4* __restrict__ b, float4* __restrict__ c,
                                                            long long n, unsigned int* __restrict__ counters, int n_counters) {
   sm100::griddep_launch_dependents();
+  sm100::griddep_wait();          // (nothing to wait for in an ordinary launch)
   const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
   const long long stride = (long long)gridDim.x * blockDim.x;
   if (counters)
@@ -700,7 +701,6 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         float s = s0 + s1;
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-        if (a == 0 && !RAGGED && !p.wait_at_start) griddep_wait();            // the kernel that zeroes out_norms
         if (lane == 0) atomicAdd(p.out_norms + b_begin + a, s);
       } else {
         // CH columns per tensor-memory read: 32, or 16 where the running sums leave few registers (NT = 192; the three
