@@ -42,7 +42,7 @@ struct DeviceInfo {
   std::atomic<int> state{0};     // 0 unknown, 1 ready, -1 failed
   int cc_major = 0, sm_count = 0;
   unsigned int* status_ptr = nullptr;
-  bool tc_attr_set[32] = {};
+  bool tc_attr_set[64] = {};
   bool tok_attr_set = false;
 };
 static DeviceInfo g_dev[MAX_DEVICES];
@@ -183,36 +183,61 @@ constexpr UnitCost COST_ALL_192 = {192, 0.375 / 128, 0.60 / 128, 0.05, 0.95, 11.
 constexpr UnitCost COST_ALL_128 = {128, 0.35 / 128, 0.44 / 128, 0.16, 0.55, 9.5};
 constexpr UnitCost COST_ALL_SHORT = {128, 0.05 / 32, 0.10 / 32, 0.0, 0.54, 9.5};
 
+// One pair per two SMs that walks over the tiles (PERSIST) instead of a pair per tile.  It saves the prologue and the teardown, and
+// tensor work of the next tile overlaps the write-out.  What is lost: pairs that run faster cannot take more tiles (64 x 256 x 512 x 16384,
+// three statistics: 321 -> 328 us).  Slices of the last wave stay one to a pair: 40 x 200 x 640 x 8000 (54 tiles left), both outputs, 104 us
+// unsplit, 125 to 135 in 2 to 5 slices.
+constexpr double PERSIST_SAVES = 3.5;             // per unit after a pair's first
+constexpr double PERSIST_DRIFT = 1.025;
+constexpr double TAIL_SPLIT_OUTPUT = 3.5;         // per output of a unit whose sums are added: exchange over the lanes, atomic adds
+
+struct LaunchCost {
+  double us;
+  int tail_split;             // 0: a pair per tile; otherwise one pair per two SMs, the tiles of the last wave in this many slices
+};
 // Time of a launch of `tiles` tiles in ns slices of the batch: waves of `slots` pairs, the last one with fewer pairs.
-static double launch_cost(const UnitCost& c, long long tiles, int B, double T, int slots, int ns, double out_bytes) {
-  const long long units = tiles * ns, full = units / slots, rest = units % slots;
-  const double per = (double)(((long long)B + ns - 1) / ns);
-  auto unit = [&](double busy) {
+static LaunchCost launch_cost(const UnitCost& c, long long tiles, int B, double T, int slots, int ns, int outputs, double out_bytes, bool may_persist) {
+  auto unit = [&](long long examples, double busy) {
     const double ex = T * (c.token_lo + (c.token_hi - c.token_lo) * busy) + c.example;
-    return per * (ex > c.example_min ? ex : c.example_min) + c.fixed + (ns > 1 ? SPLIT_FIXED : 0.0);
+    return examples * (ex > c.example_min ? ex : c.example_min);
   };
-  return full * unit(1.0) + (rest ? unit((double)rest / slots) : 0.0) + (ns > 1 ? out_bytes / ZERO_BYTES_PER_US : 0.0);
+  const long long units = tiles * ns, full = units / slots, rest = units % slots, per = ((long long)B + ns - 1) / ns;
+  const double fixed = c.fixed + (ns > 1 ? SPLIT_FIXED : 0.0), last = (double)rest / slots;
+  LaunchCost best = {full * (unit(per, 1.0) + fixed) + (rest ? unit(per, last) + fixed : 0.0) + (ns > 1 ? out_bytes / ZERO_BYTES_PER_US : 0.0), 0};
+  if (!may_persist || ns > 1 || tiles <= slots) return best;
+  const double whole = full * (unit(per, 1.0) * PERSIST_DRIFT + c.fixed - PERSIST_SAVES) + PERSIST_SAVES;
+  const double plain = whole + (rest ? unit(per, last) + c.fixed - PERSIST_SAVES : 0.0);
+  if (plain < best.us) best = {plain, 1};
+  // the last wave's tiles in slices, as many as leave one unit to a pair
+  const int k = rest ? (int)std::min<long long>(slots / rest, B) : 1;
+  if (k > 1) {
+    const double split = whole + unit(((long long)B + k - 1) / k, last * k) + c.fixed - PERSIST_SAVES + outputs * TAIL_SPLIT_OUTPUT;
+    if (split < best.us) best = {split, k};
+  }
+  return best;
 }
 struct TilePlan {
   int choice, ns;             // index into the candidates, batch slices
+  int tail_split;             // as in LaunchCost
 };
 // The cheapest of the candidate kernels and slice counts.
-static TilePlan plan_tiles(const UnitCost* cand, int n_cand, int B, double T, int d_in, int d_out, int slots, int max_split, int outputs) {
-  TilePlan best = {0, 1};
+static TilePlan plan_tiles(const UnitCost* cand, int n_cand, int B, double T, int d_in, int d_out, int slots, int max_split, int outputs,
+                           bool may_persist = false) {
+  TilePlan best = {0, 1, 0};
   double best_cost = 1e300;
   const long long pairs_m = ((long long)d_out + TC_PAIR_M - 1) / TC_PAIR_M;
   const double out_bytes = 4.0 * outputs * d_in * d_out;
   for (int k = 0; k < n_cand; ++k) {
     const long long tiles = pairs_m * ((d_in + cand[k].nt - 1) / cand[k].nt);
     for (int ns = 1; ns <= max_split && ns <= B && (ns == 1 || tiles * (ns - 1) < 16ll * slots); ++ns) {
-      const double cost = launch_cost(cand[k], tiles, B, T, slots, ns, out_bytes);
-      if (cost < best_cost * 0.995) { best_cost = cost; best = {k, ns}; }
+      const LaunchCost cost = launch_cost(cand[k], tiles, B, T, slots, ns, outputs, out_bytes, may_persist);
+      if (cost.us < best_cost * 0.995) { best_cost = cost.us; best = {k, ns, cost.tail_split}; }
     }
   }
   return best;
 }
 
-// Pair rows per band of the tile order (tc_tile_of_block).  Thread blocks start in the order of their index, `slots`
+// Pair rows per band of the tile order (tc_tile_of_pair).  Thread blocks start in the order of their index, `slots`
 // CTA pairs at a time, the batch slices one after the other; such a wave streams, for every example of its slice, the dY
 // panels of the pair rows and the X panels of the column tiles it touches, and between two waves the batch has passed
 // through L2.  So the bytes a launch reads from HBM follow the sum over waves of (pair rows x 256 + column tiles x nt):
@@ -300,7 +325,7 @@ static pe_status_t zero_for_split(DeviceInfo* di, float* a, float* b, size_t n, 
 }
 
 // mxt, myt: the maps of the zero-padded tail groups of a packed batch (RAGGED); any valid map otherwise.
-template <int PHI, bool TF32, int NT, int MEAN, int BKT = tc_default_bk(TF32, NT), bool RAGGED = false, int OPT = OPT_NONE, bool F8 = false, bool CHUNKED = false>
+template <int PHI, bool TF32, int NT, int MEAN, int BKT = tc_default_bk(TF32, NT), bool RAGGED = false, int OPT = OPT_NONE, bool F8 = false, bool CHUNKED = false, bool PERSIST = false>
 static pe_status_t launch_tc_inst(DeviceInfo* di, int slot, const CUtensorMap& mx, const CUtensorMap& my, const CUtensorMap& mm,
                                   const CUtensorMap& ms, const CUtensorMap& msgn, const TcParams& p, dim3 grid, cudaStream_t st,
                                   const CUtensorMap* mxt = nullptr, const CUtensorMap* myt = nullptr, const FusedOpt* opt = nullptr) {
@@ -308,15 +333,24 @@ static pe_status_t launch_tc_inst(DeviceInfo* di, int slot, const CUtensorMap& m
   {
     std::lock_guard<std::mutex> lock(g_dev_mutex);
     if (!di->tc_attr_set[slot]) {
-      if (cudaFuncSetAttribute(tc_stats_kernel<PHI, TF32, NT, MEAN, BKT, RAGGED, OPT, F8, CHUNKED>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+      if (cudaFuncSetAttribute(tc_stats_kernel<PHI, TF32, NT, MEAN, BKT, RAGGED, OPT, F8, CHUNKED, PERSIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
         cudaGetLastError();
         return PE_ERR_CUDA;
       }
       di->tc_attr_set[slot] = true;
     }
   }
-  return launch_dependent(tc_stats_kernel<PHI, TF32, NT, MEAN, BKT, RAGGED, OPT, F8, CHUNKED>, grid, TC_THREADS, smem, st, mx, my, mm, ms, msgn,
+  return launch_dependent(tc_stats_kernel<PHI, TF32, NT, MEAN, BKT, RAGGED, OPT, F8, CHUNKED, PERSIST>, grid, TC_THREADS, smem, st, mx, my, mm, ms, msgn,
                             mxt ? *mxt : mx, myt ? *myt : my, p, opt ? *opt : FusedOpt{});
+}
+
+// The same with one tile per pair, or (persist) one pair per two SMs that walks over the tiles.
+template <int PHI, int NT, int MEAN, int BKT = tc_default_bk(false, NT), bool CHUNKED = false>
+static pe_status_t launch_tc_tiles(DeviceInfo* di, int slot, bool persist, const CUtensorMap& mx, const CUtensorMap& my, const CUtensorMap& mm,
+                                   const CUtensorMap& ms, const CUtensorMap& msgn, const TcParams& p, dim3 grid, cudaStream_t st) {
+  if (!persist) return launch_tc_inst<PHI, false, NT, MEAN, BKT, false, OPT_NONE, false, CHUNKED>(di, slot, mx, my, mm, ms, msgn, p, grid, st);
+  grid.x = 2 * (di->sm_count / 2);
+  return launch_tc_inst<PHI, false, NT, MEAN, BKT, false, OPT_NONE, false, CHUNKED, true>(di, 32 + slot, mx, my, mm, ms, msgn, p, grid, st);
 }
 
 // Tensor-core launch.  per_example = 0 runs the plain contraction over all B*T rows (its result goes
@@ -345,7 +379,11 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
   } else {
     cand[n_cand++] = !per_example ? COST_PLAIN : phi == PE_PHI_SIGN ? COST_SIGN : COST_STAT;
   }
-  const TilePlan plan = plan_tiles(cand, n_cand, B, T, d_in, d_out, slots, max_split, (out_mean ? 1 : 0) + (out_stat ? 1 : 0) + (out_sign ? 1 : 0));
+  // Several tiles per pair: rows of whole 32-byte sectors (others, written in parts of sectors, 12 x 100 x 900 x 20001, three statistics: 160 us
+  // against 252), and 16-bit counts of examples.
+  const bool may_persist = per_example && !accumulate && d_in % 8 == 0 && aligned(out_mean, 32) && aligned(out_stat, 32) && aligned(out_sign, 32) &&
+                           !(triple && B > TC_SIGN_COUNT_MAX);
+  const TilePlan plan = plan_tiles(cand, n_cand, B, T, d_in, d_out, slots, max_split, (out_mean ? 1 : 0) + (out_stat ? 1 : 0) + (out_sign ? 1 : 0), may_persist);
   const long long pad192 = (long long)((d_in + 191) / 192) * 192, pad128 = (long long)((d_in + 127) / 128) * 128;
   const bool mean_tmem = both && !triple && !runs && forced != PE_PATH_TENSOR_NARROW && forced != PE_PATH_TENSOR_WIDE && T >= TC_MEAN_TMEM_MIN_T &&
                          pad192 * 100 > pad128 * (100 + TC_WIDE_MAX_PAD_PERCENT);
@@ -388,34 +426,46 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
   p.out_mean = out_mean; p.out_stat = out_stat; p.out_sign = out_sign; p.out_norms = nullptr; p.dev_status = di->status_ptr;
   p.seq_offsets = nullptr; p.sq_norms = sq_norms; p.clip_norm = clip_norm; p.scale_x = scale_x; p.scale_y = scale_y;
   dim3 grid(2 * pairs_m * tiles_n, 1, ns);
-  if (phi == PHI_UNSCALE) return launch_tc_inst<4, false, 256, MEAN_NONE>(di, 30, mx, my, mm, ms, msgn, p, grid, st);
-  if (phi == PHI_CLIP_SCALE) return launch_tc_inst<3, false, 256, MEAN_NONE>(di, 14, mx, my, mm, ms, msgn, p, grid, st);
-  if (runs) {
-    if (phi == PE_PHI_SQUARE) return launch_tc_inst<1, false, 128, MEAN_REGS, 128, false, OPT_NONE, false, true>(di, 28, mx, my, mm, ms, msgn, p, grid, st);
-    return launch_tc_inst<2, false, 128, MEAN_REGS, 128, false, OPT_NONE, false, true>(di, 29, mx, my, mm, ms, msgn, p, grid, st);
+  const bool persist = plan.tail_split > 0 && ns == 1 && !mean_tmem;
+  if (persist) {
+    const int tiles = pairs_m * tiles_n;
+    p.tail_split = plan.tail_split;
+    p.whole_tiles = plan.tail_split > 1 ? tiles - tiles % slots : tiles;
+    if (plan.tail_split > 1) {
+      p.wait_at_start = 0;
+      zero_tail_tiles_kernel<<<di->sm_count, 256, 0, st>>>(p, nt);
+      rc = check_launch();
+      if (rc != PE_OK) return rc;
+    }
   }
-  if (triple && wide) return launch_tc_inst<1, false, 192, MEAN_HYBRID_SIGN>(di, 26, mx, my, mm, ms, msgn, p, grid, st);
-  if (triple && short_seq) return launch_tc_inst<1, false, 128, MEAN_REGS_SIGN, TC_SHORT_BK>(di, 27, mx, my, mm, ms, msgn, p, grid, st);
-  if (triple) return launch_tc_inst<1, false, 128, MEAN_REGS_SIGN>(di, 10, mx, my, mm, ms, msgn, p, grid, st);
+  if (phi == PHI_UNSCALE) return launch_tc_tiles<4, 256, MEAN_NONE>(di, 30, persist, mx, my, mm, ms, msgn, p, grid, st);
+  if (phi == PHI_CLIP_SCALE) return launch_tc_tiles<3, 256, MEAN_NONE>(di, 14, persist, mx, my, mm, ms, msgn, p, grid, st);
+  if (runs) {
+    if (phi == PE_PHI_SQUARE) return launch_tc_tiles<1, 128, MEAN_REGS, 128, true>(di, 28, persist, mx, my, mm, ms, msgn, p, grid, st);
+    return launch_tc_tiles<2, 128, MEAN_REGS, 128, true>(di, 29, persist, mx, my, mm, ms, msgn, p, grid, st);
+  }
+  if (triple && wide) return launch_tc_tiles<1, 192, MEAN_HYBRID_SIGN>(di, 26, persist, mx, my, mm, ms, msgn, p, grid, st);
+  if (triple && short_seq) return launch_tc_tiles<1, 128, MEAN_REGS_SIGN, TC_SHORT_BK>(di, 27, persist, mx, my, mm, ms, msgn, p, grid, st);
+  if (triple) return launch_tc_tiles<1, 128, MEAN_REGS_SIGN>(di, 10, persist, mx, my, mm, ms, msgn, p, grid, st);
   if (!per_example) return launch_tc_inst<0, false, 256, MEAN_NONE>(di, 4, mx, my, mm, ms, msgn, p, grid, st);
   if (short_seq) {
-    if (phi == PE_PHI_SQUARE) return launch_tc_inst<1, false, 128, MEAN_REGS, TC_SHORT_BK>(di, 8, mx, my, mm, ms, msgn, p, grid, st);
-    return launch_tc_inst<2, false, 128, MEAN_REGS, TC_SHORT_BK>(di, 9, mx, my, mm, ms, msgn, p, grid, st);
+    if (phi == PE_PHI_SQUARE) return launch_tc_tiles<1, 128, MEAN_REGS, TC_SHORT_BK>(di, 8, persist, mx, my, mm, ms, msgn, p, grid, st);
+    return launch_tc_tiles<2, 128, MEAN_REGS, TC_SHORT_BK>(di, 9, persist, mx, my, mm, ms, msgn, p, grid, st);
   }
   if (wide) {
-    if (phi == PE_PHI_SQUARE) return launch_tc_inst<1, false, 192, MEAN_REGS>(di, 12, mx, my, mm, ms, msgn, p, grid, st);
-    return launch_tc_inst<2, false, 192, MEAN_REGS>(di, 13, mx, my, mm, ms, msgn, p, grid, st);
+    if (phi == PE_PHI_SQUARE) return launch_tc_tiles<1, 192, MEAN_REGS>(di, 12, persist, mx, my, mm, ms, msgn, p, grid, st);
+    return launch_tc_tiles<2, 192, MEAN_REGS>(di, 13, persist, mx, my, mm, ms, msgn, p, grid, st);
   }
   if (mean_regs) {
-    if (phi == PE_PHI_SQUARE) return launch_tc_inst<1, false, 128, MEAN_REGS>(di, 0, mx, my, mm, ms, msgn, p, grid, st);
-    return launch_tc_inst<2, false, 128, MEAN_REGS>(di, 1, mx, my, mm, ms, msgn, p, grid, st);
+    if (phi == PE_PHI_SQUARE) return launch_tc_tiles<1, 128, MEAN_REGS>(di, 0, persist, mx, my, mm, ms, msgn, p, grid, st);
+    return launch_tc_tiles<2, 128, MEAN_REGS>(di, 1, persist, mx, my, mm, ms, msgn, p, grid, st);
   }
   if (both) {
     if (phi == PE_PHI_SQUARE) return launch_tc_inst<1, false, 256, MEAN_TMEM>(di, 6, mx, my, mm, ms, msgn, p, grid, st);
     return launch_tc_inst<2, false, 256, MEAN_TMEM>(di, 7, mx, my, mm, ms, msgn, p, grid, st);
   }
-  if (phi == PE_PHI_SQUARE) return launch_tc_inst<1, false, 256, MEAN_NONE>(di, 2, mx, my, mm, ms, msgn, p, grid, st);
-  return launch_tc_inst<2, false, 256, MEAN_NONE>(di, 3, mx, my, mm, ms, msgn, p, grid, st);
+  if (phi == PE_PHI_SQUARE) return launch_tc_tiles<1, 256, MEAN_NONE>(di, 2, persist, mx, my, mm, ms, msgn, p, grid, st);
+  return launch_tc_tiles<2, 256, MEAN_NONE>(di, 3, persist, mx, my, mm, ms, msgn, p, grid, st);
 }
 
 // Per-example squared norms on the tensor cores: the statistic-only 256 x 256 schedule, but every

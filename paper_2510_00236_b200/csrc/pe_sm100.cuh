@@ -340,6 +340,37 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 // predecessor has executed launch_dependents (or exited); wait() then blocks until the predecessor
 // has completed and its writes are visible.  Both are no-ops in a kernel launched the ordinary way.
 __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// One whole 32-byte sector per lane (p: 32-byte aligned).
+__device__ __forceinline__ void st_global_v8(float* p, const float* v) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]),
+               "f"(v[6]), "f"(v[7]) : "memory");
+}
+// Register transposes over the lanes, by exchanges of half of the values at a time.  Every lane holds 32 consecutive values of
+// a row of its own.  quad_transpose: afterwards lane 4g+i holds values 8i .. 8i+7 of the quad's row j in v[8j ..], so that
+// 32-byte stores of v[8j ..] by the quad cover 128 consecutive bytes.  warp_transpose: afterwards lane l holds value l of
+// row r in v[r].
+template <int S, int BLOCK>     // exchanges with the lane S away: blocks of BLOCK values whose number differs in one bit
+__device__ __forceinline__ void transpose_step(float (&v)[32], int lane) {
+  const bool high = lane & S;
+#pragma unroll
+  for (int k = 0; k < 32; ++k) {
+    if (k & BLOCK) continue;
+    const float got = __shfl_xor_sync(0xffffffffu, high ? v[k] : v[k + BLOCK], S);
+    v[k] = high ? got : v[k];
+    v[k + BLOCK] = high ? v[k + BLOCK] : got;
+  }
+}
+__device__ __forceinline__ void quad_transpose(float (&v)[32], int lane) {
+  transpose_step<2, 16>(v, lane);
+  transpose_step<1, 8>(v, lane);
+}
+__device__ __forceinline__ void warp_transpose(float (&v)[32], int lane) {
+  transpose_step<16, 16>(v, lane);
+  transpose_step<8, 8>(v, lane);
+  transpose_step<4, 4>(v, lane);
+  transpose_step<2, 2>(v, lane);
+  transpose_step<1, 1>(v, lane);
+}
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Packed fp32 pairs (two floats in one 64-bit register, one instruction for both).

@@ -26,7 +26,8 @@
 //                        tile is reduced and added to out_norms[b]                 -- per-example squared norms
 //   PHI = 0,   NT = 256: no per-example reset (accumulate in tensor memory)        -- plain contraction over all rows
 // Further template arguments: RAGGED (packed batches with per-example token ranges), OPT (the parameter
-// update applied by the block that completes a tile's sums), F8 (e4m3 operands for the plain contraction).
+// update applied by the block that completes a tile's sums), F8 (e4m3 operands for the plain contraction), CHUNKED (several
+// accumulators per example), PERSIST (several tiles per pair).
 //
 // Warp roles per block (12 warps): 0 = TMA producer of the dY boxes, 2 = TMEM allocator, then TMA
 // producer of the X boxes, 1 = MMA issuer (leader block only), 3 idle, 4..11 = epilogue (warp w reads
@@ -41,6 +42,14 @@
 // earlier ones.  (MEAN_TMEM has one accumulator: while the epilogue drains it the producers keep filling
 // the ring, and the issuer then works the backlog off at full tensor rate, which absorbs the pause as long
 // as the operand supply, not the tensor pipe, is what bounds the example.)
+//
+// PERSIST: layers of more tiles than pairs.  A pair per two SMs takes every (gridDim.x / 2)-th unit: the tensor work of a tile starts
+// while the one before is written out (two accumulators ahead; the write-out goes from registers to memory, past the ring), and
+// prologue and teardown are paid once.  The tiles of the last, partial wave are contracted in slices of the batch, as many
+// as leave every pair one, and added to outputs zeroed beforehand.  Bound by the epilogue (short sequences) or the operand supply as
+// before.  8 x 256 x 1024 x 32104, both outputs 231 -> 174 us, sign 165 -> 121; 128 x 32 x 4096^2, three statistics 577 -> 497;
+// 64 x 256 x 512 x 32768 565 -> 527 (of which the slices 40), sign 477 -> 420; 16 x 1024 x 2048 x 8192, sign 460 -> 405, but
+// sequences of 256 tokens and more gain nothing by the walk alone (64 x 256 x 512 x 16384, three statistics, 321 -> 328 us).
 //
 // Barriers.  full[s] lives in the leader block: its producer posts the byte count of BOTH blocks'
 // loads, and the follower's TMA loads credit their bytes to it through the cluster window.
@@ -135,6 +144,8 @@ struct TcParams {
   int B, T, d_in, d_out;
   int pairs_m, tiles_n, band;   // tile grid: 256-row pair rows x NT-column tiles; pair rows per band of the tile order
   int nsplit;          // batch slices (gridDim.z); > 1 => outputs pre-zeroed, partials added atomically
+  int whole_tiles;     // PERSIST: tiles that one pair contracts over the whole batch; each of the others goes to
+  int tail_split;      // this many pairs, by slices of the batch, whose sums are added to (zeroed) outputs
   int per_example;     // 1: reset the accumulator for every example and apply phi (statistics)
                        // 0: one accumulation over the whole slice (plain contraction, phi = identity)
   int half_operands;   // 16-bit operands are IEEE half instead of bf16 (the staged per-token statistic)
@@ -153,6 +164,18 @@ struct TcParams {
   float clip_norm;          // PHI == 3 only: C of c_b = min(1, C / sqrt(N_b))
   unsigned int* dev_status;
 };
+
+// PERSIST: unit u of the launch, a tile and the examples it is contracted over.
+struct TcUnit {
+  int tile, b_begin, b_end;
+  bool whole;
+};
+__device__ __forceinline__ int tc_units(const TcParams& p) { return p.whole_tiles + (p.pairs_m * p.tiles_n - p.whole_tiles) * p.tail_split; }
+__device__ __forceinline__ TcUnit tc_unit(const TcParams& p, int u) {
+  if (u < p.whole_tiles) return {u, 0, p.B, true};
+  const int rest = p.pairs_m * p.tiles_n - p.whole_tiles, v = u - p.whole_tiles, slice = v / rest;
+  return {p.whole_tiles + v - slice * rest, (int)((long long)p.B * slice / p.tail_split), (int)((long long)p.B * (slice + 1) / p.tail_split), p.tail_split == 1};
+}
 
 // Where an example's tokens are and how many pipeline stages they take.  Fixed-length batches: the
 // operand maps are 3-D (d, T, B), an example is the coordinate `seq` of the last dimension and its
@@ -206,8 +229,7 @@ __device__ __forceinline__ int ragged_slice_begin(const int* offsets, int B, int
 // pair indices sweep the d_in tiles inside a band of p.band pair rows before moving to the next band:
 // the ~74 resident pairs then touch about band*256 columns of dY and 74/band*NT columns of X per
 // example instead of all of dY.  Returns this block's 128-row tile of d_out and NT-column tile of d_in.
-__device__ __forceinline__ void tc_tile_of_block(const TcParams& p, uint32_t rank, int& tile_m, int& tile_n) {
-  const int pair_id = blockIdx.x >> 1;
+__device__ __forceinline__ void tc_tile_of_pair(const TcParams& p, int pair_id, uint32_t rank, int& tile_m, int& tile_n) {
   const int per_band = p.band * p.tiles_n;
   const int band = pair_id / per_band, r = pair_id - band * per_band;
   const int rows = min(p.band, p.pairs_m - band * p.band);      // pair rows in this (possibly last, shorter) band
@@ -274,6 +296,26 @@ __global__ void __launch_bounds__(256) zero_outputs_kernel(float4* __restrict__ 
     reinterpret_cast<float*>(a)[k] = 0.f;
     if (b) reinterpret_cast<float*>(b)[k] = 0.f;
     if (c) reinterpret_cast<float*>(c)[k] = 0.f;
+  }
+}
+
+// Zeroes the tiles from the p.whole_tiles-th on (256 rows x nt columns each) of up to three outputs, for the launch whose last
+// tiles are split over the batch; a warp takes a row of a tile.  At most half a wave of tiles (29 MB for both outputs), while the
+// contraction of the others already runs.
+__global__ void __launch_bounds__(256) zero_tail_tiles_kernel(TcParams p, int nt) {
+  sm100::griddep_launch_dependents();
+  const int rest = p.pairs_m * p.tiles_n - p.whole_tiles, lane = threadIdx.x & 31;
+  for (int k = blockIdx.x * 8 + (threadIdx.x >> 5); k < rest * TC_PAIR_M; k += gridDim.x * 8) {
+    int tile_m, tile_n;
+    tc_tile_of_pair(p, p.whole_tiles + k / TC_PAIR_M, 0, tile_m, tile_n);
+    const int row = tile_m * TC_TILE_M + k % TC_PAIR_M, end = min(p.d_in, (tile_n + 1) * nt);
+    if (row >= p.d_out) continue;
+    for (int col = tile_n * nt + lane; col < end; col += 32) {
+      const long long at = (long long)row * p.d_in + col;
+      if (p.out_mean) p.out_mean[at] = 0.f;
+      if (p.out_stat) p.out_stat[at] = 0.f;
+      if (p.out_sign) p.out_sign[at] = 0.f;
+    }
   }
 }
 
@@ -367,7 +409,7 @@ __device__ __forceinline__ void fused_update_piece(const FusedOpt& o, const TcPa
 // fp32 FMAs in order give too.  64 more registers per epilogue thread, hence the 256 x 128 tile.
 // OPT: the parameter update applied by the block that completes a tile's sums (OPT_ADAM needs both running
 // sums, OPT_SIGN the sign statistic alone); `o` is ignored when OPT == OPT_NONE.
-template <int PHI, bool TF32, int NT, int MEAN, int BKT = tc_default_bk(TF32, NT), bool RAGGED = false, int OPT = OPT_NONE, bool F8 = false, bool CHUNKED = false>
+template <int PHI, bool TF32, int NT, int MEAN, int BKT = tc_default_bk(TF32, NT), bool RAGGED = false, int OPT = OPT_NONE, bool F8 = false, bool CHUNKED = false, bool PERSIST = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
 tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_dy,
                 const __grid_constant__ CUtensorMap tmap_mean, const __grid_constant__ CUtensorMap tmap_stat,
@@ -388,6 +430,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   static_assert(!RAGGED || (!TF32 && MEAN != MEAN_TMEM), "packed batches: 16-bit operands, several accumulators");
   static_assert((PHI != 3 && PHI != 4) || MEAN == MEAN_NONE, "the clipped sum and the scaled contraction are statistic-only passes");
   static_assert(!CHUNKED || (MEAN == MEAN_REGS && NT == 128 && !RAGGED && OPT == OPT_NONE && Op::GROUP == 1), "runs of an example: the two-sum kernel on the 256 x 128 tile");
+  static_assert(!PERSIST || (!RAGGED && OPT == OPT_NONE && MEAN != MEAN_TMEM && !NORMS && PHI != 0), "several tiles per pair: fixed-length batches, whole sums written");
   constexpr int CHUNK_STAGES = CHUNKED ? TC_CHUNK_TOKENS / BKT : 1;
   constexpr int REGS_CONTROL = CHUNKED ? 40 : Op::REGS_CONTROL, REGS_EPILOGUE = CHUNKED ? 232 : Op::REGS_EPILOGUE;
   static_assert(128 * REGS_CONTROL + 256 * REGS_EPILOGUE <= TC_THREADS * TC_REGS_AT_LAUNCH, "setmaxnreg: the epilogue's increase must fit what the control warps give up");
@@ -427,8 +470,9 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       b_end = max(b_begin, ragged_slice_begin(p.seq_offsets, p.B, blockIdx.z + 1, p.nsplit, lane));
     }
   }
-  const int nb = b_end - b_begin;
-  const int nu = (nb + GROUP - 1) / GROUP;          // units of work: groups of GROUP examples (GROUP = 1: the examples)
+  int nb = b_end - b_begin;
+  const int n_units = PERSIST ? tc_units(p) : 1;      // PERSIST: this pair takes every (gridDim.x / 2)-th of them
+  int nu = (nb + GROUP - 1) / GROUP;          // units of work: groups of GROUP examples (GROUP = 1: the examples)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
@@ -461,11 +505,8 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       // Warp 0 loads this block's rows of dY^T (and, in the leader, posts the stage's byte count);
       // warp 2 loads this block's half of the X^T rows.  Both wait for the same "stage empty" phase.
       const bool is_a = (warp == 0);
-      int tile_m, tile_n;
-      tc_tile_of_block(p, rank, tile_m, tile_n);
       const CUtensorMap* tmap = is_a ? &tmap_dy : &tmap_x;
       const CUtensorMap* tmap_tail = is_a ? &tmap_dy_tail : &tmap_x_tail;
-      const int c0 = is_a ? tile_m * TC_TILE_M : tile_n * NT + (int)rank * Op::B_FEATS;   // first feature of this warp's boxes
       const int n_boxes = is_a ? Op::A_BOXES : Op::B_BOXES;
       const int box_feats = is_a ? Op::BOX_FEATS : Op::B_BOX_FEATS;
       const int box_bytes = is_a ? BOX_BYTES : Op::B_BOX_BYTES;
@@ -477,27 +518,39 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       uint32_t ph = 1;
       bool ok = true;
       bool side_ready = false;        // RAGGED: the side buffer is complete
-      for (int e = 0; e < nu && ok; ++e) {
-        const SeqGeom g = seq_geom<RAGGED>(p, b_begin + GROUP * e, BK);
-        for (int kc = 0; kc < g.nk; ++kc) {
-          if (!mbar_wait_warp(empty_bar(s), ph, abort_flag, p.dev_status, TC_WAIT_EMPTY, strict)) { ok = false; break; }
-          if (elect_one()) {
-            const bool tail = RAGGED && kc >= g.nk_main;       // the zero-padded last partial group, from the side buffer (boxes 16 tokens tall)
-            if (is_a && rank == 0) mbar_arrive_expect_tx(full_bar(s), tail ? 2 * STAGE_BYTES / (BK / 16) : 2 * STAGE_BYTES);     // both blocks' bytes
-            const uint32_t leader_full = map_to_cta(full_bar(s), 0);
-            const uint32_t dst = smem_base + s * STAGE_BYTES + (is_a ? 0 : A_BYTES);
-            if (tail && !side_ready) griddep_wait();
-            const CUtensorMap* tm = tail ? tmap_tail : tmap;
-            const int c1 = tail ? 0 : g.row0 + kc * BK;
-            // (grouped examples: the box is GROUP examples deep; past the batch's end it reads zeros)
-            const int c2 = RAGGED ? (tail ? b_begin + e : 0) : b_begin + GROUP * e;
-            for (int b = 0; b < n_boxes; ++b) tma_load_3d_pair(dst + b * box_bytes, tm, leader_full, c0 + b * box_feats, c1, c2);
-          }
-          __syncwarp();
-          if (RAGGED && kc >= g.nk_main) side_ready = true;
-          if (++s == STAGES) { s = 0; ph ^= 1u; }
+      int unit = blockIdx.x >> 1;
+      do {
+        int tile_m, tile_n;
+        if (PERSIST) {
+          const TcUnit t = tc_unit(p, unit);
+          b_begin = t.b_begin; b_end = t.b_end; nb = b_end - b_begin; nu = (nb + GROUP - 1) / GROUP;
+          tc_tile_of_pair(p, t.tile, rank, tile_m, tile_n);
+        } else {
+          tc_tile_of_pair(p, unit, rank, tile_m, tile_n);
         }
-      }
+        const int c0 = is_a ? tile_m * TC_TILE_M : tile_n * NT + (int)rank * Op::B_FEATS;   // first feature of this warp's boxes
+        for (int e = 0; e < nu && ok; ++e) {
+          const SeqGeom g = seq_geom<RAGGED>(p, b_begin + GROUP * e, BK);
+          for (int kc = 0; kc < g.nk; ++kc) {
+            if (!mbar_wait_warp(empty_bar(s), ph, abort_flag, p.dev_status, TC_WAIT_EMPTY, strict)) { ok = false; break; }
+            if (elect_one()) {
+              const bool tail = RAGGED && kc >= g.nk_main;       // the zero-padded last partial group, from the side buffer (boxes 16 tokens tall)
+              if (is_a && rank == 0) mbar_arrive_expect_tx(full_bar(s), tail ? 2 * STAGE_BYTES / (BK / 16) : 2 * STAGE_BYTES);     // both blocks' bytes
+              const uint32_t leader_full = map_to_cta(full_bar(s), 0);
+              const uint32_t dst = smem_base + s * STAGE_BYTES + (is_a ? 0 : A_BYTES);
+              if (tail && !side_ready) griddep_wait();
+              const CUtensorMap* tm = tail ? tmap_tail : tmap;
+              const int c1 = tail ? 0 : g.row0 + kc * BK;
+              // (grouped examples: the box is GROUP examples deep; past the batch's end it reads zeros)
+              const int c2 = RAGGED ? (tail ? b_begin + e : 0) : b_begin + GROUP * e;
+              for (int b = 0; b < n_boxes; ++b) tma_load_3d_pair(dst + b * box_bytes, tm, leader_full, c0 + b * box_feats, c1, c2);
+            }
+            __syncwarp();
+            if (RAGGED && kc >= g.nk_main) side_ready = true;
+            if (++s == STAGES) { s = 0; ph ^= 1u; }
+          }
+        }
+      } while (PERSIST && ok && (unit += gridDim.x >> 1) < n_units);
     } else if (rank == 0 && warp == 1) {
       // ---------------------------------------------------------- MMA issuer (leader block)
       // Unit e (an example, or GROUP of them) goes to accumulator unit e % UNITS.  A plain contraction (per_example == 0)
@@ -506,57 +559,65 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       const uint32_t idesc = (F8 || (!TF32 && p.half_operands)) ? make_idesc_half_mn_major(TC_PAIR_M, NT) : make_idesc_mn_major(TC_PAIR_M, NT, TF32);
       int s = 0;
       uint32_t ph = 0;
-      int run = 0;                    // CHUNKED: accumulators filled so far
+      int run = 0;                    // accumulators filled so far (CHUNKED: several per example)
       bool ok = true;
-      for (int e = 0; e < nu && ok; ++e) {
-        const SeqGeom sg = seq_geom<RAGGED>(p, b_begin + GROUP * e, BK);
-        int buf = e % UNITS;
-        if (p.per_example && !CHUNKED) {
-          if (!mbar_wait_warp(acc_empty_bar(buf), ((uint32_t)(e / UNITS) & 1u) ^ 1u, abort_flag, p.dev_status, TC_WAIT_ACC_EMPTY, strict)) break;
-          tc_fence_after();
+      int unit = blockIdx.x >> 1;
+      do {
+        if (PERSIST) {
+          const TcUnit t = tc_unit(p, unit);
+          b_begin = t.b_begin; b_end = t.b_end; nb = b_end - b_begin; nu = (nb + GROUP - 1) / GROUP;
         }
-        const bool last_of_acc = p.per_example || e + UNITS >= nu;
-        for (int kc = 0; kc < sg.nk; ++kc) {
-          const int kin = CHUNKED ? kc % CHUNK_STAGES : kc;           // stage within its accumulator
-          const bool acc_done = kc == sg.nk - 1 || (CHUNKED && kin == CHUNK_STAGES - 1);
-          if (CHUNKED && kin == 0) {
-            buf = run % UNITS;
-            if (!mbar_wait_warp(acc_empty_bar(buf), ((uint32_t)(run / UNITS) & 1u) ^ 1u, abort_flag, p.dev_status, TC_WAIT_ACC_EMPTY, strict)) { ok = false; break; }
+        for (int e = 0; e < nu && ok; ++e) {
+          const SeqGeom sg = seq_geom<RAGGED>(p, b_begin + GROUP * e, BK);
+          int buf = (PERSIST ? run : e) % UNITS;
+          if (p.per_example && !CHUNKED) {
+            if (!mbar_wait_warp(acc_empty_bar(buf), ((uint32_t)((PERSIST ? run : e) / UNITS) & 1u) ^ 1u, abort_flag, p.dev_status, TC_WAIT_ACC_EMPTY, strict)) { ok = false; break; }
             tc_fence_after();
-            ++run;
+            if (PERSIST) ++run;
           }
-          const uint32_t d_tmem = tmem_base + (uint32_t)(buf * GROUP * NT);
-          if (!mbar_wait_warp(full_bar(s), ph, abort_flag, p.dev_status, TC_WAIT_FULL, strict)) { ok = false; break; }
-          tc_fence_after();
-          if (elect_one()) {
-            const uint32_t a_src = smem_base + s * STAGE_BYTES;
-            const uint32_t b_src = a_src + A_BYTES;
-            // tokens of this example in this stage: the rest of its whole 16-token groups, or the padded tail group
-            const int t_left = (RAGGED && kc >= sg.nk_main) ? 16 : sg.main - kc * BK;
+          const bool last_of_acc = p.per_example || e + UNITS >= nu;
+          for (int kc = 0; kc < sg.nk; ++kc) {
+            const int kin = CHUNKED ? kc % CHUNK_STAGES : kc;           // stage within its accumulator
+            const bool acc_done = kc == sg.nk - 1 || (CHUNKED && kin == CHUNK_STAGES - 1);
+            if (CHUNKED && kin == 0) {
+              buf = run % UNITS;
+              if (!mbar_wait_warp(acc_empty_bar(buf), ((uint32_t)(run / UNITS) & 1u) ^ 1u, abort_flag, p.dev_status, TC_WAIT_ACC_EMPTY, strict)) { ok = false; break; }
+              tc_fence_after();
+              ++run;
+            }
+            const uint32_t d_tmem = tmem_base + (uint32_t)(buf * GROUP * NT);
+            if (!mbar_wait_warp(full_bar(s), ph, abort_flag, p.dev_status, TC_WAIT_FULL, strict)) { ok = false; break; }
+            tc_fence_after();
+            if (elect_one()) {
+              const uint32_t a_src = smem_base + s * STAGE_BYTES;
+              const uint32_t b_src = a_src + A_BYTES;
+              // tokens of this example in this stage: the rest of its whole 16-token groups, or the padded tail group
+              const int t_left = (RAGGED && kc >= sg.nk_main) ? 16 : sg.main - kc * BK;
 #pragma unroll
-            for (int j = 0; j < GROUP; ++j) {
-              // grouped examples: example j of the group sits BK tokens further in every box and has its own accumulator
-              if (GROUP > 1 && GROUP * e + j >= nb) break;
-              uint32_t accumulate = (kin > 0 || (!p.per_example && e >= UNITS)) ? 1u : 0u;
+              for (int j = 0; j < GROUP; ++j) {
+                // grouped examples: example j of the group sits BK tokens further in every box and has its own accumulator
+                if (GROUP > 1 && GROUP * e + j >= nb) break;
+                uint32_t accumulate = (kin > 0 || (!p.per_example && e >= UNITS)) ? 1u : 0u;
 #pragma unroll
-              for (int k = 0; k < BK / Op::MMA_K; ++k) {
-                // rows past T are zero-filled by TMA; whole MMA steps past T are skipped
-                if (k * Op::MMA_K < t_left) {
-                  const uint64_t ad = make_smem_desc(a_src + j * (BK * 128) + k * Op::K_STEP_BYTES, BOX_BYTES, Op::SBO_BYTES, Op::DESC_LAYOUT);
-                  const uint64_t bd = make_smem_desc(b_src + j * (BK * Op::B_ROW_BYTES) + k * Op::B_K_STEP_BYTES, Op::B_BOX_BYTES, Op::B_SBO_BYTES,
-                                                     Op::B_DESC_LAYOUT);
-                  umma_ss_pair<TF32 ? 1 : (F8 ? 2 : 0)>(d_tmem + (uint32_t)(j * NT), ad, bd, idesc, accumulate);
-                  accumulate = 1;
+                for (int k = 0; k < BK / Op::MMA_K; ++k) {
+                  // rows past T are zero-filled by TMA; whole MMA steps past T are skipped
+                  if (k * Op::MMA_K < t_left) {
+                    const uint64_t ad = make_smem_desc(a_src + j * (BK * 128) + k * Op::K_STEP_BYTES, BOX_BYTES, Op::SBO_BYTES, Op::DESC_LAYOUT);
+                    const uint64_t bd = make_smem_desc(b_src + j * (BK * Op::B_ROW_BYTES) + k * Op::B_K_STEP_BYTES, Op::B_BOX_BYTES, Op::B_SBO_BYTES,
+                                                       Op::B_DESC_LAYOUT);
+                    umma_ss_pair<TF32 ? 1 : (F8 ? 2 : 0)>(d_tmem + (uint32_t)(j * NT), ad, bd, idesc, accumulate);
+                    accumulate = 1;
+                  }
                 }
               }
+              umma_commit_pair(empty_bar(s));                // stage reusable in both blocks once these MMAs retire
+              if (last_of_acc && acc_done) umma_commit_pair(acc_full_bar(buf));   // accumulator complete, both blocks
             }
-            umma_commit_pair(empty_bar(s));                // stage reusable in both blocks once these MMAs retire
-            if (last_of_acc && acc_done) umma_commit_pair(acc_full_bar(buf));   // accumulator complete, both blocks
+            __syncwarp();
+            if (++s == STAGES) { s = 0; ph ^= 1u; }
           }
-          __syncwarp();
-          if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
-      }
+      } while (PERSIST && ok && (unit += gridDim.x >> 1) < n_units);
     }
   } else {
     // ------------------------------------------------------------ epilogue (both blocks)
@@ -582,8 +643,17 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
 #pragma unroll
     for (int j = 0; j < N_MEAN; ++j) acc_mean[j] = 0.f;
     bool ok = true;
+    int unit = blockIdx.x >> 1, a0 = 0;    // PERSIST: accumulators of the units before this one
+    do {        // (the body keeps the function's indentation)
     int tile_m, tile_n;
-    tc_tile_of_block(p, rank, tile_m, tile_n);
+    bool whole = true;
+    if (PERSIST) {
+      const TcUnit t = tc_unit(p, unit);
+      b_begin = t.b_begin; b_end = t.b_end; nb = b_end - b_begin; nu = (nb + GROUP - 1) / GROUP; whole = t.whole;
+      tc_tile_of_pair(p, t.tile, rank, tile_m, tile_n);
+    } else {
+      tc_tile_of_pair(p, unit, rank, tile_m, tile_n);
+    }
     // per-example mode: one accumulator unit per example (or group), in order; plain mode: each accumulator once
     const int n_runs = CHUNKED ? (p.T + TC_CHUNK_TOKENS - 1) / TC_CHUNK_TOKENS : 1;      // accumulators per example
     const int n_acc = p.per_example ? nu * n_runs : min(nu, UNITS);
@@ -593,8 +663,8 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     for (int j = 0; j < N_RUN; ++j) acc_run[j] = 0.f;
     const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
     for (int a = 0; a < n_acc; ++a) {
-      const int buf = a % UNITS;
-      const uint32_t acc_ph = (uint32_t)(a / UNITS) & 1u;
+      const int buf = (a0 + a) % UNITS;
+      const uint32_t acc_ph = (uint32_t)((a0 + a) / UNITS) & 1u;
       // PHI == 3: this example's clipping coefficient c_b = min(1, C / sqrt(N_b)); the load is issued before
       // the wait for the accumulator, which hides its latency.  N_b = 0 (a zero gradient) gives 1.
       uint64_t coef2 = 0;
@@ -828,6 +898,77 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
 #pragma unroll
       for (int j = 0; j < N_STAT; ++j) acc_stat[j] = fmaf(2.f, acc_stat[j], -nbf);
     }
+    if constexpr (PERSIST) {
+      // Several tiles per pair: straight from the registers, since the operand ring already fills for the next tile.  Lanes
+      // exchange their rows' values first, so that four of them store 128 bytes side by side (stores of 32 bytes to 32 rows: 8 x 256
+      // x 1024 x 32104, both outputs, 201 us against 179).  Slices of a tile add 128 bytes of a row per instruction (16-byte adds, 32
+      // bytes to a lane: 128 x 32 x 4096^2, both outputs, 241 us against 235).
+      const int row0 = tile_m * TC_TILE_M + q * 32, col0 = tile_n * NT + h * COLS;
+      if (!whole) griddep_wait();                                   // the kernel that zeroes this tile
+      auto put = [&](float* out, int c, float (&v)[32]) {           // 32 columns from the c-th on
+        if (whole) {
+          const int row = row0 + (lane & ~3), col = col0 + c + 8 * (lane & 3);
+          quad_transpose(v, lane);
+          if (ok && col < p.d_in) {                                 // d_in is a multiple of 8: a group is all in or all out
+            float* const dst = out + (long long)row * p.d_in + col;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (row + j < p.d_out) st_global_v8(dst + (long long)j * p.d_in, &v[8 * j]);
+          }
+        } else {
+          const int col = col0 + c + lane;
+          warp_transpose(v, lane);
+          if (ok && col < p.d_in) {
+            float* const dst = out + (long long)row0 * p.d_in + col;
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (row0 + j < p.d_out) atomicAdd(dst + (long long)j * p.d_in, v[j]);
+          }
+        }
+      };
+      if (p.out_stat) {
+#pragma unroll
+        for (int c = 0; c < COLS; c += 32) {
+          float v[32];
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = acc_stat[c + j];
+          put(p.out_stat, c, v);
+        }
+      }
+      if (p.out_mean && (KEEP_MEAN || HYBRID)) {
+#pragma unroll
+        for (int c = 0; c < COLS; c += 32) {
+          float v[32];
+          if (HYBRID && c < HYB_TMEM_COLS) {
+            uint32_t m[32];
+            tmem_ld_32x32b_x32_wait(lane_base + (uint32_t)(HYB_COL0 + h * HYB_TMEM_COLS) + c, m);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(m[j]);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = acc_mean[HYBRID ? (c - HYB_TMEM_COLS + j) & 31 : (KEEP_MEAN ? c + j : 0)];
+          }
+          put(p.out_mean, c, v);
+        }
+      }
+      if constexpr (TRIPLE) {
+        const float nbf = (float)nb;
+#pragma unroll
+        for (int c = 0; c < COLS; c += 32) {
+          float v[32];
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = (float)((acc_cnt[(c + j) >> 1] >> (16 * (j & 1))) & 0xFFFFu) - nbf;
+          if (p.out_sign) put(p.out_sign, c, v);
+        }
+#pragma unroll
+        for (int j = 0; j < N_CNT; ++j) acc_cnt[j] = 0u;
+      }
+#pragma unroll
+      for (int j = 0; j < N_STAT; ++j) acc_stat[j] = 0.f;
+#pragma unroll
+      for (int j = 0; j < N_MEAN; ++j) acc_mean[j] = 0.f;
+      a0 += n_acc;
+    } else {
     constexpr int PANELS = COLS / 32;
     // each epilogue warp stages in its own eighth of the operand ring: 6 panels of 4 KiB (7 at NT = 192)
     constexpr int WARP_PANELS = (STAGES * STAGE_BYTES / 8) / 4096;
@@ -972,6 +1113,8 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       }
       __syncwarp();
     }
+    }
+    } while (PERSIST && ok && (unit += gridDim.x >> 1) < n_units);
   }
 
   // ---------------------------------------------------------------- teardown
