@@ -163,12 +163,13 @@ pe_status_t pe_linear_stats_all(const void* X, const void* dY, int B, int T, int
                                 float* out_mean, float* out_square, float* out_sign, pe_stream_t stream);
 
 /*
- * The same statistics for widths that are no multiples of 8.  TMA, which feeds the tensor-core kernel, wants 16-byte row
- * pitches; pe_linear_stats runs such layers on the SIMT kernel.  With a workspace this call first copies the
- * operands concerned to a padded pitch and contracts the copies on the tensor cores.  accumulate != 0: as
- * pe_linear_stats_accumulate; out_sign != NULL (phi square, accumulate 0): as pe_linear_stats_all.
+ * The same statistics by way of copies of the operands.  Widths that are no multiples of 8: TMA, which feeds the tensor-core
+ * kernel, wants 16-byte row pitches; pe_linear_stats runs such layers on the SIMT kernel.  With a workspace this call first copies
+ * the operands concerned to a padded pitch and contracts the copies on the tensor cores.  Examples of one token (T == 1):
+ * G_b is an outer product, so that the sums over b are contractions of the operands' exact squares (as pairs of bf16) and
+ * signs, which are written to the workspace; no G_b is formed.  accumulate != 0: as pe_linear_stats_accumulate; out_sign != NULL (phi square, accumulate 0): as pe_linear_stats_all.
  * workspace: device memory, 256-byte aligned, pe_linear_stats_padded_workspace_bytes() bytes, contents undefined
- * afterwards.  That function returns 0 where nothing is to be gained (widths that are multiples of 8, layers too small, a forced
+ * afterwards.  That function returns 0 where nothing is to be gained (widths that are multiples of 8 with T > 1, layers too small, a forced
  * path): the call is then the ordinary one and ignores the workspace.  Other arguments, alignments and results as for
  * pe_linear_stats.
  */

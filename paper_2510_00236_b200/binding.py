@@ -190,9 +190,9 @@ def pe_linear_stats_padded_workspace_bytes(B, T, d_in, d_out) -> int:
 
 
 def _padded(X, dY, B, T, d_in, d_out, phi, accumulate, out_mean, out_stat, out_sign) -> bool:
-    """Runs pe_linear_stats_padded with a workspace from torch's allocator if the widths are no multiples of 8 and the
-    library says that it pays; False if the ordinary call is the one to make."""
-    if not (d_in & 7 or d_out & 7):
+    """Runs pe_linear_stats_padded with a workspace from torch's allocator if the widths are no multiples of 8 or the
+    examples single tokens, and the library says that it pays; False if the ordinary call is the one to make."""
+    if not (d_in & 7 or d_out & 7 or T == 1):
         return False
     need = pe_linear_stats_padded_workspace_bytes(B, T, d_in, d_out)
     if need == 0:
@@ -202,7 +202,8 @@ def _padded(X, dY, B, T, d_in, d_out, phi, accumulate, out_mean, out_stat, out_s
 
 
 def pe_linear_stats_padded(X, dY, phi, accumulate, out_mean, out_stat, out_sign, workspace):
-    """The C entry point: statistics of a layer whose widths are no multiples of 8 by way of padded copies in `workspace`
+    """The C entry point: statistics of a layer whose widths are no multiples of 8, or whose examples are single tokens, by way of
+    copies in `workspace`
     (uint8, pe_linear_stats_padded_workspace_bytes(...) bytes; None where that is 0).  pe_linear_stats, _accumulate and
     _all call it where it pays."""
     B, T, d_in, d_out = _io_check(X, dY, torch.bfloat16)

@@ -325,7 +325,7 @@ static pe_status_t zero_for_split(DeviceInfo* di, float* a, float* b, size_t n, 
 }
 
 // mxt, myt: the maps of the zero-padded tail groups of a packed batch (RAGGED); any valid map otherwise.
-template <int PHI, bool TF32, int NT, int MEAN, int BKT = tc_default_bk(TF32, NT), bool RAGGED = false, int OPT = OPT_NONE, bool F8 = false, bool CHUNKED = false, bool PERSIST = false>
+template <int PHI, bool TF32, int NT, int MEAN, int BKT = tc_default_bk(TF32, NT), bool RAGGED = false, int OPT = OPT_NONE, bool F8 = false, bool CHUNKED = false, bool PERSIST = false, bool PARTS = false>
 static pe_status_t launch_tc_inst(DeviceInfo* di, int slot, const CUtensorMap& mx, const CUtensorMap& my, const CUtensorMap& mm,
                                   const CUtensorMap& ms, const CUtensorMap& msgn, const TcParams& p, dim3 grid, cudaStream_t st,
                                   const CUtensorMap* mxt = nullptr, const CUtensorMap* myt = nullptr, const FusedOpt* opt = nullptr) {
@@ -333,14 +333,14 @@ static pe_status_t launch_tc_inst(DeviceInfo* di, int slot, const CUtensorMap& m
   {
     std::lock_guard<std::mutex> lock(g_dev_mutex);
     if (!di->tc_attr_set[slot]) {
-      if (cudaFuncSetAttribute(tc_stats_kernel<PHI, TF32, NT, MEAN, BKT, RAGGED, OPT, F8, CHUNKED, PERSIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+      if (cudaFuncSetAttribute(tc_stats_kernel<PHI, TF32, NT, MEAN, BKT, RAGGED, OPT, F8, CHUNKED, PERSIST, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
         cudaGetLastError();
         return PE_ERR_CUDA;
       }
       di->tc_attr_set[slot] = true;
     }
   }
-  return launch_dependent(tc_stats_kernel<PHI, TF32, NT, MEAN, BKT, RAGGED, OPT, F8, CHUNKED, PERSIST>, grid, TC_THREADS, smem, st, mx, my, mm, ms, msgn,
+  return launch_dependent(tc_stats_kernel<PHI, TF32, NT, MEAN, BKT, RAGGED, OPT, F8, CHUNKED, PERSIST, PARTS>, grid, TC_THREADS, smem, st, mx, my, mm, ms, msgn,
                             mxt ? *mxt : mx, myt ? *myt : my, p, opt ? *opt : FusedOpt{});
 }
 
@@ -1007,8 +1007,109 @@ static bool padding_pays(int B, int T, int d_in, int d_out) {
          (double)B * T * d_in * d_out >= (double)PAD_MIN_MACS && (long long)B * T < (1ll << 31);
 }
 
+// Examples of one token: the four copies of each operand, in n chunks of `chunk` rows.  A chunk is what one accumulator takes, and the
+// accumulators are added in registers; the square's error against fp64, 2-norm, at 1024 x 1024^2: 1.4e-6 with 512 rows, 3.0e-7 with
+// 128, 1.7e-7 with 64, and 2.4e-7 with the kernel that forms every G_b.  64 rows cost 25.1 us there, 128 rows 22.8.
+constexpr int ONE_TOKEN_CHUNK = 64;
+struct OneTokenLayout {
+  int chunk, n, pitch_x, pitch_y;
+  size_t x_bytes, y_bytes;
+};
+static OneTokenLayout one_token_layout(int B, int d_in, int d_out) {
+  OneTokenLayout l;
+  l.n = (B + ONE_TOKEN_CHUNK - 1) / ONE_TOKEN_CHUNK;
+  l.chunk = ((B + l.n - 1) / l.n + 15) / 16 * 16;
+  l.pitch_x = (d_in + 7) & ~7;
+  l.pitch_y = (d_out + 7) & ~7;
+  l.x_bytes = align_up((size_t)4 * l.n * l.chunk * l.pitch_x * 2, 256);
+  l.y_bytes = align_up((size_t)4 * l.n * l.chunk * l.pitch_y * 2, 256);
+  return l;
+}
+// From this many entries of all G_b on, the two launches (16 us at least, and 8 us more of host time) beat the kernel that forms every
+// G_b and is bound by reading them: mean and square, three statistics, sign alone, us: 128 x 1024^2 26.8, 49.6, 31.0 -> 16.7, 17.8,
+// 15.7 (64 x 1024^2 18.7, 31.0, 20.7 stays); 1024 x 1024^2 133, 313, 162 -> 25, 31, 16; 512 x 4096^2 781, 2145, 1112 -> 123, 157, 48.
+constexpr double ONE_TOKEN_MIN_MACS = 1.2e8;
+static bool one_token_pays(int B, int T, int d_in, int d_out) {
+  return T == 1 && B > 0 && B <= (1 << 24) && tc_shape_ok(B, T, (d_in + 7) & ~7, (d_out + 7) & ~7) && (double)B * d_in * d_out >= ONE_TOKEN_MIN_MACS;
+}
+// Slices of each product's chunks: units of at most `len` chunks of a tile, by the estimated time of the launch: the units shared out
+// over the pairs, at least the longest.
+static void one_token_slices(const OneTokenLayout& l, const bool (&want)[3], long long tiles, int slots, double out_bytes, int (&slices)[3]) {
+  const double per_chunk = l.chunk * (COST_PLAIN.token_lo + COST_PLAIN.token_hi) * 0.5;
+  const int counts[3] = {4 * l.n, l.n, l.n};
+  double best = 1e300;
+  for (int parts = 1; parts <= 4 * l.n && parts <= 128; ++parts) {
+    const int len = (4 * l.n + parts - 1) / parts;
+    double work = 0.0, longest = 0.0;
+    int s[3];
+    bool split = false;
+    for (int k = 0; k < 3; ++k) {
+      s[k] = want[k] ? (counts[k] + len - 1) / len : 0;
+      if (s[k] > 1) split = true;
+    }
+    for (int k = 0; k < 3; ++k) {
+      if (!s[k]) continue;
+      const double unit = (double)((counts[k] + s[k] - 1) / s[k]) * per_chunk + COST_PLAIN.fixed + (split ? SPLIT_FIXED : 0.0);
+      work += unit * s[k] * tiles;
+      longest = std::max(longest, unit);
+    }
+    const double units = (double)tiles * (s[0] + s[1] + s[2]);
+    const double us = std::max(longest, work / units * std::ceil(units / slots)) + (split ? out_bytes / ZERO_BYTES_PER_US : 0.0);
+    if (us < best * 0.995) {
+      best = us;
+      for (int k = 0; k < 3; ++k) slices[k] = s[k];
+    }
+  }
+}
+static pe_status_t one_token_stats(DeviceInfo* di, const void* X, const void* dY, int B, int d_in, int d_out, float* out_mean, float* out_square,
+                                   float* out_sign, bool accumulate, void* workspace, cudaStream_t st) {
+  const OneTokenLayout l = one_token_layout(B, d_in, d_out);
+  const OneTokenTensor tx = {static_cast<const uint16_t*>(X), static_cast<uint16_t*>(workspace), d_in, l.pitch_x};
+  const OneTokenTensor ty = {static_cast<const uint16_t*>(dY), reinterpret_cast<uint16_t*>(static_cast<char*>(workspace) + l.x_bytes), d_out, l.pitch_y};
+  const int tiles_n = (d_in + 255) / 256, pairs_m = (d_out + TC_PAIR_M - 1) / TC_PAIR_M;
+  if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
+  const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
+  float* const outs[3] = {out_square, out_mean, out_sign};
+  const bool want[3] = {out_square != nullptr, out_mean != nullptr, out_sign != nullptr};
+  TcParams p{};
+  one_token_slices(l, want, (long long)tiles_n * pairs_m, slots, 4.0 * (want[0] + want[1] + want[2]) * d_in * d_out, p.part_slices);
+  const bool split = p.part_slices[0] > 1 || p.part_slices[1] > 1 || p.part_slices[2] > 1;
+  OneTokenOutputs zero = {{nullptr, nullptr, nullptr}, (long long)d_in * d_out};
+  if (split && !accumulate)
+    for (int k = 0; k < 3; ++k) zero.out[k] = outs[k];
+  const int rows = l.n * l.chunk, zero_blocks = split && !accumulate ? 2 * di->sm_count : 0;
+  one_token_operands_kernel<<<rows + zero_blocks, LAYOUT_THREADS, 0, st>>>(tx, ty, B, l.chunk, l.n, want[0] ? 1 : 0, want[1] ? 1 : 0, want[2] ? 1 : 0, zero);
+  pe_status_t rc = check_launch();
+  if (rc != PE_OK) return rc;
+  CUtensorMap mx, my;
+  constexpr int box_feats = TcOperand<false, 256>::BOX_FEATS, box_tokens = TcOperand<false, 256>::BK;
+  rc = make_operand_map(&mx, tx.dst, 4 * l.n, l.chunk, d_in, false, box_feats, box_tokens, false, 1, l.pitch_x);
+  if (rc == PE_OK) rc = make_operand_map(&my, ty.dst, 4 * l.n, l.chunk, d_out, false, box_feats, box_tokens, false, 1, l.pitch_y);
+  if (rc != PE_OK) return rc;
+  const bool scalar_out = d_in % 4 != 0;
+  CUtensorMap mo[3] = {mx, mx, mx};
+  for (int k = 0; k < 3 && !scalar_out; ++k) {
+    if (!outs[k]) continue;
+    rc = make_output_map(&mo[k], outs[k], d_in, d_out);
+    if (rc != PE_OK) return rc;
+  }
+  p.B = 6 * l.n; p.T = l.chunk; p.d_in = d_in; p.d_out = d_out; p.nsplit = split ? 2 : 1; p.per_example = 1;
+  p.accumulate = accumulate ? 1 : 0; p.scalar_out = scalar_out ? 1 : 0; p.wait_at_start = 1; p.part_chunks = l.n;
+  p.pairs_m = pairs_m; p.tiles_n = tiles_n;
+  const int units = p.part_slices[0] + p.part_slices[1] + p.part_slices[2];
+  p.band = choose_band(pairs_m, tiles_n, 256, units, slots);
+  p.out_stat = out_square; p.out_mean = out_mean; p.out_sign = out_sign; p.dev_status = di->status_ptr;
+  return launch_tc_inst<0, false, 256, MEAN_NONE, tc_default_bk(false, 256), false, OPT_NONE, false, false, false, true>(
+      di, 31, mx, my, mo[1], mo[0], mo[2], p, dim3(2 * pairs_m * tiles_n, 1, units), st);
+}
+
 size_t pe_linear_stats_padded_workspace_bytes(int B, int T, int d_in, int d_out) {
-  if (B < 1 || T < 1 || d_in < 1 || d_out < 1 || g_path.load() != PE_PATH_AUTO || !padding_pays(B, T, d_in, d_out)) return 0;
+  if (B < 1 || T < 1 || d_in < 1 || d_out < 1 || g_path.load() != PE_PATH_AUTO) return 0;
+  if (one_token_pays(B, T, d_in, d_out)) {
+    const OneTokenLayout l = one_token_layout(B, d_in, d_out);
+    return l.x_bytes + l.y_bytes;
+  }
+  if (!padding_pays(B, T, d_in, d_out)) return 0;
   const PaddedLayout l = padded_layout(B, T, d_in, d_out, false);
   return l.x_bytes + l.y_bytes;
 }
@@ -1018,7 +1119,8 @@ pe_status_t pe_linear_stats_padded(const void* X, const void* dY, int B, int T, 
                                    pe_stream_t stream) {
   const size_t need = pe_linear_stats_padded_workspace_bytes(B, T, d_in, d_out);
   if (out_sign && (accumulate || phi != PE_PHI_SQUARE)) return PE_ERR_PHI;
-  if (need == 0) {
+  const bool plain = T == 1 && phi == PE_PHI_IDENTITY && d_in % 8 == 0 && d_out % 8 == 0;       // a contraction of the operands as they are
+  if (need == 0 || plain) {
     if (out_sign) return pe_linear_stats_all(X, dY, B, T, d_in, d_out, out_mean, out_stat, out_sign, stream);
     return accumulate ? pe_linear_stats_accumulate(X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, stream)
                       : pe_linear_stats(X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, stream);
@@ -1034,8 +1136,16 @@ pe_status_t pe_linear_stats_padded(const void* X, const void* dY, int B, int T, 
   rc = device_info(&di);
   if (rc != PE_OK) return rc;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const PaddedLayout l = padded_layout(B, T, d_in, d_out, false);
   const long long rows = (long long)B * T;
+  if (one_token_pays(B, T, d_in, d_out)) {
+    g_last_path.store(PE_PATH_TENSOR);
+    if (phi == PE_PHI_SQUARE) return one_token_stats(di, X, dY, B, d_in, d_out, out_mean, out_stat, out_sign, accumulate != 0, workspace, st);
+    if (phi == PE_PHI_SIGN) return one_token_stats(di, X, dY, B, d_in, d_out, out_mean, nullptr, out_stat, accumulate != 0, workspace, st);
+    rc = one_token_stats(di, X, dY, B, d_in, d_out, out_mean ? out_mean : out_stat, nullptr, nullptr, accumulate != 0, workspace, st);
+    if (rc != PE_OK || !out_mean || !out_stat) return rc;
+    return one_token_stats(di, X, dY, B, d_in, d_out, out_stat, nullptr, nullptr, accumulate != 0, workspace, st);
+  }
+  const PaddedLayout l = padded_layout(B, T, d_in, d_out, false);
   PadTensor px = {static_cast<const uint16_t*>(X), static_cast<uint16_t*>(workspace), d_in, l.pitch_x};
   PadTensor py = {static_cast<const uint16_t*>(dY), reinterpret_cast<uint16_t*>(static_cast<char*>(workspace) + l.x_bytes), d_out, l.pitch_y};
   const bool pad_x = l.x_bytes > 0, pad_y = l.y_bytes > 0;

@@ -27,7 +27,7 @@
 //   PHI = 0,   NT = 256: no per-example reset (accumulate in tensor memory)        -- plain contraction over all rows
 // Further template arguments: RAGGED (packed batches with per-example token ranges), OPT (the parameter
 // update applied by the block that completes a tile's sums), F8 (e4m3 operands for the plain contraction), CHUNKED (several
-// accumulators per example), PERSIST (several tiles per pair).
+// accumulators per example), PERSIST (several tiles per pair), PARTS (several contractions in one launch).
 //
 // Warp roles per block (12 warps): 0 = TMA producer of the dY boxes, 2 = TMEM allocator, then TMA
 // producer of the X boxes, 1 = MMA issuer (leader block only), 3 idle, 4..11 = epilogue (warp w reads
@@ -146,6 +146,8 @@ struct TcParams {
   int nsplit;          // batch slices (gridDim.z); > 1 => outputs pre-zeroed, partials added atomically
   int whole_tiles;     // PERSIST: tiles that one pair contracts over the whole batch; each of the others goes to
   int tail_split;      // this many pairs, by slices of the batch, whose sums are added to (zeroed) outputs
+  int part_chunks;     // PARTS: chunks of rows per part, slices of the square's, the mean's and the sign's chunks
+  int part_slices[3];
   int per_example;     // 1: reset the accumulator for every example and apply phi (statistics)
                        // 0: one accumulation over the whole slice (plain contraction, phi = identity)
   int half_operands;   // 16-bit operands are IEEE half instead of bf16 (the staged per-token statistic)
@@ -164,6 +166,13 @@ struct TcParams {
   float clip_norm;          // PHI == 3 only: C of c_b = min(1, C / sqrt(N_b))
   unsigned int* dev_status;
 };
+
+// PARTS: chunk c of the launch is chunk c % n of product c / n, the operands of which are copies 0 (as it is), 1 and 2 (upper and lower
+// half of the squares) and 3 (sign): dY0 X0 | dY1 X1, dY2 X1, dY1 X2, dY2 X2 | dY3 X3.  Where that chunk is in the operand.
+__device__ __forceinline__ int tc_part_chunk(const TcParams& p, int c, bool of_dy) {
+  const int product = c / p.part_chunks;
+  return (int)(((of_dy ? 0x321210u : 0x322110u) >> (4 * product)) & 15u) * p.part_chunks + c - product * p.part_chunks;
+}
 
 // PERSIST: unit u of the launch, a tile and the examples it is contracted over.
 struct TcUnit {
@@ -409,7 +418,7 @@ __device__ __forceinline__ void fused_update_piece(const FusedOpt& o, const TcPa
 // fp32 FMAs in order give too.  64 more registers per epilogue thread, hence the 256 x 128 tile.
 // OPT: the parameter update applied by the block that completes a tile's sums (OPT_ADAM needs both running
 // sums, OPT_SIGN the sign statistic alone); `o` is ignored when OPT == OPT_NONE.
-template <int PHI, bool TF32, int NT, int MEAN, int BKT = tc_default_bk(TF32, NT), bool RAGGED = false, int OPT = OPT_NONE, bool F8 = false, bool CHUNKED = false, bool PERSIST = false>
+template <int PHI, bool TF32, int NT, int MEAN, int BKT = tc_default_bk(TF32, NT), bool RAGGED = false, int OPT = OPT_NONE, bool F8 = false, bool CHUNKED = false, bool PERSIST = false, bool PARTS = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
 tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_dy,
                 const __grid_constant__ CUtensorMap tmap_mean, const __grid_constant__ CUtensorMap tmap_stat,
@@ -430,6 +439,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   static_assert(!RAGGED || (!TF32 && MEAN != MEAN_TMEM), "packed batches: 16-bit operands, several accumulators");
   static_assert((PHI != 3 && PHI != 4) || MEAN == MEAN_NONE, "the clipped sum and the scaled contraction are statistic-only passes");
   static_assert(!CHUNKED || (MEAN == MEAN_REGS && NT == 128 && !RAGGED && OPT == OPT_NONE && Op::GROUP == 1), "runs of an example: the two-sum kernel on the 256 x 128 tile");
+  static_assert(!PARTS || (PHI == 0 && !TF32 && !F8 && !RAGGED && !PERSIST && OPT == OPT_NONE), "the statistics of one-token examples are plain contractions");
   static_assert(!PERSIST || (!RAGGED && OPT == OPT_NONE && MEAN != MEAN_TMEM && !NORMS && PHI != 0), "several tiles per pair: fixed-length batches, whole sums written");
   constexpr int CHUNK_STAGES = CHUNKED ? TC_CHUNK_TOKENS / BKT : 1;
   constexpr int REGS_CONTROL = CHUNKED ? 40 : Op::REGS_CONTROL, REGS_EPILOGUE = CHUNKED ? 232 : Op::REGS_EPILOGUE;
@@ -469,6 +479,16 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       b_begin = ragged_slice_begin(p.seq_offsets, p.B, blockIdx.z, p.nsplit, lane);
       b_end = max(b_begin, ragged_slice_begin(p.seq_offsets, p.B, blockIdx.z + 1, p.nsplit, lane));
     }
+  }
+  int which = 0;                                    // PARTS: 0 the square, 1 the mean, 2 the sign
+  if constexpr (PARTS) {
+    int z = blockIdx.z;
+    if (z >= p.part_slices[0]) { z -= p.part_slices[0]; which = 1; }
+    if (which == 1 && z >= p.part_slices[1]) { z -= p.part_slices[1]; which = 2; }
+    const int first = which == 0 ? p.part_chunks : which == 1 ? 0 : 5 * p.part_chunks;
+    const long long count = which == 0 ? 4ll * p.part_chunks : p.part_chunks;
+    b_begin = first + (int)(count * z / p.part_slices[which]);
+    b_end = first + (int)(count * (z + 1) / p.part_slices[which]);
   }
   int nb = b_end - b_begin;
   const int n_units = PERSIST ? tc_units(p) : 1;      // PERSIST: this pair takes every (gridDim.x / 2)-th of them
@@ -542,7 +562,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
               const CUtensorMap* tm = tail ? tmap_tail : tmap;
               const int c1 = tail ? 0 : g.row0 + kc * BK;
               // (grouped examples: the box is GROUP examples deep; past the batch's end it reads zeros)
-              const int c2 = RAGGED ? (tail ? b_begin + e : 0) : b_begin + GROUP * e;
+              const int c2 = PARTS ? tc_part_chunk(p, b_begin + e, is_a) : RAGGED ? (tail ? b_begin + e : 0) : b_begin + GROUP * e;
               for (int b = 0; b < n_boxes; ++b) tma_load_3d_pair(dst + b * box_bytes, tm, leader_full, c0 + b * box_feats, c1, c2);
             }
             __syncwarp();
@@ -1018,14 +1038,19 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
           bulk_commit_group();
         }
       };
+      if constexpr (PARTS) {
+#pragma unroll
+        for (int c = 0; c < PANELS; ++c) put_panel(stage_base + c * 4096, &acc_mean[c * 32]);
+        send(which == 0 ? &tmap_stat : which == 1 ? &tmap_mean : &tmap_sign, which == 0 ? p.out_stat : which == 1 ? p.out_mean : p.out_sign, stage_base);
+      }
       // sum_b phi(G_b), or the plain contraction when PHI == 0
-      if (p.out_stat || stage_for_update) {
+      if (!PARTS && (p.out_stat || stage_for_update)) {
 #pragma unroll
         for (int c = 0; c < PANELS; ++c) put_panel(stage_base + c * 4096, (PHI != 0) ? &acc_stat[c * 32] : &acc_mean[c * 32]);
         if (p.out_stat) send(&tmap_stat, p.out_stat, stage_base);
       }
       // sum_b G_b
-      if ((p.out_mean || (stage_for_update && OPT == OPT_ADAM)) && (KEEP_MEAN || MEAN == MEAN_TMEM || HYBRID)) {
+      if (!PARTS && (p.out_mean || (stage_for_update && OPT == OPT_ADAM)) && (KEEP_MEAN || MEAN == MEAN_TMEM || HYBRID)) {
         uint32_t first = stage_base + PANELS * 4096;          // MEAN_REGS / PHI == 0: second half of the warp's 16 KiB
         if constexpr (HYBRID) {
           // two panels from tensor memory, the third from registers; staged behind the statistic's three panels
