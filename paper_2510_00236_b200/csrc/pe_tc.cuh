@@ -271,6 +271,14 @@ __device__ __forceinline__ uint32_t sign_plus_one_packed(uint64_t g2) {
   return __byte_perm(__float_as_uint(t0), __float_as_uint(t1), 0x5410);
 }
 
+// The same for the sum over two examples, sign + sign + 2 in {0 .. 4}: the saturated halves are added before the integer is
+// extracted (1.5 * 2^22 has steps of 0.5).
+__device__ __forceinline__ uint32_t signs_plus_two_packed(uint64_t g2, uint64_t h2) {
+  float t0, t1;
+  sm100::f32x2_unpack(sm100::f32x2_add(sm100::f32x2_add(sign_half2(g2), sm100::f32x2_pack(6291456.f, 6291456.f)), sign_half2(h2)), t0, t1);
+  return __byte_perm(__float_as_uint(t0), __float_as_uint(t1), 0x5410);
+}
+
 template <int PHI>
 __device__ __forceinline__ float phi_apply(float g) {
   if (PHI == 1) return g * g;
@@ -442,7 +450,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   static_assert(!PARTS || (PHI == 0 && !TF32 && !F8 && !RAGGED && !PERSIST && OPT == OPT_NONE), "the statistics of one-token examples are plain contractions");
   static_assert(!PERSIST || (!RAGGED && OPT == OPT_NONE && MEAN != MEAN_TMEM && !NORMS && PHI != 0), "several tiles per pair: fixed-length batches, whole sums written");
   constexpr int CHUNK_STAGES = CHUNKED ? TC_CHUNK_TOKENS / BKT : 1;
-  constexpr int REGS_CONTROL = CHUNKED ? 40 : Op::REGS_CONTROL, REGS_EPILOGUE = CHUNKED ? 232 : Op::REGS_EPILOGUE;
+  constexpr int REGS_CONTROL = CHUNKED || TRIPLE ? 40 : Op::REGS_CONTROL, REGS_EPILOGUE = CHUNKED || TRIPLE ? 232 : Op::REGS_EPILOGUE;
   static_assert(128 * REGS_CONTROL + 256 * REGS_EPILOGUE <= TC_THREADS * TC_REGS_AT_LAUNCH, "setmaxnreg: the epilogue's increase must fit what the control warps give up");
   static_assert(OPT != OPT_ADAM || (MEAN == MEAN_REGS && PHI == 1), "the Adam family consumes sum_b G_b and sum_b G_b^2");
   static_assert(OPT != OPT_SIGN || (MEAN == MEAN_NONE && PHI == 2), "MicroSignSGD consumes sum_b sign(G_b)");
@@ -663,15 +671,21 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
 #pragma unroll
     for (int j = 0; j < N_MEAN; ++j) acc_mean[j] = 0.f;
     bool ok = true;
+    // What of the unit stays in registers during the loop over its examples was measured (8 x 256 x 1024 x 32104, both outputs, 186 us with
+    // the tile found before the loop, 196 to 207 otherwise; three statistics 1 %, one statistic 2 % the other way round).
+    constexpr bool TILE_FIRST = PHI == 4 || (!TRIPLE && !(PERSIST && MEAN == MEAN_NONE));
     int unit = blockIdx.x >> 1, a0 = 0;    // PERSIST: accumulators of the units before this one
     do {        // (the body keeps the function's indentation)
     int tile_m, tile_n;
     bool whole = true;
     if (PERSIST) {
       const TcUnit t = tc_unit(p, unit);
-      b_begin = t.b_begin; b_end = t.b_end; nb = b_end - b_begin; nu = (nb + GROUP - 1) / GROUP; whole = t.whole;
-      tc_tile_of_pair(p, t.tile, rank, tile_m, tile_n);
-    } else {
+      b_begin = t.b_begin; b_end = t.b_end; nb = b_end - b_begin; nu = (nb + GROUP - 1) / GROUP;
+      if constexpr (TILE_FIRST) {
+        whole = t.whole;
+        tc_tile_of_pair(p, t.tile, rank, tile_m, tile_n);
+      }
+    } else if constexpr (TILE_FIRST) {
       tc_tile_of_pair(p, unit, rank, tile_m, tile_n);
     }
     // per-example mode: one accumulator unit per example (or group), in order; plain mode: each accumulator once
@@ -851,7 +865,37 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         // per example, which is what bounds short sequences (the three-statistic epilogue, bound by its instruction
         // count, gains 2-3 %).
         constexpr bool PIPELINED = (CH == 32 && PHI != 3 && PHI != 4) || (TRIPLE && NT == 128);
-        if constexpr (PIPELINED) {
+        if constexpr (TRIPLE && GROUP == 2) {
+          // The two examples side by side, 8 columns at a time: their signs are counted with one extraction for both, which the
+          // epilogue, bound by its instructions, shows in full: 1024 x 32 x 1024^2 315 -> 276 us, 128 x 32 x 4096^2 492 -> 475.  One pair of
+          // reads in flight (the scheduler's other warp hides its latency) and the larger register share: with two pairs it spills,
+          // 283 us; with 216 registers 291.  An example missing from the last unit counts as a gradient of zeros.
+          constexpr int STEPS = COLS / 8;
+          uint32_t g[8], h[8];
+          auto fold_two = [&](int c) {
+            if (in_unit < 2) {
+#pragma unroll
+              for (int j = 0; j < 8; ++j) h[j] = 0u;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) {
+              const int k = c * 8 + j;
+              const uint64_t g2 = f32x2_pack(__uint_as_float(g[j]), __uint_as_float(g[j + 1]));
+              const uint64_t h2 = f32x2_pack(__uint_as_float(h[j]), __uint_as_float(h[j + 1]));
+              f32x2_unpack(f32x2_add(f32x2_add(f32x2_pack(acc_mean[k], acc_mean[k + 1]), g2), h2), acc_mean[k], acc_mean[k + 1]);
+              f32x2_unpack(f32x2_fma(h2, h2, f32x2_fma(g2, g2, f32x2_pack(acc_stat[k], acc_stat[k + 1]))), acc_stat[k], acc_stat[k + 1]);
+              acc_cnt[k >> 1] += signs_plus_two_packed(g2, h2);
+            }
+          };
+#pragma unroll
+          for (int k = 0; k < STEPS; ++k) {
+            tmem_ld_issue(taddr + k * 8, g);
+            tmem_ld_issue(taddr + NT + k * 8, h);
+            tmem_ld_wait_for(g, h);
+            if (k == STEPS - 1) release_unit();
+            fold_two(k);
+          }
+        } else if constexpr (PIPELINED) {
           constexpr int TOTAL = GROUP * NCH;          // reads per unit when every example of the group exists
           const int n_reads = in_unit * NCH;
           uint32_t ra[CH], rb[CH];
@@ -912,6 +956,11 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     // whatever lies outside the matrix.  The tensor-memory loads are warp-wide instructions: the
     // condition around them is made uniform over the warp.
     ok = __all_sync(0xffffffffu, ok);
+    if constexpr (!TILE_FIRST) {
+      const TcUnit t = PERSIST ? tc_unit(p, unit) : TcUnit{unit, 0, 0, true};
+      whole = t.whole;
+      tc_tile_of_pair(p, t.tile, rank, tile_m, tile_n);
+    }
     if constexpr (PHI == 2) {
       // sum_b (sign(G_b) + 1) / 2  ->  sum_b sign(G_b)
       const float nbf = (float)nb;
@@ -972,7 +1021,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         }
       }
       if constexpr (TRIPLE) {
-        const float nbf = (float)nb;
+        const float nbf = (float)(GROUP * nu);
 #pragma unroll
         for (int c = 0; c < COLS; c += 32) {
           float v[32];
@@ -1090,7 +1139,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         if (p.out_sign) {
           if (elect_one()) bulk_wait_read_all();
           __syncwarp();
-          const float nbf = (float)nb;
+          const float nbf = (float)(GROUP * nu);
 #pragma unroll
           for (int c = 0; c < PANELS; ++c) {
             float v[32];
