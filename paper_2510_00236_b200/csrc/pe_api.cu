@@ -6,6 +6,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <cmath>
+#include <functional>
 #include <mutex>
 #include <vector>
 
@@ -353,6 +354,10 @@ static pe_status_t launch_tc_tiles(DeviceInfo* di, int slot, bool persist, const
   return launch_tc_inst<PHI, false, NT, MEAN, BKT, false, OPT_NONE, false, CHUNKED, true>(di, 32 + slot, mx, my, mm, ms, msgn, p, grid, st);
 }
 
+// What makes the operands of a launch (a layout kernel): called with the outputs to zero by the way.
+using LayoutStep = std::function<pe_status_t(const LayoutZero&)>;
+static bool any_output(const LayoutZero& z) { return z.out[0] || z.out[1] || z.out[2]; }
+
 // Tensor-core launch.  per_example = 0 runs the plain contraction over all B*T rows (its result goes
 // to whichever of out_mean / out_stat is not NULL).  With per_example = 1 and both outputs wanted the
 // pair tile is 256 x 128 (two running sums per thread); with only out_stat it is 256 x 256.
@@ -360,7 +365,7 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
                              int per_example, float* out_mean, float* out_stat, cudaStream_t st, bool half_ops = false,
                              float* out_sign = nullptr, bool accumulate = false, const float* sq_norms = nullptr, float clip_norm = 0.f,
                              int pitch_x = 0, int pitch_y = 0, bool chunked = false, const float* scale_x = nullptr,
-                             const float* scale_y = nullptr) {
+                             const float* scale_y = nullptr, const LayoutStep& before = nullptr) {
   const bool triple = out_sign != nullptr;       // mean + square + sign in one pass (phi = square, all three outputs given)
   const bool both = per_example && ((out_mean && out_stat) || chunked);
   const bool runs = chunked && T > TC_CHUNK_TOKENS;     // several accumulators per example
@@ -415,13 +420,18 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
   if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
   int ns = mean_tmem ? plan_tiles(&COST_STAT, 1, B, T, d_in, d_out, slots, max_split, 2).ns : plan.ns;
   if (triple && (B + ns - 1) / ns > TC_SIGN_COUNT_MAX) ns = (B + TC_SIGN_COUNT_MAX - 1) / TC_SIGN_COUNT_MAX;   // 16-bit sign counters
-  if (ns > 1 && !accumulate) {
+  const bool to_zero = ns > 1 && !accumulate;
+  if (before) {
+    LayoutZero zero = {{nullptr, nullptr, nullptr}, (long long)d_in * d_out};
+    if (to_zero) { zero.out[0] = out_mean; zero.out[1] = out_stat; zero.out[2] = out_sign; }
+    rc = before(zero);
+  } else if (to_zero) {
     rc = zero_for_split(di, out_mean, out_stat, (size_t)d_in * d_out, st, out_sign);
-    if (rc != PE_OK) return rc;
   }
+  if (rc != PE_OK) return rc;
   TcParams p{};
   p.B = B; p.T = T; p.d_in = d_in; p.d_out = d_out; p.nsplit = ns; p.per_example = per_example; p.half_operands = half_ops ? 1 : 0;
-  p.accumulate = accumulate ? 1 : 0; p.scalar_out = scalar_out ? 1 : 0; p.wait_at_start = ns == 1 || accumulate ? 1 : 0;
+  p.accumulate = accumulate ? 1 : 0; p.scalar_out = scalar_out ? 1 : 0; p.wait_at_start = !to_zero || before ? 1 : 0;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, nt, ns, di->sm_count / 2);
   p.out_mean = out_mean; p.out_stat = out_stat; p.out_sign = out_sign; p.out_norms = nullptr; p.dev_status = di->status_ptr;
   p.seq_offsets = nullptr; p.sq_norms = sq_norms; p.clip_norm = clip_norm; p.scale_x = scale_x; p.scale_y = scale_y;
@@ -728,14 +738,16 @@ static void regroup_rows(int& B, int& T) {
 
 // pe_linear_stats on the tensor cores.
 static pe_status_t tc_linear_stats(DeviceInfo* di, const void* X, const void* dY, int B, int T, int d_in, int d_out, int phi, float* out_mean,
-                                   float* out_stat, bool accumulate, cudaStream_t st) {
+                                   float* out_stat, bool accumulate, cudaStream_t st, const LayoutStep& before = nullptr) {
   g_last_path.store(PE_PATH_TENSOR);
-  auto plain = [&](float* out) { return launch_tc(di, X, dY, B, T, d_in, d_out, phi, 0, out, nullptr, st, false, nullptr, accumulate); };
+  auto plain = [&](float* out, const LayoutStep& first = nullptr) {
+    return launch_tc(di, X, dY, B, T, d_in, d_out, phi, 0, out, nullptr, st, false, nullptr, accumulate, nullptr, 0.f, 0, 0, false, nullptr, nullptr, first);
+  };
   if (phi == PE_PHI_IDENTITY || !out_stat) {
     // phi = identity, or only sum_b G_b wanted: the plain contraction over all B*T rows, where B and T only enter
     // through B*T: regroup short sequences into full two-stage "examples" when the rows divide evenly.
     regroup_rows(B, T);
-    pe_status_t rc = plain(out_mean ? out_mean : out_stat);
+    pe_status_t rc = plain(out_mean ? out_mean : out_stat, before);
     if (rc != PE_OK || !out_mean || !out_stat) return rc;
     if (accumulate) return plain(out_stat);          // a copy would overwrite: contract once more into the second
     if (cudaMemcpyAsync(out_stat, out_mean, (size_t)d_in * d_out * sizeof(float), cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
@@ -744,7 +756,8 @@ static pe_status_t tc_linear_stats(DeviceInfo* di, const void* X, const void* dY
     }
     return PE_OK;
   }
-  return launch_tc(di, X, dY, B, T, d_in, d_out, phi, 1, out_mean, out_stat, st, false, nullptr, accumulate);
+  return launch_tc(di, X, dY, B, T, d_in, d_out, phi, 1, out_mean, out_stat, st, false, nullptr, accumulate, nullptr, 0.f, 0, 0, false, nullptr, nullptr,
+                   before);
 }
 
 // The same for layers that the SIMT kernel would otherwise serve, from copies whose rows are pitch_x, pitch_y elements
@@ -753,13 +766,14 @@ static pe_status_t tc_linear_stats(DeviceInfo* di, const void* X, const void* dY
 // pe_linear_stats_all (phi = square).
 static pe_status_t tc_linear_stats_pitched(DeviceInfo* di, const void* X, const void* dY, int B, int T, int d_in, int d_out, int phi,
                                            float* out_mean, float* out_stat, float* out_sign, bool accumulate, int pitch_x, int pitch_y,
-                                           cudaStream_t st) {
+                                           cudaStream_t st, const LayoutStep& before) {
   g_last_path.store(PE_PATH_TENSOR);
-  auto run = [&](int f, float* mean, float* stat, float* sign) {
-    return launch_tc(di, X, dY, B, T, d_in, d_out, f, 1, mean, stat, st, false, sign, accumulate, nullptr, 0.f, pitch_x, pitch_y, true);
+  auto run = [&](int f, float* mean, float* stat, float* sign, const LayoutStep& first = nullptr) {
+    return launch_tc(di, X, dY, B, T, d_in, d_out, f, 1, mean, stat, st, false, sign, accumulate, nullptr, 0.f, pitch_x, pitch_y, true, nullptr, nullptr,
+                     first);
   };
   if (phi == PE_PHI_IDENTITY) {
-    pe_status_t rc = run(PE_PHI_SQUARE, out_mean ? out_mean : out_stat, nullptr, nullptr);
+    pe_status_t rc = run(PE_PHI_SQUARE, out_mean ? out_mean : out_stat, nullptr, nullptr, before);
     if (rc != PE_OK || !out_mean || !out_stat) return rc;
     if (accumulate) return run(PE_PHI_SQUARE, out_stat, nullptr, nullptr);
     if (cudaMemcpyAsync(out_stat, out_mean, (size_t)d_in * d_out * sizeof(float), cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
@@ -769,10 +783,10 @@ static pe_status_t tc_linear_stats_pitched(DeviceInfo* di, const void* X, const 
     return PE_OK;
   }
   if (out_sign && T > TC_CHUNK_TOKENS) {
-    pe_status_t rc = run(PE_PHI_SQUARE, out_mean, out_stat, nullptr);
+    pe_status_t rc = run(PE_PHI_SQUARE, out_mean, out_stat, nullptr, before);
     return rc == PE_OK ? run(PE_PHI_SIGN, nullptr, out_sign, nullptr) : rc;
   }
-  return run(phi, out_mean, out_stat, out_sign);
+  return run(phi, out_mean, out_stat, out_sign, before);
 }
 
 template <typename TIn>
@@ -1009,7 +1023,7 @@ static bool padding_pays(int B, int T, int d_in, int d_out) {
 
 // Examples of one token: the four copies of each operand, in n chunks of `chunk` rows.  A chunk is what one accumulator takes, and the
 // accumulators are added in registers; the square's error against fp64, 2-norm, at 1024 x 1024^2: 1.4e-6 with 512 rows, 3.0e-7 with
-// 128, 1.7e-7 with 64, and 2.4e-7 with the kernel that forms every G_b.  64 rows cost 25.1 us there, 128 rows 22.8.
+// 128, 1.7e-7 with 64, and 2.4e-7 with the kernel that forms every G_b.  64 rows cost 10 % there.
 constexpr int ONE_TOKEN_CHUNK = 64;
 struct OneTokenLayout {
   int chunk, n, pitch_x, pitch_y;
@@ -1027,7 +1041,7 @@ static OneTokenLayout one_token_layout(int B, int d_in, int d_out) {
 }
 // From this many entries of all G_b on, the two launches (16 us at least, and 8 us more of host time) beat the kernel that forms every
 // G_b and is bound by reading them: mean and square, three statistics, sign alone, us: 128 x 1024^2 26.8, 49.6, 31.0 -> 16.7, 17.8,
-// 15.7 (64 x 1024^2 18.7, 31.0, 20.7 stays); 1024 x 1024^2 133, 313, 162 -> 25, 31, 16; 512 x 4096^2 781, 2145, 1112 -> 123, 157, 48.
+// 15.7 (64 x 1024^2 18.7, 31.0, 20.7 stays); 1024 x 1024^2 133, 313, 162 -> 23, 28, 16; 512 x 4096^2 781, 2145, 1112 -> 123, 157, 48.
 constexpr double ONE_TOKEN_MIN_MACS = 1.2e8;
 static bool one_token_pays(int B, int T, int d_in, int d_out) {
   return T == 1 && B > 0 && B <= (1 << 24) && tc_shape_ok(B, T, (d_in + 7) & ~7, (d_out + 7) & ~7) && (double)B * d_in * d_out >= ONE_TOKEN_MIN_MACS;
@@ -1074,12 +1088,12 @@ static pe_status_t one_token_stats(DeviceInfo* di, const void* X, const void* dY
   TcParams p{};
   one_token_slices(l, want, (long long)tiles_n * pairs_m, slots, 4.0 * (want[0] + want[1] + want[2]) * d_in * d_out, p.part_slices);
   const bool split = p.part_slices[0] > 1 || p.part_slices[1] > 1 || p.part_slices[2] > 1;
-  OneTokenOutputs zero = {{nullptr, nullptr, nullptr}, (long long)d_in * d_out};
+  LayoutZero zero = {{nullptr, nullptr, nullptr}, (long long)d_in * d_out};
   if (split && !accumulate)
     for (int k = 0; k < 3; ++k) zero.out[k] = outs[k];
   const int rows = l.n * l.chunk, zero_blocks = split && !accumulate ? 2 * di->sm_count : 0;
-  one_token_operands_kernel<<<rows + zero_blocks, LAYOUT_THREADS, 0, st>>>(tx, ty, B, l.chunk, l.n, want[0] ? 1 : 0, want[1] ? 1 : 0, want[2] ? 1 : 0, zero);
-  pe_status_t rc = check_launch();
+  pe_status_t rc = launch_dependent(one_token_operands_kernel, dim3(rows + zero_blocks), LAYOUT_THREADS, 0, st, tx, ty, B, l.chunk, l.n, want[0] ? 1 : 0,
+                                    want[1] ? 1 : 0, want[2] ? 1 : 0, zero);
   if (rc != PE_OK) return rc;
   CUtensorMap mx, my;
   constexpr int box_feats = TcOperand<false, 256>::BOX_FEATS, box_tokens = TcOperand<false, 256>::BK;
@@ -1152,11 +1166,11 @@ pe_status_t pe_linear_stats_padded(const void* X, const void* dY, int B, int T, 
   const long long groups = rows * ((pad_x && pad_y ? std::max(l.pitch_x, l.pitch_y) : pad_x ? l.pitch_x : l.pitch_y) / 8);
   long long blocks = (groups + 4 * LAYOUT_THREADS - 1) / (4 * LAYOUT_THREADS);
   if (blocks > 16ll * di->sm_count) blocks = 16ll * di->sm_count;
-  pad_rows_kernel<<<dim3((unsigned)blocks, pad_x && pad_y ? 2 : 1), LAYOUT_THREADS, 0, st>>>(pad_x ? px : py, py, rows);
-  rc = check_launch();
-  if (rc != PE_OK) return rc;
+  const LayoutStep pad = [&](const LayoutZero& zero) {
+    return launch_dependent(any_output(zero) ? pad_rows_kernel<true> : pad_rows_kernel<false>, dim3((unsigned)blocks, pad_x && pad_y ? 2 : 1), LAYOUT_THREADS, 0, st, pad_x ? px : py, py, rows, zero);
+  };
   return tc_linear_stats_pitched(di, pad_x ? (const void*)px.dst : X, pad_y ? (const void*)py.dst : dY, B, T, d_in, d_out, phi, out_mean, out_stat, out_sign,
-                         accumulate != 0, l.pitch_x, l.pitch_y, st);
+                         accumulate != 0, l.pitch_x, l.pitch_y, st, pad);
 }
 
 // Tile of the unfolding kernel: output positions of one row and channels per round, so that a block's shared memory (input rows
@@ -1230,11 +1244,13 @@ pe_status_t pe_conv2d_stats(const void* x, const void* grad_out, int B, int C, i
   o.vec = T % 8 == 0 && aligned(grad_out, 16) ? 1 : 0;
   const long long blocks = o.unfold_blocks + (long long)o.t_tiles * o.f_tiles * B;
   if (blocks >= (1ll << 31)) return PE_ERR_DIM;
-  conv_operands_kernel<<<(unsigned)blocks, LAYOUT_THREADS, std::max(t.smem, 64 * TRANSPOSE_PITCH * 2), st>>>(o, g);
-  if ((rc = check_launch()) != PE_OK) return rc;
-  if (forced != PE_PATH_SIMT && whole) return tc_linear_stats(di, X, dY, B, T, d_in, F, phi, out_mean, out_stat, false, st);
+  const LayoutStep operands = [&](const LayoutZero& zero) {
+    return launch_dependent(any_output(zero) ? conv_operands_kernel<true> : conv_operands_kernel<false>, dim3((unsigned)blocks), LAYOUT_THREADS, std::max(t.smem, 64 * TRANSPOSE_PITCH * 2), st, o, g, zero);
+  };
+  if (forced != PE_PATH_SIMT && whole) return tc_linear_stats(di, X, dY, B, T, d_in, F, phi, out_mean, out_stat, false, st, operands);
   if (forced != PE_PATH_SIMT && padding_pays(B, T, d_in, F))
-    return tc_linear_stats_pitched(di, X, dY, B, T, d_in, F, phi, out_mean, out_stat, nullptr, false, l.pitch_x, l.pitch_y, st);
+    return tc_linear_stats_pitched(di, X, dY, B, T, d_in, F, phi, out_mean, out_stat, nullptr, false, l.pitch_x, l.pitch_y, st, operands);
+  if ((rc = operands(LayoutZero{})) != PE_OK) return rc;
   g_last_path.store(PE_PATH_SIMT);
   return launch_simt<__nv_bfloat16, MODE_STATS>(di, reinterpret_cast<const __nv_bfloat16*>(X), reinterpret_cast<const __nv_bfloat16*>(dY), B, T, d_in, F,
                                                 (int)phi, out_mean, out_stat, st, false, SimtExtra{}, nullptr, l.pitch_x, l.pitch_y);

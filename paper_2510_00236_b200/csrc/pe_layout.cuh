@@ -7,10 +7,29 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "pe_sm100.cuh"
+
 namespace pe {
 
 constexpr int LAYOUT_THREADS = 256;
 constexpr int UNFOLD_SMEM_BYTES = 48 * 1024;
+
+// These kernels also zero the outputs of a split batch, which saves a launch between them and the statistics kernel, and are launched as
+// programmatic dependents: 8 x 64 x 257 x 511 19.6 -> 17.3 us, 16 x 100 x 333 x 2001 24.9 -> 21.6, 16 images of 16 x 56 x 56 under 3 x 3 filters
+// 33.5 -> 29.4.  ZERO = false where there is nothing to zero: the loops alone cost 30 x 50 x 900 x 1501 27.1 -> 28.9 us.
+struct LayoutZero {
+  float* out[3];                // NULL: none; 16-byte aligned
+  long long n;                  // floats per output
+};
+// first, step: this thread's share of the floats, in groups of four
+__device__ __forceinline__ void zero_share(const LayoutZero& z, long long first, long long step) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    if (!z.out[k]) continue;
+    for (long long i = first; i < z.n >> 2; i += step) reinterpret_cast<float4*>(z.out[k])[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (long long i = (z.n & ~3ll) + first; i < z.n; i += step) z.out[k][i] = 0.f;
+  }
+}
 
 // dst[r, 0..d) = src[r, 0..d): src rows back to back, dst rows `pitch` elements apart (a multiple of 8, at least d).
 // A thread writes 16-byte groups; their eight source elements start at any even byte, so it reads the two aligned 16-byte
@@ -21,8 +40,12 @@ struct PadTensor {
   uint16_t* dst;
   int d, pitch;
 };
+template <bool ZERO>
 __global__ void __launch_bounds__(LAYOUT_THREADS)
-pad_rows_kernel(PadTensor ta, PadTensor tb, long long rows) {
+pad_rows_kernel(PadTensor ta, PadTensor tb, long long rows, LayoutZero zero) {
+  sm100::griddep_launch_dependents();
+  sm100::griddep_wait();
+  if (ZERO) zero_share(zero, ((long long)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x, (long long)gridDim.x * gridDim.y * blockDim.x);
   const PadTensor& t = blockIdx.y == 0 ? ta : tb;
   const int groups = t.pitch >> 3;
   const long long total = rows * groups, elems = rows * t.d;
@@ -165,9 +188,13 @@ __device__ __forceinline__ void transpose_block(const ConvOperands& o, int F, in
     *reinterpret_cast<uint4*>(o.dY + ((long long)b * T + t0 + t) * o.pitch_y + f0 + f) = make_uint4(v[0], v[1], v[2], v[3]);
   }
 }
+template <bool ZERO>
 __global__ void __launch_bounds__(LAYOUT_THREADS)
-conv_operands_kernel(ConvOperands o, ConvGeom g) {
+conv_operands_kernel(ConvOperands o, ConvGeom g, LayoutZero zero) {
   extern __shared__ __align__(16) uint16_t layout_smem[];
+  sm100::griddep_launch_dependents();
+  sm100::griddep_wait();
+  if (ZERO) zero_share(zero, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
   if ((long long)blockIdx.x < o.unfold_blocks) unfold_block(o, g, layout_smem);
   else transpose_block(o, g.F, g.Ho * g.Wo, layout_smem);
 }
@@ -181,15 +208,11 @@ conv_operands_kernel(ConvOperands o, ConvGeom g) {
 //
 // Copy k (0 as it is, 1 and 2 the halves, 3 the sign) of an operand is [n][chunk][pitch], rows past B zero.  A block takes a row; blocks
 // past the rows zero the outputs.  Bound by launch latency and HBM: two reads of 2 bytes and up to 8 written per element.  The whole
-// call, mean and square: 1024 x 1024^2 133 -> 25 us, 512 x 4096^2 781 -> 123, against forming every G_b.
+// call, mean and square: 1024 x 1024^2 133 -> 23 us, 512 x 4096^2 781 -> 123, against forming every G_b.
 struct OneTokenTensor {
   const uint16_t* src;
   uint16_t* dst;
   int d, pitch;
-};
-struct OneTokenOutputs {
-  float* out[3];
-  long long n;                  // floats per output
 };
 __device__ __forceinline__ void one_token_load(const uint16_t* row, int d, int g, bool vec, uint32_t (&w)[8]) {
   if (vec) {
@@ -202,16 +225,12 @@ __device__ __forceinline__ void one_token_load(const uint16_t* row, int d, int g
   }
 }
 __global__ void __launch_bounds__(LAYOUT_THREADS)
-one_token_operands_kernel(OneTokenTensor tx, OneTokenTensor ty, int B, int chunk, int n, int want_square, int want_mean, int want_sign, OneTokenOutputs zero) {
+one_token_operands_kernel(OneTokenTensor tx, OneTokenTensor ty, int B, int chunk, int n, int want_square, int want_mean, int want_sign, LayoutZero zero) {
+  sm100::griddep_launch_dependents();
+  sm100::griddep_wait();
   const int rows = n * chunk, b = blockIdx.x;
   if (b >= rows) {
-    const long long first = (long long)(b - rows) * LAYOUT_THREADS + threadIdx.x, step = (long long)(gridDim.x - rows) * LAYOUT_THREADS;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      if (!zero.out[k]) continue;
-      for (long long i = first; i < zero.n >> 2; i += step) reinterpret_cast<float4*>(zero.out[k])[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (long long i = (zero.n & ~3ll) + first; i < zero.n; i += step) zero.out[k][i] = 0.f;
-    }
+    zero_share(zero, (long long)(b - rows) * LAYOUT_THREADS + threadIdx.x, (long long)(gridDim.x - rows) * LAYOUT_THREADS);
     return;
   }
   const bool vx = tx.d % 8 == 0, vy = ty.d % 8 == 0;
