@@ -233,6 +233,10 @@ def pe_conv2d_stats(x, grad_out, kernel_size, phi, stride, padding, dilation, ou
     need = pe_conv2d_stats_workspace_bytes(B, C, H, W, F, *kernel_size, stride, padding, dilation)
     if need == 0:
         return False
+    # the library sees bare pointers: sizes it derives from x must be those that grad_out has
+    sizes = tuple((n + 2 * p - d * (k - 1) - 1) // s + 1 for n, p, d, k, s in zip((H, W), padding, dilation, kernel_size, stride))
+    if tuple(grad_out.shape) != (B, F, *sizes) or grad_out.device != x.device:
+        raise ValueError("grad_out must be [B, F, H_out, W_out] of this convolution, on x's device")
     workspace = x.new_empty((need,), dtype=torch.uint8)
     _launch("pe_conv2d_stats", x, x.data_ptr(), grad_out.data_ptr(), B, C, H, W, F, *kernel_size, *stride, *padding, *dilation, _phi(phi),
             _ptr(out_mean), _ptr(out_stat), workspace.data_ptr(), need)

@@ -1,0 +1,24 @@
+"""What the binding refuses before the library, which sees bare pointers, is called.  Nothing here needs a GPU."""
+import pytest
+import torch
+
+import paper_2510_00236_b200 as pe
+
+BF16 = torch.bfloat16
+
+
+# x 2 x 3 x 9 x 8 under a 3 x 3 kernel, stride (2, 1), padding (1, 0), dilation (1, 2): 5 x 4 positions
+@pytest.mark.parametrize("shape,device", [((2, 4, 5, 3), "cpu"), ((2, 4, 4, 4), "cpu"), ((1, 4, 5, 4), "cpu"), ((2, 4, 4, 5), "cpu"),
+                                          ((2, 4, 6, 4), "cpu"), ((2, 4, 5, 4), "meta")])
+def test_convolution_refuses_cotangents_of_another_size_or_device(shape, device):
+    x, grad_out = torch.zeros((2, 3, 9, 8), dtype=BF16), torch.zeros(shape, dtype=BF16, device=device)
+    mean, stat = torch.zeros((4, 27)), torch.zeros((4, 27))
+    with pytest.raises(ValueError, match="grad_out"):
+        pe.pe_conv2d_stats(x, grad_out, (3, 3), "square", (2, 1), (1, 0), (1, 2), mean, stat)
+
+
+def test_convolution_of_the_right_size_reaches_the_library():
+    x, grad_out = torch.zeros((2, 3, 9, 8), dtype=BF16), torch.zeros((2, 4, 5, 4), dtype=BF16)
+    mean, stat = torch.zeros((4, 27)), torch.zeros((4, 27))
+    with pytest.raises(pe.PestatsError):            # a tensor on the CPU
+        pe.pe_conv2d_stats(x, grad_out, (3, 3), "square", (2, 1), (1, 0), (1, 2), mean, stat)
