@@ -209,6 +209,8 @@ def pe_linear_stats_padded(X, dY, phi, accumulate, out_mean, out_stat, out_sign,
     B, T, d_in, d_out = _io_check(X, dY, torch.bfloat16)
     for name, t in (("out_mean", out_mean), ("out_stat", out_stat), ("out_sign", out_sign)):
         _out_check(name, t, d_out, d_in)
+    if workspace is not None and (workspace.device != X.device or not workspace.is_contiguous()):
+        raise ValueError("workspace must be a contiguous tensor on X's device")
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     _launch("pe_linear_stats_padded", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, _phi(phi), int(bool(accumulate)), _ptr(out_mean),
             _ptr(out_stat), _ptr(out_sign), _ptr(workspace), ws_bytes)

@@ -22,3 +22,11 @@ def test_convolution_of_the_right_size_reaches_the_library():
     mean, stat = torch.zeros((4, 27)), torch.zeros((4, 27))
     with pytest.raises(pe.PestatsError):            # a tensor on the CPU
         pe.pe_conv2d_stats(x, grad_out, (3, 3), "square", (2, 1), (1, 0), (1, 2), mean, stat)
+
+
+@pytest.mark.parametrize("workspace", [torch.empty(4096, dtype=torch.uint8, device="meta"), torch.zeros(1, dtype=torch.uint8).expand(1 << 20),
+                                       torch.zeros(8192, dtype=torch.uint8)[::2]])
+def test_padded_call_refuses_a_workspace_the_kernels_cannot_write(workspace):
+    X, out = torch.zeros((2, 4, 9), dtype=BF16), torch.zeros((9, 9))
+    with pytest.raises(ValueError, match="workspace"):
+        pe.pe_linear_stats_padded(X, X, "square", 0, out, torch.zeros((9, 9)), None, workspace)
