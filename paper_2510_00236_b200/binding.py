@@ -149,8 +149,9 @@ def _phi(phi) -> int:
 # The two lookups every call makes, in their cheapest form (0.1 us each): torch.cuda.current_stream builds a Stream object
 # (2.3 us) and torch.cuda.device switches and restores the device (1.6 us) even when it is the current one already, together
 # a third of a small call's host time.
-_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-_current_device = getattr(torch._C, "_cuda_getDevice", None)
+# They are private names of torch: where one is missing, the public call does the same.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda dev: torch.cuda.current_stream(dev).cuda_stream)
+_current_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
 
 
 def _launch(name, t, *args):

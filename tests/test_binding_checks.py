@@ -1,8 +1,12 @@
 """What the binding refuses before the library, which sees bare pointers, is called.  Nothing here needs a GPU."""
+import importlib.util
+import types
+
 import pytest
 import torch
 
 import paper_2510_00236_b200 as pe
+from paper_2510_00236_b200 import binding
 
 BF16 = torch.bfloat16
 
@@ -30,3 +34,14 @@ def test_padded_call_refuses_a_workspace_the_kernels_cannot_write(workspace):
     X, out = torch.zeros((2, 4, 9), dtype=BF16), torch.zeros((9, 9))
     with pytest.raises(ValueError, match="workspace"):
         pe.pe_linear_stats_padded(X, X, "square", 0, out, torch.zeros((9, 9)), None, workspace)
+
+
+def test_lookups_without_torch_private_functions(monkeypatch):
+    for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+        monkeypatch.delattr(torch._C, name, raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda dev: types.SimpleNamespace(cuda_stream=1000 + dev))
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    spec = importlib.util.spec_from_file_location("paper_2510_00236_b200.binding_again", binding.__file__)
+    again = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(again)
+    assert again._raw_stream(2) == 1002 and again._current_device() == 3
