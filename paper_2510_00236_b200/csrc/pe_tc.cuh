@@ -1192,6 +1192,9 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   }
 
   // ---------------------------------------------------------------- teardown
+  // Sequences of whole 16-token groups need nothing of the side buffer, and with an unsplit batch nothing above has waited for the kernel
+  // that fills it.  This one may not complete before it does: the next call may fill the same workspace.
+  if constexpr (RAGGED) griddep_wait();
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
