@@ -168,7 +168,7 @@ pe_status_t pe_linear_stats_all(const void* X, const void* dY, int B, int T, int
  * the operands concerned to a padded pitch and contracts the copies on the tensor cores.  Examples of one token (T == 1):
  * G_b is an outer product, so that the sums over b are contractions of the operands' exact squares (as pairs of bf16) and
  * signs, which are written to the workspace; no G_b is formed.  accumulate != 0: as pe_linear_stats_accumulate; out_sign != NULL (phi square, accumulate 0): as pe_linear_stats_all.
- * workspace: device memory, 256-byte aligned, pe_linear_stats_padded_workspace_bytes() bytes, contents undefined
+ * workspace: device memory, 256-byte aligned, pe_linear_stats_padded_workspace_bytes() bytes (whatever the outputs are), contents undefined
  * afterwards.  That function returns 0 where nothing is to be gained (widths that are multiples of 8 with T > 1, layers too small, a forced
  * path): the call is then the ordinary one and ignores the workspace.  Other arguments, alignments and results as for
  * pe_linear_stats.
@@ -177,6 +177,11 @@ pe_status_t pe_linear_stats_padded(const void* X, const void* dY, int B, int T, 
                                    int accumulate, float* out_mean, float* out_stat, float* out_sign, void* workspace,
                                    size_t workspace_bytes, pe_stream_t stream);
 size_t pe_linear_stats_padded_workspace_bytes(int B, int T, int d_in, int d_out);
+/* The same for a call with this phi and these outputs (want_*: nonzero for one that is given): all that pe_linear_stats_padded asks for.
+ * Examples of one token: one copy of each operand for the mean, two for the square, one for the sign; none for the mean alone of widths
+ * that are multiples of 8. */
+size_t pe_linear_stats_padded_workspace_bytes_for(int B, int T, int d_in, int d_out, pe_phi_t phi, int want_mean, int want_stat,
+                                                  int want_sign);
 
 /*
  * pe_linear_stats for the weight [F, C, Kh, Kw] of a 2-D convolution (Appendix B.4): every output position is a token, its

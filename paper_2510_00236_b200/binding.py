@@ -21,7 +21,7 @@ __all__ = [
     "pe_linear_stats_ragged", "pe_linear_stats_ragged_workspace_bytes", "pe_example_sqnorms_ragged", "pe_linear_clipped_sum",
     "pe_linear_microadam_step", "pe_linear_microadam_step_f32", "pe_linear_microsignsgd_step", "pe_linear_fused_workspace_bytes",
     "pe_token_sqstats_fp8", "pe_token_sqstats_fp8_workspace_bytes", "pe_set_wait_limit_cycles", "pe_tile_order_band",
-    "pe_linear_stats_padded", "pe_linear_stats_padded_workspace_bytes", "pe_conv2d_stats", "pe_conv2d_stats_workspace_bytes",
+    "pe_linear_stats_padded", "pe_linear_stats_padded_workspace_bytes", "pe_linear_stats_padded_workspace_bytes_for", "pe_conv2d_stats", "pe_conv2d_stats_workspace_bytes",
     "pe_set_fused_update", "FUSED_AUTO", "FUSED_ALWAYS", "FUSED_NEVER",
 ]
 
@@ -39,7 +39,7 @@ EXPORTED_SYMBOLS = [
     "pe_linear_stats_ragged", "pe_linear_stats_ragged_workspace_bytes", "pe_example_sqnorms_ragged", "pe_linear_clipped_sum",
     "pe_linear_microadam_step", "pe_linear_microadam_step_f32", "pe_linear_microsignsgd_step", "pe_linear_fused_workspace_bytes",
     "pe_token_sqstats_fp8", "pe_token_sqstats_fp8_workspace_bytes", "pe_set_wait_limit_cycles", "pe_tile_order_band",
-    "pe_set_fused_update", "pe_linear_stats_padded", "pe_linear_stats_padded_workspace_bytes", "pe_conv2d_stats",
+    "pe_set_fused_update", "pe_linear_stats_padded", "pe_linear_stats_padded_workspace_bytes", "pe_linear_stats_padded_workspace_bytes_for", "pe_conv2d_stats",
     "pe_conv2d_stats_workspace_bytes",
 ]
 ADAM_VARIANTS = {"adam": 0, "microadam": 1, "microadam_var": 2, "microadam_msq": 3}      # pe_adam_variant_t
@@ -76,6 +76,8 @@ def load_library() -> ctypes.CDLL:
     lib.pe_linear_stats_padded.argtypes = [vp, vp, i, i, i, i, i, i, vp, vp, vp, vp, sz, vp]
     lib.pe_linear_stats_padded_workspace_bytes.argtypes = [i] * 4
     lib.pe_linear_stats_padded_workspace_bytes.restype = sz
+    lib.pe_linear_stats_padded_workspace_bytes_for.argtypes = [i] * 8
+    lib.pe_linear_stats_padded_workspace_bytes_for.restype = sz
     lib.pe_conv2d_stats.argtypes = [vp, vp] + [i] * 14 + [vp, vp, vp, sz, vp]
     lib.pe_conv2d_stats_workspace_bytes.argtypes = [i] * 13
     lib.pe_conv2d_stats_workspace_bytes.restype = sz
@@ -190,22 +192,34 @@ def pe_linear_stats_padded_workspace_bytes(B, T, d_in, d_out) -> int:
     return int(load_library().pe_linear_stats_padded_workspace_bytes(int(B), int(T), int(d_in), int(d_out)))
 
 
+def pe_linear_stats_padded_workspace_bytes_for(B, T, d_in, d_out, phi, want_mean, want_stat, want_sign=False) -> int:
+    """What pe_linear_stats_padded asks for with this phi and these outputs."""
+    return int((_lib or load_library()).pe_linear_stats_padded_workspace_bytes_for(B, T, d_in, d_out, _phi(phi), bool(want_mean), bool(want_stat),
+                                                                                   bool(want_sign)))
+
+
 def _padded(X, dY, B, T, d_in, d_out, phi, accumulate, out_mean, out_stat, out_sign) -> bool:
     """Runs pe_linear_stats_padded with a workspace from torch's allocator if the widths are no multiples of 8 or the
-    examples single tokens, and the library says that it pays; False if the ordinary call is the one to make."""
+    examples single tokens, and the library says that it pays; False if the ordinary call is the one to make, which it also is when
+    there is no memory for the workspace: it needs none."""
     if not (d_in & 7 or d_out & 7 or T == 1):
         return False
-    need = pe_linear_stats_padded_workspace_bytes(B, T, d_in, d_out)
+    need = pe_linear_stats_padded_workspace_bytes_for(B, T, d_in, d_out, phi, out_mean is not None, out_stat is not None, out_sign is not None)
     if need == 0:
         return False
-    pe_linear_stats_padded(X, dY, phi, accumulate, out_mean, out_stat, out_sign, X.new_empty((need,), dtype=torch.uint8))
+    try:
+        workspace = X.new_empty((need,), dtype=torch.uint8)
+    except torch.OutOfMemoryError:
+        return False
+    pe_linear_stats_padded(X, dY, phi, accumulate, out_mean, out_stat, out_sign, workspace)
     return True
 
 
 def pe_linear_stats_padded(X, dY, phi, accumulate, out_mean, out_stat, out_sign, workspace):
     """The C entry point: statistics of a layer whose widths are no multiples of 8, or whose examples are single tokens, by way of
     copies in `workspace`
-    (uint8, pe_linear_stats_padded_workspace_bytes(...) bytes; None where that is 0).  pe_linear_stats, _accumulate and
+    (uint8, pe_linear_stats_padded_workspace_bytes_for(...) bytes, or pe_linear_stats_padded_workspace_bytes(...) for any
+    outputs; None where that is 0).  pe_linear_stats, _accumulate and
     _all call it where it pays."""
     B, T, d_in, d_out = _io_check(X, dY, torch.bfloat16)
     for name, t in (("out_mean", out_mean), ("out_stat", out_stat), ("out_sign", out_sign)):

@@ -1021,7 +1021,21 @@ static bool padding_pays(int B, int T, int d_in, int d_out) {
          (double)B * T * d_in * d_out >= (double)PAD_MIN_MACS && (long long)B * T < (1ll << 31);
 }
 
-// Examples of one token: the four copies of each operand, in n chunks of `chunk` rows.  A chunk is what one accumulator takes, and the
+// Examples of one token: the statistics that are wanted, and where their copies of the operands are among those that are made (the mean
+// needs the operands as they are, the square the two halves of their squares, the sign their signs).
+struct OneTokenWant {
+  bool mean, square, sign;
+  int first_half() const { return mean ? 1 : 0; }
+  int first_sign() const { return first_half() + (square ? 2 : 0); }
+  int copies() const { return first_sign() + (sign ? 1 : 0); }
+};
+static OneTokenWant one_token_want(int phi, bool mean, bool stat, bool sign) {
+  if (phi == PE_PHI_IDENTITY) return {mean || stat, false, false};
+  if (phi == PE_PHI_SIGN) return {mean, false, stat};
+  return {mean, stat, sign};
+}
+
+// The copies of each operand, in n chunks of `chunk` rows.  A chunk is what one accumulator takes, and the
 // accumulators are added in registers; the square's error against fp64, 2-norm, at 1024 x 1024^2: 1.4e-6 with 512 rows, 3.0e-7 with
 // 128, 1.7e-7 with 64, and 2.4e-7 with the kernel that forms every G_b.  64 rows cost 10 % there.
 constexpr int ONE_TOKEN_CHUNK = 64;
@@ -1029,14 +1043,14 @@ struct OneTokenLayout {
   int chunk, n, pitch_x, pitch_y;
   size_t x_bytes, y_bytes;
 };
-static OneTokenLayout one_token_layout(int B, int d_in, int d_out) {
+static OneTokenLayout one_token_layout(int B, int d_in, int d_out, int copies) {
   OneTokenLayout l;
   l.n = (B + ONE_TOKEN_CHUNK - 1) / ONE_TOKEN_CHUNK;
   l.chunk = ((B + l.n - 1) / l.n + 15) / 16 * 16;
   l.pitch_x = (d_in + 7) & ~7;
   l.pitch_y = (d_out + 7) & ~7;
-  l.x_bytes = align_up((size_t)4 * l.n * l.chunk * l.pitch_x * 2, 256);
-  l.y_bytes = align_up((size_t)4 * l.n * l.chunk * l.pitch_y * 2, 256);
+  l.x_bytes = align_up((size_t)copies * l.n * l.chunk * l.pitch_x * 2, 256);
+  l.y_bytes = align_up((size_t)copies * l.n * l.chunk * l.pitch_y * 2, 256);
   return l;
 }
 // From this many entries of all G_b on, the two launches (16 us at least, and 8 us more of host time) beat the kernel that forms every
@@ -1077,28 +1091,29 @@ static void one_token_slices(const OneTokenLayout& l, const bool (&want)[3], lon
 }
 static pe_status_t one_token_stats(DeviceInfo* di, const void* X, const void* dY, int B, int d_in, int d_out, float* out_mean, float* out_square,
                                    float* out_sign, bool accumulate, void* workspace, cudaStream_t st) {
-  const OneTokenLayout l = one_token_layout(B, d_in, d_out);
+  const OneTokenWant want = {out_mean != nullptr, out_square != nullptr, out_sign != nullptr};
+  const OneTokenLayout l = one_token_layout(B, d_in, d_out, want.copies());
   const OneTokenTensor tx = {static_cast<const uint16_t*>(X), static_cast<uint16_t*>(workspace), d_in, l.pitch_x};
   const OneTokenTensor ty = {static_cast<const uint16_t*>(dY), reinterpret_cast<uint16_t*>(static_cast<char*>(workspace) + l.x_bytes), d_out, l.pitch_y};
   const int tiles_n = (d_in + 255) / 256, pairs_m = (d_out + TC_PAIR_M - 1) / TC_PAIR_M;
   if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
   const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
   float* const outs[3] = {out_square, out_mean, out_sign};
-  const bool want[3] = {out_square != nullptr, out_mean != nullptr, out_sign != nullptr};
   TcParams p{};
-  one_token_slices(l, want, (long long)tiles_n * pairs_m, slots, 4.0 * (want[0] + want[1] + want[2]) * d_in * d_out, p.part_slices);
+  one_token_slices(l, {want.square, want.mean, want.sign}, (long long)tiles_n * pairs_m, slots, 4.0 * (want.mean + want.square + want.sign) * d_in * d_out,
+                   p.part_slices);
   const bool split = p.part_slices[0] > 1 || p.part_slices[1] > 1 || p.part_slices[2] > 1;
   LayoutZero zero = {{nullptr, nullptr, nullptr}, (long long)d_in * d_out};
   if (split && !accumulate)
     for (int k = 0; k < 3; ++k) zero.out[k] = outs[k];
   const int rows = l.n * l.chunk, zero_blocks = split && !accumulate ? 2 * di->sm_count : 0;
-  pe_status_t rc = launch_dependent(one_token_operands_kernel, dim3(rows + zero_blocks), LAYOUT_THREADS, 0, st, tx, ty, B, l.chunk, l.n, want[0] ? 1 : 0,
-                                    want[1] ? 1 : 0, want[2] ? 1 : 0, zero);
+  pe_status_t rc = launch_dependent(one_token_operands_kernel, dim3(rows + zero_blocks), LAYOUT_THREADS, 0, st, tx, ty, B, l.chunk, l.n, want.mean ? 0 : -1,
+                                    want.square ? want.first_half() : -1, want.sign ? want.first_sign() : -1, zero);
   if (rc != PE_OK) return rc;
   CUtensorMap mx, my;
   constexpr int box_feats = TcOperand<false, 256>::BOX_FEATS, box_tokens = TcOperand<false, 256>::BK;
-  rc = make_operand_map(&mx, tx.dst, 4 * l.n, l.chunk, d_in, false, box_feats, box_tokens, false, 1, l.pitch_x);
-  if (rc == PE_OK) rc = make_operand_map(&my, ty.dst, 4 * l.n, l.chunk, d_out, false, box_feats, box_tokens, false, 1, l.pitch_y);
+  rc = make_operand_map(&mx, tx.dst, want.copies() * l.n, l.chunk, d_in, false, box_feats, box_tokens, false, 1, l.pitch_x);
+  if (rc == PE_OK) rc = make_operand_map(&my, ty.dst, want.copies() * l.n, l.chunk, d_out, false, box_feats, box_tokens, false, 1, l.pitch_y);
   if (rc != PE_OK) return rc;
   const bool scalar_out = d_in % 4 != 0;
   CUtensorMap mo[3] = {mx, mx, mx};
@@ -1109,6 +1124,10 @@ static pe_status_t one_token_stats(DeviceInfo* di, const void* X, const void* dY
   }
   p.B = 6 * l.n; p.T = l.chunk; p.d_in = d_in; p.d_out = d_out; p.nsplit = split ? 2 : 1; p.per_example = 1;
   p.accumulate = accumulate ? 1 : 0; p.scalar_out = scalar_out ? 1 : 0; p.wait_at_start = 1; p.part_chunks = l.n;
+  // the copies that products 0 to 5 take (tc_part_chunk), four bits each: mean | upper and lower halves of dY by those of X | sign
+  const unsigned int half = want.first_half(), sign = want.first_sign();
+  p.part_dy = half * 0x11110u + 0x10100u + (sign << 20);
+  p.part_x = half * 0x11110u + 0x11000u + (sign << 20);
   p.pairs_m = pairs_m; p.tiles_n = tiles_n;
   const int units = p.part_slices[0] + p.part_slices[1] + p.part_slices[2];
   p.band = choose_band(pairs_m, tiles_n, 256, units, slots);
@@ -1117,10 +1136,12 @@ static pe_status_t one_token_stats(DeviceInfo* di, const void* X, const void* dY
       di, 31, mx, my, mo[1], mo[0], mo[2], p, dim3(2 * pairs_m * tiles_n, 1, units), st);
 }
 
-size_t pe_linear_stats_padded_workspace_bytes(int B, int T, int d_in, int d_out) {
+static size_t padded_workspace_bytes(int B, int T, int d_in, int d_out, const OneTokenWant& want) {
   if (B < 1 || T < 1 || d_in < 1 || d_out < 1 || g_path.load() != PE_PATH_AUTO) return 0;
   if (one_token_pays(B, T, d_in, d_out)) {
-    const OneTokenLayout l = one_token_layout(B, d_in, d_out);
+    // the mean alone of widths that TMA can address is a contraction of the operands as they are
+    if (!want.square && !want.sign && (!want.mean || (d_in % 8 == 0 && d_out % 8 == 0))) return 0;
+    const OneTokenLayout l = one_token_layout(B, d_in, d_out, want.copies());
     return l.x_bytes + l.y_bytes;
   }
   if (!padding_pays(B, T, d_in, d_out)) return 0;
@@ -1128,13 +1149,19 @@ size_t pe_linear_stats_padded_workspace_bytes(int B, int T, int d_in, int d_out)
   return l.x_bytes + l.y_bytes;
 }
 
+size_t pe_linear_stats_padded_workspace_bytes(int B, int T, int d_in, int d_out) {
+  return padded_workspace_bytes(B, T, d_in, d_out, {true, true, true});
+}
+size_t pe_linear_stats_padded_workspace_bytes_for(int B, int T, int d_in, int d_out, pe_phi_t phi, int want_mean, int want_stat, int want_sign) {
+  return padded_workspace_bytes(B, T, d_in, d_out, one_token_want(phi, want_mean != 0, want_stat != 0, want_sign != 0));
+}
+
 pe_status_t pe_linear_stats_padded(const void* X, const void* dY, int B, int T, int d_in, int d_out, pe_phi_t phi, int accumulate,
                                    float* out_mean, float* out_stat, float* out_sign, void* workspace, size_t workspace_bytes,
                                    pe_stream_t stream) {
-  const size_t need = pe_linear_stats_padded_workspace_bytes(B, T, d_in, d_out);
+  const size_t need = pe_linear_stats_padded_workspace_bytes_for(B, T, d_in, d_out, phi, out_mean != nullptr, out_stat != nullptr, out_sign != nullptr);
   if (out_sign && (accumulate || phi != PE_PHI_SQUARE)) return PE_ERR_PHI;
-  const bool plain = T == 1 && phi == PE_PHI_IDENTITY && d_in % 8 == 0 && d_out % 8 == 0;       // a contraction of the operands as they are
-  if (need == 0 || plain) {
+  if (need == 0) {
     if (out_sign) return pe_linear_stats_all(X, dY, B, T, d_in, d_out, out_mean, out_stat, out_sign, stream);
     return accumulate ? pe_linear_stats_accumulate(X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, stream)
                       : pe_linear_stats(X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, stream);

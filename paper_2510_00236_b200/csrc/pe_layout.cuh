@@ -206,7 +206,8 @@ conv_operands_kernel(ConvOperands o, ConvGeom g, LayoutZero zero) {
 // equal magnitude (nothing changes in the product), so that the squares leave the range of fp32 only where G_b^2 does.
 // A lower half of zero is written as 2^-60 of the upper one, which no sum shows, so that infinities meet no zero they did not meet in G_b.
 //
-// Copy k (0 as it is, 1 and 2 the halves, 3 the sign) of an operand is [n][chunk][pitch], rows past B zero.  A block takes a row; blocks
+// A copy of an operand is [n][chunk][pitch], rows past B zero.  at_mean, at_halves, at_sign: the number of the copy as it is, of the upper half
+// (the lower one follows) and of the sign, -1 for one that is not wanted.  A block takes a row; blocks
 // past the rows zero the outputs.  Bound by launch latency and HBM: two reads of 2 bytes and up to 8 written per element.  The whole
 // call, mean and square: 1024 x 1024^2 133 -> 23 us, 512 x 4096^2 781 -> 123, against forming every G_b.
 struct OneTokenTensor {
@@ -225,7 +226,7 @@ __device__ __forceinline__ void one_token_load(const uint16_t* row, int d, int g
   }
 }
 __global__ void __launch_bounds__(LAYOUT_THREADS)
-one_token_operands_kernel(OneTokenTensor tx, OneTokenTensor ty, int B, int chunk, int n, int want_square, int want_mean, int want_sign, LayoutZero zero) {
+one_token_operands_kernel(OneTokenTensor tx, OneTokenTensor ty, int B, int chunk, int n, int at_mean, int at_halves, int at_sign, LayoutZero zero) {
   sm100::griddep_launch_dependents();
   sm100::griddep_wait();
   const int rows = n * chunk, b = blockIdx.x;
@@ -237,7 +238,7 @@ one_token_operands_kernel(OneTokenTensor tx, OneTokenTensor ty, int B, int chunk
   const uint16_t* const x = tx.src + (long long)b * tx.d;
   const uint16_t* const y = ty.src + (long long)b * ty.d;
   float scale_x = 1.f, scale_y = 1.f;
-  if (want_square && b < B) {
+  if (at_halves >= 0 && b < B) {
     __shared__ uint32_t top[2][LAYOUT_THREADS / 32];
     uint32_t mx = 0u, my = 0u, w[8];
     for (int g = threadIdx.x; g < tx.pitch / 8; g += LAYOUT_THREADS) {
@@ -282,9 +283,9 @@ one_token_operands_kernel(OneTokenTensor tx, OneTokenTensor ty, int B, int chunk
         *reinterpret_cast<uint4*>(dst + k * copy + 8 * g) = make_uint4((v[0] >> shift) | (v[1] >> shift << 16), (v[2] >> shift) | (v[3] >> shift << 16),
                                                                        (v[4] >> shift) | (v[5] >> shift << 16), (v[6] >> shift) | (v[7] >> shift << 16));
       };
-      if (want_mean) put(0, w, 16);
-      if (want_square) { put(1, hi, 0); put(2, lo, 0); }
-      if (want_sign) put(3, sg, 0);
+      if (at_mean >= 0) put(at_mean, w, 16);
+      if (at_halves >= 0) { put(at_halves, hi, 0); put(at_halves + 1, lo, 0); }
+      if (at_sign >= 0) put(at_sign, sg, 0);
     }
   };
   write(tx, x, vx, scale_x);

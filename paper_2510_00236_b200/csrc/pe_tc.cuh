@@ -148,6 +148,7 @@ struct TcParams {
   int tail_split;      // this many pairs, by slices of the batch, whose sums are added to (zeroed) outputs
   int part_chunks;     // PARTS: chunks of rows per part, slices of the square's, the mean's and the sign's chunks
   int part_slices[3];
+  unsigned int part_dy, part_x;   // PARTS: the copies of dY and of X that each product takes
   int per_example;     // 1: reset the accumulator for every example and apply phi (statistics)
                        // 0: one accumulation over the whole slice (plain contraction, phi = identity)
   int half_operands;   // 16-bit operands are IEEE half instead of bf16 (the staged per-token statistic)
@@ -167,11 +168,12 @@ struct TcParams {
   unsigned int* dev_status;
 };
 
-// PARTS: chunk c of the launch is chunk c % n of product c / n, the operands of which are copies 0 (as it is), 1 and 2 (upper and lower
-// half of the squares) and 3 (sign): dY0 X0 | dY1 X1, dY2 X1, dY1 X2, dY2 X2 | dY3 X3.  Where that chunk is in the operand.
+// PARTS: chunk c of the launch is chunk c % n of product c / n: the operands as they are | the upper half of dY's squares by that of X's, lower
+// by upper, upper by lower, lower by lower | the signs.  part_dy, part_x: the copy that a product takes, four bits each.  Where that
+// chunk is in the operand.
 __device__ __forceinline__ int tc_part_chunk(const TcParams& p, int c, bool of_dy) {
   const int product = c / p.part_chunks;
-  return (int)(((of_dy ? 0x321210u : 0x322110u) >> (4 * product)) & 15u) * p.part_chunks + c - product * p.part_chunks;
+  return (int)(((of_dy ? p.part_dy : p.part_x) >> (4 * product)) & 15u) * p.part_chunks + c - product * p.part_chunks;
 }
 
 // PERSIST: unit u of the launch, a tile and the examples it is contracted over.

@@ -45,3 +45,36 @@ def test_lookups_without_torch_private_functions(monkeypatch):
     again = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(again)
     assert again._raw_stream(2) == 1002 and again._current_device() == 3
+
+
+@pytest.mark.parametrize("phi,mean,stat,sign,copies", [("square", 1, 1, 1, 4), ("square", 1, 1, 0, 3), ("square", 0, 1, 0, 2), ("sign", 1, 1, 0, 2),
+                                                       ("sign", 0, 1, 0, 1), ("identity", 1, 1, 0, 0), ("identity", 0, 1, 0, 0), ("square", 1, 0, 0, 0)])
+def test_one_token_workspace_follows_the_outputs(phi, mean, stat, sign, copies):
+    B, d_in, d_out = 4096, 512, 1024
+    one = 2 * B * (d_in + d_out)
+    need = pe.pe_linear_stats_padded_workspace_bytes_for(B, 1, d_in, d_out, phi, mean, stat, sign)
+    assert copies * one <= need <= copies * (one + 2 * B)       # beside the copies: a few bytes per example
+    assert need <= pe.pe_linear_stats_padded_workspace_bytes(B, 1, d_in, d_out)
+    if copies == 0:             # widths that TMA cannot address need a copy for the mean too
+        assert pe.pe_linear_stats_padded_workspace_bytes_for(B, 1, 513, d_out, phi, mean, stat, sign) >= 2 * B * (513 + d_out)
+
+
+class _NoMemory(torch.Tensor):
+    def new_empty(self, size, dtype=None, **kw):
+        if dtype == torch.uint8:
+            raise torch.OutOfMemoryError("no memory for a workspace")
+        return super().new_empty(size, dtype=dtype, **kw)
+
+
+# single tokens, and a width that is no multiple of 8
+@pytest.mark.parametrize("B,T,d_in,d_out", [(128, 1, 1024, 1024), (64, 8, 513, 512)])
+def test_calls_without_memory_for_a_workspace_are_the_ordinary_ones(monkeypatch, B, T, d_in, d_out):
+    X, dY = (torch.zeros((B, T, d), dtype=BF16).as_subclass(_NoMemory) for d in (d_in, d_out))
+    outs = [torch.empty((d_out, d_in)) for _ in range(3)]
+    assert pe.pe_linear_stats_padded_workspace_bytes(B, T, d_in, d_out) > 0
+    called = []
+    monkeypatch.setattr(binding, "_launch", lambda name, *args: called.append(name))
+    pe.pe_linear_stats(X, dY, "square", outs[0], outs[1])
+    pe.pe_linear_stats_accumulate(X, dY, "sign", outs[0], outs[1])
+    pe.pe_linear_stats_all(X, dY, *outs)
+    assert called == ["pe_linear_stats", "pe_linear_stats_accumulate", "pe_linear_stats_all"]
