@@ -1041,16 +1041,18 @@ static OneTokenWant one_token_want(int phi, bool mean, bool stat, bool sign) {
 constexpr int ONE_TOKEN_CHUNK = 64;
 struct OneTokenLayout {
   int chunk, n, pitch_x, pitch_y;
-  size_t x_bytes, y_bytes;
+  size_t x_bytes, y_bytes, odd_bytes;     // odd: a byte per row (the marks of one_token_operands_kernel)
+  size_t total() const { return x_bytes + y_bytes + odd_bytes; }
 };
-static OneTokenLayout one_token_layout(int B, int d_in, int d_out, int copies) {
+static OneTokenLayout one_token_layout(int B, int d_in, int d_out, const OneTokenWant& want) {
   OneTokenLayout l;
   l.n = (B + ONE_TOKEN_CHUNK - 1) / ONE_TOKEN_CHUNK;
   l.chunk = ((B + l.n - 1) / l.n + 15) / 16 * 16;
   l.pitch_x = (d_in + 7) & ~7;
   l.pitch_y = (d_out + 7) & ~7;
-  l.x_bytes = align_up((size_t)copies * l.n * l.chunk * l.pitch_x * 2, 256);
-  l.y_bytes = align_up((size_t)copies * l.n * l.chunk * l.pitch_y * 2, 256);
+  l.x_bytes = align_up((size_t)want.copies() * l.n * l.chunk * l.pitch_x * 2, 256);
+  l.y_bytes = align_up((size_t)want.copies() * l.n * l.chunk * l.pitch_y * 2, 256);
+  l.odd_bytes = want.square || want.sign ? align_up((size_t)l.n * l.chunk, 256) : 0;
   return l;
 }
 // From this many entries of all G_b on, the two launches (16 us at least, and 8 us more of host time) beat the kernel that forms every
@@ -1092,7 +1094,8 @@ static void one_token_slices(const OneTokenLayout& l, const bool (&want)[3], lon
 static pe_status_t one_token_stats(DeviceInfo* di, const void* X, const void* dY, int B, int d_in, int d_out, float* out_mean, float* out_square,
                                    float* out_sign, bool accumulate, void* workspace, cudaStream_t st) {
   const OneTokenWant want = {out_mean != nullptr, out_square != nullptr, out_sign != nullptr};
-  const OneTokenLayout l = one_token_layout(B, d_in, d_out, want.copies());
+  const OneTokenLayout l = one_token_layout(B, d_in, d_out, want);
+  uint8_t* const odd = static_cast<uint8_t*>(workspace) + l.x_bytes + l.y_bytes;
   const OneTokenTensor tx = {static_cast<const uint16_t*>(X), static_cast<uint16_t*>(workspace), d_in, l.pitch_x};
   const OneTokenTensor ty = {static_cast<const uint16_t*>(dY), reinterpret_cast<uint16_t*>(static_cast<char*>(workspace) + l.x_bytes), d_out, l.pitch_y};
   const int tiles_n = (d_in + 255) / 256, pairs_m = (d_out + TC_PAIR_M - 1) / TC_PAIR_M;
@@ -1107,7 +1110,7 @@ static pe_status_t one_token_stats(DeviceInfo* di, const void* X, const void* dY
   if (split && !accumulate)
     for (int k = 0; k < 3; ++k) zero.out[k] = outs[k];
   const int rows = l.n * l.chunk, zero_blocks = split && !accumulate ? 2 * di->sm_count : 0;
-  pe_status_t rc = launch_dependent(one_token_operands_kernel, dim3(rows + zero_blocks), LAYOUT_THREADS, 0, st, tx, ty, B, l.chunk, l.n, want.mean ? 0 : -1,
+  pe_status_t rc = launch_dependent(one_token_operands_kernel, dim3(rows + zero_blocks), LAYOUT_THREADS, 0, st, tx, ty, odd, B, l.chunk, l.n, want.mean ? 0 : -1,
                                     want.square ? want.first_half() : -1, want.sign ? want.first_sign() : -1, zero);
   if (rc != PE_OK) return rc;
   CUtensorMap mx, my;
@@ -1128,6 +1131,7 @@ static pe_status_t one_token_stats(DeviceInfo* di, const void* X, const void* dY
   const unsigned int half = want.first_half(), sign = want.first_sign();
   p.part_dy = half * 0x11110u + 0x10100u + (sign << 20);
   p.part_x = half * 0x11110u + 0x11000u + (sign << 20);
+  p.odd_rows = odd; p.rows_dy = static_cast<const uint16_t*>(dY); p.rows_x = static_cast<const uint16_t*>(X);
   p.pairs_m = pairs_m; p.tiles_n = tiles_n;
   const int units = p.part_slices[0] + p.part_slices[1] + p.part_slices[2];
   p.band = choose_band(pairs_m, tiles_n, 256, units, slots);
@@ -1141,8 +1145,7 @@ static size_t padded_workspace_bytes(int B, int T, int d_in, int d_out, const On
   if (one_token_pays(B, T, d_in, d_out)) {
     // the mean alone of widths that TMA can address is a contraction of the operands as they are
     if (!want.square && !want.sign && (!want.mean || (d_in % 8 == 0 && d_out % 8 == 0))) return 0;
-    const OneTokenLayout l = one_token_layout(B, d_in, d_out, want.copies());
-    return l.x_bytes + l.y_bytes;
+    return one_token_layout(B, d_in, d_out, want).total();
   }
   if (!padding_pays(B, T, d_in, d_out)) return 0;
   const PaddedLayout l = padded_layout(B, T, d_in, d_out, false);

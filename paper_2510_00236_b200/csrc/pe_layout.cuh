@@ -202,31 +202,74 @@ conv_operands_kernel(ConvOperands o, ConvGeom g, LayoutZero zero) {
 // Operands of the statistics of examples of a single token, where G_b[o,i] = dY[b,o] X[b,i] and the sums over b are contractions of
 // row-wise functions of the operands: sum G_b = dY^T X, sum G_b^2 = (dY o dY)^T (X o X), sum sign(G_b) = sign(dY)^T sign(X).
 // The square of a bf16 has 16 significant bits: its upper and lower half are bf16 numbers, exactly, and four products of halves make up
-// the contraction without a rounding of the operands.  Each example's two rows are first scaled by 2^s and 2^-s to maxima of
-// equal magnitude (nothing changes in the product), so that the squares leave the range of fp32 only where G_b^2 does.
-// A lower half of zero is written as 2^-60 of the upper one, which no sum shows, so that infinities meet no zero they did not meet in G_b.
+// the contraction without a rounding of the operands.  Each example's two rows are first scaled by 2^-s and 2^s (nothing changes in the
+// product), which keeps the squares finite and their lower halves normal while the magnitudes that matter (those whose product with
+// the other row's largest has a square in fp32) lie within 2^-55 .. 2^63 after it.  s is the one that does so and is nearest to that of equal
+// maxima.  An example for which there is none, or that holds an infinity or a NaN, is left out of the halves and marked in `odd`, as is one with
+// a product of nonzero entries that may be zero in fp32, whose sign would count: the contraction forms G_b of those, entry by entry.
 //
 // A copy of an operand is [n][chunk][pitch], rows past B zero.  at_mean, at_halves, at_sign: the number of the copy as it is, of the upper half
 // (the lower one follows) and of the sign, -1 for one that is not wanted.  A block takes a row; blocks
 // past the rows zero the outputs.  Bound by launch latency and HBM: two reads of 2 bytes and up to 8 written per element.  The whole
-// call, mean and square: 1024 x 1024^2 133 -> 23 us, 512 x 4096^2 781 -> 123, against forming every G_b.
+// call, mean and square: 1024 x 1024^2 160 -> 23 us, 512 x 4096^2 1061 -> 124, against forming every G_b.  Finding the rows' ranges costs 0 to
+// 2.5 us of that.
+enum : int { ONE_TOKEN_ODD_SQUARE = 1, ONE_TOKEN_ODD_SIGN = 2 };
 struct OneTokenTensor {
   const uint16_t* src;
   uint16_t* dst;
   int d, pitch;
 };
-__device__ __forceinline__ void one_token_load(const uint16_t* row, int d, int g, bool vec, uint32_t (&w)[8]) {
-  if (vec) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(row) + g);
-    w[0] = v.x << 16; w[1] = v.x & 0xffff0000u; w[2] = v.y << 16; w[3] = v.y & 0xffff0000u;
-    w[4] = v.z << 16; w[5] = v.z & 0xffff0000u; w[6] = v.w << 16; w[7] = v.w & 0xffff0000u;
-  } else {
+// Eight entries as four words.
+__device__ __forceinline__ uint4 one_token_load(const uint16_t* row, int d, int g, bool vec) {
+  if (vec) return __ldg(reinterpret_cast<const uint4*>(row) + g);
+  uint32_t v[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) w[j] = 8 * g + j < d ? (uint32_t)__ldg(row + 8 * g + j) << 16 : 0u;
+  for (int j = 0; j < 8; ++j) v[j] = 8 * g + j < d ? (uint32_t)__ldg(row + 8 * g + j) : 0u;
+  return make_uint4(v[0] | v[1] << 16, v[2] | v[3] << 16, v[4] | v[5] << 16, v[6] | v[7] << 16);
+}
+// Largest and smallest nonzero magnitude of what a thread sees, as bf16 patterns, two entries at a time.  low: the pattern plus 0x7fff, which
+// as a signed number orders the nonzero patterns and puts zero last.
+struct PairExtremes {
+  uint32_t top = 0u, low = 0x7fff7fffu;
+  __device__ __forceinline__ void see(uint4 v) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t m = w[j] & 0x7fff7fffu;
+      top = __vmaxu2(top, m);
+      low = __vmins2(low, m + 0x7fff7fffu);
+    }
+  }
+  __device__ __forceinline__ int top_bits() const { return (int)max(top & 0xffffu, top >> 16); }
+  __device__ __forceinline__ int low_bits() const { return min((int)(int16_t)(low & 0xffffu), (int)(int16_t)(low >> 16)) + 0x8001; }
+};
+// Exponent of a nonzero magnitude; a subnormal counts as the smallest there is.
+__device__ __forceinline__ int one_token_exponent(int bits) { return bits < 0x80 ? -133 : (bits >> 7) - 127; }
+struct RowExtremes {
+  int top, low;
+  __device__ __forceinline__ bool zero() const { return top == 0; }
+  __device__ __forceinline__ bool finite() const { return top < 0x7f80; }
+  __device__ __forceinline__ int top_exponent() const { return max(1, top >> 7) - 127; }
+  __device__ __forceinline__ int low_exponent() const { return one_token_exponent(low); }
+};
+__device__ __forceinline__ void block_extremes(const PairExtremes& px, const PairExtremes& py, RowExtremes& x, RowExtremes& y) {
+  __shared__ int part[4][LAYOUT_THREADS / 32];
+  x = {__reduce_max_sync(0xffffffffu, px.top_bits()), __reduce_min_sync(0xffffffffu, px.low_bits())};
+  y = {__reduce_max_sync(0xffffffffu, py.top_bits()), __reduce_min_sync(0xffffffffu, py.low_bits())};
+  if ((threadIdx.x & 31) == 0) {
+    const int warp = threadIdx.x >> 5;
+    part[0][warp] = x.top; part[1][warp] = x.low; part[2][warp] = y.top; part[3][warp] = y.low;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < LAYOUT_THREADS / 32; ++k) {
+    x.top = max(x.top, part[0][k]); x.low = min(x.low, part[1][k]);
+    y.top = max(y.top, part[2][k]); y.low = min(y.low, part[3][k]);
   }
 }
 __global__ void __launch_bounds__(LAYOUT_THREADS)
-one_token_operands_kernel(OneTokenTensor tx, OneTokenTensor ty, int B, int chunk, int n, int at_mean, int at_halves, int at_sign, LayoutZero zero) {
+one_token_operands_kernel(OneTokenTensor tx, OneTokenTensor ty, uint8_t* odd, int B, int chunk, int n, int at_mean, int at_halves, int at_sign,
+                          LayoutZero zero) {
   sm100::griddep_launch_dependents();
   sm100::griddep_wait();
   const int rows = n * chunk, b = blockIdx.x;
@@ -237,59 +280,70 @@ one_token_operands_kernel(OneTokenTensor tx, OneTokenTensor ty, int B, int chunk
   const bool vx = tx.d % 8 == 0, vy = ty.d % 8 == 0;
   const uint16_t* const x = tx.src + (long long)b * tx.d;
   const uint16_t* const y = ty.src + (long long)b * ty.d;
-  float scale_x = 1.f, scale_y = 1.f;
+  float scale_x = 0.f, scale_y = 0.f;
+  bool in_halves = false;
+  PairExtremes px, py;
+  int flags = 0;
   if (at_halves >= 0 && b < B) {
-    __shared__ uint32_t top[2][LAYOUT_THREADS / 32];
-    uint32_t mx = 0u, my = 0u, w[8];
-    for (int g = threadIdx.x; g < tx.pitch / 8; g += LAYOUT_THREADS) {
-      one_token_load(x, tx.d, g, vx, w);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) mx = max(mx, w[j] & 0x7fffffffu);
-    }
-    for (int g = threadIdx.x; g < ty.pitch / 8; g += LAYOUT_THREADS) {
-      one_token_load(y, ty.d, g, vy, w);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) my = max(my, w[j] & 0x7fffffffu);
-    }
-    mx = __reduce_max_sync(0xffffffffu, mx);
-    my = __reduce_max_sync(0xffffffffu, my);
-    if ((threadIdx.x & 31) == 0) { top[0][threadIdx.x >> 5] = mx; top[1][threadIdx.x >> 5] = my; }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < LAYOUT_THREADS / 32; ++k) { mx = max(mx, top[0][k]); my = max(my, top[1][k]); }
-    const int ex = (int)(mx >> 23), ey = (int)(my >> 23);
-    if (ex > 0 && ex < 255 && ey > 0 && ey < 255) {
-      const int s = (ex - ey) / 2;                           // -126 .. 126
+    for (int g = threadIdx.x; g < tx.pitch / 8; g += LAYOUT_THREADS) px.see(one_token_load(x, tx.d, g, vx));
+    for (int g = threadIdx.x; g < ty.pitch / 8; g += LAYOUT_THREADS) py.see(one_token_load(y, ty.d, g, vy));
+    RowExtremes ex, ey;
+    block_extremes(px, py, ex, ey);
+    const bool finite = ex.finite() && ey.finite(), some = !ex.zero() && !ey.zero();
+    if (finite && some) {
+      const int top_x = ex.top_exponent(), top_y = ey.top_exponent();
+      // entries below these: a product with the other row's largest under 2^-75, a square that fp32 does not have
+      const int low_x = max(ex.low_exponent(), -76 - top_y), low_y = max(ey.low_exponent(), -76 - top_x);
+      const int least = max(max(top_x - 62, -55 - low_y), -126), most = min(min(62 - top_y, low_x + 55), 126);
+      const int s = min(max((top_x - top_y) / 2, least), most);
+      in_halves = least <= most;
       scale_x = __uint_as_float((uint32_t)(127 - s) << 23);
       scale_y = __uint_as_float((uint32_t)(127 + s) << 23);
     }
+    // (a row of zeros and one without infinities: G_b is zero, as the zeros in the copies make it)
+    if (!in_halves && (some || !finite)) flags = ONE_TOKEN_ODD_SQUARE;
+    if (at_sign >= 0 && some && ex.low_exponent() + ey.low_exponent() < -149) flags |= ONE_TOKEN_ODD_SIGN;
   }
-  auto write = [&](const OneTokenTensor& t, const uint16_t* row, bool vec, float scale) {
+  const bool look = at_halves < 0 && at_sign >= 0 && b < B;            // the smallest entries are found on the way
+  auto write = [&](const OneTokenTensor& t, const uint16_t* row, bool vec, float scale, PairExtremes& e) {
     const long long copy = (long long)rows * t.pitch;
     uint16_t* const dst = t.dst + (long long)b * t.pitch;
     for (int g = threadIdx.x; g < t.pitch / 8; g += LAYOUT_THREADS) {
-      uint32_t w[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u}, hi[8], lo[8], sg[8];
-      if (b < B) one_token_load(row, t.d, g, vec, w);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const float v = __uint_as_float(w[j]) * scale, q = v * v, up = __uint_as_float(__float_as_uint(q) & 0xffff0000u);
-        const float down = q - up;                           // exact; NaN where q is infinite
-        hi[j] = __float_as_uint(up) >> 16;
-        lo[j] = __float_as_uint(down > 0.f ? down : up * 0x1p-60f) >> 16;
-        const float f = __uint_as_float(w[j]);
-        sg[j] = f > 0.f ? 0x3f80u : f < 0.f ? 0xbf80u : 0u;
-      }
-      auto put = [&](int k, const uint32_t (&v)[8], int shift) {
-        *reinterpret_cast<uint4*>(dst + k * copy + 8 * g) = make_uint4((v[0] >> shift) | (v[1] >> shift << 16), (v[2] >> shift) | (v[3] >> shift << 16),
-                                                                       (v[4] >> shift) | (v[5] >> shift << 16), (v[6] >> shift) | (v[7] >> shift << 16));
+      const uint4 v = b < B ? one_token_load(row, t.d, g, vec) : make_uint4(0u, 0u, 0u, 0u);
+      if (look) e.see(v);
+      const uint32_t w[8] = {v.x << 16, v.x & 0xffff0000u, v.y << 16, v.y & 0xffff0000u, v.z << 16, v.z & 0xffff0000u, v.w << 16, v.w & 0xffff0000u};
+      auto put = [&](int k, const uint32_t (&v)[8]) {                  // the upper halves of the words
+        *reinterpret_cast<uint4*>(dst + k * copy + 8 * g) = make_uint4(__byte_perm(v[0], v[1], 0x7632), __byte_perm(v[2], v[3], 0x7632),
+                                                                       __byte_perm(v[4], v[5], 0x7632), __byte_perm(v[6], v[7], 0x7632));
       };
-      if (at_mean >= 0) put(at_mean, w, 16);
-      if (at_halves >= 0) { put(at_halves, hi, 0); put(at_halves + 1, lo, 0); }
-      if (at_sign >= 0) put(at_sign, sg, 0);
+      if (at_mean >= 0) *reinterpret_cast<uint4*>(dst + at_mean * copy + 8 * g) = v;
+      if (at_halves >= 0) {
+        uint32_t hi[8], lo[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const float f = in_halves ? __uint_as_float(w[j]) * scale : 0.f, q = f * f;
+          hi[j] = __float_as_uint(q);
+          lo[j] = __float_as_uint(q - __uint_as_float(hi[j] & 0xffff0000u));      // exact
+        }
+        put(at_halves, hi);
+        put(at_halves + 1, lo);
+      }
+      if (at_sign >= 0) {
+        uint32_t sg[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const float f = __uint_as_float(w[j]);
+          sg[j] = f > 0.f ? 0x3f800000u : f < 0.f ? 0xbf800000u : 0u;
+        }
+        put(at_sign, sg);
+      }
     }
   };
-  write(tx, x, vx, scale_x);
-  write(ty, y, vy, scale_y);
+  write(tx, x, vx, scale_x, px);
+  write(ty, y, vy, scale_y, py);
+  // a product below 2^-149 has a factor below 2^-74
+  if (look && __syncthreads_or(one_token_exponent(px.low_bits()) < -74 || one_token_exponent(py.low_bits()) < -74)) flags = ONE_TOKEN_ODD_SIGN;
+  if (threadIdx.x == 0 && (at_halves >= 0 || at_sign >= 0)) odd[b] = (uint8_t)flags;
 }
 
 }  // namespace pe

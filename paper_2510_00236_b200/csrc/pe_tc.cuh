@@ -149,6 +149,9 @@ struct TcParams {
   int part_chunks;     // PARTS: chunks of rows per part, slices of the square's, the mean's and the sign's chunks
   int part_slices[3];
   unsigned int part_dy, part_x;   // PARTS: the copies of dY and of X that each product takes
+  const uint8_t* odd_rows;        // PARTS: [part_chunks * T] examples whose square (1) or sign (2) the copies do not carry, formed from
+  const uint16_t* rows_dy;        // the operands themselves, [.., d_out] and [.., d_in]
+  const uint16_t* rows_x;
   int per_example;     // 1: reset the accumulator for every example and apply phi (statistics)
                        // 0: one accumulation over the whole slice (plain contraction, phi = identity)
   int half_operands;   // 16-bit operands are IEEE half instead of bf16 (the staged per-token statistic)
@@ -697,6 +700,22 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     float acc_run[N_RUN];           // CHUNKED: the sum of the example's runs so far
 #pragma unroll
     for (int j = 0; j < N_RUN; ++j) acc_run[j] = 0.f;
+    // PARTS: this unit's share of the marked examples, looked up while the first operands are on their way
+    int odd_begin = 0, odd_end = 0;
+    bool any_odd = false;
+    if constexpr (PARTS) {
+      if (which != 1) {
+        const int z = (int)blockIdx.z - (which == 2 ? p.part_slices[0] + p.part_slices[1] : 0), groups = p.part_chunks * p.T / 16;
+        odd_begin = (int)((long long)groups * z / p.part_slices[which]) * 16;
+        odd_end = (int)((long long)groups * (z + 1) / p.part_slices[which]) * 16;
+        uint32_t seen = 0u;
+        for (int r = odd_begin + 16 * lane; r < odd_end; r += 512) {
+          const uint4 v = *reinterpret_cast<const uint4*>(p.odd_rows + r);
+          seen |= v.x | v.y | v.z | v.w;
+        }
+        any_odd = __any_sync(0xffffffffu, (seen & (which == 0 ? 0x01010101u : 0x02020202u)) != 0u);
+      }
+    }
     const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
     for (int a = 0; a < n_acc; ++a) {
       const int buf = (a0 + a) % UNITS;
@@ -962,6 +981,64 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       const TcUnit t = PERSIST ? tc_unit(p, unit) : TcUnit{unit, 0, 0, true};
       whole = t.whole;
       tc_tile_of_pair(p, t.tile, rank, tile_m, tile_n);
+    }
+    if constexpr (PARTS) {
+      // The marked examples, in fp32 as G_b: a row per lane, the columns' entries of X handed round two at a time.  Bound by the exchanges (square)
+      // and by the instructions of a comparison per entry (sign).  Every example marked for both and every piece holding a zero product,
+      // three statistics: 1024 x 1024^2 1075 us (ordinary examples 29; 288 with the kernel that forms every G_b for all), 512 x 4096^2 3364 (159;
+      // 2058).  Both rows have to span more than 2^33 for that (or hold an infinity or NaN).
+      if (ok && any_odd) {
+        const int row = tile_m * TC_TILE_M + q * 32 + lane, col0 = tile_n * NT + h * COLS;
+        // +-1 or 0 as bf16
+        auto sgn = [](uint32_t bits) { return (bits & 0x7fffu) != 0u && (bits & 0x7fffu) <= 0x7f80u ? 0x3f80u | (bits & 0x8000u) : 0u; };
+        auto lowest = [](uint32_t bits) { return (bits & 0x7fffu) != 0u ? (int)(bits & 0x7fffu) : 0x7fff; };
+        for (int r0 = odd_begin; r0 < odd_end; r0 += 32) {
+          unsigned int todo = __ballot_sync(0xffffffffu, r0 + lane < odd_end && (p.odd_rows[r0 + lane] & (which == 0 ? 1 : 2)) != 0);
+          for (; todo != 0u; todo &= todo - 1u) {
+            const long long b = r0 + __ffs((int)todo) - 1;
+            const uint32_t yb = row < p.d_out ? p.rows_dy[b * p.d_out + row] : 0u;
+            const float y = __uint_as_float(yb << 16);
+            const uint16_t* const xb = p.rows_x + b * p.d_in;
+            uint32_t mine[COLS / 64];
+            int low = 0x7fff;
+#pragma unroll
+            for (int c = 0; c < COLS / 64; ++c) {
+              const int col = col0 + 64 * c + 2 * lane;
+              const uint32_t x0 = col < p.d_in ? xb[col] : 0u, x1 = col + 1 < p.d_in ? xb[col + 1] : 0u;
+              mine[c] = x0 | x1 << 16;
+              low = min(low, min(lowest(x0), lowest(x1)));
+            }
+            if (which == 0) {
+#pragma unroll
+              for (int c = 0; c < COLS / 64; ++c) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                  const uint32_t x2 = __shfl_sync(0xffffffffu, mine[c], j);
+                  const int k = 64 * c + 2 * j;
+                  const uint64_t g2 = f32x2_mul(f32x2_pack(__uint_as_float(x2 << 16), __uint_as_float(x2 & 0xffff0000u)), f32x2_pack(y, y));
+                  f32x2_unpack(f32x2_fma(g2, g2, f32x2_pack(acc_mean[k], acc_mean[k + 1])), acc_mean[k], acc_mean[k + 1]);
+                }
+              }
+            } else {
+              // counted by the signs of its factors: taken back where the product is zero, if one of this piece may be
+              const int ex = __reduce_min_sync(0xffffffffu, low) >> 7, ey = __reduce_min_sync(0xffffffffu, lowest(yb)) >> 7;
+              if ((ex > 0 ? ex : -6) + (ey > 0 ? ey : -6) >= 254 - 149) continue;
+              const float sy = __uint_as_float(sgn(yb) << 16);
+#pragma unroll
+              for (int c = 0; c < COLS / 64; ++c) {
+                const uint32_t signs = sgn(mine[c] & 0xffffu) | sgn(mine[c] >> 16) << 16;
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                  const uint32_t x2 = __shfl_sync(0xffffffffu, mine[c], j), s2 = __shfl_sync(0xffffffffu, signs, j);
+                  const int k = 64 * c + 2 * j;
+                  if (__uint_as_float(x2 << 16) * y == 0.f) acc_mean[k] -= __uint_as_float(s2 << 16) * sy;
+                  if (__uint_as_float(x2 & 0xffff0000u) * y == 0.f) acc_mean[k + 1] -= __uint_as_float(s2 & 0xffff0000u) * sy;
+                }
+              }
+            }
+          }
+        }
+      }
     }
     if constexpr (PHI == 2) {
       // sum_b (sign(G_b) + 1) / 2  ->  sum_b sign(G_b)
