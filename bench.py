@@ -596,8 +596,8 @@ def main():
     alg_bytes = 2.0 * B * T * (d_in + d_out)
     specs = [("tc_stats_kernel<mean + square + sign>", "all", peaks["bf16_tflops"], "bf16", alg_bytes + 12.0 * d_in * d_out),
              ("tok_sqstats_kernel", "token", 0.5 * peaks["bf16_tflops"], "tf32", alg_bytes + 4.0 * d_in * d_out)]
-    if st["tok_ws"] is not None:      # two-pass form: three streaming kernels around the half contraction
-        specs[1] = ("pe_token_sqstats_staged: column_max + square_to_half + tc_stats_kernel<identity, half> + unscale", "token_staged",
+    if st["tok_ws"] is not None:      # staged form: one streaming kernel in front of the contraction of the half squares
+        specs[1] = ("pe_token_sqstats_staged: square_chunks + tc_stats_kernel<unscale, half>", "token_staged",
                     peaks["bf16_tflops"], "f16", alg_bytes + 4.0 * d_in * d_out)
     by_kernel = []
     for (kname, key, peak, op_dtype, nbytes), ms in zip(specs, call_ms):

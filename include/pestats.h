@@ -73,7 +73,8 @@ typedef struct CUstream_st* pe_stream_t; /* a cudaStream_t */
  * When the batch is split across thread blocks the outputs are zeroed first and every block adds its
  * partial tile with fp32 reduce-add bulk stores (the SIMT kernel adds up to eight slices in a fixed order
  * and only the sums of more slices with fp32 atomics), so the low bits of out_mean / the square statistic
- * may differ between runs; the sign statistic is always exact-integer valued.
+ * may differ between runs.  On layers of more tiles than fit the chip at once the tiles of the last wave alone may be split so, and added with
+ * fp32 atomics.  The sign statistic is always exact-integer valued.
  */
 pe_status_t pe_linear_stats(const void* X, const void* dY, int B, int T, int d_in, int d_out,
                             pe_phi_t phi, float* out_mean, float* out_stat, pe_stream_t stream);

@@ -242,7 +242,7 @@ static TilePlan plan_tiles(const UnitCost* cand, int n_cand, int B, double T, in
 // CTA pairs at a time, the batch slices one after the other; such a wave streams, for every example of its slice, the dY
 // panels of the pair rows and the X panels of the column tiles it touches, and between two waves the batch has passed
 // through L2.  So the bytes a launch reads from HBM follow the sum over waves of (pair rows x 256 + column tiles x nt):
-// measured on the 8192 x 2048 layer with 256 sequences of 1024 tokens, 18.5 GB with bands of 8 pair rows, which the
+// measured on the 8192 x 2048 layer with 256 sequences of 1024 tokens in five slices, 18.5 GB with bands of 8 pair rows, which the
 // waves cut unevenly there, against 13.0 GB with bands of 1 (the model gives 2.54 and 1.88 times the operands' size).
 // The candidates are walked on the host; the previous default is kept unless another band saves more than 3 %.
 static int choose_band(int pairs_m, int tiles_n, int nt, int nsplit, int slots) {
@@ -1012,9 +1012,10 @@ static PaddedLayout padded_layout(int B, int T, int d_in, int d_out, bool always
   return l;
 }
 // Widths that are no multiples of 8: from this many multiply-adds on, copying the operands to a padded pitch and
-// contracting them on the tensor cores beats the SIMT kernel.  Three launches against one, 20.8 us of host time per call:
-// 4 x 64 x 129 x 255 (2^23) 10.4 us SIMT, 8 x 64 x 257 x 511 (2^26) 24.0, 8 x 256 x 129 x 257 (2^26) 22.7,
-// 16 x 64 x 513 x 511 (2^28) 49.4, 16 x 128 x 513 x 511 (2^29) 87.2.
+// contracting them on the tensor cores beats the SIMT kernel.  Two launches against one, at least 15 us of host and device time per call.
+// SIMT / padded, us: 8 x 64 x 129 x 257 (2^24) 10.4 / 16.4, 8 x 64 x 257 x 255 (2^25) 12.4 / 16.3, 8 x 128 x 129 x 257 (2^25) 14.5 / 15.2,
+// 8 x 64 x 257 x 511 (2^26) 18.6 / 16.5, 32 x 8 x 513 x 511 (2^26) 26.5 / 23.7, 8 x 256 x 129 x 257 (2^26) 22.7 / 15.3, 2 x 2048 x 129 x 255 (2^27)
+// 61.6 / 20.7.  (One width below 16, where the SIMT tile is mostly empty, would gain earlier: 64 x 256 x 1024 x 1 (2^24) 94 / 17.)
 constexpr long long PAD_MIN_MACS = 1ll << 26;
 static bool padding_pays(int B, int T, int d_in, int d_out) {
   return B > 0 && T > 0 && (d_in % 8 || d_out % 8) && tc_shape_ok(B, T, (d_in + 7) & ~7, (d_out + 7) & ~7) &&
@@ -1510,7 +1511,11 @@ struct StagedLayout {
   long long chunks;           // 0: two passes over the inputs
   size_t total() const { return max_bytes + x_bytes + y_bytes; }
 };
-// From this many input elements on (1.2e8: 419 -> 352 us, 1.7e8: 646 -> 557); below it callers take the one-kernel form.
+// From this many input elements on.  The line is where callers begin to prefer a staged form to the one-kernel one; it is not where the
+// one-pass staging begins to win, and a workspace of the two-pass form's size stays enough below it.  One kernel / one-pass / two-pass, us:
+// 16 x 128 x 512 x 2048 (5e6) 19 / 23 / 35, 64 x 256 x 512 x 2048 (4e7) 69 / 68 / 88, 64 x 256 x 1024 x 4096 (8e7) 225 / 154 / 203,
+// 40 x 1000 x 1024 x 1400 (9.7e7) 212 / 171 / 223, 40 x 1000 x 1024 x 1600 (1.05e8) 269 / 190 / 243, 16 x 1024 x 2048 x 8192 (1.7e8) 941 / 491 / 672,
+// 128 x 512 x 512 x 1024 (1.0e8, few tiles) 141 / 151 / 196.
 constexpr double STAGE_CHUNKS_MIN_ELEMS = 1e8;
 static StagedLayout chunked_layout(int B, int T, int d_in, int d_out) {
   StagedLayout l;

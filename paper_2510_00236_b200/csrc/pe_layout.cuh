@@ -1,7 +1,8 @@
 // Layout kernels in front of the tensor-core contraction.  For operands whose rows TMA cannot address (it wants 16-byte
 // row pitches): rows of a width that is no multiple of 8 copied to a padded pitch, and the operands of a convolution's
 // weight gradient (Appendix B.4) unfolded straight into that form.  For the contractions that stand for the statistics of one-token
-// examples: the halves of their squares and their signs.  Streaming kernels, bound by HBM bandwidth; the columns
+// examples: the halves of their squares and their signs.  The padding kernel is bound by HBM bandwidth, the unfolding kernel by its
+// gathers from shared memory (58 MB in 25 us), the one-token kernel by launch latency and HBM.  The columns
 // between the width and the pitch are never read (the tensor maps end at the width).
 #pragma once
 #include <cuda_runtime.h>
@@ -34,7 +35,7 @@ __device__ __forceinline__ void zero_share(const LayoutZero& z, long long first,
 // dst[r, 0..d) = src[r, 0..d): src rows back to back, dst rows `pitch` elements apart (a multiple of 8, at least d).
 // A thread writes 16-byte groups; their eight source elements start at any even byte, so it reads the two aligned 16-byte
 // words around them (the second one is its neighbour's first: an L1 hit) and shifts.  gridDim.y = 1 or 2 picks the tensor.
-// Bound by HBM: each element is read and written once (8 x 256 x 1024 x 32101, the whole call: 8192 -> 271 us, was SIMT).
+// Bound by HBM: each element is read and written once (8 x 256 x 1024 x 32101, the whole call: 8192 -> 240 us, was SIMT).
 struct PadTensor {
   const uint16_t* src;
   uint16_t* dst;

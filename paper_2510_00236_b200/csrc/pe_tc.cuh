@@ -46,7 +46,8 @@
 // PERSIST: layers of more tiles than pairs.  A pair per two SMs takes every (gridDim.x / 2)-th unit: the tensor work of a tile starts
 // while the one before is written out (two accumulators ahead; the write-out goes from registers to memory, past the ring), and
 // prologue and teardown are paid once.  The tiles of the last, partial wave are contracted in slices of the batch, as many
-// as leave every pair one, and added to outputs zeroed beforehand.  Bound by the epilogue (short sequences) or the operand supply as
+// as leave every pair one, and added to outputs zeroed beforehand, in no fixed order (more than two slices: the low bits may differ between
+// runs).  Bound by the epilogue (short sequences) or the operand supply as
 // before.  8 x 256 x 1024 x 32104, both outputs 231 -> 174 us, sign 165 -> 121; 128 x 32 x 4096^2, three statistics 577 -> 497 (474 since);
 // 64 x 256 x 512 x 32768 565 -> 527 (of which the slices 40), sign 477 -> 420; 16 x 1024 x 2048 x 8192, sign 460 -> 405, but
 // sequences of 256 tokens and more gain nothing by the walk alone (64 x 256 x 512 x 16384, three statistics, 321 -> 328 us).
