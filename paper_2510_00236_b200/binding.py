@@ -194,8 +194,7 @@ def pe_linear_stats_padded_workspace_bytes(B, T, d_in, d_out) -> int:
 
 def pe_linear_stats_padded_workspace_bytes_for(B, T, d_in, d_out, phi, want_mean, want_stat, want_sign=False) -> int:
     """What pe_linear_stats_padded asks for with this phi and these outputs."""
-    return int((_lib or load_library()).pe_linear_stats_padded_workspace_bytes_for(B, T, d_in, d_out, _phi(phi), bool(want_mean), bool(want_stat),
-                                                                                   bool(want_sign)))
+    return (_lib or load_library()).pe_linear_stats_padded_workspace_bytes_for(B, T, d_in, d_out, _phi(phi), want_mean, want_stat, want_sign)
 
 
 def _padded(X, dY, B, T, d_in, d_out, phi, accumulate, out_mean, out_stat, out_sign) -> bool:
@@ -211,7 +210,9 @@ def _padded(X, dY, B, T, d_in, d_out, phi, accumulate, out_mean, out_stat, out_s
         workspace = X.new_empty((need,), dtype=torch.uint8)
     except torch.OutOfMemoryError:
         return False
-    pe_linear_stats_padded(X, dY, phi, accumulate, out_mean, out_stat, out_sign, workspace)
+    # (the callers have checked the tensors)
+    _launch("pe_linear_stats_padded", X, X.data_ptr(), dY.data_ptr(), B, T, d_in, d_out, phi, accumulate, _ptr(out_mean), _ptr(out_stat), _ptr(out_sign),
+            workspace.data_ptr(), need)
     return True
 
 
