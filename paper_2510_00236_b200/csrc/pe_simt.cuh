@@ -64,23 +64,22 @@ __device__ __forceinline__ float apply_phi(float g, int phi, float coef) {
   return g;
 }
 
-// Columns c .. c+3 of a row of `width` elements.  vec: a group inside the row is one aligned load.
-__device__ __forceinline__ float4 load_group(const float* row, int c, int width, bool vec) {
-  if (vec && c + 3 < width) return __ldg(reinterpret_cast<const float4*>(row + c));
+// Four elements from p on, `left` of which are inside the row.  whole: all four, as one aligned load.
+__device__ __forceinline__ float4 load_group(const float* p, int left, bool whole) {
+  if (whole) return __ldg(reinterpret_cast<const float4*>(p));
   float v[4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) v[j] = c + j < width ? __ldg(row + c + j) : 0.f;
+  for (int j = 0; j < 4; ++j) v[j] = j < left ? __ldg(p + j) : 0.f;
   return make_float4(v[0], v[1], v[2], v[3]);
 }
-__device__ __forceinline__ float4 load_group(const __nv_bfloat16* row, int c, int width, bool vec) {
+__device__ __forceinline__ float4 load_group(const __nv_bfloat16* p, int left, bool whole) {
   uint32_t w[4];
-  if (vec && c + 3 < width) {
-    const uint2 u = __ldg(reinterpret_cast<const uint2*>(row + c));
+  if (whole) {
+    const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
     w[0] = u.x << 16; w[1] = u.x & 0xFFFF0000u; w[2] = u.y << 16; w[3] = u.y & 0xFFFF0000u;
   } else {
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-      w[j] = c + j < width ? (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(row + c + j)) << 16 : 0u;
+    for (int j = 0; j < 4; ++j) w[j] = j < left ? (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(p) + j) << 16 : 0u;
   }
   return make_float4(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]), __uint_as_float(w[3]));
 }
@@ -184,19 +183,29 @@ simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, 
   }
   if (b < b_end) open_example();
 
+  // A thread's groups of a chunk lie in one column, Y_STEP and X_STEP tokens apart, so that a chunk's addresses take one multiplication per
+  // operand: spelled out per group, their 64-bit multiplications were a fifth of the FMA pipe's work.
+  constexpr int Y_STEP = 4 * SIMT_THREADS / ROWS, X_STEP = 4 * SIMT_THREADS / COLS;
+  static_assert(Y_STEP * ROWS == 4 * SIMT_THREADS && X_STEP * COLS == 4 * SIMT_THREADS, "whole rows of groups per round");
+  const int y_tok = threadIdx.x / (ROWS / 4), x_tok = threadIdx.x / (COLS / 4);
+  const int y_col = o0 + 4 * (threadIdx.x % (ROWS / 4)), x_col = i0 + 4 * (threadIdx.x % (COLS / 4));
+  const bool y_whole = vec_y != 0 && y_col + 3 < d_out, x_whole = vec_x != 0 && x_col + 3 < d_in;
   float4 sy[Tile::YV], sx[Tile::XV];
   auto load_chunk = [&]() {            // zero past the example's end and past the matrix edge
+    const TIn* yp = dY + (row0 + t + y_tok) * (long long)ldy + y_col;
+    const TIn* xp = X + (row0 + t + x_tok) * (long long)ldx + x_col;
+    const int y_left = y_col < d_out ? Tb - t - y_tok : 0, x_left = x_col < d_in ? Tb - t - x_tok : 0;
 #pragma unroll
     for (int k = 0; k < Tile::YV; ++k) {
-      const int v = threadIdx.x + k * SIMT_THREADS, tt = t + v / (ROWS / 4), c = o0 + 4 * (v % (ROWS / 4));
       sy[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (tt < Tb && c < d_out) sy[k] = load_group(dY + (size_t)(row0 + tt) * ldy, c, d_out, vec_y != 0);
+      if (k * Y_STEP < y_left) sy[k] = load_group(yp, d_out - y_col, y_whole);
+      yp += (size_t)Y_STEP * ldy;
     }
 #pragma unroll
     for (int k = 0; k < Tile::XV; ++k) {
-      const int v = threadIdx.x + k * SIMT_THREADS, tt = t + v / (COLS / 4), c = i0 + 4 * (v % (COLS / 4));
       sx[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (tt < Tb && c < d_in) sx[k] = load_group(X + (size_t)(row0 + tt) * ldx, c, d_in, vec_x != 0);
+      if (k * X_STEP < x_left) sx[k] = load_group(xp, d_in - x_col, x_whole);
+      xp += (size_t)X_STEP * ldx;
     }
   };
   auto put = [&](float* at, float4 v) {
