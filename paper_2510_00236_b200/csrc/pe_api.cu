@@ -18,6 +18,7 @@
 #include "pe_layout.cuh"
 #include "pe_optim.cuh"
 #include "pe_stage.cuh"
+#include "pe_short.cuh"
 #include "pe_simt.cuh"
 #include "pe_tc.cuh"
 #include "pe_tok.cuh"
@@ -179,10 +180,8 @@ constexpr UnitCost COST_TOKEN = {TOK_NT, 0.42 / TOK_BK, 0.45 / TOK_BK, 0.0, 0.0,
 constexpr UnitCost COST_PLAIN_FP8 = {256, 0.28 / 128, 0.40 / 128, 0.0, 0.0, 8.5};
 constexpr UnitCost COST_BOTH_192 = {192, 0.375 / 128, 0.55 / 128, 0.02, 0.35, 10.0};     // two sums
 constexpr UnitCost COST_BOTH_128 = {128, 0.35 / 128, 0.44 / 128, 0.12, 0.20, 8.3};
-constexpr UnitCost COST_BOTH_SHORT = {128, 0.05 / 32, 0.10 / 32, 0.0, 0.245, 8.3};       // two examples per stage (T <= 32)
 constexpr UnitCost COST_ALL_192 = {192, 0.375 / 128, 0.60 / 128, 0.05, 0.95, 11.0};      // three statistics
 constexpr UnitCost COST_ALL_128 = {128, 0.35 / 128, 0.44 / 128, 0.16, 0.55, 9.5};
-constexpr UnitCost COST_ALL_SHORT = {128, 0.05 / 32, 0.10 / 32, 0.0, 0.54, 9.5};
 
 // One pair per two SMs that walks over the tiles (PERSIST) instead of a pair per tile.  It saves the prologue and the teardown, and
 // tensor work of the next tile overlaps the write-out.  What is lost: pairs that run faster cannot take more tiles (64 x 256 x 512 x 16384,
@@ -358,6 +357,94 @@ static pe_status_t launch_tc_tiles(DeviceInfo* di, int slot, bool persist, const
 using LayoutStep = std::function<pe_status_t(const LayoutZero&)>;
 static bool any_output(const LayoutZero& z) { return z.out[0] || z.out[1] || z.out[2]; }
 
+// Statistics of short sequences (T <= SHORT_T).  out_mean, out_square, out_sign: those wanted; out_mean and out_sign with or without
+// out_square, out_square with or without out_mean.
+struct ShortCost {
+  double example, fixed, add;      // us per example of a tile, per tile, more for a tile whose sums are added
+};
+static ShortCost short_cost(bool mean, bool square, bool sign) {
+  if (mean && square && sign) return {0.45, 2.2, 3.2};
+  if (mean && sign) return {0.345, 1.5, 2.3};
+  if (mean) return {0.19, 1.5, 2.3};
+  return sign ? ShortCost{0.28, 1.0, 1.5} : ShortCost{0.155, 1.0, 1.5};
+}
+static pe_status_t launch_short(DeviceInfo* di, const void* X, const void* dY, int B, int T, int d_in, int d_out, float* out_mean, float* out_square,
+                                float* out_sign, cudaStream_t st, bool accumulate, int pitch_x, int pitch_y, const LayoutStep& before) {
+  CUtensorMap mx, my;
+  pe_status_t rc = make_operand_map(&mx, X, B, T, d_in, false, 64, SHORT_T, false, SHORT_G, pitch_x);
+  if (rc == PE_OK) rc = make_operand_map(&my, dY, B, T, d_out, false, 64, SHORT_T, false, SHORT_G, pitch_y);
+  if (rc != PE_OK) return rc;
+  const int tiles_n = (d_in + SHORT_NT - 1) / SHORT_NT, pairs_m = (d_out + TC_PAIR_M - 1) / TC_PAIR_M;
+  if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
+  const long long tiles = (long long)tiles_n * pairs_m;
+  const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
+  // Every pair takes whole tiles in turn; the tiles of a last partial wave, or all of them where that is cheaper, go to several
+  // pairs each, by slices of the batch.
+  const ShortCost c = short_cost(out_mean, out_square, out_sign);
+  int whole = 0, split = 1;
+  double best = 1e300;
+  for (int pass = 0; pass < 2; ++pass) {
+    const long long w = pass == 0 ? 0 : tiles - tiles % slots, rest = tiles - w;
+    if (pass == 1 && (w == 0 || rest == 0)) break;
+    for (int k = 1; k <= B && k <= 4 * slots && (k == 1 || rest * (k - 1) < 16ll * slots); ++k) {
+      const double per = (double)((B + k - 1) / k);
+      const bool add = k > 1 || accumulate;
+      const double us = (double)(w / slots) * (B * c.example + c.fixed) +
+                        (double)((rest * k + slots - 1) / slots) * (per * c.example + c.fixed + (add ? c.add : 0.0)) + (add && !accumulate ? 2.0 : 0.0);
+      if (per <= TC_SIGN_COUNT_MAX && us < best * 0.995) { best = us; whole = (int)(k == 1 ? tiles : w); split = k; }
+    }
+  }
+  if (best == 1e300) { whole = 0; split = (B + TC_SIGN_COUNT_MAX - 1) / TC_SIGN_COUNT_MAX; }
+  TcParams p{};
+  p.B = B; p.T = T; p.d_in = d_in; p.d_out = d_out; p.accumulate = accumulate ? 1 : 0;
+  p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, SHORT_NT, whole == 0 ? split : 1, slots);
+  p.whole_tiles = whole; p.tail_split = split;
+  p.scalar_out = d_in % 4 != 0 ? 1 : 0;
+  CUtensorMap mm = mx, msq = mx, msgn = mx;           // an output that is not wanted gets a map that is never used
+  if (!p.scalar_out) {
+    if (out_mean) rc = make_output_map(&mm, out_mean, d_in, d_out);
+    if (rc == PE_OK && out_square) rc = make_output_map(&msq, out_square, d_in, d_out);
+    if (rc == PE_OK && out_sign) rc = make_output_map(&msgn, out_sign, d_in, d_out);
+    if (rc != PE_OK) return rc;
+  }
+  p.out_mean = out_mean; p.out_stat = out_square; p.out_sign = out_sign; p.dev_status = di->status_ptr;
+  const bool to_zero = split > 1 && !accumulate;
+  p.wait_at_start = !to_zero || before ? 1 : 0;
+  if (before) {
+    LayoutZero zero = {{nullptr, nullptr, nullptr}, (long long)d_in * d_out};
+    if (to_zero) { zero.out[0] = out_mean; zero.out[1] = out_square; zero.out[2] = out_sign; }
+    rc = before(zero);
+  } else if (to_zero && whole > 0) {
+    zero_tail_tiles_kernel<<<di->sm_count, 256, 0, st>>>(p, SHORT_NT);
+    rc = check_launch();
+  } else if (to_zero) {
+    float* const outs[3] = {out_mean, out_square, out_sign};
+    float* list[3] = {nullptr, nullptr, nullptr};
+    int n = 0;
+    for (float* o : outs)
+      if (o) list[n++] = o;
+    rc = zero_for_split(di, list[0], list[1], (size_t)d_in * d_out, st, list[2]);
+  }
+  if (rc != PE_OK) return rc;
+  const long long units = whole + (tiles - whole) * split;
+  const dim3 grid((unsigned)(2 * std::min<long long>(slots, units)));
+  auto run = [&](auto kernel, int slot) {
+    {
+      std::lock_guard<std::mutex> lock(g_dev_mutex);
+      if (!di->tc_attr_set[slot]) {
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SHORT_SMEM_BYTES) != cudaSuccess) { cudaGetLastError(); return PE_ERR_CUDA; }
+        di->tc_attr_set[slot] = true;
+      }
+    }
+    return launch_dependent(kernel, grid, TC_THREADS, SHORT_SMEM_BYTES, st, mx, my, mm, msq, msgn, p);
+  };
+  if (out_sign && out_mean && out_square) return run(short_stats_kernel<true, true, true>, 8);
+  if (out_sign && out_mean) return run(short_stats_kernel<true, false, true>, 9);
+  if (out_sign) return run(short_stats_kernel<false, false, true>, 27);
+  if (out_mean) return run(short_stats_kernel<true, true, false>, 40);
+  return run(short_stats_kernel<false, true, false>, 41);
+}
+
 // Tensor-core launch.  per_example = 0 runs the plain contraction over all B*T rows (its result goes
 // to whichever of out_mean / out_stat is not NULL).  With per_example = 1 and both outputs wanted the
 // pair tile is 256 x 128 (two running sums per thread); with only out_stat it is 256 x 256.
@@ -370,17 +457,18 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
   const bool both = per_example && ((out_mean && out_stat) || chunked);
   const bool runs = chunked && T > TC_CHUNK_TOKENS;     // several accumulators per example
   const int forced = g_path.load();
+  if (per_example && T <= SHORT_T && forced != PE_PATH_TENSOR_WIDE && (phi == PE_PHI_SQUARE || phi == PE_PHI_SIGN))
+    return launch_short(di, X, dY, B, T, d_in, d_out, out_mean, phi == PE_PHI_SQUARE ? out_stat : nullptr, phi == PE_PHI_SIGN ? out_stat : out_sign, st,
+                        accumulate, pitch_x, pitch_y, before);
   const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1, max_split = std::max(16, slots);
   // Tile and batch slices by estimated time.  Both outputs: 256 x 192 or 256 x 128 (22 % more operand traffic per flop, but
-  // less padding and more even waves on some layers: 64 x 256 x 512 x 32768 528 us against 497); T <= 32: 256 x 128 with two
-  // examples per stage.
+  // less padding and more even waves on some layers: 64 x 256 x 512 x 32768 528 us against 497).
   UnitCost cand[2];
   int n_cand = 0;
   bool cand_wide[2] = {false, false};
   if (both) {
-    const bool short_t = T <= TC_SHORT_T;
-    if (forced != PE_PATH_TENSOR_NARROW && !runs && (!short_t || forced == PE_PATH_TENSOR_WIDE)) { cand_wide[n_cand] = true; cand[n_cand++] = triple ? COST_ALL_192 : COST_BOTH_192; }
-    if (forced != PE_PATH_TENSOR_WIDE || n_cand == 0) cand[n_cand++] = short_t ? (triple ? COST_ALL_SHORT : COST_BOTH_SHORT) : (triple ? COST_ALL_128 : COST_BOTH_128);
+    if (forced != PE_PATH_TENSOR_NARROW && !runs) { cand_wide[n_cand] = true; cand[n_cand++] = triple ? COST_ALL_192 : COST_BOTH_192; }
+    if (forced != PE_PATH_TENSOR_WIDE || n_cand == 0) cand[n_cand++] = triple ? COST_ALL_128 : COST_BOTH_128;
   } else {
     cand[n_cand++] = !per_example ? COST_PLAIN : phi == PE_PHI_SIGN ? COST_SIGN : COST_STAT;
   }
@@ -396,15 +484,12 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
   const bool mean_regs = both && !mean_tmem;
   const int nt = mean_regs ? (wide ? 192 : 128) : 256;
   const int box_feats = TcOperand<false, 256>::BOX_FEATS;
-  const bool short_seq = mean_regs && !wide && T <= TC_SHORT_T;      // many short examples, both sums in registers: small stages
-  const int box_tokens = short_seq ? TC_SHORT_BK : tc_default_bk(false, nt);
+  const int box_tokens = tc_default_bk(false, nt);
   CUtensorMap mx, my;
-  // short sequences: a box is two examples deep (a stage holds two examples of 32 tokens each)
-  const int box_examples = short_seq ? TcOperand<false, 128, TC_SHORT_BK>::GROUP : 1;
   pe_status_t rc = wide ? make_operand_map(&mx, X, B, T, d_in, false, TcOperand<false, 192>::B_BOX_FEATS, box_tokens, true, 1, pitch_x)
-                        : make_operand_map(&mx, X, B, T, d_in, false, box_feats, box_tokens, false, box_examples, pitch_x);
+                        : make_operand_map(&mx, X, B, T, d_in, false, box_feats, box_tokens, false, 1, pitch_x);
   if (rc != PE_OK) return rc;
-  rc = make_operand_map(&my, dY, B, T, d_out, false, box_feats, box_tokens, false, box_examples, pitch_y);
+  rc = make_operand_map(&my, dY, B, T, d_out, false, box_feats, box_tokens, false, 1, pitch_y);
   if (rc != PE_OK) return rc;
   // an output that is not wanted gets the other one's map and is never used; rows that are no 16-byte multiples cannot be
   // described by a map at all and are written without one (scalar_out)
@@ -455,13 +540,8 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
     return launch_tc_tiles<2, 128, MEAN_REGS, 128, true>(di, 29, persist, mx, my, mm, ms, msgn, p, grid, st);
   }
   if (triple && wide) return launch_tc_tiles<1, 192, MEAN_HYBRID_SIGN>(di, 26, persist, mx, my, mm, ms, msgn, p, grid, st);
-  if (triple && short_seq) return launch_tc_tiles<1, 128, MEAN_REGS_SIGN, TC_SHORT_BK>(di, 27, persist, mx, my, mm, ms, msgn, p, grid, st);
   if (triple) return launch_tc_tiles<1, 128, MEAN_REGS_SIGN>(di, 10, persist, mx, my, mm, ms, msgn, p, grid, st);
   if (!per_example) return launch_tc_inst<0, false, 256, MEAN_NONE>(di, 4, mx, my, mm, ms, msgn, p, grid, st);
-  if (short_seq) {
-    if (phi == PE_PHI_SQUARE) return launch_tc_tiles<1, 128, MEAN_REGS, TC_SHORT_BK>(di, 8, persist, mx, my, mm, ms, msgn, p, grid, st);
-    return launch_tc_tiles<2, 128, MEAN_REGS, TC_SHORT_BK>(di, 9, persist, mx, my, mm, ms, msgn, p, grid, st);
-  }
   if (wide) {
     if (phi == PE_PHI_SQUARE) return launch_tc_tiles<1, 192, MEAN_REGS>(di, 12, persist, mx, my, mm, ms, msgn, p, grid, st);
     return launch_tc_tiles<2, 192, MEAN_REGS>(di, 13, persist, mx, my, mm, ms, msgn, p, grid, st);

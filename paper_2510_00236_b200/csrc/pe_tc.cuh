@@ -11,7 +11,7 @@
 // 128 x 128 tile would need 128 B/clk at full tensor rate, a 256 x 128 pair 96, a 256 x 192 pair 75, a
 // 256 x 256 pair 64.
 //
-//   MEAN_REGS, NT = 128: two running sums per thread (64 + 64 registers)         -- both outputs, short sequences
+//   MEAN_REGS, NT = 128: two running sums per thread (64 + 64 registers)         -- both outputs
 //   MEAN_REGS, NT = 192: two running sums per thread (96 + 96 registers; the control
 //                        warps shrink to 40 registers so that the epilogue warps can take 232) -- both outputs
 //   MEAN_REGS_SIGN, NT = 128: the same plus sum_b sign(G_b), counted in 16-bit halves
@@ -84,11 +84,8 @@ __host__ __device__ constexpr int tc_smem_budget(int nt) { return (nt == 192 ? 2
 // statistics; tf32 (kind::tf32, fp32 storage, 8 tokens per instruction) for the per-token statistic,
 // whose squared operands need more than bf16's 8 significant bits.  NT = d_in columns per pair tile.
 // Default tokens per pipeline stage: 128 for the 256 x 128 tile, 64 for the 256 x 256 tile, 32 for
-// tf32.  With both outputs and short sequences (T <= 32) the 256 x 128 tile takes 32-token stages
-// instead: a 128-token box would be mostly zero fill, and 16 small slots keep more examples in flight.
+// tf32.  (The statistics of sequences of at most 32 tokens have a kernel of their own, pe_short.cuh.)
 __host__ __device__ constexpr int tc_default_bk(bool tf32, int nt) { return tf32 ? 32 : (nt == 256 ? 64 : 128); }
-constexpr int TC_SHORT_BK = 32;
-constexpr int TC_SHORT_T = 32;
 constexpr int TC_CHUNK_TOKENS = 512;    // CHUNKED: tokens per accumulator
 // F8: 8-bit operands (kind::f8f6f4, e4m3, 32 tokens per instruction): the scaled squares of the two-pass
 // per-token statistic's fp8 form.
@@ -100,11 +97,7 @@ struct TcOperand {
   // tokens per pipeline stage (one TMA box is BK tokens tall)
   static constexpr int BK = BK_;
   static constexpr int MMA_K = 32 / ELEM_BYTES;                 // tokens per MMA instruction: 16 | 8 | 32
-  // Short sequences (the 32-token stages of the 256 x 128 tile): a stage holds TWO examples (the TMA box is
-  // two examples deep, 32 tokens each), the issuer fills both of its accumulators from it and the epilogue
-  // drains both behind one barrier: half the barrier hand-offs per example, which is what bounds T <= 32.
-  static constexpr int GROUP = (!TF32 && !F8 && NT == 128 && BK_ == TC_SHORT_BK) ? 2 : 1;
-  static constexpr int BOX_BYTES = 128 * BK * GROUP;            // one box: GROUP x BK tokens x 128 bytes
+  static constexpr int BOX_BYTES = 128 * BK;                    // one box: BK tokens x 128 bytes
   static constexpr int A_BOXES = TC_TILE_M / BOX_FEATS;         // this block's 128 rows of dY^T
   static constexpr int B_FEATS = NT / 2;                        // this block's half of the tile's d_in columns
   // NT = 192: 96 columns of X per block are one and a half 128-byte rows.  X is then loaded in
@@ -114,12 +107,12 @@ struct TcOperand {
   static_assert(!B_NARROW || !TF32, "64-byte rows are only set up for 16-bit operands");
   static constexpr int B_ROW_BYTES = B_NARROW ? 64 : 128;
   static constexpr int B_BOX_FEATS = B_ROW_BYTES / ELEM_BYTES;  // 64 | 32
-  static constexpr int B_BOX_BYTES = B_ROW_BYTES * BK * GROUP;
+  static constexpr int B_BOX_BYTES = B_ROW_BYTES * BK;
   static constexpr int B_BOXES = B_FEATS / B_BOX_FEATS;         // 1 | 2 | 3
   static constexpr int A_BYTES = A_BOXES * BOX_BYTES;           // 32 KiB (BK = 128) | 16 KiB
   static constexpr int B_BYTES = B_BOXES * B_BOX_BYTES;         // 16 KiB | 24 KiB (NT = 192)
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;         // per block: 48 KiB | 56 KiB | 32 KiB
-  static constexpr int STAGES = tc_smem_budget(NT) / STAGE_BYTES;   // 4 | 4 | 6 | 8 with the grouped 32-token stages
+  static constexpr int STAGES = tc_smem_budget(NT) / STAGE_BYTES;   // 4 | 4 | 6
   static constexpr int K_STEP_BYTES = MMA_K * 128;              // smem advance per MMA: 2048 | 1024
   static constexpr int B_K_STEP_BYTES = MMA_K * B_ROW_BYTES;
   static constexpr int ACC_BUFS = TC_TMEM_COLS / NT;            // 4 | 2 | 2 accumulators in tensor memory
@@ -274,14 +267,6 @@ __device__ __forceinline__ uint64_t sign_half2(uint64_t g2) {
 __device__ __forceinline__ uint32_t sign_plus_one_packed(uint64_t g2) {
   float t0, t1;
   sm100::f32x2_unpack(sm100::f32x2_fma(sign_half2(g2), sm100::f32x2_pack(2.f, 2.f), sm100::f32x2_pack(12582912.f, 12582912.f)), t0, t1);
-  return __byte_perm(__float_as_uint(t0), __float_as_uint(t1), 0x5410);
-}
-
-// The same for the sum over two examples, sign + sign + 2 in {0 .. 4}: the saturated halves are added before the integer is
-// extracted (1.5 * 2^22 has steps of 0.5).
-__device__ __forceinline__ uint32_t signs_plus_two_packed(uint64_t g2, uint64_t h2) {
-  float t0, t1;
-  sm100::f32x2_unpack(sm100::f32x2_add(sm100::f32x2_add(sign_half2(g2), sm100::f32x2_pack(6291456.f, 6291456.f)), sign_half2(h2)), t0, t1);
   return __byte_perm(__float_as_uint(t0), __float_as_uint(t1), 0x5410);
 }
 
@@ -452,7 +437,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   static_assert(MEAN != MEAN_TMEM || (NT == 256 && PHI != 0), "the tensor-memory mean sits beside one 256-column accumulator");
   static_assert(!RAGGED || (!TF32 && MEAN != MEAN_TMEM), "packed batches: 16-bit operands, several accumulators");
   static_assert((PHI != 3 && PHI != 4) || MEAN == MEAN_NONE, "the clipped sum and the scaled contraction are statistic-only passes");
-  static_assert(!CHUNKED || (MEAN == MEAN_REGS && NT == 128 && !RAGGED && OPT == OPT_NONE && Op::GROUP == 1), "runs of an example: the two-sum kernel on the 256 x 128 tile");
+  static_assert(!CHUNKED || (MEAN == MEAN_REGS && NT == 128 && !RAGGED && OPT == OPT_NONE), "runs of an example: the two-sum kernel on the 256 x 128 tile");
   static_assert(!PARTS || (PHI == 0 && !TF32 && !F8 && !RAGGED && !PERSIST && OPT == OPT_NONE), "the statistics of one-token examples are plain contractions");
   static_assert(!PERSIST || (!RAGGED && OPT == OPT_NONE && MEAN != MEAN_TMEM && !NORMS && PHI != 0), "several tiles per pair: fixed-length batches, whole sums written");
   constexpr int CHUNK_STAGES = CHUNKED ? TC_CHUNK_TOKENS / BKT : 1;
@@ -463,12 +448,6 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   constexpr int STAGES = Op::STAGES, BK = Op::BK;
   constexpr int BOX_BYTES = Op::BOX_BYTES, A_BYTES = Op::A_BYTES, STAGE_BYTES = Op::STAGE_BYTES;
   constexpr int ACC_BUFS = (MEAN == MEAN_TMEM) ? 1 : Op::ACC_BUFS;
-  // GROUP examples share a stage and a pair of accumulator barriers (short sequences): the unit of work of
-  // the producers, the issuer and the epilogue warps is then a group of GROUP consecutive examples
-  constexpr int GROUP = Op::GROUP;
-  constexpr int UNITS = ACC_BUFS / GROUP;            // accumulator units (of GROUP buffers, one barrier pair each)
-  static_assert(GROUP == 1 || ((MEAN == MEAN_REGS || MEAN == MEAN_REGS_SIGN) && !RAGGED && OPT == OPT_NONE),
-                "grouped examples: the short-sequence variants of the two- and three-sum kernels");
   constexpr int MEAN_COL0 = 256;                    // first tensor-memory column of the MEAN_TMEM running sum
   constexpr int COLS = NT / 2;                      // accumulator columns per epilogue thread
   extern __shared__ uint8_t smem_raw[];
@@ -506,7 +485,6 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   }
   int nb = b_end - b_begin;
   const int n_units = PERSIST ? tc_units(p) : 1;      // PERSIST: this pair takes every (gridDim.x / 2)-th of them
-  int nu = (nb + GROUP - 1) / GROUP;          // units of work: groups of GROUP examples (GROUP = 1: the examples)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
@@ -557,14 +535,14 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         int tile_m, tile_n;
         if (PERSIST) {
           const TcUnit t = tc_unit(p, unit);
-          b_begin = t.b_begin; b_end = t.b_end; nb = b_end - b_begin; nu = (nb + GROUP - 1) / GROUP;
+          b_begin = t.b_begin; b_end = t.b_end; nb = b_end - b_begin;
           tc_tile_of_pair(p, t.tile, rank, tile_m, tile_n);
         } else {
           tc_tile_of_pair(p, unit, rank, tile_m, tile_n);
         }
         const int c0 = is_a ? tile_m * TC_TILE_M : tile_n * NT + (int)rank * Op::B_FEATS;   // first feature of this warp's boxes
-        for (int e = 0; e < nu && ok; ++e) {
-          const SeqGeom g = seq_geom<RAGGED>(p, b_begin + GROUP * e, BK);
+        for (int e = 0; e < nb && ok; ++e) {
+          const SeqGeom g = seq_geom<RAGGED>(p, b_begin + e, BK);
           for (int kc = 0; kc < g.nk; ++kc) {
             if (!mbar_wait_warp(empty_bar(s), ph, abort_flag, p.dev_status, TC_WAIT_EMPTY, strict)) { ok = false; break; }
             if (elect_one()) {
@@ -575,8 +553,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
               if (tail && !side_ready) griddep_wait();
               const CUtensorMap* tm = tail ? tmap_tail : tmap;
               const int c1 = tail ? 0 : g.row0 + kc * BK;
-              // (grouped examples: the box is GROUP examples deep; past the batch's end it reads zeros)
-              const int c2 = PARTS ? tc_part_chunk(p, b_begin + e, is_a) : RAGGED ? (tail ? b_begin + e : 0) : b_begin + GROUP * e;
+              const int c2 = PARTS ? tc_part_chunk(p, b_begin + e, is_a) : RAGGED ? (tail ? b_begin + e : 0) : b_begin + e;
               for (int b = 0; b < n_boxes; ++b) tma_load_3d_pair(dst + b * box_bytes, tm, leader_full, c0 + b * box_feats, c1, c2);
             }
             __syncwarp();
@@ -587,7 +564,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       } while (PERSIST && ok && (unit += gridDim.x >> 1) < n_units);
     } else if (rank == 0 && warp == 1) {
       // ---------------------------------------------------------- MMA issuer (leader block)
-      // Unit e (an example, or GROUP of them) goes to accumulator unit e % UNITS.  A plain contraction (per_example == 0)
+      // Example e goes to accumulator e % ACC_BUFS.  A plain contraction (per_example == 0)
       // alternates the same way but resets each accumulator only once, and the epilogue adds them up.
       // operand format code 0 is IEEE half under kind::f16 and e4m3 under kind::f8f6f4
       const uint32_t idesc = (F8 || (!TF32 && p.half_operands)) ? make_idesc_half_mn_major(TC_PAIR_M, NT) : make_idesc_mn_major(TC_PAIR_M, NT, TF32);
@@ -599,27 +576,27 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       do {
         if (PERSIST) {
           const TcUnit t = tc_unit(p, unit);
-          b_begin = t.b_begin; b_end = t.b_end; nb = b_end - b_begin; nu = (nb + GROUP - 1) / GROUP;
+          b_begin = t.b_begin; b_end = t.b_end; nb = b_end - b_begin;
         }
-        for (int e = 0; e < nu && ok; ++e) {
-          const SeqGeom sg = seq_geom<RAGGED>(p, b_begin + GROUP * e, BK);
-          int buf = (PERSIST ? run : e) % UNITS;
+        for (int e = 0; e < nb && ok; ++e) {
+          const SeqGeom sg = seq_geom<RAGGED>(p, b_begin + e, BK);
+          int buf = (PERSIST ? run : e) % ACC_BUFS;
           if (p.per_example && !CHUNKED) {
-            if (!mbar_wait_warp(acc_empty_bar(buf), ((uint32_t)((PERSIST ? run : e) / UNITS) & 1u) ^ 1u, abort_flag, p.dev_status, TC_WAIT_ACC_EMPTY, strict)) { ok = false; break; }
+            if (!mbar_wait_warp(acc_empty_bar(buf), ((uint32_t)((PERSIST ? run : e) / ACC_BUFS) & 1u) ^ 1u, abort_flag, p.dev_status, TC_WAIT_ACC_EMPTY, strict)) { ok = false; break; }
             tc_fence_after();
             if (PERSIST) ++run;
           }
-          const bool last_of_acc = p.per_example || e + UNITS >= nu;
+          const bool last_of_acc = p.per_example || e + ACC_BUFS >= nb;
           for (int kc = 0; kc < sg.nk; ++kc) {
             const int kin = CHUNKED ? kc % CHUNK_STAGES : kc;           // stage within its accumulator
             const bool acc_done = kc == sg.nk - 1 || (CHUNKED && kin == CHUNK_STAGES - 1);
             if (CHUNKED && kin == 0) {
-              buf = run % UNITS;
-              if (!mbar_wait_warp(acc_empty_bar(buf), ((uint32_t)(run / UNITS) & 1u) ^ 1u, abort_flag, p.dev_status, TC_WAIT_ACC_EMPTY, strict)) { ok = false; break; }
+              buf = run % ACC_BUFS;
+              if (!mbar_wait_warp(acc_empty_bar(buf), ((uint32_t)(run / ACC_BUFS) & 1u) ^ 1u, abort_flag, p.dev_status, TC_WAIT_ACC_EMPTY, strict)) { ok = false; break; }
               tc_fence_after();
               ++run;
             }
-            const uint32_t d_tmem = tmem_base + (uint32_t)(buf * GROUP * NT);
+            const uint32_t d_tmem = tmem_base + (uint32_t)(buf * NT);
             if (!mbar_wait_warp(full_bar(s), ph, abort_flag, p.dev_status, TC_WAIT_FULL, strict)) { ok = false; break; }
             tc_fence_after();
             if (elect_one()) {
@@ -627,21 +604,15 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
               const uint32_t b_src = a_src + A_BYTES;
               // tokens of this example in this stage: the rest of its whole 16-token groups, or the padded tail group
               const int t_left = (RAGGED && kc >= sg.nk_main) ? 16 : sg.main - kc * BK;
+              uint32_t accumulate = (kin > 0 || (!p.per_example && e >= ACC_BUFS)) ? 1u : 0u;
 #pragma unroll
-              for (int j = 0; j < GROUP; ++j) {
-                // grouped examples: example j of the group sits BK tokens further in every box and has its own accumulator
-                if (GROUP > 1 && GROUP * e + j >= nb) break;
-                uint32_t accumulate = (kin > 0 || (!p.per_example && e >= UNITS)) ? 1u : 0u;
-#pragma unroll
-                for (int k = 0; k < BK / Op::MMA_K; ++k) {
-                  // rows past T are zero-filled by TMA; whole MMA steps past T are skipped
-                  if (k * Op::MMA_K < t_left) {
-                    const uint64_t ad = make_smem_desc(a_src + j * (BK * 128) + k * Op::K_STEP_BYTES, BOX_BYTES, Op::SBO_BYTES, Op::DESC_LAYOUT);
-                    const uint64_t bd = make_smem_desc(b_src + j * (BK * Op::B_ROW_BYTES) + k * Op::B_K_STEP_BYTES, Op::B_BOX_BYTES, Op::B_SBO_BYTES,
-                                                       Op::B_DESC_LAYOUT);
-                    umma_ss_pair<TF32 ? 1 : (F8 ? 2 : 0)>(d_tmem + (uint32_t)(j * NT), ad, bd, idesc, accumulate);
-                    accumulate = 1;
-                  }
+              for (int k = 0; k < BK / Op::MMA_K; ++k) {
+                // rows past T are zero-filled by TMA; whole MMA steps past T are skipped
+                if (k * Op::MMA_K < t_left) {
+                  const uint64_t ad = make_smem_desc(a_src + k * Op::K_STEP_BYTES, BOX_BYTES, Op::SBO_BYTES, Op::DESC_LAYOUT);
+                  const uint64_t bd = make_smem_desc(b_src + k * Op::B_K_STEP_BYTES, Op::B_BOX_BYTES, Op::B_SBO_BYTES, Op::B_DESC_LAYOUT);
+                  umma_ss_pair<TF32 ? 1 : (F8 ? 2 : 0)>(d_tmem, ad, bd, idesc, accumulate);
+                  accumulate = 1;
                 }
               }
               umma_commit_pair(empty_bar(s));                // stage reusable in both blocks once these MMAs retire
@@ -686,7 +657,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     bool whole = true;
     if (PERSIST) {
       const TcUnit t = tc_unit(p, unit);
-      b_begin = t.b_begin; b_end = t.b_end; nb = b_end - b_begin; nu = (nb + GROUP - 1) / GROUP;
+      b_begin = t.b_begin; b_end = t.b_end; nb = b_end - b_begin;
       if constexpr (TILE_FIRST) {
         whole = t.whole;
         tc_tile_of_pair(p, t.tile, rank, tile_m, tile_n);
@@ -694,9 +665,9 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     } else if constexpr (TILE_FIRST) {
       tc_tile_of_pair(p, unit, rank, tile_m, tile_n);
     }
-    // per-example mode: one accumulator unit per example (or group), in order; plain mode: each accumulator once
+    // per-example mode: one accumulator per example, in order; plain mode: each accumulator once
     const int n_runs = CHUNKED ? (p.T + TC_CHUNK_TOKENS - 1) / TC_CHUNK_TOKENS : 1;      // accumulators per example
-    const int n_acc = p.per_example ? nu * n_runs : min(nu, UNITS);
+    const int n_acc = p.per_example ? nb * n_runs : min(nb, ACC_BUFS);
     constexpr int N_RUN = CHUNKED ? COLS : 1;
     float acc_run[N_RUN];           // CHUNKED: the sum of the example's runs so far
 #pragma unroll
@@ -719,8 +690,8 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     }
     const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
     for (int a = 0; a < n_acc; ++a) {
-      const int buf = (a0 + a) % UNITS;
-      const uint32_t acc_ph = (uint32_t)((a0 + a) / UNITS) & 1u;
+      const int buf = (a0 + a) % ACC_BUFS;
+      const uint32_t acc_ph = (uint32_t)((a0 + a) / ACC_BUFS) & 1u;
       // PHI == 3: this example's clipping coefficient c_b = min(1, C / sqrt(N_b)); the load is issued before
       // the wait for the accumulator, which hides its latency.  N_b = 0 (a zero gradient) gives 1.
       uint64_t coef2 = 0;
@@ -740,7 +711,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       // instructions, so no lane may leave the loop alone when its own wait is the one that gives up
       if (!mbar_wait_warp(acc_full_bar(buf), acc_ph, abort_flag, p.dev_status, TC_WAIT_ACC_FULL)) { ok = false; break; }
       tc_fence_after();
-      const uint32_t taddr = lane_base + (uint32_t)(buf * GROUP * NT + h * COLS);
+      const uint32_t taddr = lane_base + (uint32_t)(buf * NT + h * COLS);
       if constexpr (MEAN == MEAN_TMEM) {
         // sum_b G_b lives in tensor-memory columns MEAN_COL0.. of the same lanes: read it with G_b,
         // add, write it back (the first example just writes G_b).
@@ -833,8 +804,6 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         // statistics on the 256 x 128 tile, whose 160 registers of sums leave room for two reads of 16 in flight, not 32)
         constexpr int CH = (NT == 192 || TRIPLE || CHUNKED) ? 16 : 32;
         constexpr int NCH = COLS / CH;                // reads per example
-        // grouped examples: the unit's accumulators one after the other; the unit is released after the last read
-        const int in_unit = (GROUP > 1) ? min(GROUP, nb - GROUP * a) : 1;
         // phi and the running sums for one read of CH columns (chunk c of this thread's COLS columns)
         float4 col_scale[PHI == 4 ? CH / 4 : 1];
         auto fold = [&](const uint32_t (&r)[CH], int c) {
@@ -875,7 +844,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
             }
           }
         };
-        auto release_unit = [&]() {
+        auto release_acc = [&]() {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(map_to_cta(acc_empty_bar(buf), 0));   // buffer(s) free for the issuer's next example(s)
@@ -887,85 +856,47 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         // per example, which is what bounds short sequences (the three-statistic epilogue, bound by its instruction
         // count, gains 2-3 %).
         constexpr bool PIPELINED = (CH == 32 && PHI != 3 && PHI != 4) || (TRIPLE && NT == 128);
-        if constexpr (TRIPLE && GROUP == 2) {
-          // The two examples side by side, 8 columns at a time: their signs are counted with one extraction for both, which the
-          // epilogue, bound by its instructions, shows in full: 1024 x 32 x 1024^2 315 -> 276 us, 128 x 32 x 4096^2 492 -> 475.  One pair of
-          // reads in flight (the scheduler's other warp hides its latency) and the larger register share: with two pairs it spills,
-          // 283 us; with 216 registers 291.  An example missing from the last unit counts as a gradient of zeros.
-          constexpr int STEPS = COLS / 8;
-          uint32_t g[8], h[8];
-          auto fold_two = [&](int c) {
-            if (in_unit < 2) {
-#pragma unroll
-              for (int j = 0; j < 8; ++j) h[j] = 0u;
-            }
-#pragma unroll
-            for (int j = 0; j < 8; j += 2) {
-              const int k = c * 8 + j;
-              const uint64_t g2 = f32x2_pack(__uint_as_float(g[j]), __uint_as_float(g[j + 1]));
-              const uint64_t h2 = f32x2_pack(__uint_as_float(h[j]), __uint_as_float(h[j + 1]));
-              f32x2_unpack(f32x2_add(f32x2_add(f32x2_pack(acc_mean[k], acc_mean[k + 1]), g2), h2), acc_mean[k], acc_mean[k + 1]);
-              f32x2_unpack(f32x2_fma(h2, h2, f32x2_fma(g2, g2, f32x2_pack(acc_stat[k], acc_stat[k + 1]))), acc_stat[k], acc_stat[k + 1]);
-              acc_cnt[k >> 1] += signs_plus_two_packed(g2, h2);
-            }
-          };
-#pragma unroll
-          for (int k = 0; k < STEPS; ++k) {
-            tmem_ld_issue(taddr + k * 8, g);
-            tmem_ld_issue(taddr + NT + k * 8, h);
-            tmem_ld_wait_for(g, h);
-            if (k == STEPS - 1) release_unit();
-            fold_two(k);
-          }
-        } else if constexpr (PIPELINED) {
-          constexpr int TOTAL = GROUP * NCH;          // reads per unit when every example of the group exists
-          const int n_reads = in_unit * NCH;
+        if constexpr (PIPELINED) {
           uint32_t ra[CH], rb[CH];
           tmem_ld_issue(taddr, ra);
 #pragma unroll
-          for (int k = 0; k < TOTAL; ++k) {
-            if (GROUP > 1 && k >= n_reads) break;
+          for (int k = 0; k < NCH; ++k) {
             if (k & 1) tmem_ld_wait_for(rb); else tmem_ld_wait_for(ra);
-            if (k + 1 < n_reads) {
-              const uint32_t next = taddr + (uint32_t)(((k + 1) / NCH) * NT + ((k + 1) % NCH) * CH);
+            if (k + 1 < NCH) {
+              const uint32_t next = taddr + (uint32_t)((k + 1) * CH);
               if (k & 1) tmem_ld_issue(next, ra); else tmem_ld_issue(next, rb);
             } else {
-              release_unit();
+              release_acc();
             }
-            if (k & 1) fold(rb, k % NCH); else fold(ra, k % NCH);
+            if (k & 1) fold(rb, k); else fold(ra, k);
           }
         } else {
 #pragma unroll
-          for (int ju = 0; ju < GROUP; ++ju) {
-            if (GROUP > 1 && ju >= in_unit) break;
-            const uint32_t taddr_j = taddr + (uint32_t)(ju * NT);
+          for (int c = 0; c < NCH; ++c) {
+            uint32_t r[CH];
+            if constexpr (PHI == 4) {
+              const int col = tile_n * NT + h * COLS + c * CH;
 #pragma unroll
-            for (int c = 0; c < NCH; ++c) {
-              uint32_t r[CH];
-              if constexpr (PHI == 4) {
-                const int col = tile_n * NT + h * COLS + c * CH;
+              for (int j = 0; j < CH / 4; ++j)
+                col_scale[j] = col + 4 * j < p.d_in ? __ldg(reinterpret_cast<const float4*>(p.scale_x + (long long)(b_begin + a) * p.d_in + col) + j)
+                                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            if constexpr (CH == 32) tmem_ld_32x32b_x32_wait(taddr + c * CH, r);
+            else tmem_ld_32x32b_x16_wait(taddr + c * CH, r);
+            if (c == NCH - 1) release_acc();
+            if constexpr (CHUNKED) {
+              const bool last_run = a % n_runs == n_runs - 1;
 #pragma unroll
-                for (int j = 0; j < CH / 4; ++j)
-                  col_scale[j] = col + 4 * j < p.d_in ? __ldg(reinterpret_cast<const float4*>(p.scale_x + (long long)(b_begin + a) * p.d_in + col) + j)
-                                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+              for (int j = 0; j < CH; j += 2) {
+                float lo, hi;
+                f32x2_unpack(f32x2_add(f32x2_pack(acc_run[c * CH + j], acc_run[c * CH + j + 1]), f32x2_pack(__uint_as_float(r[j]), __uint_as_float(r[j + 1]))), lo, hi);
+                r[j] = __float_as_uint(lo); r[j + 1] = __float_as_uint(hi);
+                acc_run[c * CH + j] = last_run ? 0.f : lo;
+                acc_run[c * CH + j + 1] = last_run ? 0.f : hi;
               }
-              if constexpr (CH == 32) tmem_ld_32x32b_x32_wait(taddr_j + c * CH, r);
-              else tmem_ld_32x32b_x16_wait(taddr_j + c * CH, r);
-              if (c == NCH - 1 && ju == in_unit - 1) release_unit();
-              if constexpr (CHUNKED) {
-                const bool last_run = a % n_runs == n_runs - 1;
-#pragma unroll
-                for (int j = 0; j < CH; j += 2) {
-                  float lo, hi;
-                  f32x2_unpack(f32x2_add(f32x2_pack(acc_run[c * CH + j], acc_run[c * CH + j + 1]), f32x2_pack(__uint_as_float(r[j]), __uint_as_float(r[j + 1]))), lo, hi);
-                  r[j] = __float_as_uint(lo); r[j + 1] = __float_as_uint(hi);
-                  acc_run[c * CH + j] = last_run ? 0.f : lo;
-                  acc_run[c * CH + j + 1] = last_run ? 0.f : hi;
-                }
-                if (last_run) fold(r, c);
-              } else {
-                fold(r, c);
-              }
+              if (last_run) fold(r, c);
+            } else {
+              fold(r, c);
             }
           }
         }
@@ -1101,7 +1032,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         }
       }
       if constexpr (TRIPLE) {
-        const float nbf = (float)(GROUP * nu);
+        const float nbf = (float)nb;
 #pragma unroll
         for (int c = 0; c < COLS; c += 32) {
           float v[32];
@@ -1219,7 +1150,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         if (p.out_sign) {
           if (elect_one()) bulk_wait_read_all();
           __syncwarp();
-          const float nbf = (float)(GROUP * nu);
+          const float nbf = (float)nb;
 #pragma unroll
           for (int c = 0; c < PANELS; ++c) {
             float v[32];

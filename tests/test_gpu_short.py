@@ -1,0 +1,44 @@
+"""Sequences of at most 32 tokens: the kernel of its own that contracts two examples per hand-off."""
+import pytest
+import torch
+
+import paper_2510_00236_b200 as pe
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+# one and two MMA steps, odd batches (a last unit of one example), one example, partial 128- and 32-column pieces, tiles on both sides of the
+# number of pairs, batches split so finely that a slice holds one example, widths that go by way of padded copies (rows of 4 k and of odd length)
+@pytest.mark.parametrize("B,T,d_in,d_out", [(1, 1, 8, 8), (5, 16, 136, 264), (4, 17, 128, 256), (33, 32, 200, 520), (2, 31, 264, 40), (9, 2, 96, 76 * 256),
+                                            (3, 32, 1032, 21 * 256 + 8), (200, 3, 64, 72), (70, 9, 612, 1037), (64, 32, 333, 520)])
+@pytest.mark.parametrize("zeros", [False, True])
+def test_short_sequences_against_fp64(B, T, d_in, d_out, zeros):
+    g = torch.Generator(device=DEV).manual_seed(B * T)
+    X = torch.randn((B, T, d_in), generator=g, device=DEV).bfloat16()
+    dY = (torch.randn((B, T, d_out), generator=g, device=DEV) * T ** -0.5).bfloat16()
+    if zeros:       # columns, rows and whole examples whose G_b is exactly zero
+        X[::2, :, ::3] = 0
+        dY[1::3, :, 1::5] = 0
+        X[B // 2] = 0
+    new = lambda: torch.full((d_out, d_in), float("nan"), device=DEV)       # noqa: E731
+    mean, square, sign, mean1, square1, mean2, sign2, square3, sign3 = (new() for _ in range(9))
+    pe.pe_linear_stats_all(X, dY, mean, square, sign)
+    pe.pe_linear_stats(X, dY, "square", mean1, square1)
+    pe.pe_linear_stats(X, dY, "sign", mean2, sign2)
+    pe.pe_linear_stats(X, dY, "square", None, square3)
+    pe.pe_linear_stats(X, dY, "sign", None, sign3)
+    more = [t.clone() for t in (mean1, square1)]
+    pe.pe_linear_stats_accumulate(X, dY, "square", *more)
+    assert pe.pe_get_async_status(DEV) == (0, 0)
+    G = torch.einsum("bto,bti->boi", dY.double(), X.double())
+    # a term of G_b is exact in fp32 and its sum is taken in fp32, truncated: (T + B) * 2^-23 of the sum of magnitudes at most
+    mag = torch.einsum("bto,bti->boi", dY.double().abs(), X.double().abs())
+    eps = (T + B) * 2.0 ** -23
+    for got, times in ((mean, 1), (mean1, 1), (mean2, 1), (more[0], 2)):
+        assert torch.all((got.double() - times * G.sum(0)).abs() <= times * eps * mag.sum(0))
+    for got, times in ((square, 1), (square1, 1), (square3, 1), (more[1], 2)):
+        assert torch.all((got.double() - times * (G * G).sum(0)).abs() <= times * 3 * eps * (mag * mag).sum(0))
+    unsure = ((G.abs() <= eps * mag) & (mag > 0)).sum(0)
+    for got in (sign, sign2, sign3):
+        assert torch.all((got.double() - G.sign().sum(0)).abs() <= 2 * unsure)
