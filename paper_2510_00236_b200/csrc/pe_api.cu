@@ -1284,12 +1284,12 @@ pe_status_t pe_linear_stats_padded(const void* X, const void* dY, int B, int T, 
                          accumulate != 0, l.pitch_x, l.pitch_y, st, pad);
 }
 
-// Tile of the unfolding kernel: output positions of one row and channels per round, so that a block's shared memory (input rows
-// and feature table) stays within its budget.  False: a receptive field too large for that.
+// Tile of the unfolding kernel: output positions across and down, and channels per round, so that a block's shared memory (the input
+// rows) stays within its budget.  False: a receptive field too large for that.
 struct UnfoldTile {
-  int tile_w, chan, cols, smem;
+  int tile_w, tile_h, chan, cols, img_rows, row_step, kh_step, smem;
 };
-static bool unfold_tile(const ConvGeom& g, UnfoldTile* t) {
+static bool unfold_tile(const ConvGeom& g, int sm_count, UnfoldTile* t) {
   const int kk = g.Kh * g.Kw;
   auto smem = [&](int chan, int cols) { return (long long)((chan * kk + 7) / 8 * 8) * 4 + ((long long)chan * g.Kh * cols + 8) * 2; };
   auto cols_of = [&](int w) { return (long long)(w - 1) * g.sw + (long long)(g.Kw - 1) * g.dw + 1; };
@@ -1297,7 +1297,19 @@ static bool unfold_tile(const ConvGeom& g, UnfoldTile* t) {
     const long long cols = cols_of(w);
     for (int chan = g.C; chan > 0; chan = chan > 8 ? (chan - 1) / 8 * 8 : 0) {
       if ((long long)chan * kk < (1 << 14) && cols < (1 << 16) && smem(chan, (int)cols) <= UNFOLD_SMEM_BYTES) {
-        *t = {w, chan, (int)cols, (int)smem(chan, (int)cols)};
+        // one output row: the kernel's rows alone.  (An extra column where pairs have to start at an even one, and a whole pair at the end: less than
+        // the 4 bytes per feature counted above.)
+        const int even = ((int)cols + 2) & ~1;
+        *t = {w, 1, chan, even, g.Kh, g.dh, 1, chan * g.Kh * even * 2};
+        // Several output rows share their input rows, as long as about four blocks are left to an SM: fewer blocks hide less of each other's
+        // latency (8 images of 64 x 28 x 28, 3 x 3, one row to a block 32 us, eight 39 before the loads were batched).
+        const long long w_tiles = (g.Wo + w - 1) / w;
+        for (int h = 8; h > 1; h /= 2) {
+          const long long rows = (long long)(h - 1) * g.sh + (long long)(g.Kh - 1) * g.dh + 1, bytes = chan * rows * even * 2;
+          if (h > g.Ho || bytes > UNFOLD_SMEM_BYTES || w_tiles * ((g.Ho + h - 1) / h) * g.B < 4ll * sm_count) continue;
+          *t = {w, h, chan, even, (int)rows, 1, g.dh, (int)bytes};
+          break;
+        }
         return true;
       }
     }
@@ -1317,7 +1329,7 @@ size_t pe_conv2d_stats_workspace_bytes(int B, int C, int H, int W, int F, int Kh
                                        int dil_h, int dil_w) {
   ConvGeom g;
   UnfoldTile t;
-  if (!conv_geom(B, C, H, W, F, Kh, Kw, stride_h, stride_w, pad_h, pad_w, dil_h, dil_w, &g) || !unfold_tile(g, &t)) return 0;
+  if (!conv_geom(B, C, H, W, F, Kh, Kw, stride_h, stride_w, pad_h, pad_w, dil_h, dil_w, &g) || !unfold_tile(g, 0, &t)) return 0;
   const PaddedLayout l = padded_layout(B, g.Ho * g.Wo, C * Kh * Kw, F, true);
   return l.x_bytes + l.y_bytes;
 }
@@ -1328,7 +1340,7 @@ pe_status_t pe_conv2d_stats(const void* x, const void* grad_out, int B, int C, i
   ConvGeom g;
   UnfoldTile t;
   if (!conv_geom(B, C, H, W, F, Kh, Kw, stride_h, stride_w, pad_h, pad_w, dil_h, dil_w, &g)) return PE_ERR_DIM;
-  if (!unfold_tile(g, &t)) return PE_ERR_UNSUPPORTED_SHAPE;
+  if (!unfold_tile(g, 0, &t)) return PE_ERR_UNSUPPORTED_SHAPE;
   if (!x || !grad_out) return PE_ERR_NULL;
   const int T = g.Ho * g.Wo, d_in = C * Kh * Kw;
   const PaddedLayout l = padded_layout(B, T, d_in, F, true);
@@ -1349,8 +1361,13 @@ pe_status_t pe_conv2d_stats(const void* x, const void* grad_out, int B, int C, i
   ConvOperands o;
   o.x = static_cast<const uint16_t*>(x); o.gy = static_cast<const uint16_t*>(grad_out); o.X = X; o.dY = dY;
   o.pitch_x = l.pitch_x; o.pitch_y = l.pitch_y;
-  o.tile_w = t.tile_w; o.chan = t.chan; o.cols = t.cols; o.w_tiles = (g.Wo + t.tile_w - 1) / t.tile_w;
-  o.unfold_blocks = (long long)o.w_tiles * g.Ho * B;
+  unfold_tile(g, di->sm_count, &t);
+  o.tile_w = t.tile_w; o.tile_h = t.tile_h; o.chan = t.chan; o.cols = t.cols; o.img_rows = t.img_rows; o.row_step = t.row_step; o.kh_step = t.kh_step;
+  o.pairs = W % 2 == 0 && aligned(x, 4) ? 1 : 0;
+  const uint32_t per_row = (uint32_t)(o.pairs ? t.cols / 2 : t.cols);
+  o.per_row_magic = (uint32_t)(((1ull << 32) + per_row - 1) / per_row); o.img_rows_magic = (uint32_t)(((1ull << 32) + t.img_rows - 1) / t.img_rows);
+  o.w_tiles = (g.Wo + t.tile_w - 1) / t.tile_w; o.h_tiles = (g.Ho + t.tile_h - 1) / t.tile_h;
+  o.unfold_blocks = (long long)o.w_tiles * o.h_tiles * B;
   o.t_tiles = (T + 63) / 64; o.f_tiles = (l.pitch_y + 63) / 64;
   o.vec = T % 8 == 0 && aligned(grad_out, 16) ? 1 : 0;
   const long long blocks = o.unfold_blocks + (long long)o.t_tiles * o.f_tiles * B;

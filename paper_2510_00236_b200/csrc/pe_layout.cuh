@@ -2,7 +2,7 @@
 // row pitches): rows of a width that is no multiple of 8 copied to a padded pitch, and the operands of a convolution's
 // weight gradient (Appendix B.4) unfolded straight into that form.  For the contractions that stand for the statistics of one-token
 // examples: the halves of their squares and their signs.  The padding kernel is bound by HBM bandwidth, the unfolding kernel by its
-// gathers from shared memory (58 MB in 25 us), the one-token kernel by launch latency and HBM.  The columns
+// gathers from shared memory, the one-token kernel by launch latency and HBM.  The columns
 // between the width and the pitch are never read (the tensor maps end at the width).
 #pragma once
 #include <cuda_runtime.h>
@@ -91,68 +91,92 @@ struct ConvGeom {
 // transpose the cotangents.
 //
 // Unfolding: X[(b, oh, ow), f] = x[b, c, oh*sh - ph + kh*dh, ow*sw - pw + kw*dw] (0 outside the image), f = (c*Kh + kh)*Kw + kw: one
-// row of pitch_x bf16 per output position.  A block handles a run of tile_w positions of one output row: the input rows it touches go
-// to shared memory once, `chan` channels at a time and with the image's border as zeros, and every 16-byte group of the
-// result is gathered from there; a thread keeps its group, whose eight offsets stay in registers, and walks over the positions.
+// row of pitch_x bf16 per output position.  A block handles tile_h x tile_w output positions: the input rows they touch go to shared
+// memory once, `chan` channels at a time, two elements per load where the rows allow, and with the image's border as zeros; every 16-byte
+// group of the result is gathered from there.  A thread keeps its group, whose eight offsets stay in registers, and walks over the positions.
 // chan is a multiple of 8 or C, so that a round's features start on a group.
 //
 // Transposing: dY[b, t, f] = gy[b, f, t], [B, F, T] -> [B, T, pitch_y], through 64 x 64 tiles of shared memory; vec: rows of gy are
 // 16-byte multiples and read as such.
 //
-// 32 images of 3 x 112 x 112, 7 x 7, stride 2, 64 filters (43 MB written): 45 -> 25 us against two launches, an offset table read from
-// shared memory for every group and 2-byte reads of the cotangents; the whole call was 1158 us with torch's unfold, which launches
-// one kernel per image, in fp32, before a transpose and two conversions.
+// Bound by the gathers' instructions and the latency of a block's loads.  Whole calls, against a block per output row whose warps load one input row
+// after the other: 32 images of 3 x 112 x 112, 7 x 7, stride 2, 64 filters (43 MB written) 46 -> 39 us; 32 of 64 x 14 x 14, 3 x 3, 128 filters
+// 34 -> 20; 64 of 64 x 15 x 15, 3 x 3, stride 2, 96 filters 30 -> 21; 16 of 16 x 56 x 56, 3 x 3, 96 filters 33 -> 31.
 struct ConvOperands {
   const uint16_t* x;
   const uint16_t* gy;
   uint16_t* X;
   uint16_t* dY;
   int pitch_x, pitch_y;
-  int tile_w, chan, cols;       // unfolding: positions per block, channels per round, image columns per row in shared memory
-  int w_tiles;                  // ceil(Wo / tile_w)
-  long long unfold_blocks;      // w_tiles * Ho * B
+  int tile_w, tile_h, chan;     // unfolding: positions per block, across and down, channels per round
+  int cols, img_rows;           // image columns and rows per channel in shared memory
+  int row_step, kh_step;        // image rows from one of those to the next; of those from one kernel row to the next
+  int pairs;                    // the image's rows are whole aligned pairs of elements
+  uint32_t per_row_magic, img_rows_magic;     // ceil(2^32 / loads per row), ceil(2^32 / img_rows): exact quotients of numbers below 2^16 (not by 1)
+  int w_tiles, h_tiles;         // ceil(Wo / tile_w), ceil(Ho / tile_h)
+  long long unfold_blocks;      // w_tiles * h_tiles * B
   int t_tiles, f_tiles;         // transposing: ceil(T / 64), ceil(pitch_y / 64)
   int vec;
 };
 __device__ __forceinline__ void unfold_block(const ConvOperands& o, const ConvGeom& g, uint16_t* smem) {
   const int kk = g.Kh * g.Kw;
-  const int chunk_feats = (o.chan * kk + 7) & ~7;
-  int* const off = reinterpret_cast<int*>(smem);                     // [chunk_feats]: element offset of a feature at position 0, -1 beyond
-  uint16_t* const img = smem + 2 * chunk_feats;                      // [chan][Kh][cols]
   const int ow0 = (int)(blockIdx.x % o.w_tiles) * o.tile_w;
-  const int rest = (int)(blockIdx.x / o.w_tiles), oh = rest % g.Ho, b = rest / g.Ho;
-  const int n_ow = min(o.tile_w, g.Wo - ow0);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rest = (int)(blockIdx.x / o.w_tiles), oh0 = rest % o.h_tiles * o.tile_h, b = rest / o.h_tiles;
+  const int n_ow = min(o.tile_w, g.Wo - ow0), positions = min(o.tile_h, g.Ho - oh0) * n_ow;
+  const int shift = o.pairs ? (ow0 * g.sw - g.pw) & 1 : 0;           // pairs start at even columns of the image
+  const int iw0 = ow0 * g.sw - g.pw - shift, ih0 = oh0 * g.sh - g.ph;
   for (int c0 = 0; c0 < g.C; c0 += o.chan) {
     const int nc = min(o.chan, g.C - c0);
     const int feats = nc * kk, groups = (feats + 7) >> 3;
-    for (int r = warp; r < nc * g.Kh; r += LAYOUT_THREADS / 32) {
-      const int ch = r / g.Kh, kh = r - ch * g.Kh, ih = oh * g.sh - g.ph + kh * g.dh;
-      const uint16_t* const row = o.x + (((long long)b * g.C + c0 + ch) * g.H + ih) * g.W;
-      for (int w = lane; w < o.cols; w += 32) {
-        const int iw = ow0 * g.sw - g.pw + w;
-        img[r * o.cols + w] = (ih >= 0 && ih < g.H && iw >= 0 && iw < g.W) ? __ldg(row + iw) : (uint16_t)0;
+    // smem: [nc][img_rows][cols], eight loads of a thread in flight (a warp per row, one after the other, spent 20 us on latency)
+    const int per_row = o.pairs ? o.cols / 2 : o.cols, total = nc * o.img_rows * per_row;
+    for (int base = threadIdx.x; base < total; base += 8 * LAYOUT_THREADS) {
+      uint32_t v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const uint32_t k = (uint32_t)(base + j * LAYOUT_THREADS);
+        const uint32_t r = per_row > 1 ? __umulhi(k, o.per_row_magic) : k, ch = o.img_rows > 1 ? __umulhi(r, o.img_rows_magic) : r;
+        const int ih = ih0 + (int)(r - ch * o.img_rows) * o.row_step, iw = iw0 + (int)(k - r * per_row) * (o.pairs ? 2 : 1);
+        v[j] = 0u;
+        if ((int)k < total && ih >= 0 && ih < g.H && iw >= 0 && iw < g.W) {
+          const uint16_t* const at = o.x + (((long long)b * g.C + c0 + ch) * g.H + ih) * g.W + iw;
+          v[j] = o.pairs ? __ldg(reinterpret_cast<const uint32_t*>(at)) : (uint32_t)__ldg(at);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int k = base + j * LAYOUT_THREADS;
+        if (k >= total) break;
+        if (o.pairs) reinterpret_cast<uint32_t*>(smem)[k] = v[j];
+        else smem[k] = (uint16_t)v[j];
       }
     }
-    for (int f = threadIdx.x; f < groups * 8; f += LAYOUT_THREADS) {
-      const int r = f / g.Kw, kw = f - r * g.Kw;                     // r = ch * Kh + kh
-      off[f] = f < feats ? r * o.cols + kw * g.dw : -1;
-    }
     __syncthreads();
-    uint16_t* const out = o.X + (((long long)b * g.Ho + oh) * g.Wo + ow0) * o.pitch_x + c0 * kk;
     for (int g0 = 0; g0 < groups; g0 += LAYOUT_THREADS) {
       const int width = min(groups - g0, LAYOUT_THREADS), together = LAYOUT_THREADS / width;      // groups side by side, positions at once
       const int grp = g0 + (int)threadIdx.x % width, first = (int)threadIdx.x / width;
       if (first >= together) continue;
-      const int4 o0 = *reinterpret_cast<const int4*>(off + 8 * grp), o1 = *reinterpret_cast<const int4*>(off + 8 * grp + 4);
-      const int at[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
+      // features past the last one: any element will do, those columns are never read
+      int at[8];
+      int ch = 8 * grp / kk, kh = (8 * grp - ch * kk) / g.Kw, kw = 8 * grp - ch * kk - kh * g.Kw;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        at[j] = 8 * grp + j < feats ? (ch * o.img_rows + kh * o.kh_step) * o.cols + kw * g.dw + shift : 0;
+        if (++kw == g.Kw) {
+          kw = 0;
+          if (++kh == g.Kh) { kh = 0; ++ch; }
+        }
+      }
+      uint16_t* const out = o.X + (((long long)b * g.Ho + oh0) * g.Wo + ow0) * o.pitch_x + c0 * kk + 8 * grp;
+      int r = first / n_ow, w = first - r * n_ow;
 #pragma unroll 2
-      for (int tok = first; tok < n_ow; tok += together) {
+      for (int pos = first; pos < positions; pos += together) {
+        const uint16_t* const img = smem + r * g.sh * o.cols + w * g.sw;
         uint32_t v[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = at[j] >= 0 ? (uint32_t)img[at[j] + tok * g.sw] : 0u;
-        *reinterpret_cast<uint4*>(out + (long long)tok * o.pitch_x + 8 * grp) =
-            make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+        for (int j = 0; j < 8; ++j) v[j] = img[at[j]];
+        *reinterpret_cast<uint4*>(out + ((long long)r * g.Wo + w) * o.pitch_x) = make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+        for (w += together; w >= n_ow; w -= n_ow) ++r;
       }
     }
     __syncthreads();
