@@ -177,6 +177,10 @@ constexpr UnitCost COST_SIGN = {256, 0.51 / 128, 0.68 / 128, 0.0, 0.66, 8.5};
 constexpr UnitCost COST_NORMS = {256, 0.51 / 128, 0.68 / 128, 0.0, 0.30, 7.0};
 constexpr UnitCost COST_PLAIN = {256, 0.51 / 128, 0.68 / 128, 0.0, 0.0, 8.5};
 constexpr UnitCost COST_TOKEN = {TOK_NT, 0.42 / TOK_BK, 0.45 / TOK_BK, 0.0, 0.0, 8.5};     // an "example" is one 32-row stage
+// The per-token statistic's chunks dealt out evenly over the pairs: two tiles instead of one to write out per pair, and rows that are read at
+// different times for the tiles that share them.  64 x 256 x 512 x 2048 (16 tiles) 68.9 -> 63.0 us, 64 x 256 x 1024 x 2048 (32) 125 -> 111, 100 x 100 x 776 x 3000
+// (48) 116 -> 108; 128 x 512 x 512 x 1024 (8 tiles, whose nine slices leave two pairs idle) 117 -> 119, which stays in slices.
+constexpr double TOK_EVEN_FIXED = 4.0;
 constexpr UnitCost COST_PLAIN_FP8 = {256, 0.28 / 128, 0.40 / 128, 0.0, 0.0, 8.5};
 constexpr UnitCost COST_BOTH_192 = {192, 0.375 / 128, 0.55 / 128, 0.02, 0.35, 10.0};     // two sums
 constexpr UnitCost COST_BOTH_128 = {128, 0.35 / 128, 0.44 / 128, 0.12, 0.20, 8.3};
@@ -988,8 +992,14 @@ static pe_status_t launch_tok(DeviceInfo* di, const void* X, const void* dY, lon
   const long long n_chunks = (rows + TOK_BK - 1) / TOK_BK;
   const int units = n_chunks > (1 << 30) ? (1 << 30) : (int)n_chunks;
   const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
+  const long long tiles = (long long)tiles_n * pairs_m;
   const int ns = plan_tiles(&COST_TOKEN, 1, units, TOK_BK, d_in, d_out, slots, std::max(32, slots), 1).ns;
-  if (ns > 1) {
+  // The chunks of all tiles dealt out evenly, where that saves more than the second tile that most pairs then write out.
+  const double in_slices = launch_cost(COST_TOKEN, tiles, units, TOK_BK, slots, ns, 1, 4.0 * d_in * d_out, false).us;
+  const double evenly = std::ceil((double)tiles * units / slots) * TOK_BK * COST_TOKEN.token_hi + COST_TOKEN.fixed + SPLIT_FIXED + 4.0 * d_in * d_out / ZERO_BYTES_PER_US +
+                        TOK_EVEN_FIXED;
+  const bool even = tiles <= slots && tiles * units >= slots && evenly < in_slices;
+  if (ns > 1 || even) {
     rc = zero_for_split(di, out, nullptr, (size_t)d_in * d_out, st);
     if (rc != PE_OK) return rc;
   }
@@ -1005,8 +1015,8 @@ static pe_status_t launch_tok(DeviceInfo* di, const void* X, const void* dY, lon
   }
   TokParams p;
   p.rows = rows; p.d_in = d_in; p.d_out = d_out; p.pairs_m = pairs_m; p.tiles_n = tiles_n;
-  p.band = choose_band(pairs_m, tiles_n, TOK_NT, ns, di->sm_count / 2); p.nsplit = ns; p.dev_status = di->status_ptr;
-  return launch_dependent(tok_sqstats_kernel, dim3(2 * pairs_m * tiles_n, 1, ns), TOK_THREADS, TOK_SMEM_BYTES, st, mx, my, mo, p);
+  p.band = choose_band(pairs_m, tiles_n, TOK_NT, even ? 1 : ns, di->sm_count / 2); p.nsplit = even ? 1 : ns; p.even = even ? 1 : 0; p.dev_status = di->status_ptr;
+  return launch_dependent(tok_sqstats_kernel, even ? dim3(2 * slots) : dim3(2 * pairs_m * tiles_n, 1, ns), TOK_THREADS, TOK_SMEM_BYTES, st, mx, my, mo, p);
 }
 
 }  // namespace pe

@@ -175,7 +175,6 @@ short_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
       int tile_m, tile_n;
       tc_tile_of_pair(p, t.tile, rank, tile_m, tile_n);
       const int row0 = tile_m * TC_TILE_M + q * 32, col0 = tile_n * SHORT_NT + h * COLS;
-      const bool row_inside = row0 + lane < p.d_out;
       uint32_t g[2][W], f[2][W];              // the two examples' entries, two reads in turn
       bool read_ahead = false;
       for (int b = t.b_begin; b < t.b_end; b += SHORT_G) {

@@ -11,7 +11,9 @@
 // two-pass variant on large layers and faster on small ones, with a third of the HBM traffic.
 //
 // Work unit: a CTA pair owns a 256 x 256 tile of the [d_out, d_in] output and a contiguous range of
-// 32-row chunks of the B*T rows (gridDim.z slices; partial sums are added by TMA reduce).
+// 32-row chunks of the B*T rows (gridDim.z slices; partial sums are added by TMA reduce).  With at most as many tiles as pairs, and where whole slices
+// leave pairs idle (16 tiles: 64 of 74), the chunks of all tiles are dealt out evenly instead, tile after tile: a pair then holds the end of one
+// tile and the start of the next, in the two accumulators that tensor memory has room for, and writes both out at the end.
 //
 // Shared memory per block: 4 "raw" stages of 16 KiB (bf16: 128 rows of dY^T as two 64-feature boxes,
 // this block's 128 rows of X^T as two more; 128-byte swizzle with 16-byte chunks, as TMA writes it)
@@ -52,6 +54,7 @@ struct TokParams {
   int d_in, d_out;
   int pairs_m, tiles_n, band;   // tile grid and tile order, as in TcParams
   int nsplit;          // slices of the row range (gridDim.z); > 1 => output pre-zeroed, partial sums added
+  int even;            // the chunks of all tiles are dealt out evenly over gridDim.x / 2 pairs (output pre-zeroed, sums added); tiles <= pairs
   unsigned int* dev_status;
 };
 
@@ -97,17 +100,41 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();          // 0 = leader of the pair
-  int tile_m, tile_n;                               // 128-row tile of d_out, 256-column tile of d_in (banded tile order)
-  {
-    const int pair_id = blockIdx.x >> 1;
+  const long long n_chunks = (p.rows + TOK_BK - 1) / TOK_BK;
+  // one or two pieces: a tile (128-row tile of d_out, 256-column tile of d_in, in the banded tile order) and a range of chunks
+  struct Piece {
+    int tile_m, tile_n;
+    long long begin, end;
+  };
+  Piece piece[2];
+  int n_pieces = 1;
+  auto tile_of = [&](Piece& t, int pair_id) {
     const int per_band = p.band * p.tiles_n;
     const int band = pair_id / per_band, r = pair_id - band * per_band;
     const int rows_in_band = min(p.band, p.pairs_m - band * p.band);
-    tile_n = r / rows_in_band;
-    tile_m = 2 * (band * p.band + (r - tile_n * rows_in_band)) + (int)rank;
+    t.tile_n = r / rows_in_band;
+    t.tile_m = 2 * (band * p.band + (r - t.tile_n * rows_in_band)) + (int)rank;
+  };
+  if (p.even) {
+    const long long total = n_chunks * p.pairs_m * p.tiles_n, pairs = gridDim.x >> 1;
+    const long long first = total * (blockIdx.x >> 1) / pairs, last = total * ((blockIdx.x >> 1) + 1) / pairs;
+    const int tile = (int)(first / n_chunks);
+    tile_of(piece[0], tile);
+    piece[0].begin = first - tile * n_chunks;
+    piece[0].end = min(n_chunks, piece[0].begin + last - first);
+    if (last > (tile + 1) * n_chunks) {
+      n_pieces = 2;
+      tile_of(piece[1], tile + 1);
+      piece[1].begin = 0;
+      piece[1].end = last - (tile + 1) * n_chunks;
+    }
+  } else {
+    tile_of(piece[0], blockIdx.x >> 1);
+    piece[0].begin = n_chunks * blockIdx.z / p.nsplit;
+    piece[0].end = n_chunks * (blockIdx.z + 1) / p.nsplit;
   }
-  const long long n_chunks = (p.rows + TOK_BK - 1) / TOK_BK;
-  const long long c_begin = n_chunks * blockIdx.z / p.nsplit, c_end = n_chunks * (blockIdx.z + 1) / p.nsplit;
+  if (n_pieces == 1) piece[1] = {0, 0, 0, 0};
+  const bool add = p.nsplit > 1 || p.even;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < TOK_RAW_STAGES; ++s) { mbar_init(raw_full(s), 1); mbar_init(raw_empty(s), 4); }
@@ -122,7 +149,7 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   griddep_launch_dependents();            // as in the statistics kernel
-  if (p.nsplit == 1) griddep_wait();
+  if (!add) griddep_wait();
 
   if (warp < 4) {
     const bool strict = wait_cycle_limit() < WAIT_CYCLE_LIMIT_STRICT;
@@ -130,11 +157,14 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
       // ---------------------------------------------------------- TMA producers (each block for itself)
       const bool is_a = (warp == 0);
       const CUtensorMap* tmap = is_a ? &tmap_dy : &tmap_x;
-      const int c0 = is_a ? tile_m * TC_TILE_M : tile_n * TOK_NT + (int)rank * (TOK_NT / 2);
       if (elect_one()) prefetch_tensormap(tmap);
       int s = 0; uint32_t ph = 1;
-      for (long long ch = c_begin; ch < c_end; ++ch) {
-        if (!mbar_wait_warp(raw_empty(s), ph, abort_flag, p.dev_status, TOK_WAIT_RAW_EMPTY, strict)) break;
+      bool ok = true;
+      for (int k = 0; k < 2 && ok; ++k) {
+      const Piece t = k ? piece[1] : piece[0];
+      const int c0 = is_a ? t.tile_m * TC_TILE_M : t.tile_n * TOK_NT + (int)rank * (TOK_NT / 2);
+      for (long long ch = t.begin; ch < t.end; ++ch) {
+        if (!mbar_wait_warp(raw_empty(s), ph, abort_flag, p.dev_status, TOK_WAIT_RAW_EMPTY, strict)) { ok = false; break; }
         if (elect_one()) {
           if (is_a) mbar_arrive_expect_tx(raw_full(s), TOK_RAW_STAGE);          // this block's four boxes
           const uint32_t dst = smem_base + s * TOK_RAW_STAGE + (is_a ? 0 : 2 * TOK_BOX_BYTES);
@@ -144,12 +174,17 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         __syncwarp();
         if (++s == TOK_RAW_STAGES) { s = 0; ph ^= 1u; }
       }
+      }
     } else if (rank == 0 && warp == 1) {
       // ---------------------------------------------------------- MMA issuer (leader block)
       constexpr uint32_t idesc = make_idesc_mn_major(TC_PAIR_M, TOK_NT, true);
       int c = 0; uint32_t ph = 0;
-      for (long long ch = c_begin; ch < c_end; ++ch) {
-        if (!mbar_wait_warp(cooked_full(c), ph, abort_flag, p.dev_status, TOK_WAIT_COOKED_FULL, strict)) break;
+      bool ok = true;
+      for (int piece_no = 0; piece_no < 2 && ok; ++piece_no) {
+      const Piece t = piece_no ? piece[1] : piece[0];
+      const uint32_t d_tmem = tmem_base + (uint32_t)(piece_no * TOK_NT);
+      for (long long ch = t.begin; ch < t.end; ++ch) {
+        if (!mbar_wait_warp(cooked_full(c), ph, abort_flag, p.dev_status, TOK_WAIT_COOKED_FULL, strict)) { ok = false; break; }
         tc_fence_after();
         if (elect_one()) {
           const uint32_t a_src = cooked_base + c * TOK_COOKED_STAGE;
@@ -158,13 +193,14 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
           for (int k = 0; k < TOK_BK / TOK_MMA_K; ++k) {       // rows past the end are zero: no need to skip them
             const uint64_t ad = make_smem_desc(a_src + k * TOK_MMA_K * 128, TOK_BOX_BYTES, 512u, 1u);
             const uint64_t bd = make_smem_desc(b_src + k * TOK_MMA_K * 128, TOK_BOX_BYTES, 512u, 1u);
-            umma_ss_pair<1>(tmem_base, ad, bd, idesc, (k > 0 || ch > c_begin) ? 1u : 0u);
+            umma_ss_pair<1>(d_tmem, ad, bd, idesc, (k > 0 || ch > t.begin) ? 1u : 0u);
           }
           umma_commit_pair(cooked_empty(c));             // cooked stage reusable in both blocks once these MMAs retire
-          if (ch == c_end - 1) umma_commit_pair(acc_full);        // accumulator complete, both blocks
+          if (ch == t.end - 1 && piece_no == n_pieces - 1) umma_commit_pair(acc_full);        // accumulators complete, both blocks
         }
         __syncwarp();
         if (++c == TOK_COOKED_STAGES) { c = 0; ph ^= 1u; }
+      }
       }
     }
   } else {
@@ -176,7 +212,8 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
       // The sixteen warps work as four groups of four, group g on the stages n = g, g + 4, ... (ring slot g),
       // so that the groups' shared-memory round trips and barrier hand-offs overlap one another's arithmetic.
       const int grp = w >> 2, wl = w & 3;
-      for (long long n = grp; n < c_end - c_begin; n += TOK_CONV_GROUPS) {
+      const long long stages = piece[0].end - piece[0].begin + piece[1].end - piece[1].begin;
+      for (long long n = grp; n < stages; n += TOK_CONV_GROUPS) {
         const int s = (int)(n % TOK_RAW_STAGES);          // raw and cooked rings advance together (same depth)
         const uint32_t ph = (uint32_t)(n / TOK_RAW_STAGES) & 1u;
         // every lane polls, the warp acts on one answer (what follows contains warp-wide instructions)
@@ -220,38 +257,42 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     }
     static_assert(TOK_RAW_STAGES == TOK_COOKED_STAGES && TOK_RAW_STAGES % 2 == 0, "the two rings advance together; each slot belongs to one converter group");
     ok = __all_sync(0xffffffffu, ok);
-    if (ok && w < 8) ok = mbar_wait_warp(acc_full, 0, abort_flag, p.dev_status, TOK_WAIT_ACC);
+    const int mine = w >> 3;                  // the first eight warps write the first piece's tile out, the others the second's
+    if (ok && mine < n_pieces) ok = mbar_wait_warp(acc_full, 0, abort_flag, p.dev_status, TOK_WAIT_ACC);
     ok = __all_sync(0xffffffffu, ok);
-    if (ok && w < 8) {
-      // Write-out as in the statistics kernel: 32 rows x 128 columns per warp, staged in the idle ring
-      // as four 128-byte-swizzled 4 KiB panels, stored (or added, with a split row range) by TMA.
+    if (ok && mine < n_pieces) {
+      // Write-out as in the statistics kernel: 32 rows x 128 columns per warp, staged in the idle ring, 32 columns (a 128-byte-swizzled 4 KiB
+      // panel) at a time in two panels per warp, stored (or added) by TMA.
       tc_fence_after();
-      const int q = warp & 3, h = w >> 2;
-      const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * 128);
-      const uint32_t stage_base = smem_base + (uint32_t)w * (4u * 4096u);
-      const int row0 = tile_m * TC_TILE_M + q * 32, col0 = tile_n * TOK_NT + h * 128;
+      const Piece t = mine ? piece[1] : piece[0];
+      const int q = warp & 3, h = (w >> 2) & 1;
+      const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(mine * TOK_NT + h * 128);
+      const uint32_t stage_base = smem_base + (uint32_t)w * (2u * 4096u);
+      const int row0 = t.tile_m * TC_TILE_M + q * 32, col0 = t.tile_n * TOK_NT + h * 128;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         uint32_t r[32];
         tmem_ld_32x32b_x32_wait(lane_base + c * 32, r);
-        uint8_t* dst = smem_gen + (stage_base - smem_base) + c * 4096 + lane * 128;
+        if (c == 2) {                             // the panels are used again
+          if (elect_one()) bulk_wait_read_all();
+          __syncwarp();
+        }
+        const uint32_t panel = stage_base + (c & 1) * 4096;
+        uint8_t* dst = smem_gen + (panel - smem_base) + lane * 128;
 #pragma unroll
         for (int k = 0; k < 8; ++k)
           *reinterpret_cast<uint4*>(dst + ((k ^ (lane & 7)) << 4)) = make_uint4(r[4 * k], r[4 * k + 1], r[4 * k + 2], r[4 * k + 3]);
-      }
-      fence_async_smem();
-      __syncwarp();
-      if (row0 < p.d_out && elect_one()) {
-        if (p.nsplit > 1) griddep_wait();         // the kernel that zeroes the output may still be running
-        for (int c = 0; c < 4; ++c) {
-          if (col0 + c * 32 < p.d_in) {
-            if (p.nsplit == 1) tma_store_2d<false>(&tmap_out, stage_base + c * 4096, col0 + c * 32, row0);
-            else tma_store_2d<true>(&tmap_out, stage_base + c * 4096, col0 + c * 32, row0);
-          }
+        fence_async_smem();
+        __syncwarp();
+        if (row0 < p.d_out && col0 + c * 32 < p.d_in && elect_one()) {
+          if (c == 0 && add) griddep_wait();         // the kernel that zeroes the output may still be running
+          if (add) tma_store_2d<true>(&tmap_out, panel, col0 + c * 32, row0);
+          else tma_store_2d<false>(&tmap_out, panel, col0 + c * 32, row0);
+          bulk_commit_group();
         }
-        bulk_commit_group();
-        bulk_wait_read_all();               // shared memory must outlive TMA's reads
+        __syncwarp();
       }
+      if (elect_one()) bulk_wait_read_all();               // shared memory must outlive TMA's reads
     }
     __syncwarp();
   }
