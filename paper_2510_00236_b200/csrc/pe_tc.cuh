@@ -140,6 +140,7 @@ struct TcParams {
   int nsplit;          // batch slices (gridDim.z); > 1 => outputs pre-zeroed, partials added atomically
   int whole_tiles;     // PERSIST: tiles that one pair contracts over the whole batch; each of the others goes to
   int tail_split;      // this many pairs, by slices of the batch, whose sums are added to (zeroed) outputs
+  int slice_examples;  // 0, or the examples of such a slice (the last one may have fewer): where slices are short, 64-bit divisions would show
   int part_chunks;     // PARTS: chunks of rows per part, slices of the square's, the mean's and the sign's chunks
   int part_slices[3];
   unsigned int part_dy, part_x;   // PARTS: the copies of dY and of X that each product takes
@@ -182,6 +183,7 @@ __device__ __forceinline__ int tc_units(const TcParams& p) { return p.whole_tile
 __device__ __forceinline__ TcUnit tc_unit(const TcParams& p, int u) {
   if (u < p.whole_tiles) return {u, 0, p.B, true};
   const int rest = p.pairs_m * p.tiles_n - p.whole_tiles, v = u - p.whole_tiles, slice = v / rest;
+  if (p.slice_examples) return {p.whole_tiles + v - slice * rest, slice * p.slice_examples, min(p.B, (slice + 1) * p.slice_examples), false};
   return {p.whole_tiles + v - slice * rest, (int)((long long)p.B * slice / p.tail_split), (int)((long long)p.B * (slice + 1) / p.tail_split), p.tail_split == 1};
 }
 
@@ -439,7 +441,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   static_assert((PHI != 3 && PHI != 4) || MEAN == MEAN_NONE, "the clipped sum and the scaled contraction are statistic-only passes");
   static_assert(!CHUNKED || (MEAN == MEAN_REGS && NT == 128 && !RAGGED && OPT == OPT_NONE), "runs of an example: the two-sum kernel on the 256 x 128 tile");
   static_assert(!PARTS || (PHI == 0 && !TF32 && !F8 && !RAGGED && !PERSIST && OPT == OPT_NONE), "the statistics of one-token examples are plain contractions");
-  static_assert(!PERSIST || (!RAGGED && OPT == OPT_NONE && MEAN != MEAN_TMEM && !NORMS && PHI != 0), "several tiles per pair: fixed-length batches, whole sums written");
+  static_assert(!PERSIST || (!RAGGED && OPT == OPT_NONE && MEAN != MEAN_TMEM && PHI != 0), "several tiles per pair: fixed-length batches");
   constexpr int CHUNK_STAGES = CHUNKED ? TC_CHUNK_TOKENS / BKT : 1;
   constexpr int REGS_CONTROL = CHUNKED || TRIPLE ? 40 : Op::REGS_CONTROL, REGS_EPILOGUE = CHUNKED || TRIPLE ? 232 : Op::REGS_EPILOGUE;
   static_assert(128 * REGS_CONTROL + 256 * REGS_EPILOGUE <= TC_THREADS * TC_REGS_AT_LAUNCH, "setmaxnreg: the epilogue's increase must fit what the control warps give up");
@@ -689,6 +691,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       }
     }
     const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
+    float norm_kept = 0.f;          // NORMS
     for (int a = 0; a < n_acc; ++a) {
       const int buf = (a0 + a) % ACC_BUFS;
       const uint32_t acc_ph = (uint32_t)((a0 + a) / ACC_BUFS) & 1u;
@@ -775,30 +778,38 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       } else if constexpr (NORMS) {
         // this thread's share of ||G_b||_F^2 (its row, its 128 columns; rows and columns outside the
         // matrix are exact zeros), then the warp's, then one atomic per warp and example
-        uint64_t sa = f32x2_pack(0.f, 0.f), sb = sa;
+        // All reads at once and the accumulator released behind them, before the arithmetic.
+        constexpr int READS = COLS / 32;
+        uint32_t r[READS][32];
 #pragma unroll
-        for (int c = 0; c < COLS / 32; ++c) {
-          uint32_t r[32];
-          tmem_ld_32x32b_x32_wait(taddr + c * 32, r);
-          if (c == COLS / 32 - 1) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(map_to_cta(acc_empty_bar(buf), 0));
-          }
+        for (int c = 0; c < READS; ++c) tmem_ld_issue(taddr + c * 32, r[c]);
 #pragma unroll
-          for (int j = 0; j < 32; j += 4) {
-            const uint64_t g0 = f32x2_pack(__uint_as_float(r[j]), __uint_as_float(r[j + 1]));
-            const uint64_t g1 = f32x2_pack(__uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
-            sa = f32x2_fma(g0, g0, sa);
-            sb = f32x2_fma(g1, g1, sb);
+        for (int c = 0; c < READS; ++c) tmem_ld_wait_for(r[c]);
+        tc_fence_before();
+        __syncwarp();
+        mbar_arrive_cluster_if(lane == 0, map_to_cta(acc_empty_bar(buf), 0));
+        uint64_t part[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) part[i] = f32x2_pack(0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < READS; ++c)
+#pragma unroll
+          for (int j = 0; j < 32; j += 2) {
+            const uint64_t g2 = f32x2_pack(__uint_as_float(r[c][j]), __uint_as_float(r[c][j + 1]));
+            part[(j / 2) % 4] = f32x2_fma(g2, g2, part[(j / 2) % 4]);
           }
-        }
         float s0, s1;
-        f32x2_unpack(f32x2_add(sa, sb), s0, s1);
+        f32x2_unpack(f32x2_add(f32x2_add(part[0], part[1]), f32x2_add(part[2], part[3])), s0, s1);
         float s = s0 + s1;
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-        if (lane == 0) atomicAdd(p.out_norms + b_begin + a, s);
+        // lane l keeps the sum of the unit's example 32 k + l: one coalesced add per 32 examples.  An add per example and warp met the other tiles' at one
+        // address of L2, 2048 of them per example on 128 tiles: 128 x 64 x 2048 x 4096 254 -> 109 us, 50 x 120 x 1400 x 2000 80 -> 40, 64 x 128 x 512 x 2048 20 -> 16.
+        if (lane == (a & 31)) norm_kept = s;
+        if ((a & 31) == 31 || a == n_acc - 1) {
+          const int first = a & ~31;
+          if (first + lane <= a) atomicAdd(p.out_norms + b_begin + first + lane, norm_kept);
+        }
       } else {
         // CH columns per tensor-memory read: 32, or 16 where the running sums leave few registers (NT = 192; the three
         // statistics on the 256 x 128 tile, whose 160 registers of sums leave room for two reads of 16 in flight, not 32)
@@ -978,7 +989,9 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
 #pragma unroll
       for (int j = 0; j < N_STAT; ++j) acc_stat[j] = fmaf(2.f, acc_stat[j], -nbf);
     }
-    if constexpr (PERSIST) {
+    if constexpr (PERSIST && NORMS) {
+      a0 += n_acc;                  // (nothing to write out)
+    } else if constexpr (PERSIST) {
       // Several tiles per pair: straight from the registers, since the operand ring already fills for the next tile.  Lanes
       // exchange their rows' values first, so that four of them store 128 bytes side by side (stores of 32 bytes to 32 rows: 8 x 256
       // x 1024 x 32104, both outputs, 201 us against 179).  Slices of a tile add 128 bytes of a row per instruction (16-byte adds, 32
