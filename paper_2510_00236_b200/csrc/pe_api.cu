@@ -310,22 +310,23 @@ static pe_status_t launch_dependent(Kernel kernel, dim3 grid, int threads, int s
   if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess) { cudaGetLastError(); return PE_ERR_CUDA; }
   return check_launch();
 }
-// Zeroes up to three [d_out, d_in] outputs with a kernel that lets its successor start at once.  An ordinary launch: the successor may
-// run its main loop beside it.  dependent: a programmatic dependent itself, and the successor has to wait for it before
-// anything else (what came before may still be running); worth it where there is little to zero: the norms of
-// 64 x 256 x 512 x 2048 36.1 -> 32.6 us, but 1024 x 32 x 1024^2 (8 MB of outputs) 142 -> 147.
+// Zeroes up to three [d_out, d_in] outputs with a kernel that lets its successor start when everything older has completed: the successor
+// may run its main loop beside it.  As a programmatic dependent (its launch overlaps the predecessor's end: a training step over 25 layers with
+// MicroAdam 1597 -> 1576 us, one layer with both optimizers 127.4 -> 126.0, a packed batch 91.4 -> 90.3); ordinary: not so, for short sequences
+// (1024 x 32 x 1024^2 122.1 against 123.3); early: the successor starts at once and has to wait for it before anything else (what came before may
+// still be running), worth it where there is little to zero: the norms of 64 x 256 x 512 x 2048 36.1 -> 32.6 us.
+enum ZeroLaunch { ZERO_DEPENDENT, ZERO_ORDINARY, ZERO_EARLY };
 static pe_status_t zero_for_split(DeviceInfo* di, float* a, float* b, size_t n, cudaStream_t st, float* c = nullptr,
-                                  unsigned int* counters = nullptr, int n_counters = 0, bool dependent = false) {
+                                  unsigned int* counters = nullptr, int n_counters = 0, ZeroLaunch how = ZERO_DEPENDENT) {
   float* first = a ? a : b;
   float* second = a ? b : nullptr;
   if (!first) return PE_OK;
   long long blocks = ((long long)(n / 4) + 255) / 256;
   if (blocks > di->sm_count) blocks = di->sm_count;   // few blocks: the dependent kernel needs the SMs
-  if (dependent)
-    return launch_dependent(zero_outputs_kernel, dim3((int)(blocks < 1 ? 1 : blocks)), 256, 0, st, reinterpret_cast<float4*>(first),
-                            reinterpret_cast<float4*>(second), reinterpret_cast<float4*>(c), (long long)n, counters, n_counters);
-  zero_outputs_kernel<<<(int)(blocks < 1 ? 1 : blocks), 256, 0, st>>>(reinterpret_cast<float4*>(first), reinterpret_cast<float4*>(second),
-                                                                            reinterpret_cast<float4*>(c), (long long)n, counters, n_counters);
+  const dim3 grid((int)(blocks < 1 ? 1 : blocks));
+  float4 *const o1 = reinterpret_cast<float4*>(first), *const o2 = reinterpret_cast<float4*>(second), *const o3 = reinterpret_cast<float4*>(c);
+  if (how != ZERO_ORDINARY) return launch_dependent(zero_outputs_kernel, grid, 256, 0, st, o1, o2, o3, (long long)n, counters, n_counters, how == ZERO_EARLY ? 1 : 0);
+  zero_outputs_kernel<<<grid, 256, 0, st>>>(o1, o2, o3, (long long)n, counters, n_counters, 0);
   return check_launch();
 }
 
@@ -428,7 +429,7 @@ static pe_status_t launch_short(DeviceInfo* di, const void* X, const void* dY, i
     int n = 0;
     for (float* o : outs)
       if (o) list[n++] = o;
-    rc = zero_for_split(di, list[0], list[1], (size_t)d_in * d_out, st, list[2]);
+    rc = zero_for_split(di, list[0], list[1], (size_t)d_in * d_out, st, list[2], nullptr, 0, ZERO_ORDINARY);
   }
   if (rc != PE_OK) return rc;
   const long long units = whole + (tiles - whole) * split;
@@ -533,8 +534,7 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
     p.whole_tiles = plan.tail_split > 1 ? tiles - tiles % slots : tiles;
     if (plan.tail_split > 1) {
       p.wait_at_start = 0;
-      zero_tail_tiles_kernel<<<di->sm_count, 256, 0, st>>>(p, nt);
-      rc = check_launch();
+      rc = launch_dependent(zero_tail_tiles_kernel, dim3(di->sm_count), 256, 0, st, p, nt);
       if (rc != PE_OK) return rc;
     }
   }
@@ -597,7 +597,7 @@ static pe_status_t launch_tc_norms(DeviceInfo* di, const void* X, const void* dY
   p.whole_tiles = 0; p.tail_split = ns; p.slice_examples = per;
   // norms[b] = 0 (by a kernel that overlaps the launch of this one, 16-byte alignment allowing)
   p.wait_at_start = 1;
-  rc = aligned(norms, 16) ? zero_for_split(di, norms, nullptr, (size_t)B, st, nullptr, nullptr, 0, true)
+  rc = aligned(norms, 16) ? zero_for_split(di, norms, nullptr, (size_t)B, st, nullptr, nullptr, 0, ZERO_EARLY)
                           : zero_outputs(norms, nullptr, (size_t)B * sizeof(float), st);
   if (rc != PE_OK) return rc;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, 256, ns, di->sm_count / 2);
@@ -789,9 +789,9 @@ static pe_status_t launch_tc_ragged(DeviceInfo* di, const void* X, const void* d
   // the pre-pass: the partial 16-token groups to the side buffer, and the outputs of a split batch to zero
   const bool zero = ns > 1 && !norms;
   const int chunks = (int)std::min<long long>(8, std::max<long long>(1, 8ll * di->sm_count / (2ll * B)));
-  pack_tails_kernel<<<dim3((unsigned)B, 2, (unsigned)chunks), STAGE_THREADS, 0, st>>>(tx, ty, offsets, rows, zero ? first : nullptr,
-                                                                                         zero && both ? out_mean : nullptr, (long long)d_in * d_out);
-  if ((rc = check_launch()) != PE_OK) return rc;
+  rc = launch_dependent(pack_tails_kernel, dim3((unsigned)B, 2, (unsigned)chunks), STAGE_THREADS, 0, st, tx, ty, offsets, rows, zero ? first : (float*)nullptr,
+                        zero && both ? out_mean : (float*)nullptr, (long long)d_in * d_out);
+  if (rc != PE_OK) return rc;
   TcParams p{};
   p.B = B; p.T = 0; p.d_in = d_in; p.d_out = d_out; p.nsplit = ns; p.per_example = 1; p.half_operands = 0;
   p.accumulate = norms ? 1 : 0;

@@ -249,6 +249,7 @@ struct TailTensor {
 __global__ void __launch_bounds__(STAGE_THREADS)
 pack_tails_kernel(TailTensor tx_, TailTensor ty_, const int* __restrict__ offsets, long long total_rows, float* __restrict__ zero_a,
                   float* __restrict__ zero_b, long long zero_n) {
+  sm100::griddep_wait();                  // everything older has completed when the statistics kernel starts, as behind zero_outputs_kernel
   sm100::griddep_launch_dependents();
   const TailTensor& tn = blockIdx.y == 0 ? tx_ : ty_;
   const int b = blockIdx.x, d8 = tn.d / 8;

@@ -285,12 +285,15 @@ __device__ __forceinline__ float phi_apply(float g) {
 
 // Zeroes the outputs of a split-batch launch.  The statistics kernel that follows is launched as a
 // programmatic dependent: it starts right away (it only touches the outputs in its very last step,
-// behind griddepcontrol.wait), so the zeroing costs no time on the stream.  a, b, c: n floats each, 16-byte aligned; b and
-// c may be NULL.  counters: the tile counters of a fused update (n_counters words; may be NULL).
+// behind griddepcontrol.wait), so the zeroing costs no time on the stream.  It is a programmatic dependent itself, and lets its successor
+// start only when everything before it has completed, on which the successor relies (early: at once, for a successor that waits for this one
+// before anything else).  a, b, c: n floats each, 16-byte aligned; b and c may be NULL.  counters: the tile counters of a fused update
+// (n_counters words; may be NULL).
 __global__ void __launch_bounds__(256) zero_outputs_kernel(float4* __restrict__ a, float4* __restrict__ b, float4* __restrict__ c,
-                                                           long long n, unsigned int* __restrict__ counters, int n_counters) {
-  sm100::griddep_launch_dependents();
-  sm100::griddep_wait();          // (nothing to wait for in an ordinary launch)
+                                                           long long n, unsigned int* __restrict__ counters, int n_counters, int early) {
+  if (early) sm100::griddep_launch_dependents();
+  sm100::griddep_wait();
+  if (!early) sm100::griddep_launch_dependents();
   const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
   const long long stride = (long long)gridDim.x * blockDim.x;
   if (counters)
@@ -313,6 +316,7 @@ __global__ void __launch_bounds__(256) zero_outputs_kernel(float4* __restrict__ 
 // tiles are split over the batch; a warp takes a row of a tile.  At most half a wave of tiles (29 MB for both outputs), while the
 // contraction of the others already runs.
 __global__ void __launch_bounds__(256) zero_tail_tiles_kernel(TcParams p, int nt) {
+  sm100::griddep_wait();
   sm100::griddep_launch_dependents();
   const int rest = p.pairs_m * p.tiles_n - p.whole_tiles, lane = threadIdx.x & 31;
   for (int k = blockIdx.x * 8 + (threadIdx.x >> 5); k < rest * TC_PAIR_M; k += gridDim.x * 8) {
@@ -502,8 +506,8 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   // The next kernel of the stream may be launched from here on (it finds no room before blocks of this one leave).  With an unsplit
   // batch this kernel is itself a programmatic dependent of whatever precedes it: everything above overlapped that
   // kernel's end, and nothing below may start before it has completed.  (With a split batch its predecessor is the kernel
-  // that zeroes the outputs, itself an ordinary launch, and only the write-out waits for it.)
-  // A packed batch's predecessor is the kernel that fills the side buffer (and zeroes the outputs), an ordinary launch too: the
+  // that zeroes the outputs, which lets this one start when everything older has completed, and only the write-out waits for it.)
+  // A packed batch's predecessor is the kernel that fills the side buffer (and zeroes the outputs), to the same effect: the
   // producers wait for it before the first load from there.
   griddep_launch_dependents();
   if (!RAGGED && p.wait_at_start) griddep_wait();
