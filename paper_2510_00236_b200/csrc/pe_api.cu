@@ -609,38 +609,54 @@ static pe_status_t launch_tc_norms(DeviceInfo* di, const void* X, const void* dY
   return launch_tc_inst<1, false, 256, MEAN_NORMS>(di, 11, mx, my, mx, mx, mx, p, dim3(2 * pairs_m * tiles_n, 1, ns), st);
 }
 
-// Tile and batch slices of a SIMT launch: the cheapest by an estimate in microseconds, fitted to a sweep of all tiles and slice
-// counts over 14 layers from 48 x 48 to 1024 x 1024 (the choice within 6 % of the sweep's best, geometric mean).  A chunk of
+// Tile and batch slices of a SIMT launch: the cheapest by an estimate in microseconds, fitted to sweeps of all tiles and slice
+// counts over layers from 48 x 48 to 1100 x 1100 (the choice 5 % above the sweep's best, geometric mean).  A chunk of
 // tokens costs its FMAs times the blocks that share the SM, but for a block alone at least that and a latency.
+constexpr int SIMT_MAX_D_OUT = 65535 * 128;
 struct SimtPlan {
-  int tile, slices, cluster;      // tile: index into the four shapes, largest first
+  int tile, slices, cluster;      // tile: index into the five shapes
 };
-static SimtPlan plan_simt(DeviceInfo* di, int mode, int B, int T, int d_in, int d_out) {
-  static constexpr int rows[4] = {SimtTile84::ROWS, SimtTile44::ROWS, SimtTile22::ROWS, SimtTile11::ROWS};
-  static constexpr int cols[4] = {SimtTile84::COLS, SimtTile44::COLS, SimtTile22::COLS, SimtTile11::COLS};
-  static constexpr int kt[4] = {SimtTile84::KT, SimtTile44::KT, SimtTile22::KT, SimtTile11::KT};
-  static constexpr int per_sm[4] = {2, 2, 3, 4};                      // blocks an SM holds
-  static constexpr double chunk_us[4] = {1.95, 0.60, 0.85, 0.80};     // a full chunk's FMAs, one block
-  static constexpr double latency_us[4] = {0.25, 0.35, 0.45, 0.50};
-  static constexpr double fold_us[4] = {0.35, 0.10, 0.05, 0.05};      // phi and the sums at the end of an example
+static SimtPlan plan_simt(DeviceInfo* di, int mode, bool two_sums, int B, int T, int d_in, int d_out) {
+  constexpr int HALF = 4;
+  static constexpr int rows[5] = {SimtTile84::ROWS, SimtTile44::ROWS, SimtTile22::ROWS, SimtTile11::ROWS, SimtTileHalf<MODE_STATS>::ROWS};
+  static constexpr int cols[5] = {SimtTile84::COLS, SimtTile44::COLS, SimtTile22::COLS, SimtTile11::COLS, SimtTileHalf<MODE_STATS>::COLS};
+  const int kt[5] = {SimtTile84::KT, SimtTile44::KT, SimtTile22::KT, SimtTile11::KT, mode == MODE_TOKEN ? SimtTileHalf<MODE_TOKEN>::KT : SimtTileHalf<MODE_STATS>::KT};
+  static constexpr int per_sm[5] = {2, 2, 3, 4, 4};                           // blocks an SM holds
+  static constexpr double chunk_us[5] = {1.95, 0.60, 0.85, 0.80, 0.46};       // a full chunk's FMAs, one block
+  static constexpr double latency_us[5] = {0.25, 0.35, 0.45, 0.50, 0.0};
+  static constexpr double fold_us[5] = {0.35, 0.10, 0.05, 0.05, 0.0};         // phi and the sums at the end of an example
   const bool by_rows = mode == MODE_TOKEN;                            // what the slices divide: rows or examples
   const long long units = by_rows ? (long long)B * T : B;
+  const int loose = (d_in % 4 != 0) + (d_out % 4 != 0);
   SimtPlan best = {0, 1, 1};
   double best_cost = 1e300;
-  for (int k = 0; k < 4; ++k) {
+  for (int k = 0; k < 5; ++k) {
     const long long tiles = (long long)((d_in + cols[k] - 1) / cols[k]) * ((d_out + rows[k] - 1) / rows[k]);
     for (int s = 1; s <= 32 && s <= units; s *= 2) {
       const long long blocks = tiles * s, slots = (long long)per_sm[k] * di->sm_count;
-      double sharing = (double)std::min<long long>(per_sm[k], (blocks + di->sm_count - 1) / di->sm_count);
-      if (k == 0 && s >= SIMT_MAX_CLUSTER && blocks <= di->sm_count) sharing = 1.5;      // clusters of eight are placed densely
       const long long per = (units + s - 1) / s;
       const double tokens = (double)(by_rows ? per : (long long)T), whole = std::floor(tokens / kt[k]);
       const double rest = (double)(((long long)(tokens - whole * kt[k]) + 7) / 8 * 8) / kt[k];
-      auto chunk = [&](double f) { return std::max(sharing * chunk_us[k] * f, latency_us[k] + chunk_us[k] * f); };
-      double walk = whole * chunk(1.0) + (rest > 0.0 ? chunk(rest) : 0.0);
-      if (!by_rows) walk = per * (walk + fold_us[k] * sharing);
-      const double waves = (double)((blocks + slots - 1) / slots);
-      const double cost = waves * (walk + 2.0) + 1.5 + 0.12 * s + (s > SIMT_MAX_CLUSTER ? 3.0 : 0.0);
+      double cost;
+      if (k == HALF) {
+        // whole rounds of blocks, then those that are left: blocks that share an SM take turns, one alone is as long as 1.27
+        const double chunk = by_rows ? 2 * chunk_us[k] : chunk_us[k], edge = 0.195 + 0.075 * loose, fold = by_rows ? 0.0 : two_sums ? 0.294 : 0.05;
+        auto round = [&](double together) {
+          const double share = std::max(together, 1.27);
+          return (by_rows ? 1.0 : (double)per) * (((whole + rest) * chunk + fold) * share + (whole + (rest > 0.0 ? 1.0 : 0.0)) * edge) + 4.7;
+        };
+        const long long most = (blocks + di->sm_count - 1) / di->sm_count, left = most % per_sm[k];
+        cost = (double)(most / per_sm[k]) * round(per_sm[k]) + (left ? round((double)left) : 0.0) + 1.86 + (s > 1 ? 1.475 : 0.0) + (s > SIMT_MAX_CLUSTER ? 5.0 : 0.0);
+        cost *= 0.88;          // (both estimates are high; chosen only where it is the faster one: at 70 layers never more than 2 % behind)
+      } else {
+        double sharing = (double)std::min<long long>(per_sm[k], (blocks + di->sm_count - 1) / di->sm_count);
+        if (k == 0 && s >= SIMT_MAX_CLUSTER && blocks <= di->sm_count) sharing = 1.5;      // clusters of eight are placed densely
+        auto chunk = [&](double f) { return std::max(sharing * chunk_us[k] * f, latency_us[k] + chunk_us[k] * f); };
+        double walk = whole * chunk(1.0) + (rest > 0.0 ? chunk(rest) : 0.0);
+        if (!by_rows) walk = per * (walk + fold_us[k] * sharing);
+        const double waves = (double)((blocks + slots - 1) / slots);
+        cost = waves * (walk + 2.0) + 1.5 + 0.12 * s + (s > SIMT_MAX_CLUSTER ? 3.0 : 0.0);
+      }
       if (cost < best_cost) { best_cost = cost; best = {k, s, s < SIMT_MAX_CLUSTER ? s : SIMT_MAX_CLUSTER}; }
     }
   }
@@ -667,9 +683,10 @@ static pe_status_t launch_simt_inst(const SimtPlan& plan, const TIn* X, const TI
   const size_t group = 4 * sizeof(TIn);
   const int vec_x = ldx % 4 == 0 && aligned(X, group) ? 1 : 0, vec_y = ldy % 4 == 0 && aligned(dY, group) ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((d_in + Tile::COLS - 1) / Tile::COLS, (d_out + Tile::ROWS - 1) / Tile::ROWS, plan.slices);
-  cfg.blockDim = dim3(SIMT_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  if (cfg.gridDim.y > 65535) return PE_ERR_DIM;
+  const long long tiles = (long long)((d_in + Tile::COLS - 1) / Tile::COLS) * ((d_out + Tile::ROWS - 1) / Tile::ROWS);
+  if (d_out > SIMT_MAX_D_OUT || tiles >= (1ll << 31)) return PE_ERR_DIM;
+  cfg.gridDim = dim3((unsigned)tiles, 1, plan.slices);
+  cfg.blockDim = dim3(Tile::THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeClusterDimension;
   attr.val.clusterDim.x = 1; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = plan.cluster;
@@ -686,9 +703,9 @@ static pe_status_t launch_simt(DeviceInfo* di, const TIn* X, const TIn* dY, int 
                                float* out_mean, float* out_stat, cudaStream_t st, bool accumulate = false, SimtExtra ex = SimtExtra{},
                                const FusedOpt* opt = nullptr, int pitch_x = 0, int pitch_y = 0) {
   const int ldx = pitch_x ? pitch_x : d_in, ldy = pitch_y ? pitch_y : d_out;
-  SimtPlan plan = plan_simt(di, MODE, B, T, d_in, d_out);
+  const bool two_sums = out_mean || (opt && opt->kind == OPT_ADAM);
+  SimtPlan plan = plan_simt(di, MODE, two_sums, B, T, d_in, d_out);
   if (opt && plan.slices > SIMT_MAX_CLUSTER) plan.slices = SIMT_MAX_CLUSTER;      // a fused update needs the whole batch in one cluster
-  if ((d_out + SimtTile11::ROWS - 1) / SimtTile11::ROWS > 65535 && plan.tile > 0) plan.tile = 0;      // gridDim.y
   if (MODE != MODE_NORMS && plan.slices > plan.cluster && !accumulate) {
     pe_status_t rc = zero_outputs(out_mean, out_stat, (size_t)d_in * d_out * sizeof(float), st);
     if (rc != PE_OK) return rc;
@@ -697,7 +714,7 @@ static pe_status_t launch_simt(DeviceInfo* di, const TIn* X, const TIn* dY, int 
   auto run = [&](auto tile) {
     using Tile = decltype(tile);
     if constexpr (MODE == MODE_STATS) {
-      if (out_mean || (opt && opt->kind == OPT_ADAM))
+      if (two_sums)
         return launch_simt_inst<TIn, MODE, Tile, 2>(plan, X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, st, accumulate, ldx, ldy, ex, o);
     }
     return launch_simt_inst<TIn, MODE, Tile, 1>(plan, X, dY, B, T, d_in, d_out, phi, out_mean, out_stat, st, accumulate, ldx, ldy, ex, o);
@@ -706,6 +723,7 @@ static pe_status_t launch_simt(DeviceInfo* di, const TIn* X, const TIn* dY, int 
     case 0: return run(SimtTile84{});
     case 1: return run(SimtTile44{});
     case 2: return run(SimtTile22{});
+    case 4: return run(SimtTileHalf<MODE>{});
     default: return run(SimtTile11{});
   }
 }

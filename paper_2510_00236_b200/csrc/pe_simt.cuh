@@ -9,33 +9,35 @@
 // contracted, across example boundaries, and the two chunk buffers need one barrier per chunk.  The batch is
 // split over the blocks of a cluster, whose partial sums meet in shared memory: nothing is zeroed first, no
 // atomics, and the result does not depend on timing (more slices than a cluster holds fall back to atomics).
-// Measured, both outputs: 8 x 256 tokens x 1024 x 16384 46 TFLOP/s; 32 x 128 x 256 x 1024 157.8 -> 75 us, 8 x 16 x 64 x 64
-// 18.7 -> 11.4 us per call, against a 64 x 64 tile of 4 x 4 entries, one buffer and scalar reads.  Not faster: 8 x 8 entries
-// (one block per SM, 38 TFLOP/s), scalar FMAs (42), two tokens instead of two columns per packed FMA (spills, 30), 16-token
-// chunks (the barrier twice as often, 32 against 34 at 8 x 256 x 1024 x 2048).
+// Measured, both outputs, against a 64 x 64 tile of 4 x 4 entries, one buffer and scalar reads: 32 x 128 x 256 x 1024 157.8 -> 65 us, 8 x 16 x 64 x 64
+// 18.7 -> 11.4 us per call; 8 x 256 x 1024 x 16384 1438 us, 48 TFLOP/s (packed FMAs from shared memory alone, in a loop: 61; of the difference a
+// seventh are the warps that wait at the chunks' barrier).  Not faster: 8 x 8 entries (one block per SM, 38 TFLOP/s), scalar FMAs (42), packed FMAs
+// over diagonals of 2 x 2 entries, which need no doubled operands (3 to 6 % slower), clusters of 16, 16-token chunks of the largest tile.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "pe_optim.cuh"
 #include "pe_sm100.cuh"
 
 namespace pe {
 
-constexpr int SIMT_THREADS = 256;       // 16 x 16 threads
 constexpr int SIMT_MAX_CLUSTER = 8;     // batch slices whose partial sums meet in shared memory
 
 enum : int { MODE_STATS = 0, MODE_TOKEN = 1, MODE_NORMS = 2 };
 
 // Tile shapes.  TM x TN entries per thread; KT tokens per chunk.  The large tile has the most FMAs per shared-memory
 // read, the small ones spread a small layer over the chip.
-template <int TM_, int TN_, int KT_>
+template <int TM_, int TN_, int KT_, int THREADS_ = 256>
 struct SimtTile {
-  static constexpr int TM = TM_, TN = TN_, KT = KT_;
-  static constexpr int ROWS = 16 * TM, COLS = 16 * TN;
+  static constexpr int TM = TM_, TN = TN_, KT = KT_, THREADS = THREADS_;
+  static constexpr int TY = THREADS / 16;                        // TY x 16 threads
+  static constexpr int ROWS = TY * TM, COLS = 16 * TN;
   static constexpr int CHUNK = KT * (ROWS + COLS);               // floats of one chunk: dY part, then X part
-  static constexpr int YV = KT * ROWS / 4 / SIMT_THREADS, XV = KT * COLS / 4 / SIMT_THREADS;   // 4-column groups per thread
-  static_assert(YV * 4 * SIMT_THREADS == KT * ROWS && XV * 4 * SIMT_THREADS == KT * COLS, "whole groups per thread");
+  static constexpr int YV = KT * ROWS / 4 / THREADS, XV = KT * COLS / 4 / THREADS;   // 4-column groups per thread
+  static_assert(YV * 4 * THREADS == KT * ROWS && XV * 4 * THREADS == KT * COLS, "whole groups per thread");
   // the largest tile keeps its running sums in shared memory (64 registers of sums beside 32 of G_b would leave one block per SM)
   static constexpr bool SUMS_IN_SMEM = TM * TN > 16;
   // the chunk buffers; the sums' exchange at the end lies behind them where the sums live there, on top of them otherwise
@@ -44,6 +46,11 @@ struct SimtTile {
   }
 };
 using SimtTile84 = SimtTile<8, 4, 32>;
+// Half of the largest tile in blocks of half the threads, four to an SM: the same FMAs per read in twice as many pieces, which spread layers of a
+// few hundred rows and columns more evenly.  10 x 200 x 800 x 400, both outputs, 78 -> 64 us, 64 x 32 x 500 x 300 43 -> 35, 8 x 256 x 1024 x 2048 255 -> 215,
+// and per token 230 -> 177.  Shorter chunks beside running sums, whose shared memory would leave room for three blocks.
+template <int MODE>
+using SimtTileHalf = SimtTile<8, 4, MODE == MODE_TOKEN ? 32 : 16, 128>;
 using SimtTile44 = SimtTile<4, 4, 16>;
 using SimtTile22 = SimtTile<2, 2, 32>;
 using SimtTile11 = SimtTile<1, 1, 64>;
@@ -84,8 +91,9 @@ __device__ __forceinline__ float4 load_group(const __nv_bfloat16* p, int left, b
   return make_float4(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]), __uint_as_float(w[3]));
 }
 
-// A thread's N operands of one token: N = 1, 2 or 4 consecutive floats, 8 as two groups of four, 64 floats apart.
-template <int N>
+// A thread's N operands of one token: N = 1, 2 or 4 consecutive floats, 8 as two groups of four, 4 * SIDE floats apart (SIDE: threads on this
+// side of the tile).
+template <int N, int SIDE>
 __device__ __forceinline__ void lds_vec(const float* p, float (&v)[N]) {
   if constexpr (N == 1) {
     v[0] = *p;
@@ -95,21 +103,21 @@ __device__ __forceinline__ void lds_vec(const float* p, float (&v)[N]) {
   } else {
 #pragma unroll
     for (int h = 0; h < N / 4; ++h) {
-      const float4 t = *reinterpret_cast<const float4*>(p + 64 * h);
+      const float4 t = *reinterpret_cast<const float4*>(p + 4 * SIDE * h);
       v[4 * h] = t.x; v[4 * h + 1] = t.y; v[4 * h + 2] = t.z; v[4 * h + 3] = t.w;
     }
   }
 }
 // Tile row (column) of entry j of a thread's N: the layout lds_vec reads.
-template <int N>
-__device__ __forceinline__ int micro_index(int thread, int j) { return N <= 4 ? thread * N + j : thread * 4 + (j & 3) + 64 * (j >> 2); }
+template <int N, int SIDE>
+__device__ __forceinline__ int micro_index(int thread, int j) { return N <= 4 ? thread * N + j : thread * 4 + (j & 3) + 4 * SIDE * (j >> 2); }
 
 // MODE_STATS: out_mean = sum_b G_b, out_stat = sum_b phi(G_b)         (Section 2.3, Eq. (2))
 // MODE_TOKEN: out_stat = sum_{b,t} dY^2 X^2; operands are squared as they are staged and the
 //             accumulator is never reset between examples             (Section 2.3, per-token form)
 // MODE_NORMS: out_stat is a [B] array, zero on entry; every tile adds its share of ||G_b||_F^2 to
 //             out_stat[b] (Section 2.3, per-example squared norms); no [d_out, d_in] output
-// gridDim = (ceil(d_in/COLS), ceil(d_out/ROWS), slices) in clusters of (1, 1, cluster), cluster a power of two that divides
+// gridDim = (ceil(d_in/COLS) * ceil(d_out/ROWS), 1, slices) in clusters of (1, 1, cluster), cluster a power of two that divides
 // slices; slice z handles examples [z*B/slices, (z+1)*B/slices), or that share of the B*T rows (MODE_TOKEN).  With more
 // slices than one cluster the outputs must be zero on entry and the clusters' sums are added atomically; with
 // accumulate != 0 the results are added to whatever the outputs hold.  opt.kind != 0 (one cluster only): the block that
@@ -118,7 +126,7 @@ __device__ __forceinline__ int micro_index(int thread, int j) { return N <= 4 ? 
 // ldx, ldy: elements from one token's row of X, dY to the next.
 // SUMS: running sums per entry: 2 = sum_b phi(G_b) and sum_b G_b, 1 = the former alone (or the contraction of MODE_TOKEN).
 template <typename TIn, int MODE, class Tile, int SUMS>
-__global__ void __launch_bounds__(SIMT_THREADS, 2)
+__global__ void __launch_bounds__(Tile::THREADS, 512 / Tile::THREADS)
 simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, int T, int d_in, int d_out,
                   int phi, float* __restrict__ out_mean, float* __restrict__ out_stat, int accumulate, int cluster, int ldx, int ldy, int vec_x, int vec_y,
                   SimtExtra ex, FusedOpt opt) {
@@ -127,7 +135,8 @@ simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, 
   extern __shared__ __align__(16) float simt_smem[];
   // a warp is 4 x 8 threads of the 16 x 16: four distinct operands of dY and eight of X per shared-memory read
   const int tx = (threadIdx.x & 7) | ((threadIdx.x >> 2) & 8), ty = ((threadIdx.x >> 3) & 3) | ((threadIdx.x >> 6) << 2);
-  const int i0 = blockIdx.x * COLS, o0 = blockIdx.y * ROWS;
+  const int tiles_in = (d_in + COLS - 1) / COLS;
+  const int i0 = (int)(blockIdx.x % tiles_in) * COLS, o0 = (int)(blockIdx.x / tiles_in) * ROWS;
   const int slices = gridDim.z;
 
   // g: this thread's entries of G_b.  Running sums ([0] = the statistic, [1] = sum_b G_b) in registers, or, IN_SMEM, in a
@@ -135,7 +144,7 @@ simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, 
   float g[TM][TN];
   float sum[IN_SMEM ? 1 : SUMS][TM][TN];
   float* const smem_sums = simt_smem + 2 * Tile::CHUNK;
-  auto slot = [&](int s, int r, int c4) { return reinterpret_cast<float4*>(smem_sums) + ((s * TM + r) * (TN / 4) + c4) * SIMT_THREADS + threadIdx.x; };
+  auto slot = [&](int s, int r, int c4) { return reinterpret_cast<float4*>(smem_sums) + ((s * TM + r) * (TN / 4) + c4) * Tile::THREADS + threadIdx.x; };
 #pragma unroll
   for (int r = 0; r < TM; ++r) {
 #pragma unroll
@@ -185,8 +194,8 @@ simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, 
 
   // A thread's groups of a chunk lie in one column, Y_STEP and X_STEP tokens apart, so that a chunk's addresses take one multiplication per
   // operand: spelled out per group, their 64-bit multiplications were a fifth of the FMA pipe's work.
-  constexpr int Y_STEP = 4 * SIMT_THREADS / ROWS, X_STEP = 4 * SIMT_THREADS / COLS;
-  static_assert(Y_STEP * ROWS == 4 * SIMT_THREADS && X_STEP * COLS == 4 * SIMT_THREADS, "whole rows of groups per round");
+  constexpr int Y_STEP = 4 * Tile::THREADS / ROWS, X_STEP = 4 * Tile::THREADS / COLS;
+  static_assert(Y_STEP * ROWS == 4 * Tile::THREADS && X_STEP * COLS == 4 * Tile::THREADS, "whole rows of groups per round");
   const int y_tok = threadIdx.x / (ROWS / 4), x_tok = threadIdx.x / (COLS / 4);
   const int y_col = o0 + 4 * (threadIdx.x % (ROWS / 4)), x_col = i0 + 4 * (threadIdx.x % (COLS / 4));
   const bool y_whole = vec_y != 0 && y_col + 3 < d_out, x_whole = vec_x != 0 && x_col + 3 < d_in;
@@ -271,9 +280,9 @@ simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, 
     float* const y = simt_smem + buf * Tile::CHUNK;
     float* const x = y + KT * ROWS;
 #pragma unroll
-    for (int k = 0; k < Tile::YV; ++k) put(y + 4 * (threadIdx.x + k * SIMT_THREADS), sy[k]);
+    for (int k = 0; k < Tile::YV; ++k) put(y + 4 * (threadIdx.x + k * Tile::THREADS), sy[k]);
 #pragma unroll
-    for (int k = 0; k < Tile::XV; ++k) put(x + 4 * (threadIdx.x + k * SIMT_THREADS), sx[k]);
+    for (int k = 0; k < Tile::XV; ++k) put(x + 4 * (threadIdx.x + k * Tile::THREADS), sx[k]);
     __syncthreads();           // a buffer is written again two chunks later, behind the barrier that follows its last reads
     // the next chunk's loads are in flight during this one's arithmetic
     t += KT;
@@ -284,14 +293,14 @@ simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, 
     }
     more = b < b_end;
     if (more) load_chunk();
-    // tokens past the example's end are zero: whole groups of 8 of them are skipped
-#pragma unroll 1
-    for (int k0 = 0; k0 < KT && k0 < left; k0 += 8) {
+    // tokens past the example's end are zero: whole groups of 8 of them are skipped.  (A whole chunk without a loop: the reads of one group overlap the
+    // FMAs of the one before; 3 to 5 %.)
+    auto tokens = [&](auto count, int k0) {
 #pragma unroll
-      for (int kk = 0; kk < 8; ++kk) {
+      for (int kk = 0; kk < decltype(count)::value; ++kk) {
         float yv[TM], xv[TN];
-        lds_vec<TM>(y + (k0 + kk) * ROWS + (TM < 4 ? TM : 4) * ty, yv);
-        lds_vec<TN>(x + (k0 + kk) * COLS + (TN < 4 ? TN : 4) * tx, xv);
+        lds_vec<TM, Tile::TY>(y + (k0 + kk) * ROWS + (TM < 4 ? TM : 4) * ty, yv);
+        lds_vec<TN, 16>(x + (k0 + kk) * COLS + (TN < 4 ? TN : 4) * tx, xv);
 #pragma unroll
         for (int r = 0; r < TM; ++r) {
           if constexpr (TN >= 2) {
@@ -306,6 +315,12 @@ simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, 
           }
         }
       }
+    };
+    if (left >= KT) {
+      tokens(std::integral_constant<int, KT>{}, 0);
+    } else {
+#pragma unroll 1
+      for (int k0 = 0; k0 < left; k0 += 8) tokens(std::integral_constant<int, 8>{}, k0);
     }
     if (ends) fold(cur_b);
   }
@@ -328,7 +343,7 @@ simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, 
         for (int r = 0; r < TM; ++r)
 #pragma unroll
           for (int c4 = 0; c4 < TN / 4; ++c4)
-            *reinterpret_cast<float4*>(xch + (s * ROWS + micro_index<TM>(ty, r)) * COLS + micro_index<TN>(tx, 4 * c4)) = v[r][c4];
+            *reinterpret_cast<float4*>(xch + (s * ROWS + micro_index<TM, Tile::TY>(ty, r)) * COLS + micro_index<TN, 16>(tx, 4 * c4)) = v[r][c4];
       }
     } else {
       __syncthreads();         // the chunk buffers are idle from here on
@@ -338,7 +353,7 @@ simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, 
         for (int r = 0; r < TM; ++r)
 #pragma unroll
           for (int c = 0; c < TN; ++c)
-            xch[(s * ROWS + micro_index<TM>(ty, r)) * COLS + micro_index<TN>(tx, c)] = MODE == MODE_TOKEN ? g[r][c] : sum[s][r][c];
+            xch[(s * ROWS + micro_index<TM, Tile::TY>(ty, r)) * COLS + micro_index<TN, 16>(tx, c)] = MODE == MODE_TOKEN ? g[r][c] : sum[s][r][c];
     }
     if (cluster > 1) sm100::cluster_sync_all();
     else __syncthreads();
@@ -346,7 +361,7 @@ simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, 
     const bool add = slices > cluster || accumulate;
     const uint32_t local = sm100::smem_u32(xch);
     const int share = ROWS / cluster;         // rows this block finishes
-    for (int e = threadIdx.x; e < share * COLS; e += SIMT_THREADS) {
+    for (int e = threadIdx.x; e < share * COLS; e += Tile::THREADS) {
       const int r = rank * share + e / COLS, c = e % COLS;
       const int o = o0 + r, i = i0 + c;
       if (o >= d_out || i >= d_in) continue;
