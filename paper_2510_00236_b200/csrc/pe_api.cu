@@ -630,9 +630,11 @@ static SimtPlan plan_simt(DeviceInfo* di, int mode, bool two_sums, int B, int T,
   const int loose = (d_in % 4 != 0) + (d_out % 4 != 0);
   SimtPlan best = {0, 1, 1};
   double best_cost = 1e300;
+  int least = 1;             // slices: sums of all rows are not to grow longer, and with them their rounding error, for the last tile's sake
   for (int k = 0; k < 5; ++k) {
+    if (k == HALF && by_rows) least = best.slices;
     const long long tiles = (long long)((d_in + cols[k] - 1) / cols[k]) * ((d_out + rows[k] - 1) / rows[k]);
-    for (int s = 1; s <= 32 && s <= units; s *= 2) {
+    for (int s = least; s <= 32 && s <= units; s *= 2) {
       const long long blocks = tiles * s, slots = (long long)per_sm[k] * di->sm_count;
       const long long per = (units + s - 1) / s;
       const double tokens = (double)(by_rows ? per : (long long)T), whole = std::floor(tokens / kt[k]);

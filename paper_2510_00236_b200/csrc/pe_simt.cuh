@@ -47,8 +47,8 @@ struct SimtTile {
 };
 using SimtTile84 = SimtTile<8, 4, 32>;
 // Half of the largest tile in blocks of half the threads, four to an SM: the same FMAs per read in twice as many pieces, which spread layers of a
-// few hundred rows and columns more evenly.  10 x 200 x 800 x 400, both outputs, 78 -> 64 us, 64 x 32 x 500 x 300 43 -> 35, 8 x 256 x 1024 x 2048 255 -> 215,
-// and per token 230 -> 177.  Shorter chunks beside running sums, whose shared memory would leave room for three blocks.
+// few hundred rows and columns more evenly.  10 x 200 x 800 x 400, both outputs, 78 -> 64 us, 64 x 32 x 500 x 300 43 -> 35, 8 x 256 x 1024 x 2048 255 -> 208,
+// and per token 230 -> 187.  Shorter chunks beside running sums, whose shared memory would leave room for three blocks.
 template <int MODE>
 using SimtTileHalf = SimtTile<8, 4, MODE == MODE_TOKEN ? 32 : 16, 128>;
 using SimtTile44 = SimtTile<4, 4, 16>;
