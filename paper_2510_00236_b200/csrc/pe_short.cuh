@@ -11,8 +11,8 @@
 //    arithmetic; it arrives by a predicated instruction (a branch around it costs about 80 cycles).  Releasing and looking ahead took 300 cycles a unit.
 //  - Results leave through a panel of shared memory of their own (TMA stores, or adds for a slice of the batch), so that the operand ring is
 //    filled for the next tile meanwhile.  Adds from registers, lanes transposed, took 7 us per tile and two sums.
-// 1024 x 32 tokens x 1024^2: both outputs 135 -> 110 us (clock cycles a unit: 901 -> 750), sign 166 -> 155, square 98 -> 89, three statistics
-// 275 -> 244; 128 x 32 x 4096^2: 219 -> 196, 304 -> 270, 178 -> 153, 472 -> 429; 512 x 2 x 1024^2: 72 -> 58, 92 -> 81, .. , 142 -> 127.
+// 1024 x 32 tokens x 1024^2: both outputs 135 -> 110 us (clock cycles a unit: 901 -> 750), sign 166 -> 155, square 98 -> 92, three statistics
+// 275 -> 244; 128 x 32 x 4096^2: 219 -> 196, 304 -> 270, 178 -> 160, 472 -> 429; 512 x 2 x 1024^2: 72 -> 58, 92 -> 81, .. , 142 -> 127.
 // (before: stages and accumulators of tc_stats_kernel with two examples each).  What is left above the arithmetic is the two units' round trip
 // from release to the next unit's reads, about 780 cycles at T = 32.  Measured and dropped: signs counted from the sign bits by byte
 // permutes and 16-bit adds with zeros looked for by three-way minima (three statistics 244 -> 228 us where G_b holds no zeros, but every zero
@@ -29,6 +29,7 @@ constexpr int SHORT_A_BOX = SHORT_G * SHORT_T * 128;              // 64 rows of 
 constexpr int SHORT_B_BOX = SHORT_G * SHORT_T * 128;              // 64 columns of X: 8 KiB
 constexpr int SHORT_STAGE = 2 * SHORT_A_BOX + SHORT_B_BOX;        // 24 KiB
 constexpr int SHORT_STAGES = 8;
+constexpr int SHORT_RUN = 16;                       // examples summed by themselves where the square alone is wanted
 constexpr int SHORT_UNITS = TC_TMEM_COLS / (SHORT_G * SHORT_NT);  // accumulator units in tensor memory: 2
 constexpr int SHORT_PANEL = 4096;                   // per epilogue warp: 32 x 32 results on their way out
 constexpr int SHORT_RING = SHORT_STAGES * SHORT_STAGE + 8 * SHORT_PANEL;
@@ -154,11 +155,16 @@ short_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     constexpr bool COUNT = SIGN && SQUARE;
     float acc_mean[MEAN ? COLS : 1], acc_stat[SQUARE || SIGN ? COLS : 1];
     uint32_t acc_cnt[COUNT ? COLS / 2 : 1];
+    // The square alone: SHORT_RUN examples at a time in sums of their own.  This tile leaves more of the batch to a pair than the 256 x 256 tile of
+    // tc_stats_kernel does, and plain sums would round more often than there.
+    constexpr bool RUNS = SQUARE && !MEAN && !SIGN;
+    float acc_run[RUNS ? COLS : 1];
     auto clear = [&]() {
 #pragma unroll
       for (int j = 0; j < COLS; ++j) {
         if (MEAN) acc_mean[j] = 0.f;
         if (SQUARE || SIGN) acc_stat[j] = 0.f;
+        if (RUNS) acc_run[j] = 0.f;
         if (COUNT && j % 2 == 0) acc_cnt[j / 2] = 0u;
       }
     };
@@ -225,10 +231,23 @@ short_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             const uint64_t g2 = f32x2_pack(__uint_as_float(gk[j]), __uint_as_float(gk[j + 1]));
             const uint64_t f2 = f32x2_pack(__uint_as_float(fk[j]), __uint_as_float(fk[j + 1]));
             if constexpr (MEAN) f32x2_unpack(f32x2_add(f32x2_add(f32x2_pack(acc_mean[c], acc_mean[c + 1]), g2), f2), acc_mean[c], acc_mean[c + 1]);
-            if constexpr (SQUARE) f32x2_unpack(f32x2_fma(f2, f2, f32x2_fma(g2, g2, f32x2_pack(acc_stat[c], acc_stat[c + 1]))), acc_stat[c], acc_stat[c + 1]);
+            if constexpr (SQUARE) {
+              float& s0 = RUNS ? acc_run[RUNS ? c : 0] : acc_stat[c];
+              float& s1 = RUNS ? acc_run[RUNS ? c + 1 : 0] : acc_stat[c + 1];
+              f32x2_unpack(f32x2_fma(f2, f2, f32x2_fma(g2, g2, f32x2_pack(s0, s1))), s0, s1);
+            }
             if constexpr (COUNT) acc_cnt[c / 2] += signs_plus_two_packed(g2, f2);
             if constexpr (SIGN && !COUNT)
               f32x2_unpack(f32x2_add(f32x2_add(f32x2_pack(acc_stat[c], acc_stat[c + 1]), sign_half2(g2)), sign_half2(f2)), acc_stat[c], acc_stat[c + 1]);
+          }
+        }
+        if constexpr (RUNS) {
+          if ((b - t.b_begin) % SHORT_RUN == SHORT_RUN - SHORT_G || b + SHORT_G >= t.b_end) {
+#pragma unroll
+            for (int j = 0; j < COLS; j += 2) {
+              f32x2_unpack(f32x2_add(f32x2_pack(acc_stat[j], acc_stat[j + 1]), f32x2_pack(acc_run[j], acc_run[j + 1])), acc_stat[j], acc_stat[j + 1]);
+              acc_run[j] = acc_run[j + 1] = 0.f;
+            }
           }
         }
         buf ^= 1;
