@@ -311,13 +311,23 @@ static pe_status_t launch_dependent(Kernel kernel, dim3 grid, int threads, int s
   return check_launch();
 }
 // Zeroes up to three [d_out, d_in] outputs with a kernel that lets its successor start when everything older has completed: the successor
-// may run its main loop beside it.  As a programmatic dependent (its launch overlaps the predecessor's end: a training step over 25 layers with
-// MicroAdam 1597 -> 1576 us, one layer with both optimizers 127.4 -> 126.0, a packed batch 91.4 -> 90.3); ordinary: not so, for short sequences
-// (1024 x 32 x 1024^2 122.1 against 123.3); early: the successor starts at once and has to wait for it before anything else (what came before may
-// still be running), worth it where there is little to zero: the norms of 64 x 256 x 512 x 2048 36.1 -> 32.6 us.
-enum ZeroLaunch { ZERO_DEPENDENT, ZERO_ORDINARY, ZERO_EARLY };
+// may run its main loop beside it.  A programmatic dependent itself: 25 layers with MicroAdam 1597 -> 1576 us against ordinary launches, 1024 x 32 x 1024^2,
+// both outputs, 113 -> 110, 64 x 32 x 256 x 4096 18.6 -> 16.2.  early: the successor starts at once and has to wait for it before anything else (what came
+// before may still be running), worth it where there is little to zero: the norms of 64 x 256 x 512 x 2048 36.1 -> 32.6 us.
+// Shared memory that these kernels do not use, so that an SM takes one block: as dependents they would else crowd the SMs that become free first, and
+// zero 8 MB from there (64 x 256 x 512 x 2048, three statistics, calls one after the other, 47.2 us against 43.4; 45.2 as ordinary launches).
+constexpr int ZERO_SMEM = 120 * 1024;
+template <typename Kernel>
+static pe_status_t one_block_per_sm(DeviceInfo* di, int slot, Kernel kernel) {
+  std::lock_guard<std::mutex> lock(g_dev_mutex);
+  if (!di->tc_attr_set[slot]) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ZERO_SMEM) != cudaSuccess) { cudaGetLastError(); return PE_ERR_CUDA; }
+    di->tc_attr_set[slot] = true;
+  }
+  return PE_OK;
+}
 static pe_status_t zero_for_split(DeviceInfo* di, float* a, float* b, size_t n, cudaStream_t st, float* c = nullptr,
-                                  unsigned int* counters = nullptr, int n_counters = 0, ZeroLaunch how = ZERO_DEPENDENT) {
+                                  unsigned int* counters = nullptr, int n_counters = 0, bool early = false) {
   float* first = a ? a : b;
   float* second = a ? b : nullptr;
   if (!first) return PE_OK;
@@ -325,9 +335,11 @@ static pe_status_t zero_for_split(DeviceInfo* di, float* a, float* b, size_t n, 
   if (blocks > di->sm_count) blocks = di->sm_count;   // few blocks: the dependent kernel needs the SMs
   const dim3 grid((int)(blocks < 1 ? 1 : blocks));
   float4 *const o1 = reinterpret_cast<float4*>(first), *const o2 = reinterpret_cast<float4*>(second), *const o3 = reinterpret_cast<float4*>(c);
-  if (how != ZERO_ORDINARY) return launch_dependent(zero_outputs_kernel, grid, 256, 0, st, o1, o2, o3, (long long)n, counters, n_counters, how == ZERO_EARLY ? 1 : 0);
-  zero_outputs_kernel<<<grid, 256, 0, st>>>(o1, o2, o3, (long long)n, counters, n_counters, 0);
-  return check_launch();
+  if (!early) {
+    const pe_status_t rc = one_block_per_sm(di, 5, zero_outputs_kernel);
+    if (rc != PE_OK) return rc;
+  }
+  return launch_dependent(zero_outputs_kernel, grid, 256, early ? 0 : ZERO_SMEM, st, o1, o2, o3, (long long)n, counters, n_counters, early ? 1 : 0);
 }
 
 // mxt, myt: the maps of the zero-padded tail groups of a packed batch (RAGGED); any valid map otherwise.
@@ -365,6 +377,9 @@ static bool any_output(const LayoutZero& z) { return z.out[0] || z.out[1] || z.o
 
 // Statistics of short sequences (T <= SHORT_T).  out_mean, out_square, out_sign: those wanted; out_mean and out_sign with or without
 // out_square, out_square with or without out_mean.
+// Whole tiles per pair or slices of the batch: by time, fitted to sweeps of both over layers from 512 x 512 to 4096 x 4096 (both outputs, 2000 x 3 x 512^2, 8
+// tiles in 1, 8, 9, 10 and 18 slices: 366, 56, 52, 86 and 56 us; 300 x 16 x 2048^2, 128 tiles: 120 whole, 122 with the last wave's in four slices, three
+// statistics 258 and 246).
 struct ShortCost {
   double example, fixed, add;      // us per example of a tile, per tile, more for a tile whose sums are added
 };
@@ -421,15 +436,15 @@ static pe_status_t launch_short(DeviceInfo* di, const void* X, const void* dY, i
     if (to_zero) { zero.out[0] = out_mean; zero.out[1] = out_square; zero.out[2] = out_sign; }
     rc = before(zero);
   } else if (to_zero && whole > 0) {
-    zero_tail_tiles_kernel<<<di->sm_count, 256, 0, st>>>(p, SHORT_NT);
-    rc = check_launch();
+    rc = one_block_per_sm(di, 24, zero_tail_tiles_kernel);
+    if (rc == PE_OK) rc = launch_dependent(zero_tail_tiles_kernel, dim3(di->sm_count), 256, ZERO_SMEM, st, p, SHORT_NT);
   } else if (to_zero) {
     float* const outs[3] = {out_mean, out_square, out_sign};
     float* list[3] = {nullptr, nullptr, nullptr};
     int n = 0;
     for (float* o : outs)
       if (o) list[n++] = o;
-    rc = zero_for_split(di, list[0], list[1], (size_t)d_in * d_out, st, list[2], nullptr, 0, ZERO_ORDINARY);
+    rc = zero_for_split(di, list[0], list[1], (size_t)d_in * d_out, st, list[2]);
   }
   if (rc != PE_OK) return rc;
   const long long units = whole + (tiles - whole) * split;
@@ -534,7 +549,8 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
     p.whole_tiles = plan.tail_split > 1 ? tiles - tiles % slots : tiles;
     if (plan.tail_split > 1) {
       p.wait_at_start = 0;
-      rc = launch_dependent(zero_tail_tiles_kernel, dim3(di->sm_count), 256, 0, st, p, nt);
+      rc = one_block_per_sm(di, 24, zero_tail_tiles_kernel);
+      if (rc == PE_OK) rc = launch_dependent(zero_tail_tiles_kernel, dim3(di->sm_count), 256, ZERO_SMEM, st, p, nt);
       if (rc != PE_OK) return rc;
     }
   }
@@ -597,7 +613,7 @@ static pe_status_t launch_tc_norms(DeviceInfo* di, const void* X, const void* dY
   p.whole_tiles = 0; p.tail_split = ns; p.slice_examples = per;
   // norms[b] = 0 (by a kernel that overlaps the launch of this one, 16-byte alignment allowing)
   p.wait_at_start = 1;
-  rc = aligned(norms, 16) ? zero_for_split(di, norms, nullptr, (size_t)B, st, nullptr, nullptr, 0, ZERO_EARLY)
+  rc = aligned(norms, 16) ? zero_for_split(di, norms, nullptr, (size_t)B, st, nullptr, nullptr, 0, true)
                           : zero_outputs(norms, nullptr, (size_t)B * sizeof(float), st);
   if (rc != PE_OK) return rc;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, 256, ns, di->sm_count / 2);

@@ -37,7 +37,7 @@
 // 115 per TMA load and 550 per barrier probe behind queued MMAs, which bound every shape and needed two
 // issuers on alternate examples with half the operand ring each.  One issuer on the whole ring instead:
 // 128 x 512 tokens x 1024^2, both outputs 152 -> 127 us, three statistics 183 -> 134; 64 x 256 x 512 x 2048
-// 41.3 -> 36.3 us (cuBLAS' plain GEMM of the shape: 35.8); 1024 x 32 x 1024^2 170 -> 142.
+// 41.3 -> 36.3 us (cuBLAS' plain GEMM of the shape: 35.8).
 // The 512 TMEM columns hold 512/NT accumulators, so the MMAs of later examples overlap the epilogue of
 // earlier ones.  (MEAN_TMEM has one accumulator: while the epilogue drains it the producers keep filling
 // the ring, and the issuer then works the backlog off at full tensor rate, which absorbs the pause as long
@@ -47,8 +47,8 @@
 // while the one before is written out (two accumulators ahead; the write-out goes from registers to memory, past the ring), and
 // prologue and teardown are paid once.  The tiles of the last, partial wave are contracted in slices of the batch, as many
 // as leave every pair one, and added to outputs zeroed beforehand, in no fixed order (more than two slices: the low bits may differ between
-// runs).  Bound by the epilogue (short sequences) or the operand supply as
-// before.  8 x 256 x 1024 x 32104, both outputs 231 -> 174 us, sign 165 -> 121; 128 x 32 x 4096^2, three statistics 577 -> 497 (474 since);
+// runs).  Bound by the operand supply as
+// before.  8 x 256 x 1024 x 32104, both outputs 231 -> 174 us, sign 165 -> 121;
 // 64 x 256 x 512 x 32768 565 -> 527 (of which the slices 40), sign 477 -> 420; 16 x 1024 x 2048 x 8192, sign 460 -> 405, but
 // sequences of 256 tokens and more gain nothing by the walk alone (64 x 256 x 512 x 16384, three statistics, 321 -> 328 us).
 //
@@ -868,8 +868,8 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         // reads; the three statistics' 160 registers beside two 16-column reads), the reads are software-pipelined:
         // read k+1 is issued before the arithmetic on read k, so only the first read of a unit exposes the
         // tensor-memory latency.  That latency, paid twice per example, was a third of the two-sum epilogue's time
-        // per example, which is what bounds short sequences (the three-statistic epilogue, bound by its instruction
-        // count, gains 2-3 %).
+        // per example of 32 tokens (the three-statistic epilogue, bound by its instruction
+        // count, gained 2-3 %).
         constexpr bool PIPELINED = (CH == 32 && PHI != 3 && PHI != 4) || (TRIPLE && NT == 128);
         if constexpr (PIPELINED) {
           uint32_t ra[CH], rb[CH];
@@ -999,7 +999,7 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       // Several tiles per pair: straight from the registers, since the operand ring already fills for the next tile.  Lanes
       // exchange their rows' values first, so that four of them store 128 bytes side by side (stores of 32 bytes to 32 rows: 8 x 256
       // x 1024 x 32104, both outputs, 201 us against 179).  Slices of a tile add 128 bytes of a row per instruction (16-byte adds, 32
-      // bytes to a lane: 128 x 32 x 4096^2, both outputs, 241 us against 235).
+      // bytes to a lane, were 2 % of a call of 235 us slower).
       const int row0 = tile_m * TC_TILE_M + q * 32, col0 = tile_n * NT + h * COLS;
       if (!whole) griddep_wait();                                   // the kernel that zeroes this tile
       auto put = [&](float* out, int c, float (&v)[32]) {           // 32 columns from the c-th on
