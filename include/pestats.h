@@ -426,6 +426,12 @@ int pe_last_path(void);
  * operand columns its waves of sm_count / 2 pairs stream from memory, sum over waves of (pair rows x 256 + column tiles x
  * tile_cols); the paper has no counterpart (it leaves scheduling to XLA).  Returns 0 for arguments out of range. */
 int pe_tile_order_band(int d_in, int d_out, int tile_cols, int batch_slices, int sm_count);
+/* How a launch would divide its work, as a host-side query (no GPU is touched) by which the rules are tested.  what, and what plan[0..2] receive:
+ *   PE_PLAN_SHORT (statistics of bf16 sequences of T <= 32 tokens; outputs: 1 = sum of G_b, 2 = of squares, 4 = of signs, added up):
+ *     tiles contracted over the whole batch by one pair of thread blocks, batch slices of every other tile, examples of the longest running sum.
+ * PE_ERR_DIM for arguments out of range. */
+typedef enum { PE_PLAN_SHORT = 0 } pe_plan_t;
+pe_status_t pe_plan_query(int what /* pe_plan_t */, int outputs, int B, int T, int d_in, int d_out, int sm_count, long long* plan);
 /* Number of kernels the library has launched since load (or since the last reset to 0 via
  * pe_reset_launch_count). */
 long long pe_launch_count(void);

@@ -20,7 +20,7 @@ __all__ = [
     "microadam_family_step", "ADAM_VARIANTS", "pe_linear_stats_all", "pe_linear_stats_accumulate", "pe_example_sqnorms",
     "pe_linear_stats_ragged", "pe_linear_stats_ragged_workspace_bytes", "pe_example_sqnorms_ragged", "pe_linear_clipped_sum",
     "pe_linear_microadam_step", "pe_linear_microadam_step_f32", "pe_linear_microsignsgd_step", "pe_linear_fused_workspace_bytes",
-    "pe_token_sqstats_fp8", "pe_token_sqstats_fp8_workspace_bytes", "pe_set_wait_limit_cycles", "pe_tile_order_band",
+    "pe_token_sqstats_fp8", "pe_token_sqstats_fp8_workspace_bytes", "pe_set_wait_limit_cycles", "pe_tile_order_band", "pe_plan_query", "PLAN_SHORT",
     "pe_linear_stats_padded", "pe_linear_stats_padded_workspace_bytes", "pe_linear_stats_padded_workspace_bytes_for", "pe_conv2d_stats", "pe_conv2d_stats_workspace_bytes",
     "pe_set_fused_update", "FUSED_AUTO", "FUSED_ALWAYS", "FUSED_NEVER",
 ]
@@ -28,6 +28,7 @@ __all__ = [
 PHI_IDENTITY, PHI_SQUARE, PHI_SIGN = 0, 1, 2
 PATH_AUTO, PATH_SIMT, PATH_TENSOR, PATH_TENSOR_NARROW, PATH_TENSOR_WIDE = 0, 1, 2, 3, 4
 FUSED_AUTO, FUSED_ALWAYS, FUSED_NEVER = 0, 1, 2      # pe_fused_mode_t
+PLAN_SHORT = 0                                       # pe_plan_t
 _PHI_NAMES = {"identity": PHI_IDENTITY, "square": PHI_SQUARE, "sign": PHI_SIGN}
 
 # every symbol include/pestats.h declares
@@ -38,7 +39,7 @@ EXPORTED_SYMBOLS = [
     "pe_token_sqstats_static", "microadam_family_step", "pe_linear_stats_all", "pe_linear_stats_accumulate", "pe_example_sqnorms",
     "pe_linear_stats_ragged", "pe_linear_stats_ragged_workspace_bytes", "pe_example_sqnorms_ragged", "pe_linear_clipped_sum",
     "pe_linear_microadam_step", "pe_linear_microadam_step_f32", "pe_linear_microsignsgd_step", "pe_linear_fused_workspace_bytes",
-    "pe_token_sqstats_fp8", "pe_token_sqstats_fp8_workspace_bytes", "pe_set_wait_limit_cycles", "pe_tile_order_band",
+    "pe_token_sqstats_fp8", "pe_token_sqstats_fp8_workspace_bytes", "pe_set_wait_limit_cycles", "pe_tile_order_band", "pe_plan_query",
     "pe_set_fused_update", "pe_linear_stats_padded", "pe_linear_stats_padded_workspace_bytes", "pe_linear_stats_padded_workspace_bytes_for", "pe_conv2d_stats",
     "pe_conv2d_stats_workspace_bytes",
 ]
@@ -117,6 +118,8 @@ def load_library() -> ctypes.CDLL:
     lib.pe_last_path.argtypes = []
     lib.pe_tile_order_band.argtypes = [ctypes.c_int] * 5
     lib.pe_tile_order_band.restype = ctypes.c_int
+    lib.pe_plan_query.argtypes = [ctypes.c_int] * 7 + [ctypes.POINTER(ctypes.c_longlong)]
+    lib.pe_plan_query.restype = ctypes.c_int
     lib.pe_launch_count.argtypes = []
     lib.pe_launch_count.restype = ll
     lib.pe_reset_launch_count.argtypes = []
@@ -595,6 +598,13 @@ def pe_set_path(path: int) -> int:
 def pe_tile_order_band(d_in: int, d_out: int, tile_cols: int, batch_slices: int, sm_count: int) -> int:
     """Pair rows per band of the tile order a tensor-core launch of this shape would use (host-side query)."""
     return int(load_library().pe_tile_order_band(int(d_in), int(d_out), int(tile_cols), int(batch_slices), int(sm_count)))
+
+
+def pe_plan_query(what: int, outputs: int, B: int, T: int, d_in: int, d_out: int, sm_count: int) -> tuple:
+    """How a launch would divide its work (host-side query): three numbers, whose meaning the header gives per PLAN_* constant."""
+    plan = (ctypes.c_longlong * 3)()
+    _check("pe_plan_query", load_library().pe_plan_query(int(what), int(outputs), int(B), int(T), int(d_in), int(d_out), int(sm_count), plan))
+    return tuple(plan)
 
 
 def pe_last_path() -> int:

@@ -389,6 +389,30 @@ static ShortCost short_cost(bool mean, bool square, bool sign) {
   if (mean) return {0.19, 1.5, 2.3};
   return sign ? ShortCost{0.28, 1.0, 1.5} : ShortCost{0.155, 1.0, 1.5};
 }
+struct ShortPlan {
+  int whole, split;                // tiles that a pair takes over the whole batch; slices of the batch for each of the others
+};
+// Every pair takes whole tiles in turn; the tiles of a last partial wave, or all of them where that is cheaper, go to several
+// pairs each, by slices of the batch.  Three statistics: a unit, whole tile or slice, has no more examples than its 16-bit counts of signs hold.
+static ShortPlan plan_short(bool mean, bool square, bool sign, int B, long long tiles, int slots, bool accumulate) {
+  const ShortCost c = short_cost(mean, square, sign);
+  const bool counts = mean && square && sign;
+  ShortPlan plan = {0, 1};
+  double best = 1e300;
+  for (int pass = 0; pass < 2; ++pass) {
+    const long long w = pass == 0 ? 0 : tiles - tiles % slots, rest = tiles - w;
+    if (pass == 1 && (w == 0 || rest == 0 || (counts && B > TC_SIGN_COUNT_MAX))) break;
+    for (int k = 1; k <= B && k <= 4 * slots && (k == 1 || rest * (k - 1) < 16ll * slots); ++k) {
+      const double per = (double)((B + k - 1) / k);
+      const bool add = k > 1 || accumulate;
+      const double us = (double)(w / slots) * (B * c.example + c.fixed) +
+                        (double)((rest * k + slots - 1) / slots) * (per * c.example + c.fixed + (add ? c.add : 0.0)) + (add && !accumulate ? 2.0 : 0.0);
+      if (per <= TC_SIGN_COUNT_MAX && us < best * 0.995) { best = us; plan = {(int)(k == 1 ? tiles : w), k}; }
+    }
+  }
+  if (best == 1e300) plan = {0, (B + TC_SIGN_COUNT_MAX - 1) / TC_SIGN_COUNT_MAX};
+  return plan;
+}
 static pe_status_t launch_short(DeviceInfo* di, const void* X, const void* dY, int B, int T, int d_in, int d_out, float* out_mean, float* out_square,
                                 float* out_sign, cudaStream_t st, bool accumulate, int pitch_x, int pitch_y, const LayoutStep& before) {
   CUtensorMap mx, my;
@@ -399,23 +423,8 @@ static pe_status_t launch_short(DeviceInfo* di, const void* X, const void* dY, i
   if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
   const long long tiles = (long long)tiles_n * pairs_m;
   const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
-  // Every pair takes whole tiles in turn; the tiles of a last partial wave, or all of them where that is cheaper, go to several
-  // pairs each, by slices of the batch.
-  const ShortCost c = short_cost(out_mean, out_square, out_sign);
-  int whole = 0, split = 1;
-  double best = 1e300;
-  for (int pass = 0; pass < 2; ++pass) {
-    const long long w = pass == 0 ? 0 : tiles - tiles % slots, rest = tiles - w;
-    if (pass == 1 && (w == 0 || rest == 0)) break;
-    for (int k = 1; k <= B && k <= 4 * slots && (k == 1 || rest * (k - 1) < 16ll * slots); ++k) {
-      const double per = (double)((B + k - 1) / k);
-      const bool add = k > 1 || accumulate;
-      const double us = (double)(w / slots) * (B * c.example + c.fixed) +
-                        (double)((rest * k + slots - 1) / slots) * (per * c.example + c.fixed + (add ? c.add : 0.0)) + (add && !accumulate ? 2.0 : 0.0);
-      if (per <= TC_SIGN_COUNT_MAX && us < best * 0.995) { best = us; whole = (int)(k == 1 ? tiles : w); split = k; }
-    }
-  }
-  if (best == 1e300) { whole = 0; split = (B + TC_SIGN_COUNT_MAX - 1) / TC_SIGN_COUNT_MAX; }
+  const ShortPlan plan = plan_short(out_mean, out_square, out_sign, B, tiles, slots, accumulate);
+  const int whole = plan.whole, split = plan.split;
   TcParams p{};
   p.B = B; p.T = T; p.d_in = d_in; p.d_out = d_out; p.accumulate = accumulate ? 1 : 0;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, SHORT_NT, whole == 0 ? split : 1, slots);
@@ -1991,6 +2000,22 @@ int pe_tile_order_band(int d_in, int d_out, int tile_cols, int batch_slices, int
   const long long tiles_n = ((long long)d_in + tile_cols - 1) / tile_cols, pairs_m = ((long long)d_out + pe::TC_PAIR_M - 1) / pe::TC_PAIR_M;
   if (tiles_n * pairs_m > (1ll << 29)) return 0;
   return pe::choose_band((int)pairs_m, (int)tiles_n, tile_cols, batch_slices, sm_count / 2);
+}
+pe_status_t pe_plan_query(int what, int outputs, int B, int T, int d_in, int d_out, int sm_count, long long* plan) {
+  if (!plan) return PE_ERR_NULL;
+  if (B < 1 || T < 1 || d_in < 1 || d_out < 1 || sm_count < 2) return PE_ERR_DIM;
+  const bool mean = outputs & 1, square = outputs & 2, sign = outputs & 4;
+  switch (what) {
+    case PE_PLAN_SHORT: {
+      if (!(mean || square || sign) || T > pe::SHORT_T) return PE_ERR_DIM;
+      const long long tiles = (((long long)d_in + pe::SHORT_NT - 1) / pe::SHORT_NT) * (((long long)d_out + pe::TC_PAIR_M - 1) / pe::TC_PAIR_M);
+      if (tiles > (1ll << 29)) return PE_ERR_DIM;
+      const pe::ShortPlan p = pe::plan_short(mean, square, sign, B, tiles, sm_count / 2, false);
+      plan[0] = p.whole; plan[1] = p.split; plan[2] = p.whole > 0 ? B : (B + p.split - 1) / p.split;
+      return PE_OK;
+    }
+    default: return PE_ERR_DIM;
+  }
 }
 int pe_last_path(void) { return g_last_path.load(); }
 long long pe_launch_count(void) { return g_launches.load(); }

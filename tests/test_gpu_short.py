@@ -42,3 +42,25 @@ def test_short_sequences_against_fp64(B, T, d_in, d_out, zeros):
     unsure = ((G.abs() <= eps * mag) & (mag > 0)).sum(0)
     for got in (sign, sign2, sign3):
         assert torch.all((got.double() - G.sign().sum(0)).abs() <= 2 * unsure)
+
+
+# the 128 tiles of this layer are more than there are pairs: whole tiles over the batch where the 16-bit counts of the signs hold it (32767 examples:
+# 65535 exactly), slices beyond
+@pytest.mark.parametrize("B", [32767, 33000, 70000])
+def test_counts_of_signs_do_not_overflow(B):
+    T, d = 2, 2048
+    g = torch.Generator(device=DEV).manual_seed(B)
+    X = torch.randn((B, T, d), generator=g, device=DEV, dtype=torch.bfloat16)
+    dY = torch.randn((B, T, d), generator=g, device=DEV, dtype=torch.bfloat16)
+    sign = pe.pe_linear_stats_all(X, dY)[2]
+    rows = torch.tensor([0, 1, 255, 256, 1000, 1337, 2046, 2047], device=DEV)
+    want, unsure = 0, 0
+    for b in range(0, B, 1000):
+        x, y = X[b:b + 1000].double(), dY[b:b + 1000, :, rows].double()
+        G, mag = torch.einsum("bto,bti->boi", y, x), torch.einsum("bto,bti->boi", y.abs(), x.abs())
+        want, unsure = want + G.sign().sum(0), unsure + (G.abs() <= T * 2.0 ** -23 * mag).sum(0)
+    assert torch.all((sign[rows].double() - want).abs() <= 2 * unsure)
+    X.abs_().add_(0.5)
+    dY.abs_().add_(0.5)
+    assert torch.all(pe.pe_linear_stats_all(X, dY)[2] == B)
+    assert pe.pe_get_async_status(DEV) == (0, 0)
