@@ -429,8 +429,10 @@ int pe_tile_order_band(int d_in, int d_out, int tile_cols, int batch_slices, int
 /* How a launch would divide its work, as a host-side query (no GPU is touched) by which the rules are tested.  what, and what plan[0..2] receive:
  *   PE_PLAN_SHORT (statistics of bf16 sequences of T <= 32 tokens; outputs: 1 = sum of G_b, 2 = of squares, 4 = of signs, added up):
  *     tiles contracted over the whole batch by one pair of thread blocks, batch slices of every other tile, examples of the longest running sum.
+ *   PE_PLAN_SIMT_STATS, _TOKEN, _NORMS (the SIMT kernel; outputs: 1 = the mean is wanted beside the statistic):
+ *     tile (0: 128 x 64, 1: 64 x 64, 2: 32 x 32, 3: 16 x 16, 4: 64 x 64 by 128 threads), slices of the batch, slices to a cluster.
  * PE_ERR_DIM for arguments out of range. */
-typedef enum { PE_PLAN_SHORT = 0 } pe_plan_t;
+typedef enum { PE_PLAN_SHORT = 0, PE_PLAN_SIMT_STATS = 1, PE_PLAN_SIMT_TOKEN = 2, PE_PLAN_SIMT_NORMS = 3 } pe_plan_t;
 pe_status_t pe_plan_query(int what /* pe_plan_t */, int outputs, int B, int T, int d_in, int d_out, int sm_count, long long* plan);
 /* Number of kernels the library has launched since load (or since the last reset to 0 via
  * pe_reset_launch_count). */

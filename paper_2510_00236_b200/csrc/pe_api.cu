@@ -641,7 +641,7 @@ constexpr int SIMT_MAX_D_OUT = 65535 * 128;
 struct SimtPlan {
   int tile, slices, cluster;      // tile: index into the five shapes
 };
-static SimtPlan plan_simt(DeviceInfo* di, int mode, bool two_sums, int B, int T, int d_in, int d_out) {
+static SimtPlan plan_simt(int sm_count, int mode, bool two_sums, int B, int T, int d_in, int d_out) {
   constexpr int HALF = 4;
   static constexpr int rows[5] = {SimtTile84::ROWS, SimtTile44::ROWS, SimtTile22::ROWS, SimtTile11::ROWS, SimtTileHalf<MODE_STATS>::ROWS};
   static constexpr int cols[5] = {SimtTile84::COLS, SimtTile44::COLS, SimtTile22::COLS, SimtTile11::COLS, SimtTileHalf<MODE_STATS>::COLS};
@@ -653,14 +653,20 @@ static SimtPlan plan_simt(DeviceInfo* di, int mode, bool two_sums, int B, int T,
   const bool by_rows = mode == MODE_TOKEN;                            // what the slices divide: rows or examples
   const long long units = by_rows ? (long long)B * T : B;
   const int loose = (d_in % 4 != 0) + (d_out % 4 != 0);
+  // roundings that a sum over the batch goes through: a slice's own examples, the slices of a cluster, the clusters
+  auto chain = [&](long long s) { const long long c = std::min<long long>(s, SIMT_MAX_CLUSTER); return (units + s - 1) / s + c + (s + c - 1) / c; };
   SimtPlan best = {0, 1, 1};
   double best_cost = 1e300;
+  int other_slices = 1;
   int least = 1;             // slices: sums of all rows are not to grow longer, and with them their rounding error, for the last tile's sake
   for (int k = 0; k < 5; ++k) {
-    if (k == HALF && by_rows) least = best.slices;
+    if (k == HALF) {
+      other_slices = best.slices;
+      if (by_rows) least = best.slices;
+    }
     const long long tiles = (long long)((d_in + cols[k] - 1) / cols[k]) * ((d_out + rows[k] - 1) / rows[k]);
     for (int s = least; s <= 32 && s <= units; s *= 2) {
-      const long long blocks = tiles * s, slots = (long long)per_sm[k] * di->sm_count;
+      const long long blocks = tiles * s, slots = (long long)per_sm[k] * sm_count;
       const long long per = (units + s - 1) / s;
       const double tokens = (double)(by_rows ? per : (long long)T), whole = std::floor(tokens / kt[k]);
       const double rest = (double)(((long long)(tokens - whole * kt[k]) + 7) / 8 * 8) / kt[k];
@@ -672,12 +678,12 @@ static SimtPlan plan_simt(DeviceInfo* di, int mode, bool two_sums, int B, int T,
           const double share = std::max(together, 1.27);
           return (by_rows ? 1.0 : (double)per) * (((whole + rest) * chunk + fold) * share + (whole + (rest > 0.0 ? 1.0 : 0.0)) * edge) + 4.7;
         };
-        const long long most = (blocks + di->sm_count - 1) / di->sm_count, left = most % per_sm[k];
+        const long long most = (blocks + sm_count - 1) / sm_count, left = most % per_sm[k];
         cost = (double)(most / per_sm[k]) * round(per_sm[k]) + (left ? round((double)left) : 0.0) + 1.86 + (s > 1 ? 1.475 : 0.0) + (s > SIMT_MAX_CLUSTER ? 5.0 : 0.0);
         cost *= 0.88;          // (both estimates are high; chosen only where it is the faster one: at 70 layers never more than 2 % behind)
       } else {
-        double sharing = (double)std::min<long long>(per_sm[k], (blocks + di->sm_count - 1) / di->sm_count);
-        if (k == 0 && s >= SIMT_MAX_CLUSTER && blocks <= di->sm_count) sharing = 1.5;      // clusters of eight are placed densely
+        double sharing = (double)std::min<long long>(per_sm[k], (blocks + sm_count - 1) / sm_count);
+        if (k == 0 && s >= SIMT_MAX_CLUSTER && blocks <= sm_count) sharing = 1.5;      // clusters of eight are placed densely
         auto chunk = [&](double f) { return std::max(sharing * chunk_us[k] * f, latency_us[k] + chunk_us[k] * f); };
         double walk = whole * chunk(1.0) + (rest > 0.0 ? chunk(rest) : 0.0);
         if (!by_rows) walk = per * (walk + fold_us[k] * sharing);
@@ -686,6 +692,14 @@ static SimtPlan plan_simt(DeviceInfo* di, int mode, bool two_sums, int B, int T,
       }
       if (cost < best_cost) { best_cost = cost; best = {k, s, s < SIMT_MAX_CLUSTER ? s : SIMT_MAX_CLUSTER}; }
     }
+  }
+  // Nor are sums over the examples: the last tile in more slices, or in as many as the best of the other tiles has (60 x 24 x 900 x 300, both sums: error of
+  // the mean 1.23e-7 at 53 us in 4 slices, 1.16e-7 at 56 in 16, 1.16e-7 at 79 on the 128 x 64 tile in 32).
+  if (best.tile == HALF && mode == MODE_STATS) {
+    int s = best.slices;
+    while (chain(s) > chain(other_slices) && s < 32 && 2ll * s <= units) s *= 2;
+    if (chain(s) > chain(other_slices)) s = other_slices;
+    best = {HALF, s, s < SIMT_MAX_CLUSTER ? s : SIMT_MAX_CLUSTER};
   }
   if (mode == MODE_NORMS) best.cluster = 1;      // nothing is exchanged
   return best;
@@ -731,7 +745,7 @@ static pe_status_t launch_simt(DeviceInfo* di, const TIn* X, const TIn* dY, int 
                                const FusedOpt* opt = nullptr, int pitch_x = 0, int pitch_y = 0) {
   const int ldx = pitch_x ? pitch_x : d_in, ldy = pitch_y ? pitch_y : d_out;
   const bool two_sums = out_mean || (opt && opt->kind == OPT_ADAM);
-  SimtPlan plan = plan_simt(di, MODE, two_sums, B, T, d_in, d_out);
+  SimtPlan plan = plan_simt(di->sm_count, MODE, two_sums, B, T, d_in, d_out);
   if (opt && plan.slices > SIMT_MAX_CLUSTER) plan.slices = SIMT_MAX_CLUSTER;      // a fused update needs the whole batch in one cluster
   if (MODE != MODE_NORMS && plan.slices > plan.cluster && !accumulate) {
     pe_status_t rc = zero_outputs(out_mean, out_stat, (size_t)d_in * d_out * sizeof(float), st);
@@ -2012,6 +2026,15 @@ pe_status_t pe_plan_query(int what, int outputs, int B, int T, int d_in, int d_o
       if (tiles > (1ll << 29)) return PE_ERR_DIM;
       const pe::ShortPlan p = pe::plan_short(mean, square, sign, B, tiles, sm_count / 2, false);
       plan[0] = p.whole; plan[1] = p.split; plan[2] = p.whole > 0 ? B : (B + p.split - 1) / p.split;
+      return PE_OK;
+    }
+    case PE_PLAN_SIMT_STATS:
+    case PE_PLAN_SIMT_TOKEN:
+    case PE_PLAN_SIMT_NORMS: {
+      if (d_out > pe::SIMT_MAX_D_OUT) return PE_ERR_DIM;
+      const int mode = what == PE_PLAN_SIMT_STATS ? pe::MODE_STATS : what == PE_PLAN_SIMT_TOKEN ? pe::MODE_TOKEN : pe::MODE_NORMS;
+      const pe::SimtPlan p = pe::plan_simt(sm_count, mode, mean, B, T, d_in, d_out);
+      plan[0] = p.tile; plan[1] = p.slices; plan[2] = p.cluster;
       return PE_OK;
     }
     default: return PE_ERR_DIM;

@@ -9,7 +9,7 @@ DEV = "cuda:0"
 
 
 # whole and partial tiles, rows of whole groups of four and of odd length, sequences of whole chunks, of remainders of 1 and 8 tokens and shorter than a
-# chunk, one and several batch slices
+# chunk, one and several batch slices (9 x 7: the rule's other side)
 @pytest.mark.parametrize("B,T,d_in,d_out", [(10, 200, 800, 400), (64, 32, 500, 300), (20, 185, 406, 881), (5, 20, 1100, 1100), (9, 7, 700, 640), (23, 168, 247, 489)])
 def test_against_fp64(B, T, d_in, d_out):
     g = torch.Generator(device=DEV).manual_seed(B * T)
@@ -21,6 +21,8 @@ def test_against_fp64(B, T, d_in, d_out):
     pe.pe_linear_stats_f32(X, dY, "sign", None, sign)
     pe.pe_token_sqstats_f32(X, dY, token)
     assert pe.pe_last_path() == pe.PATH_SIMT
+    if (B, T) != (9, 7):
+        assert 4 in (pe.pe_plan_query(what, outputs, B, T, d_in, d_out, 148)[0] for what, outputs in ((pe.PLAN_SIMT_STATS, 1), (pe.PLAN_SIMT_STATS, 0), (pe.PLAN_SIMT_TOKEN, 0)))
     G, mag = torch.einsum("bto,bti->boi", dY.double(), X.double()), torch.einsum("bto,bti->boi", dY.double().abs(), X.double().abs())
     # sums of T products and of B terms, a rounding each
     eps = (T + B) * 2.0 ** -24
