@@ -426,9 +426,10 @@ int pe_last_path(void);
  * operand columns its waves of sm_count / 2 pairs stream from memory, sum over waves of (pair rows x 256 + column tiles x
  * tile_cols); the paper has no counterpart (it leaves scheduling to XLA).  Returns 0 for arguments out of range. */
 int pe_tile_order_band(int d_in, int d_out, int tile_cols, int batch_slices, int sm_count);
-/* How a launch would divide its work, as a host-side query (no GPU is touched) by which the rules are tested.  what, and what plan[0..2] receive:
+/* How a launch would divide its work, as a host-side query (no GPU is touched) by which the rules are tested.  what, and what plan[0..3] receive:
  *   PE_PLAN_SHORT (statistics of bf16 sequences of T <= 32 tokens; outputs: 1 = sum of G_b, 2 = of squares, 4 = of signs, added up):
- *     tiles contracted over the whole batch by one pair of thread blocks, batch slices of every other tile, examples of the longest running sum.
+ *     tiles contracted over the whole batch by one pair of thread blocks, batch slices of every other tile, examples of the longest
+ *     running sum, and, for the square alone, how many of them are summed by themselves at a time.
  *   PE_PLAN_SIMT_STATS, _TOKEN, _NORMS (the SIMT kernel; outputs: 1 = the mean is wanted beside the statistic):
  *     tile (0: 128 x 64, 1: 64 x 64, 2: 32 x 32, 3: 16 x 16, 4: 64 x 64 by 128 threads), slices of the batch, slices to a cluster.
  * PE_ERR_DIM for arguments out of range. */

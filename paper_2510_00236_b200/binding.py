@@ -601,8 +601,8 @@ def pe_tile_order_band(d_in: int, d_out: int, tile_cols: int, batch_slices: int,
 
 
 def pe_plan_query(what: int, outputs: int, B: int, T: int, d_in: int, d_out: int, sm_count: int) -> tuple:
-    """How a launch would divide its work (host-side query): three numbers, whose meaning the header gives per PLAN_* constant."""
-    plan = (ctypes.c_longlong * 3)()
+    """How a launch would divide its work (host-side query): four numbers, whose meaning the header gives per PLAN_* constant."""
+    plan = (ctypes.c_longlong * 4)()
     _check("pe_plan_query", load_library().pe_plan_query(int(what), int(outputs), int(B), int(T), int(d_in), int(d_out), int(sm_count), plan))
     return tuple(plan)
 

@@ -389,28 +389,64 @@ static ShortCost short_cost(bool mean, bool square, bool sign) {
   if (mean) return {0.19, 1.5, 2.3};
   return sign ? ShortCost{0.28, 1.0, 1.5} : ShortCost{0.155, 1.0, 1.5};
 }
+// Rounding error of the sums, as variances up to a factor: p examples at a time in order, in runs of r summed by themselves, and `parts` such sums added
+// in order.  Terms of either sign (G_b): p + parts; terms of one sign (G_b^2): r^2 + p^2 / r + B parts, or p^2 + B parts without runs.  (1395 x 5 x
+// 1696 x 1336, square alone, p = 1395: errors of 5.2e-7, 1.32e-7, 9.5e-8 and 7.3e-8 without runs and in runs of 16, 32 and 64.)
+static double mean_rounding(double p, double parts) { return p + parts; }
+static double square_rounding(int B, double p, double r, double parts) { return (r < p ? r * r + p * p / r : p * p) + B * parts; }
+// The sums' lengths are bounded by those of the plan that a pair per tile and slice would have, at these costs (one, two sums, three), so that a
+// plan that takes fewer slices for the time's sake does not lose precision: 2021 x 24 x 2336 x 1728, mean and square, whole tiles 716 us with errors of 6.6e-7
+// and 5.3e-7, in five slices 733 us, 3.7e-7 and 1.5e-7; 1545 x 4 x 1624 x 2296, three statistics, 1157 and 1184.  It decides on 1 to 3 % of the layers from
+// 256 x 256 to 4096 x 4096.
+constexpr UnitCost SUMS_OF_ONE = COST_STAT;
+constexpr UnitCost SUMS_OF_TWO = {128, 0.05 / 32, 0.10 / 32, 0.0, 0.245, 8.3};
+constexpr UnitCost SUMS_OF_THREE = {128, 0.05 / 32, 0.10 / 32, 0.0, 0.54, 9.5};
 struct ShortPlan {
   int whole, split;                // tiles that a pair takes over the whole batch; slices of the batch for each of the others
+  int run;                         // the square alone: examples that are summed by themselves, a power of two
 };
 // Every pair takes whole tiles in turn; the tiles of a last partial wave, or all of them where that is cheaper, go to several
 // pairs each, by slices of the batch.  Three statistics: a unit, whole tile or slice, has no more examples than its 16-bit counts of signs hold.
-static ShortPlan plan_short(bool mean, bool square, bool sign, int B, long long tiles, int slots, bool accumulate) {
+static ShortPlan plan_short(bool mean, bool square, bool sign, int B, int T, int d_in, int d_out, int slots, bool accumulate, bool may_persist) {
   const ShortCost c = short_cost(mean, square, sign);
-  const bool counts = mean && square && sign;
-  ShortPlan plan = {0, 1};
+  const bool counts = mean && square && sign, runs = square && !mean;
+  const long long tiles = (((long long)d_in + SHORT_NT - 1) / SHORT_NT) * (((long long)d_out + TC_PAIR_M - 1) / TC_PAIR_M);
+  ShortPlan plan = {0, 1, SHORT_RUN_MIN};
+  double most_mean = 1e300, most_square = 1e300;
+  if (mean || square) {
+    const UnitCost& cost = counts ? SUMS_OF_THREE : mean ? SUMS_OF_TWO : SUMS_OF_ONE;
+    const int outputs = (mean ? 1 : 0) + (square ? 1 : 0) + (sign ? 1 : 0);
+    int ns = plan_tiles(&cost, 1, B, T, d_in, d_out, slots, std::max(16, slots), outputs, may_persist && !(counts && B > TC_SIGN_COUNT_MAX)).ns;
+    if (counts && (B + ns - 1) / ns > TC_SIGN_COUNT_MAX) ns = (B + TC_SIGN_COUNT_MAX - 1) / TC_SIGN_COUNT_MAX;
+    const double p = (B + ns - 1) / ns, parts = ns > 1 ? ns : 0;
+    if (mean) most_mean = mean_rounding(p, parts);
+    if (square) most_square = square_rounding(B, p, p, parts);
+    plan.split = ns;               // (where nothing below is good enough)
+  }
+  auto run_of = [&](double p, double parts) {        // the longest runs that round within 2 % as little as any
+    double least = 1e300;
+    for (int r = SHORT_RUN_MIN; r <= SHORT_RUN_MAX; r *= 2) least = std::min(least, square_rounding(B, p, r, parts));
+    int r = SHORT_RUN_MAX;
+    while (r > SHORT_RUN_MIN && square_rounding(B, p, r, parts) > 1.02 * least) r /= 2;
+    return r;
+  };
+  auto good = [&](double p, double parts) {
+    return (!counts || p <= TC_SIGN_COUNT_MAX) && (!mean || mean_rounding(p, parts) <= most_mean) &&
+           (!square || square_rounding(B, p, runs ? run_of(p, parts) : p, parts) <= most_square);
+  };
   double best = 1e300;
   for (int pass = 0; pass < 2; ++pass) {
     const long long w = pass == 0 ? 0 : tiles - tiles % slots, rest = tiles - w;
-    if (pass == 1 && (w == 0 || rest == 0 || (counts && B > TC_SIGN_COUNT_MAX))) break;
+    if (pass == 1 && (w == 0 || rest == 0 || !good(B, 0))) break;
     for (int k = 1; k <= B && k <= 4 * slots && (k == 1 || rest * (k - 1) < 16ll * slots); ++k) {
       const double per = (double)((B + k - 1) / k);
       const bool add = k > 1 || accumulate;
       const double us = (double)(w / slots) * (B * c.example + c.fixed) +
                         (double)((rest * k + slots - 1) / slots) * (per * c.example + c.fixed + (add ? c.add : 0.0)) + (add && !accumulate ? 2.0 : 0.0);
-      if (per <= TC_SIGN_COUNT_MAX && us < best * 0.995) { best = us; plan = {(int)(k == 1 ? tiles : w), k}; }
+      if (us < best * 0.995 && good(per, k > 1 ? k : 0)) { best = us; plan.whole = (int)(k == 1 ? tiles : w); plan.split = k; }
     }
   }
-  if (best == 1e300) plan = {0, (B + TC_SIGN_COUNT_MAX - 1) / TC_SIGN_COUNT_MAX};
+  if (runs) plan.run = plan.whole > 0 ? run_of(B, 0) : run_of((B + plan.split - 1) / plan.split, plan.split > 1 ? plan.split : 0);
   return plan;
 }
 static pe_status_t launch_short(DeviceInfo* di, const void* X, const void* dY, int B, int T, int d_in, int d_out, float* out_mean, float* out_square,
@@ -423,12 +459,13 @@ static pe_status_t launch_short(DeviceInfo* di, const void* X, const void* dY, i
   if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
   const long long tiles = (long long)tiles_n * pairs_m;
   const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
-  const ShortPlan plan = plan_short(out_mean, out_square, out_sign, B, tiles, slots, accumulate);
+  const ShortPlan plan = plan_short(out_mean, out_square, out_sign, B, T, d_in, d_out, slots, accumulate,
+                                    !accumulate && d_in % 8 == 0 && aligned(out_mean, 32) && aligned(out_square, 32) && aligned(out_sign, 32));
   const int whole = plan.whole, split = plan.split;
   TcParams p{};
   p.B = B; p.T = T; p.d_in = d_in; p.d_out = d_out; p.accumulate = accumulate ? 1 : 0;
   p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, SHORT_NT, whole == 0 ? split : 1, slots);
-  p.whole_tiles = whole; p.tail_split = split;
+  p.whole_tiles = whole; p.tail_split = split; p.sum_run = plan.run;
   p.scalar_out = d_in % 4 != 0 ? 1 : 0;
   CUtensorMap mm = mx, msq = mx, msgn = mx;           // an output that is not wanted gets a map that is never used
   if (!p.scalar_out) {
@@ -2024,8 +2061,8 @@ pe_status_t pe_plan_query(int what, int outputs, int B, int T, int d_in, int d_o
       if (!(mean || square || sign) || T > pe::SHORT_T) return PE_ERR_DIM;
       const long long tiles = (((long long)d_in + pe::SHORT_NT - 1) / pe::SHORT_NT) * (((long long)d_out + pe::TC_PAIR_M - 1) / pe::TC_PAIR_M);
       if (tiles > (1ll << 29)) return PE_ERR_DIM;
-      const pe::ShortPlan p = pe::plan_short(mean, square, sign, B, tiles, sm_count / 2, false);
-      plan[0] = p.whole; plan[1] = p.split; plan[2] = p.whole > 0 ? B : (B + p.split - 1) / p.split;
+      const pe::ShortPlan p = pe::plan_short(mean, square, sign, B, T, d_in, d_out, sm_count / 2, false, d_in % 8 == 0);
+      plan[0] = p.whole; plan[1] = p.split; plan[2] = p.whole > 0 ? B : (B + p.split - 1) / p.split; plan[3] = p.run;
       return PE_OK;
     }
     case PE_PLAN_SIMT_STATS:

@@ -141,6 +141,7 @@ struct TcParams {
   int whole_tiles;     // PERSIST: tiles that one pair contracts over the whole batch; each of the others goes to
   int tail_split;      // this many pairs, by slices of the batch, whose sums are added to (zeroed) outputs
   int slice_examples;  // 0, or the examples of such a slice (the last one may have fewer): where slices are short, 64-bit divisions would show
+  int sum_run;         // short_stats_kernel, the square alone: examples summed by themselves, a power of two
   int part_chunks;     // PARTS: chunks of rows per part, slices of the square's, the mean's and the sign's chunks
   int part_slices[3];
   unsigned int part_dy, part_x;   // PARTS: the copies of dY and of X that each product takes

@@ -1,4 +1,6 @@
 """Sequences of at most 32 tokens: the kernel of its own that contracts two examples per hand-off."""
+import math
+
 import pytest
 import torch
 
@@ -64,3 +66,26 @@ def test_counts_of_signs_do_not_overflow(B):
     dY.abs_().add_(0.5)
     assert torch.all(pe.pe_linear_stats_all(X, dY)[2] == B)
     assert pe.pe_get_async_status(DEV) == (0, 0)
+
+
+# layers of more tiles than pairs by a fraction of a wave.  Rounding to nearest leaves u^2 / 6 on average (u = 2^-24); a sum of p examples at a time has an
+# error of u sqrt(p / 6) against terms of either sign, u p / sqrt(18 B) against squares, beside the contraction's (T truncations in fp32, averaged over the batch)
+@pytest.mark.parametrize("outputs,B,T,d_in,d_out,p", [(2, 2021, 24, 2336, 1728, 405), (3, 1545, 4, 1624, 2296, 309), (1, 1395, 5, 1696, 1336, 200)])
+def test_precision_of_sums_over_many_examples(outputs, B, T, d_in, d_out, p):
+    g = torch.Generator(device=DEV).manual_seed(B)
+    X = torch.randn((B, T, d_in), generator=g, device=DEV, dtype=torch.bfloat16)
+    dY = torch.randn((B, T, d_out), generator=g, device=DEV, dtype=torch.bfloat16)
+    if outputs == 1:
+        mean, square = None, torch.empty((d_out, d_in), device=DEV)
+        pe.pe_linear_stats(X, dY, "square", None, square)
+    else:
+        mean, square = (pe.pe_linear_stats_all(X, dY) if outputs == 3 else pe.pe_linear_stats(X, dY, "square"))[:2]
+    rows = torch.randperm(d_out, generator=torch.Generator().manual_seed(1))[:96].to(DEV)
+    m, q = 0, 0
+    for b in range(0, B, 64):
+        G = torch.einsum("bto,bti->boi", dY[b:b + 64, :, rows].double(), X[b:b + 64].double())
+        m, q = m + G.sum(0), q + (G * G).sum(0)
+    u = 2.0 ** -24
+    if mean is not None:
+        assert (mean[rows].double() - m).norm() <= 1.25 * u * math.sqrt((p + B / p) / 6) * m.norm()
+    assert (square[rows].double() - q).norm() <= 1.25 * u * math.sqrt(p * p / (18 * B) + B / p / 18 + T / 6) * q.norm()

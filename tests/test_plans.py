@@ -18,16 +18,34 @@ def lib():
 @pytest.mark.parametrize("d_in,d_out", [(2048, 2048), (1600, 2048), (1024, 2048), (1024, 4096), (4096, 4096), (128, 512)])
 def test_sign_counts_of_short_sequences_fit_16_bits(d_in, d_out):
     for B in [32766, 32767, 32768, 33000, 40000, 65534, 65535, 66000, 70000, 100000, 131072, 140000, 1 << 20]:
-        whole, slices, longest = pe.pe_plan_query(pe.PLAN_SHORT, MEAN | SQUARE | SIGN, B, 2, d_in, d_out, SMS)
+        whole, slices, longest, _ = pe.pe_plan_query(pe.PLAN_SHORT, MEAN | SQUARE | SIGN, B, 2, d_in, d_out, SMS)
         assert longest == (B if whole else -(-B // slices))
         assert longest <= 32767
+
+
+# what a pair per tile and slice would have taken: five slices of 91 or 133 tiles, two of 99, and so on
+@pytest.mark.parametrize("outputs,B,T,d_in,d_out,most", [
+    (MEAN | SQUARE, 2021, 24, 2336, 1728, 405), (MEAN | SIGN, 2021, 24, 2336, 1728, 405), (MEAN | SQUARE | SIGN, 1545, 4, 1624, 2296, 309),
+    (MEAN | SQUARE, 1854, 6, 2616, 1368, 464), (MEAN | SQUARE | SIGN, 285, 2, 832, 3888, 95), (MEAN | SQUARE | SIGN, 1858, 20, 1864, 2208, 310)])
+def test_sums_of_short_sequences_are_not_lengthened(outputs, B, T, d_in, d_out, most):
+    assert pe.pe_plan_query(pe.PLAN_SHORT, outputs, B, T, d_in, d_out, SMS)[2] <= most
+
+
+# error variances up to a factor (examples in order, or runs and their sums, and the slices) against the slices of a pair per 256 x 256 tile and slice
+@pytest.mark.parametrize("B,T,d_in,d_out,slices", [(1395, 5, 1696, 1336, 7), (665, 16, 832, 2528, 5), (1010, 6, 528, 3304, 5), (800, 32, 1024, 4096, 0), (28, 32, 1024, 1024, 4)])
+def test_runs_of_the_square_alone(B, T, d_in, d_out, slices):
+    whole, split, longest, run = pe.pe_plan_query(pe.PLAN_SHORT, SQUARE, B, T, d_in, d_out, SMS)
+    variance = lambda p, r, parts: (r * r + p * p / r if r < p else p * p) + B * parts        # noqa: E731
+    assert run in (16, 32, 64, 128, 256)
+    p = -(-B // max(1, slices))
+    assert variance(longest, run, 0 if whole or split == 1 else split) <= variance(p, p, slices)
 
 
 # the tiles of 128 x 64 (32 slices), 64 x 64 by 256 threads (16) and 128 x 64 (32) are what these layers take among the other four tiles: roundings of a
 # sum over the batch are a slice's examples, the slices of a cluster of eight, the clusters
 @pytest.mark.parametrize("B,T,d_in,d_out,others", [(60, 24, 900, 300, 32), (37, 187, 356, 126, 16), (49, 37, 948, 328, 32)])
 def test_smaller_blocks_do_not_lengthen_fp32_sums(B, T, d_in, d_out, others):
-    tile, slices, cluster = pe.pe_plan_query(pe.PLAN_SIMT_STATS, MEAN, B, T, d_in, d_out, SMS)
+    tile, slices, cluster, _ = pe.pe_plan_query(pe.PLAN_SIMT_STATS, MEAN, B, T, d_in, d_out, SMS)
     chain = lambda s: -(-B // s) + min(s, 8) + -(-s // 8)        # noqa: E731
     assert tile == 4 and cluster == min(slices, 8)
     assert chain(slices) <= chain(others)
