@@ -207,6 +207,7 @@ size_t pe_conv2d_stats_workspace_bytes(int B, int C, int H, int W, int F, int Kh
  * it and B*T >= 256) one kernel squares the operands on chip (exact in fp32), rounds each square to
  * tf32 (11 significant bits, so every entry is within about 1e-3 relative of the exact sum) and
  * contracts them; nothing is staged in global memory.  Otherwise the SIMT kernel squares in fp32.
+ * Where more than two thread-block pairs share a tile of the output their sums are added in no fixed order, and low bits may differ between runs.
  */
 pe_status_t pe_token_sqstats(const void* X, const void* dY, int B, int T, int d_in, int d_out,
                              float* out_stat, pe_stream_t stream);
@@ -432,8 +433,10 @@ int pe_tile_order_band(int d_in, int d_out, int tile_cols, int batch_slices, int
  *     running sum, and, for the square alone, how many of them are summed by themselves at a time.
  *   PE_PLAN_SIMT_STATS, _TOKEN, _NORMS (the SIMT kernel; outputs: 1 = the mean is wanted beside the statistic):
  *     tile (0: 128 x 64, 1: 64 x 64, 2: 32 x 32, 3: 16 x 16, 4: 64 x 64 by 128 threads), slices of the batch, slices to a cluster.
+ *   PE_PLAN_TOKEN (pe_token_sqstats on the tensor cores): slices of the rows, a pair per 256 x 256 tile and slice; or, if the next is not 0, tiles whose 32-row
+ *     chunks are dealt out evenly, over how many pairs, and pairs in all.
  * PE_ERR_DIM for arguments out of range. */
-typedef enum { PE_PLAN_SHORT = 0, PE_PLAN_SIMT_STATS = 1, PE_PLAN_SIMT_TOKEN = 2, PE_PLAN_SIMT_NORMS = 3 } pe_plan_t;
+typedef enum { PE_PLAN_SHORT = 0, PE_PLAN_SIMT_STATS = 1, PE_PLAN_SIMT_TOKEN = 2, PE_PLAN_SIMT_NORMS = 3, PE_PLAN_TOKEN = 4 } pe_plan_t;
 pe_status_t pe_plan_query(int what /* pe_plan_t */, int outputs, int B, int T, int d_in, int d_out, int sm_count, long long* plan);
 /* Number of kernels the library has launched since load (or since the last reset to 0 via
  * pe_reset_launch_count). */

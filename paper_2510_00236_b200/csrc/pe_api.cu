@@ -178,9 +178,9 @@ constexpr UnitCost COST_SIGN = {256, 0.51 / 128, 0.68 / 128, 0.0, 0.66, 8.5};
 constexpr UnitCost COST_NORMS = {256, 0.51 / 128, 0.68 / 128, 0.0, 0.30, 7.0};
 constexpr UnitCost COST_PLAIN = {256, 0.51 / 128, 0.68 / 128, 0.0, 0.0, 8.5};
 constexpr UnitCost COST_TOKEN = {TOK_NT, 0.42 / TOK_BK, 0.45 / TOK_BK, 0.0, 0.0, 8.5};     // an "example" is one 32-row stage
-// The per-token statistic's chunks dealt out evenly over the pairs: two tiles instead of one to write out per pair, and rows that are read at
-// different times for the tiles that share them.  64 x 256 x 512 x 2048 (16 tiles) 68.9 -> 63.0 us, 64 x 256 x 1024 x 2048 (32) 125 -> 111, 100 x 100 x 776 x 3000
-// (48) 116 -> 108; 128 x 512 x 512 x 1024 (8 tiles, whose nine slices leave two pairs idle) 117 -> 119, which stays in slices.
+// The per-token statistic's chunks dealt out over the pairs: two tiles instead of one to write out per pair, and rows that are read at
+// different times for the tiles that share them.  64 x 256 x 512 x 2048 (16 tiles) 68.9 -> 63.0 us; 128 x 512 x 512 x 1024 (8 tiles, whose nine slices leave
+// two pairs idle) 117 -> 119, which stays in slices.
 constexpr double TOK_EVEN_FIXED = 4.0;
 constexpr UnitCost COST_PLAIN_FP8 = {256, 0.28 / 128, 0.40 / 128, 0.0, 0.0, 8.5};
 constexpr UnitCost COST_BOTH_192 = {192, 0.375 / 128, 0.55 / 128, 0.02, 0.35, 10.0};     // two sums
@@ -1083,6 +1083,29 @@ static pe_status_t launch_tc_fused(DeviceInfo* di, const void* X, const void* dY
   return launch_tc_inst<1, false, 128, MEAN_REGS, 128, false, OPT_ADAM>(di, 22, mx, my, mm, ms, ms, p, grid, st, nullptr, nullptr, &opt);
 }
 
+// Per-token statistic: `units` chunks of rows for each tile.  ns: slices of the rows, a pair per tile and slice; deal_tiles > 0: instead, the chunks of
+// every deal_tiles tiles (the last ones may be fewer) dealt out evenly over deal_pairs pairs, pairs in all.
+struct TokPlan {
+  int ns, deal_tiles, deal_pairs, pairs;
+};
+static TokPlan plan_tok(int units, int d_in, int d_out, int slots) {
+  const long long tiles = (((long long)d_in + TOK_NT - 1) / TOK_NT) * (((long long)d_out + TC_PAIR_M - 1) / TC_PAIR_M);
+  const double out_bytes = 4.0 * d_in * d_out;
+  TokPlan plan = {plan_tiles(&COST_TOKEN, 1, units, TOK_BK, d_in, d_out, slots, std::max(32, slots), 1).ns, 0, 0, 0};
+  if (tiles >= slots || tiles * units < slots || units < 2) return plan;
+  const double in_slices = launch_cost(COST_TOKEN, tiles, units, TOK_BK, slots, plan.ns, 1, out_bytes, false).us;
+  // Evenly over all pairs, which gives a tile three parts and more, added in no fixed order.  A call whose tiles would be whole or in two slices repeats bit for bit
+  // (two parts on zero, whatever their order), and keeps to that: groups of k tiles on k + 1 pairs, which give every tile two parts.
+  const long long k = plan.ns > 2 ? tiles : (slots - 1) / (slots - tiles), pairs = plan.ns > 2 ? slots : k + 1;
+  const double load = std::ceil((double)units * k / pairs);
+  const double dealt = load * TOK_BK * COST_TOKEN.token_hi + COST_TOKEN.fixed + SPLIT_FIXED + out_bytes / ZERO_BYTES_PER_US + TOK_EVEN_FIXED;
+  if (dealt < in_slices) {
+    plan.deal_tiles = (int)k; plan.deal_pairs = (int)pairs;
+    plan.pairs = (int)(plan.ns > 2 ? slots : tiles + (tiles + k - 1) / k);
+  }
+  return plan;
+}
+
 
 // Fused per-token statistic: squares, rounds to tf32 and contracts inside one kernel.
 static pe_status_t launch_tok(DeviceInfo* di, const void* X, const void* dY, long long rows, int d_in, int d_out, float* out,
@@ -1106,13 +1129,9 @@ static pe_status_t launch_tok(DeviceInfo* di, const void* X, const void* dY, lon
   const long long n_chunks = (rows + TOK_BK - 1) / TOK_BK;
   const int units = n_chunks > (1 << 30) ? (1 << 30) : (int)n_chunks;
   const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
-  const long long tiles = (long long)tiles_n * pairs_m;
-  const int ns = plan_tiles(&COST_TOKEN, 1, units, TOK_BK, d_in, d_out, slots, std::max(32, slots), 1).ns;
-  // The chunks of all tiles dealt out evenly, where that saves more than the second tile that most pairs then write out.
-  const double in_slices = launch_cost(COST_TOKEN, tiles, units, TOK_BK, slots, ns, 1, 4.0 * d_in * d_out, false).us;
-  const double evenly = std::ceil((double)tiles * units / slots) * TOK_BK * COST_TOKEN.token_hi + COST_TOKEN.fixed + SPLIT_FIXED + 4.0 * d_in * d_out / ZERO_BYTES_PER_US +
-                        TOK_EVEN_FIXED;
-  const bool even = tiles <= slots && tiles * units >= slots && evenly < in_slices;
+  const TokPlan plan = plan_tok(units, d_in, d_out, slots);
+  const int ns = plan.ns;
+  const bool even = plan.deal_tiles > 0;
   if (ns > 1 || even) {
     rc = zero_for_split(di, out, nullptr, (size_t)d_in * d_out, st);
     if (rc != PE_OK) return rc;
@@ -1129,8 +1148,9 @@ static pe_status_t launch_tok(DeviceInfo* di, const void* X, const void* dY, lon
   }
   TokParams p;
   p.rows = rows; p.d_in = d_in; p.d_out = d_out; p.pairs_m = pairs_m; p.tiles_n = tiles_n;
-  p.band = choose_band(pairs_m, tiles_n, TOK_NT, even ? 1 : ns, di->sm_count / 2); p.nsplit = even ? 1 : ns; p.even = even ? 1 : 0; p.dev_status = di->status_ptr;
-  return launch_dependent(tok_sqstats_kernel, even ? dim3(2 * slots) : dim3(2 * pairs_m * tiles_n, 1, ns), TOK_THREADS, TOK_SMEM_BYTES, st, mx, my, mo, p);
+  p.band = choose_band(pairs_m, tiles_n, TOK_NT, even ? 1 : ns, di->sm_count / 2); p.nsplit = even ? 1 : ns;
+  p.deal_tiles = plan.deal_tiles; p.deal_pairs = plan.deal_pairs; p.dev_status = di->status_ptr;
+  return launch_dependent(tok_sqstats_kernel, even ? dim3(2 * plan.pairs) : dim3(2 * pairs_m * tiles_n, 1, ns), TOK_THREADS, TOK_SMEM_BYTES, st, mx, my, mo, p);
 }
 
 }  // namespace pe
@@ -2072,6 +2092,12 @@ pe_status_t pe_plan_query(int what, int outputs, int B, int T, int d_in, int d_o
       const int mode = what == PE_PLAN_SIMT_STATS ? pe::MODE_STATS : what == PE_PLAN_SIMT_TOKEN ? pe::MODE_TOKEN : pe::MODE_NORMS;
       const pe::SimtPlan p = pe::plan_simt(sm_count, mode, mean, B, T, d_in, d_out);
       plan[0] = p.tile; plan[1] = p.slices; plan[2] = p.cluster;
+      return PE_OK;
+    }
+    case PE_PLAN_TOKEN: {
+      const long long chunks = ((long long)B * T + pe::TOK_BK - 1) / pe::TOK_BK;
+      const pe::TokPlan p = pe::plan_tok((int)std::min<long long>(chunks, 1 << 30), d_in, d_out, sm_count / 2);
+      plan[0] = p.ns; plan[1] = p.deal_tiles; plan[2] = p.deal_pairs; plan[3] = p.pairs;
       return PE_OK;
     }
     default: return PE_ERR_DIM;

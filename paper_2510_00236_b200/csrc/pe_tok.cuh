@@ -1,7 +1,7 @@
 // Tensor-core kernel for the per-token second moment (Section 2.3, the "per-token" alternative):
 //     S'[o,i] = sum_r dY[r,o]^2 * X[r,i]^2        over the B*T rows r,
 // a plain contraction of the SQUARED operands.  Nothing is staged in global memory: the bf16 tiles
-// arrive by TMA, the eight warps that later write the result out first square them on the fly
+// arrive by TMA, the warps that later write the result out first square them on the fly
 // (bf16^2 is exact in fp32), round to tf32 and lay them out in shared memory the way the tf32 MMA
 // wants them, and the pair-wide tcgen05 MMAs (cta_group::2, M = 256, N = 256, kind::tf32) accumulate
 // in tensor memory.  tf32 keeps 11 significant bits of each square (bf16 would keep 8), so every
@@ -11,9 +11,9 @@
 // two-pass variant on large layers and faster on small ones, with a third of the HBM traffic.
 //
 // Work unit: a CTA pair owns a 256 x 256 tile of the [d_out, d_in] output and a contiguous range of
-// 32-row chunks of the B*T rows (gridDim.z slices; partial sums are added by TMA reduce).  With at most as many tiles as pairs, and where whole slices
-// leave pairs idle (16 tiles: 64 of 74), the chunks of all tiles are dealt out evenly instead, tile after tile: a pair then holds the end of one
-// tile and the start of the next, in the two accumulators that tensor memory has room for, and writes both out at the end.
+// 32-row chunks of the B*T rows (gridDim.z slices; partial sums are added by TMA reduce).  With fewer tiles than pairs, and where whole slices
+// leave pairs idle (16 tiles: 64 of 74), the chunks of all tiles, or of k tiles at a time on k + 1 pairs, are dealt out evenly instead, tile after tile: a pair
+// then holds the end of one tile and the start of the next, in the two accumulators that tensor memory has room for, and writes both out at the end.
 //
 // Shared memory per block: 4 "raw" stages of 16 KiB (bf16: 128 rows of dY^T as two 64-feature boxes,
 // this block's 128 rows of X^T as two more; 128-byte swizzle with 16-byte chunks, as TMA writes it)
@@ -23,7 +23,7 @@
 // Warps (20 per block): 0 = TMA producer of the dY boxes (also posts the stage's byte count), 2 = TMEM
 // allocator, then TMA producer of the X boxes, 1 = MMA issuer (leader block only), 4..19 = converters
 // (sixteen warps: the conversion is a stream of dependent shared-memory round trips, and eight warps
-// only reached 1.4 instructions per clock of the SM's 4), of which 4..11 then write the result out.
+// only reached 1.4 instructions per clock of the SM's 4), of which 4..11 then write the (first) tile out, 12..19 the second.
 // Barriers: raw_full[s] / raw_empty[s] are local to each block (its own TMA, its own converters);
 // cooked_full[c] lives in the leader and collects the converter warps of both blocks (four per block
 // and stage: the sixteen warps work as four groups, group g on the stages n = g mod 4, i.e. always
@@ -54,7 +54,8 @@ struct TokParams {
   int d_in, d_out;
   int pairs_m, tiles_n, band;   // tile grid and tile order, as in TcParams
   int nsplit;          // slices of the row range (gridDim.z); > 1 => output pre-zeroed, partial sums added
-  int even;            // the chunks of all tiles are dealt out evenly over gridDim.x / 2 pairs (output pre-zeroed, sums added); tiles <= pairs
+  int deal_tiles, deal_pairs;   // 0, or: the chunks of every deal_tiles tiles are dealt out evenly over deal_pairs pairs, no fewer, and in the last group
+                                // the tiles that are left over the pairs that are left (output pre-zeroed, sums added)
   unsigned int* dev_status;
 };
 
@@ -115,16 +116,17 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     t.tile_n = r / rows_in_band;
     t.tile_m = 2 * (band * p.band + (r - t.tile_n * rows_in_band)) + (int)rank;
   };
-  if (p.even) {
-    const long long total = n_chunks * p.pairs_m * p.tiles_n, pairs = gridDim.x >> 1;
-    const long long first = total * (blockIdx.x >> 1) / pairs, last = total * ((blockIdx.x >> 1) + 1) / pairs;
+  if (p.deal_tiles) {
+    const int group = (int)(blockIdx.x >> 1) / p.deal_pairs, tile0 = group * p.deal_tiles, in_group = (int)(blockIdx.x >> 1) - group * p.deal_pairs;
+    const long long total = n_chunks * min(p.deal_tiles, p.pairs_m * p.tiles_n - tile0), pairs = min(p.deal_pairs, (int)(gridDim.x >> 1) - group * p.deal_pairs);
+    const long long first = total * in_group / pairs, last = total * (in_group + 1) / pairs;
     const int tile = (int)(first / n_chunks);
-    tile_of(piece[0], tile);
+    tile_of(piece[0], tile0 + tile);
     piece[0].begin = first - tile * n_chunks;
     piece[0].end = min(n_chunks, piece[0].begin + last - first);
     if (last > (tile + 1) * n_chunks) {
       n_pieces = 2;
-      tile_of(piece[1], tile + 1);
+      tile_of(piece[1], tile0 + tile + 1);
       piece[1].begin = 0;
       piece[1].end = last - (tile + 1) * n_chunks;
     }
@@ -134,7 +136,7 @@ tok_sqstats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     piece[0].end = n_chunks * (blockIdx.z + 1) / p.nsplit;
   }
   if (n_pieces == 1) piece[1] = {0, 0, 0, 0};
-  const bool add = p.nsplit > 1 || p.even;
+  const bool add = p.nsplit > 1 || p.deal_tiles;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < TOK_RAW_STAGES; ++s) { mbar_init(raw_full(s), 1); mbar_init(raw_empty(s), 4); }

@@ -49,3 +49,35 @@ def test_smaller_blocks_do_not_lengthen_fp32_sums(B, T, d_in, d_out, others):
     chain = lambda s: -(-B // s) + min(s, 8) + -(-s // 8)        # noqa: E731
     assert tile == 4 and cluster == min(slices, 8)
     assert chain(slices) <= chain(others)
+
+
+def _parts(rows, d_in, d_out):
+    """Per tile of the per-token statistic the chunks that each pair takes, by the plan."""
+    chunks, tiles, slots = -(-rows // 32), -(-d_in // 256) * -(-d_out // 256), SMS // 2
+    slices, deal_tiles, deal_pairs, pairs = pe.pe_plan_query(pe.PLAN_TOKEN, 0, 1, rows, d_in, d_out, SMS)
+    if not deal_tiles:
+        return slices, [[chunks * (z + 1) // slices - chunks * z // slices for z in range(slices)] for _ in range(tiles)]
+    parts = [[] for _ in range(tiles)]
+    assert deal_tiles <= deal_pairs and pairs <= slots
+    for pair in range(pairs):
+        group, i = divmod(pair, deal_pairs)
+        in_group, n = min(deal_tiles, tiles - group * deal_tiles), min(deal_pairs, pairs - group * deal_pairs)
+        first, last = chunks * in_group * i // n, chunks * in_group * (i + 1) // n
+        assert first < last <= first // chunks * chunks + 2 * chunks            # one or two tiles to a pair
+        for tile in range(first // chunks, -(-last // chunks)):
+            parts[group * deal_tiles + tile].append(min(last, (tile + 1) * chunks) - max(first, tile * chunks))
+    return slices, parts
+
+
+def test_rows_of_the_per_token_statistic_dealt_out():
+    dealt = 0
+    for rows in (33, 64, 100, 1000, 2000, 4127, 16384, 100000):
+        for d_in in (8, 256, 512, 776, 1024, 2304):
+            for d_out in (8, 520, 1280, 2048, 3000, 4864, 8192):
+                slices, parts = _parts(rows, d_in, d_out)
+                dealt += any(len(p) != slices for p in parts)
+                for p in parts:
+                    assert sum(p) == -(-rows // 32) and min(p) > 0
+                    # whole tiles and tiles in two parts repeat bit for bit, and they do so wherever whole slices would
+                    assert len(p) <= 2 or slices > 2
+    assert dealt > 20
