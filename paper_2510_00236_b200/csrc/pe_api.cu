@@ -182,6 +182,10 @@ constexpr UnitCost COST_TOKEN = {TOK_NT, 0.42 / TOK_BK, 0.45 / TOK_BK, 0.0, 0.0,
 // different times for the tiles that share them.  64 x 256 x 512 x 2048 (16 tiles) 68.9 -> 63.0 us; 128 x 512 x 512 x 1024 (8 tiles, whose nine slices leave
 // two pairs idle) 117 -> 119, which stays in slices.
 constexpr double TOK_EVEN_FIXED = 4.0;
+// ... and rows of operands that L2 does not hold (126 MB together, or a quarter of that for one beside the other's stream) are then read from HBM once for
+// every tile, at about 4 TB/s: 60000 rows x 2048 x 2304 (72 tiles) 906 us whole and 1123 dealt out, 512 x 4608 (36) 447 and 531, 256 x 6656 (26) 379 in
+// slices and 339 dealt out; 16384 x 1792 x 2560 (70) 238 and 276, 1280 x 2560 (50) 190 and 180.
+constexpr double TOK_L2_BYTES = 126e6, TOK_DEALT_BYTES_PER_US = 4.0e6;
 constexpr UnitCost COST_PLAIN_FP8 = {256, 0.28 / 128, 0.40 / 128, 0.0, 0.0, 8.5};
 constexpr UnitCost COST_BOTH_192 = {192, 0.375 / 128, 0.55 / 128, 0.02, 0.35, 10.0};     // two sums
 constexpr UnitCost COST_BOTH_128 = {128, 0.35 / 128, 0.44 / 128, 0.12, 0.20, 8.3};
@@ -1098,7 +1102,12 @@ static TokPlan plan_tok(int units, int d_in, int d_out, int slots) {
   // (two parts on zero, whatever their order), and keeps to that: groups of k tiles on k + 1 pairs, which give every tile two parts.
   const long long k = plan.ns > 2 ? tiles : (slots - 1) / (slots - tiles), pairs = plan.ns > 2 ? slots : k + 1;
   const double load = std::ceil((double)units * k / pairs);
-  const double dealt = load * TOK_BK * COST_TOKEN.token_hi + COST_TOKEN.fixed + SPLIT_FIXED + out_bytes / ZERO_BYTES_PER_US + TOK_EVEN_FIXED;
+  // Tiles that share rows read them at different times, and so from HBM, unless what they share stays in L2.
+  const double rows = (double)units * TOK_BK, x_bytes = 2.0 * rows * d_in, y_bytes = 2.0 * rows * d_out, tile_bytes = 2.0 * rows * 256;
+  const bool all_stay = x_bytes + y_bytes <= TOK_L2_BYTES;
+  const double traffic = (all_stay || x_bytes <= TOK_L2_BYTES / 4 ? x_bytes : tiles * tile_bytes) + (all_stay || y_bytes <= TOK_L2_BYTES / 4 ? y_bytes : tiles * tile_bytes);
+  const double dealt = std::max(load * TOK_BK * COST_TOKEN.token_hi, traffic / TOK_DEALT_BYTES_PER_US) + COST_TOKEN.fixed + SPLIT_FIXED + out_bytes / ZERO_BYTES_PER_US +
+                       TOK_EVEN_FIXED;
   if (dealt < in_slices) {
     plan.deal_tiles = (int)k; plan.deal_pairs = (int)pairs;
     plan.pairs = (int)(plan.ns > 2 ? slots : tiles + (tiles + k - 1) / k);

@@ -24,7 +24,7 @@ def test_rows_dealt_out_evenly(rows, d_in, d_out):
 
 
 # 38, 32, 56 and 64 tiles, which are whole or in two parts: two sums on zero are the same in either order
-@pytest.mark.parametrize("rows,d_in,d_out", [(2000, 512, 4864), (16384, 1024, 2048), (4001, 1800, 2048), (3001, 1024, 4096)])
+@pytest.mark.parametrize("rows,d_in,d_out", [(2000, 512, 4864), (16384, 1024, 2048), (4001, 1784, 2048), (3001, 1024, 4096)])
 def test_tiles_of_two_parts_repeat_bit_for_bit(rows, d_in, d_out):
     g = torch.Generator(device=DEV).manual_seed(rows)
     X = torch.randn((1, rows, d_in), generator=g, device=DEV).bfloat16()

@@ -81,3 +81,10 @@ def test_rows_of_the_per_token_statistic_dealt_out():
                     # whole tiles and tiles in two parts repeat bit for bit, and they do so wherever whole slices would
                     assert len(p) <= 2 or slices > 2
     assert dealt > 20
+
+
+# operands that L2 holds, or one small operand beside a large one that no two tiles share; 522, 338 and 134 MB that several tiles share
+@pytest.mark.parametrize("rows,d_in,d_out,dealt", [(16384, 1280, 2560, True), (16384, 512, 2048, True), (60000, 256, 6656, True), (60000, 2048, 2304, False), (60000, 1024, 2560, False),
+                                                   (16384, 2048, 2048, False)])
+def test_rows_are_dealt_out_where_they_stay_in_l2(rows, d_in, d_out, dealt):
+    assert (pe.pe_plan_query(pe.PLAN_TOKEN, 0, 1, rows, d_in, d_out, SMS)[1] > 0) == dealt
