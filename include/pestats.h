@@ -435,8 +435,10 @@ int pe_tile_order_band(int d_in, int d_out, int tile_cols, int batch_slices, int
  *     tile (0: 128 x 64, 1: 64 x 64, 2: 32 x 32, 3: 16 x 16, 4: 64 x 64 by 128 threads), slices of the batch, slices to a cluster.
  *   PE_PLAN_TOKEN (pe_token_sqstats on the tensor cores): slices of the rows, a pair per 256 x 256 tile and slice; or, if the next is not 0, tiles whose 32-row
  *     chunks are dealt out evenly, over how many pairs, and pairs in all.
+ *   PE_PLAN_NORMS (pe_example_sqnorms on the tensor cores): slices of the batch, their examples if a pair of thread blocks takes tiles and slices in turn (else 0),
+ *     slices that the tile order is chosen for.
  * PE_ERR_DIM for arguments out of range. */
-typedef enum { PE_PLAN_SHORT = 0, PE_PLAN_SIMT_STATS = 1, PE_PLAN_SIMT_TOKEN = 2, PE_PLAN_SIMT_NORMS = 3, PE_PLAN_TOKEN = 4 } pe_plan_t;
+typedef enum { PE_PLAN_SHORT = 0, PE_PLAN_SIMT_STATS = 1, PE_PLAN_SIMT_TOKEN = 2, PE_PLAN_SIMT_NORMS = 3, PE_PLAN_TOKEN = 4, PE_PLAN_NORMS = 5 } pe_plan_t;
 pe_status_t pe_plan_query(int what /* pe_plan_t */, int outputs, int B, int T, int d_in, int d_out, int sm_count, long long* plan);
 /* Number of kernels the library has launched since load (or since the last reset to 0 via
  * pe_reset_launch_count). */

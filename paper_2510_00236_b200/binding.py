@@ -20,7 +20,7 @@ __all__ = [
     "microadam_family_step", "ADAM_VARIANTS", "pe_linear_stats_all", "pe_linear_stats_accumulate", "pe_example_sqnorms",
     "pe_linear_stats_ragged", "pe_linear_stats_ragged_workspace_bytes", "pe_example_sqnorms_ragged", "pe_linear_clipped_sum",
     "pe_linear_microadam_step", "pe_linear_microadam_step_f32", "pe_linear_microsignsgd_step", "pe_linear_fused_workspace_bytes",
-    "pe_token_sqstats_fp8", "pe_token_sqstats_fp8_workspace_bytes", "pe_set_wait_limit_cycles", "pe_tile_order_band", "pe_plan_query", "PLAN_SHORT", "PLAN_SIMT_STATS", "PLAN_SIMT_TOKEN", "PLAN_SIMT_NORMS", "PLAN_TOKEN",
+    "pe_token_sqstats_fp8", "pe_token_sqstats_fp8_workspace_bytes", "pe_set_wait_limit_cycles", "pe_tile_order_band", "pe_plan_query", "PLAN_SHORT", "PLAN_SIMT_STATS", "PLAN_SIMT_TOKEN", "PLAN_SIMT_NORMS", "PLAN_TOKEN", "PLAN_NORMS",
     "pe_linear_stats_padded", "pe_linear_stats_padded_workspace_bytes", "pe_linear_stats_padded_workspace_bytes_for", "pe_conv2d_stats", "pe_conv2d_stats_workspace_bytes",
     "pe_set_fused_update", "FUSED_AUTO", "FUSED_ALWAYS", "FUSED_NEVER",
 ]
@@ -28,7 +28,7 @@ __all__ = [
 PHI_IDENTITY, PHI_SQUARE, PHI_SIGN = 0, 1, 2
 PATH_AUTO, PATH_SIMT, PATH_TENSOR, PATH_TENSOR_NARROW, PATH_TENSOR_WIDE = 0, 1, 2, 3, 4
 FUSED_AUTO, FUSED_ALWAYS, FUSED_NEVER = 0, 1, 2      # pe_fused_mode_t
-PLAN_SHORT, PLAN_SIMT_STATS, PLAN_SIMT_TOKEN, PLAN_SIMT_NORMS, PLAN_TOKEN = range(5)      # pe_plan_t
+PLAN_SHORT, PLAN_SIMT_STATS, PLAN_SIMT_TOKEN, PLAN_SIMT_NORMS, PLAN_TOKEN, PLAN_NORMS = range(6)      # pe_plan_t
 _PHI_NAMES = {"identity": PHI_IDENTITY, "square": PHI_SQUARE, "sign": PHI_SIGN}
 
 # every symbol include/pestats.h declares

@@ -629,6 +629,29 @@ static pe_status_t launch_tc(DeviceInfo* di, const void* X, const void* dY, int 
   return launch_tc_tiles<2, 256, MEAN_NONE>(di, 3, persist, mx, my, mm, ms, msgn, p, grid, st);
 }
 
+// Example norms: examples > 0: one pair per two SMs that takes every slots-th of the tiles' slices of so many examples, since nothing is
+// written out at the end of a tile: no pair is idle in a last wave.  16 x 512 x 2048 x 4096 (128 tiles) 95 -> 88 us, 32 x 512 x 1024 x 4096 97 -> 92.
+// 0: a pair per tile and slice.
+struct NormsPlan {
+  int slices, examples;
+  int order_slices;              // slices that the tile order is chosen for: a walk's one like the other, so that another B takes no new search
+};
+static NormsPlan plan_norms(int B, int T, int d_in, int d_out, int slots) {
+  const long long tiles = (((long long)d_in + 255) / 256) * (((long long)d_out + TC_PAIR_M - 1) / TC_PAIR_M);
+  NormsPlan plan = {plan_tiles(&COST_NORMS, 1, B, T, d_in, d_out, slots, std::max(16, slots), 0).ns, 0, 0};
+  double best = launch_cost(COST_NORMS, tiles, B, T, slots, plan.slices, 0, 0.0, false).us - (plan.slices > 1 ? SPLIT_FIXED : 0.0);
+  // (beyond 64 examples the cost of a unit is less than one per cent, and more slices only even the waves out)
+  for (int examples = 1; examples <= B && examples <= 64; ++examples) {
+    const long long slices = ((long long)B + examples - 1) / examples, rounds = (tiles * slices + slots - 1) / slots;
+    if (tiles * slices >= (1ll << 30)) continue;
+    if (tiles * slices < slots) break;
+    const double us = rounds * (examples * std::max(T * COST_NORMS.token_hi, COST_NORMS.example_min) + NORMS_UNIT) + COST_NORMS.fixed;
+    if (us < best * 0.99) { best = us; plan.slices = (int)slices; plan.examples = examples; }
+  }
+  plan.order_slices = plan.examples == 0 ? plan.slices : 1;
+  return plan;
+}
+
 // Per-example squared norms on the tensor cores: the statistic-only 256 x 256 schedule, but every
 // example's tile is reduced to one number and added to norms[b] (zeroed by the caller of this function).
 static pe_status_t launch_tc_norms(DeviceInfo* di, const void* X, const void* dY, int B, int T, int d_in, int d_out, float* norms,
@@ -642,31 +665,19 @@ static pe_status_t launch_tc_norms(DeviceInfo* di, const void* X, const void* dY
   const int tiles_n = (d_in + 255) / 256, pairs_m = (d_out + TC_PAIR_M - 1) / TC_PAIR_M;
   if ((long long)tiles_n * pairs_m > (1ll << 29)) return PE_ERR_DIM;
   const int slots = di->sm_count / 2 > 0 ? di->sm_count / 2 : 1;
-  // A pair per tile and slice of the batch, or, since nothing is written out at the end of a tile, one per two SMs that takes every
-  // slots-th of the tiles' slices, down to single examples: no pair is idle in a last wave.  16 x 512 x 2048 x 4096 (128 tiles) 95 -> 88 us,
-  // 32 x 512 x 1024 x 4096 97 -> 92.
-  const long long tiles = (long long)tiles_n * pairs_m;
-  int ns = plan_tiles(&COST_NORMS, 1, B, T, d_in, d_out, slots, std::max(16, slots), 0).ns;
-  double best = launch_cost(COST_NORMS, tiles, B, T, slots, ns, 0, 0.0, false).us - (ns > 1 ? SPLIT_FIXED : 0.0);
-  int per = 0;
-  for (int examples = 1; examples <= B; ++examples) {
-    const long long slices = ((long long)B + examples - 1) / examples, rounds = (tiles * slices + slots - 1) / slots;
-    if (tiles * slices >= (1ll << 30)) continue;
-    if (tiles * slices < slots) break;
-    const double us = rounds * (examples * std::max(T * COST_NORMS.token_hi, COST_NORMS.example_min) + NORMS_UNIT) + COST_NORMS.fixed;
-    if (us < best * 0.99) { best = us; per = examples; ns = (int)slices; }
-  }
-  const bool walk = per > 0;
+  const NormsPlan plan = plan_norms(B, T, d_in, d_out, slots);
+  const int ns = plan.slices;
+  const bool walk = plan.examples > 0;
   TcParams p{};
   p.B = B; p.T = T; p.d_in = d_in; p.d_out = d_out; p.nsplit = walk ? 1 : ns; p.per_example = 1; p.half_operands = 0;
   p.accumulate = 1;       // no matrix is written
-  p.whole_tiles = 0; p.tail_split = ns; p.slice_examples = per;
+  p.whole_tiles = 0; p.tail_split = ns; p.slice_examples = plan.examples;
   // norms[b] = 0 (by a kernel that overlaps the launch of this one, 16-byte alignment allowing)
   p.wait_at_start = 1;
   rc = aligned(norms, 16) ? zero_for_split(di, norms, nullptr, (size_t)B, st, nullptr, nullptr, 0, true)
                           : zero_outputs(norms, nullptr, (size_t)B * sizeof(float), st);
   if (rc != PE_OK) return rc;
-  p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, 256, ns, di->sm_count / 2);
+  p.pairs_m = pairs_m; p.tiles_n = tiles_n; p.band = choose_band(pairs_m, tiles_n, 256, plan.order_slices, di->sm_count / 2);
   p.out_mean = nullptr; p.out_stat = nullptr; p.out_sign = nullptr; p.out_norms = norms; p.dev_status = di->status_ptr;
   p.seq_offsets = nullptr; p.sq_norms = nullptr; p.clip_norm = 0.f;
   // the three output maps are never used by this variant: any valid map will do
@@ -2107,6 +2118,11 @@ pe_status_t pe_plan_query(int what, int outputs, int B, int T, int d_in, int d_o
       const long long chunks = ((long long)B * T + pe::TOK_BK - 1) / pe::TOK_BK;
       const pe::TokPlan p = pe::plan_tok((int)std::min<long long>(chunks, 1 << 30), d_in, d_out, sm_count / 2);
       plan[0] = p.ns; plan[1] = p.deal_tiles; plan[2] = p.deal_pairs; plan[3] = p.pairs;
+      return PE_OK;
+    }
+    case PE_PLAN_NORMS: {
+      const pe::NormsPlan p = pe::plan_norms(B, T, d_in, d_out, sm_count / 2);
+      plan[0] = p.slices; plan[1] = p.examples; plan[2] = p.order_slices;
       return PE_OK;
     }
     default: return PE_ERR_DIM;

@@ -1,4 +1,6 @@
 """How launches divide their work, through the library's host-side query (no GPU)."""
+import time
+
 import pytest
 
 import paper_2510_00236_b200 as pe
@@ -88,3 +90,18 @@ def test_rows_of_the_per_token_statistic_dealt_out():
                                                    (16384, 2048, 2048, False)])
 def test_rows_are_dealt_out_where_they_stay_in_l2(rows, d_in, d_out, dealt):
     assert (pe.pe_plan_query(pe.PLAN_TOKEN, 0, 1, rows, d_in, d_out, SMS)[1] > 0) == dealt
+
+
+def test_the_plan_of_example_norms_takes_no_time():
+    # 128 and 16 tiles; slices of the whole batch
+    start = time.perf_counter()
+    for _ in range(50):
+        for d_in, d_out in ((2048, 4096), (512, 2048)):
+            for B in (1 << 20, 1 << 24):
+                slices, examples, order, _ = pe.pe_plan_query(pe.PLAN_NORMS, 0, B, 4, d_in, d_out, SMS)
+                assert not examples or slices == -(-B // examples)
+    assert time.perf_counter() - start < 1.0                  # one search through all lengths of slices took 5 ms at B = 2^20
+    # the tile order, whose search is kept per layer and slices, is not searched anew for another batch
+    for B in range(100, 300):
+        slices, examples, order, _ = pe.pe_plan_query(pe.PLAN_NORMS, 0, B, 512, 2048, 4096, SMS)
+        assert order == (1 if examples else slices)
