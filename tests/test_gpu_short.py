@@ -11,9 +11,9 @@ DEV = "cuda:0"
 
 
 # one and two MMA steps, odd batches (a last unit of one example), one example, partial 128- and 32-column pieces, tiles on both sides of the
-# number of pairs, batches split so finely that a slice holds one example, widths that go by way of padded copies (rows of 4 k and of odd length)
+# number of pairs, batches split so finely that a slice holds one example, widths that go by way of padded copies (rows of 4 k and of odd length; the sliced tiles of a last wave among them)
 @pytest.mark.parametrize("B,T,d_in,d_out", [(1, 1, 8, 8), (5, 16, 136, 264), (4, 17, 128, 256), (33, 32, 200, 520), (2, 31, 264, 40), (9, 2, 96, 76 * 256),
-                                            (3, 32, 1032, 21 * 256 + 8), (200, 3, 64, 72), (70, 9, 612, 1037), (64, 32, 333, 520)])
+                                            (3, 32, 1032, 21 * 256 + 8), (200, 3, 64, 72), (70, 9, 612, 1037), (64, 32, 333, 520), (49, 2, 1123, 5035)])
 @pytest.mark.parametrize("zeros", [False, True])
 def test_short_sequences_against_fp64(B, T, d_in, d_out, zeros):
     g = torch.Generator(device=DEV).manual_seed(B * T)
