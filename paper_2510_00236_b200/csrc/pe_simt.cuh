@@ -71,7 +71,8 @@ __device__ __forceinline__ float apply_phi(float g, int phi, float coef) {
   return g;
 }
 
-// Four elements from p on, `left` of which are inside the row.  whole: all four, as one aligned load.
+// Four elements from p on, `left` of which are inside the row, as they are loaded.  whole: all four, as one aligned load.  Widened only when they are
+// written to shared memory, so that a chunk's loads are in flight together: WIDENED
 __device__ __forceinline__ float4 load_group(const float* p, int left, bool whole) {
   if (whole) return __ldg(reinterpret_cast<const float4*>(p));
   float v[4];
@@ -79,16 +80,20 @@ __device__ __forceinline__ float4 load_group(const float* p, int left, bool whol
   for (int j = 0; j < 4; ++j) v[j] = j < left ? __ldg(p + j) : 0.f;
   return make_float4(v[0], v[1], v[2], v[3]);
 }
-__device__ __forceinline__ float4 load_group(const __nv_bfloat16* p, int left, bool whole) {
-  uint32_t w[4];
+__device__ __forceinline__ uint4 load_group(const __nv_bfloat16* p, int left, bool whole) {
   if (whole) {
     const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
-    w[0] = u.x << 16; w[1] = u.x & 0xFFFF0000u; w[2] = u.y << 16; w[3] = u.y & 0xFFFF0000u;
-  } else {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) w[j] = j < left ? (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(p) + j) << 16 : 0u;
+    return make_uint4(u.x, u.y, 0u, 0u);
   }
-  return make_float4(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]), __uint_as_float(w[3]));
+  uint32_t w[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) w[j] = j < left ? (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(p) + j) : 0u;
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __forceinline__ float4 widen_group(float4 v, bool) { return v; }
+__device__ __forceinline__ float4 widen_group(uint4 v, bool whole) {
+  if (whole) return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
+  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.y << 16), __uint_as_float(v.z << 16), __uint_as_float(v.w << 16));
 }
 
 // A thread's N operands of one token: N = 1, 2 or 4 consecutive floats, 8 as two groups of four, 4 * SIDE floats apart (SIDE: threads on this
@@ -199,20 +204,21 @@ simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, 
   const int y_tok = threadIdx.x / (ROWS / 4), x_tok = threadIdx.x / (COLS / 4);
   const int y_col = o0 + 4 * (threadIdx.x % (ROWS / 4)), x_col = i0 + 4 * (threadIdx.x % (COLS / 4));
   const bool y_whole = vec_y != 0 && y_col + 3 < d_out, x_whole = vec_x != 0 && x_col + 3 < d_in;
-  float4 sy[Tile::YV], sx[Tile::XV];
+  using Group = std::conditional_t<sizeof(TIn) == 2, uint4, float4>;
+  Group sy[Tile::YV], sx[Tile::XV];
   auto load_chunk = [&]() {            // zero past the example's end and past the matrix edge
     const TIn* yp = dY + (row0 + t + y_tok) * (long long)ldy + y_col;
     const TIn* xp = X + (row0 + t + x_tok) * (long long)ldx + x_col;
     const int y_left = y_col < d_out ? Tb - t - y_tok : 0, x_left = x_col < d_in ? Tb - t - x_tok : 0;
 #pragma unroll
     for (int k = 0; k < Tile::YV; ++k) {
-      sy[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      sy[k] = Group{};
       if (k * Y_STEP < y_left) sy[k] = load_group(yp, d_out - y_col, y_whole);
       yp += (size_t)Y_STEP * ldy;
     }
 #pragma unroll
     for (int k = 0; k < Tile::XV; ++k) {
-      sx[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      sx[k] = Group{};
       if (k * X_STEP < x_left) sx[k] = load_group(xp, d_in - x_col, x_whole);
       xp += (size_t)X_STEP * ldx;
     }
@@ -280,9 +286,9 @@ simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, 
     float* const y = simt_smem + buf * Tile::CHUNK;
     float* const x = y + KT * ROWS;
 #pragma unroll
-    for (int k = 0; k < Tile::YV; ++k) put(y + 4 * (threadIdx.x + k * Tile::THREADS), sy[k]);
+    for (int k = 0; k < Tile::YV; ++k) put(y + 4 * (threadIdx.x + k * Tile::THREADS), widen_group(sy[k], y_whole));
 #pragma unroll
-    for (int k = 0; k < Tile::XV; ++k) put(x + 4 * (threadIdx.x + k * Tile::THREADS), sx[k]);
+    for (int k = 0; k < Tile::XV; ++k) put(x + 4 * (threadIdx.x + k * Tile::THREADS), widen_group(sx[k], x_whole));
     __syncthreads();           // a buffer is written again two chunks later, behind the barrier that follows its last reads
     // the next chunk's loads are in flight during this one's arithmetic
     t += KT;
