@@ -34,6 +34,7 @@ template <int TM_, int TN_, int KT_, int THREADS_ = 256>
 struct SimtTile {
   static constexpr int TM = TM_, TN = TN_, KT = KT_, THREADS = THREADS_;
   static constexpr int TY = THREADS / 16;                        // TY x 16 threads
+  static constexpr int BLOCKS = TM * TN == 4 ? 3 : 512 / THREADS;       // an SM holds at least (32 x 32: 86 to 92 registers, and two blocks, if left alone)
   static constexpr int ROWS = TY * TM, COLS = 16 * TN;
   static constexpr int CHUNK = KT * (ROWS + COLS);               // floats of one chunk: dY part, then X part
   static constexpr int YV = KT * ROWS / 4 / THREADS, XV = KT * COLS / 4 / THREADS;   // 4-column groups per thread
@@ -131,7 +132,7 @@ __device__ __forceinline__ int micro_index(int thread, int j) { return N <= 4 ? 
 // ldx, ldy: elements from one token's row of X, dY to the next.
 // SUMS: running sums per entry: 2 = sum_b phi(G_b) and sum_b G_b, 1 = the former alone (or the contraction of MODE_TOKEN).
 template <typename TIn, int MODE, class Tile, int SUMS>
-__global__ void __launch_bounds__(Tile::THREADS, 512 / Tile::THREADS)
+__global__ void __launch_bounds__(Tile::THREADS, Tile::BLOCKS)
 simt_stats_kernel(const TIn* __restrict__ X, const TIn* __restrict__ dY, int B, int T, int d_in, int d_out,
                   int phi, float* __restrict__ out_mean, float* __restrict__ out_stat, int accumulate, int cluster, int ldx, int ldy, int vec_x, int vec_y,
                   SimtExtra ex, FusedOpt opt) {
