@@ -431,7 +431,7 @@ int pe_tile_order_band(int d_in, int d_out, int tile_cols, int batch_slices, int
  *   PE_PLAN_SHORT (statistics of bf16 sequences of T <= 32 tokens; outputs: 1 = sum of G_b, 2 = of squares, 4 = of signs, added up):
  *     tiles contracted over the whole batch by one pair of thread blocks, batch slices of every other tile, examples of the longest
  *     running sum, and, for the square alone, how many of them are summed by themselves at a time.
- *   PE_PLAN_SIMT_STATS, _TOKEN, _NORMS (the SIMT kernel; outputs: 1 = the mean is wanted beside the statistic):
+ *   PE_PLAN_SIMT_STATS, _TOKEN, _NORMS (the SIMT kernel; outputs: 1 = the mean is wanted beside the statistic, 4 = signs alone):
  *     tile (0: 128 x 64, 1: 64 x 64, 2: 32 x 32, 3: 16 x 16, 4: 64 x 64 by 128 threads), slices of the batch, slices to a cluster.
  *   PE_PLAN_TOKEN (pe_token_sqstats on the tensor cores): slices of the rows, a pair per 256 x 256 tile and slice; or, if the next is not 0, tiles whose 32-row
  *     chunks are dealt out evenly, over how many pairs, and pairs in all.

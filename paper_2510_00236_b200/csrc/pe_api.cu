@@ -695,7 +695,7 @@ constexpr int SIMT_MAX_D_OUT = 65535 * 128;
 struct SimtPlan {
   int tile, slices, cluster;      // tile: index into the five shapes
 };
-static SimtPlan plan_simt(int sm_count, int mode, bool two_sums, int B, int T, int d_in, int d_out) {
+static SimtPlan plan_simt(int sm_count, int mode, bool two_sums, bool exact, int B, int T, int d_in, int d_out) {
   constexpr int HALF = 4;
   static constexpr int rows[5] = {SimtTile84::ROWS, SimtTile44::ROWS, SimtTile22::ROWS, SimtTile11::ROWS, SimtTileHalf<MODE_STATS>::ROWS};
   static constexpr int cols[5] = {SimtTile84::COLS, SimtTile44::COLS, SimtTile22::COLS, SimtTile11::COLS, SimtTileHalf<MODE_STATS>::COLS};
@@ -747,9 +747,9 @@ static SimtPlan plan_simt(int sm_count, int mode, bool two_sums, int B, int T, i
       if (cost < best_cost) { best_cost = cost; best = {k, s, s < SIMT_MAX_CLUSTER ? s : SIMT_MAX_CLUSTER}; }
     }
   }
-  // Nor are sums over the examples: the last tile in more slices, or in as many as the best of the other tiles has (60 x 24 x 900 x 300, both sums: error of
+  // Nor are sums over the examples, but for those of signs alone, which are exact: the last tile in more slices, or in as many as the best of the other tiles has (60 x 24 x 900 x 300, both sums: error of
   // the mean 1.23e-7 at 53 us in 4 slices, 1.16e-7 at 56 in 16, 1.16e-7 at 79 on the 128 x 64 tile in 32).
-  if (best.tile == HALF && mode == MODE_STATS) {
+  if (best.tile == HALF && mode == MODE_STATS && !exact) {
     int s = best.slices;
     while (chain(s) > chain(other_slices) && s < 32 && 2ll * s <= units) s *= 2;
     if (chain(s) > chain(other_slices)) s = other_slices;
@@ -799,7 +799,7 @@ static pe_status_t launch_simt(DeviceInfo* di, const TIn* X, const TIn* dY, int 
                                const FusedOpt* opt = nullptr, int pitch_x = 0, int pitch_y = 0) {
   const int ldx = pitch_x ? pitch_x : d_in, ldy = pitch_y ? pitch_y : d_out;
   const bool two_sums = out_mean || (opt && opt->kind == OPT_ADAM);
-  SimtPlan plan = plan_simt(di->sm_count, MODE, two_sums, B, T, d_in, d_out);
+  SimtPlan plan = plan_simt(di->sm_count, MODE, two_sums, phi == PE_PHI_SIGN && !two_sums, B, T, d_in, d_out);
   if (opt && plan.slices > SIMT_MAX_CLUSTER) plan.slices = SIMT_MAX_CLUSTER;      // a fused update needs the whole batch in one cluster
   if (MODE != MODE_NORMS && plan.slices > plan.cluster && !accumulate) {
     pe_status_t rc = zero_outputs(out_mean, out_stat, (size_t)d_in * d_out * sizeof(float), st);
@@ -2115,7 +2115,7 @@ pe_status_t pe_plan_query(int what, int outputs, int B, int T, int d_in, int d_o
     case PE_PLAN_SIMT_NORMS: {
       if (d_out > pe::SIMT_MAX_D_OUT) return PE_ERR_DIM;
       const int mode = what == PE_PLAN_SIMT_STATS ? pe::MODE_STATS : what == PE_PLAN_SIMT_TOKEN ? pe::MODE_TOKEN : pe::MODE_NORMS;
-      const pe::SimtPlan p = pe::plan_simt(sm_count, mode, mean, B, T, d_in, d_out);
+      const pe::SimtPlan p = pe::plan_simt(sm_count, mode, mean, sign && !mean, B, T, d_in, d_out);
       plan[0] = p.tile; plan[1] = p.slices; plan[2] = p.cluster;
       return PE_OK;
     }

@@ -53,6 +53,10 @@ def test_smaller_blocks_do_not_lengthen_fp32_sums(B, T, d_in, d_out, others):
     assert chain(slices) <= chain(others)
 
 
+def test_sums_of_signs_alone_are_exact_in_any_number_of_slices():
+    assert pe.pe_plan_query(pe.PLAN_SIMT_STATS, SIGN, 60, 24, 900, 300, SMS)[:2] == (4, 4)
+
+
 def _parts(rows, d_in, d_out):
     """Per tile of the per-token statistic the chunks that each pair takes, by the plan."""
     chunks, tiles, slots = -(-rows // 32), -(-d_in // 256) * -(-d_out // 256), SMS // 2
