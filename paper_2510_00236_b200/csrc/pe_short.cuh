@@ -191,46 +191,12 @@ short_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         uint32_t next_ph = ph;
         if (next_s == SHORT_STAGES) { next_s = 0; next_ph ^= 1u; }
         if (free_s >= SHORT_STAGES) free_s -= SHORT_STAGES;
-        if (!read_ahead) {
-          if (!mbar_wait_warp(done_bar(s), ph, abort_flag, p.dev_status, SHORT_WAIT_ACC)) { ok = false; break; }
-          tc_fence_after();
-          tmem_ld_issue(taddr, g[0]);
-          tmem_ld_issue(taddr + SHORT_NT, f[0]);
-        }
-        read_ahead = false;
-        bool next_done = false;
-#pragma unroll
-        for (int k = 0; k < STEPS; ++k) {
-          uint32_t(&gk)[W] = g[k & 1];
-          uint32_t(&fk)[W] = f[k & 1];
-          tmem_ld_wait_for(gk, fk);
-          if (k + 1 < STEPS) {
-            tmem_ld_issue(taddr + (k + 1) * W, g[(k + 1) & 1]);
-            tmem_ld_issue(taddr + SHORT_NT + (k + 1) * W, f[(k + 1) & 1]);
-            // whether the next unit is there already is asked a step before the answer is needed
-            if (k + 2 == STEPS && b + SHORT_G < t.b_end) next_done = mbar_test_wait(done_bar(next_s), next_ph);
-          }
-          if (!pair_of) {
-#pragma unroll
-            for (int j = 0; j < W; ++j) fk[j] = 0u;
-          }
-          if (k + 1 == STEPS) {
-            tc_fence_before();
-            __syncwarp();
-            mbar_arrive_cluster_if(lane == 0, leader_go + 8u * free_s);        // this accumulator unit may be filled again
-            if (__all_sync(0xffffffffu, next_done)) {
-              tc_fence_after();
-              const uint32_t ahead = lane_base + (uint32_t)((buf ^ 1) * SHORT_G * SHORT_NT);
-              tmem_ld_issue(ahead, g[0]);
-              tmem_ld_issue(ahead + SHORT_NT, f[0]);
-              read_ahead = true;
-            }
-          }
+        auto fold = [&](int k) {
 #pragma unroll
           for (int j = 0; j < W; j += 2) {
             const int c = k * W + j;
-            const uint64_t g2 = f32x2_pack(__uint_as_float(gk[j]), __uint_as_float(gk[j + 1]));
-            const uint64_t f2 = f32x2_pack(__uint_as_float(fk[j]), __uint_as_float(fk[j + 1]));
+            const uint64_t g2 = f32x2_pack(__uint_as_float(g[k & 1][j]), __uint_as_float(g[k & 1][j + 1]));
+            const uint64_t f2 = f32x2_pack(__uint_as_float(f[k & 1][j]), __uint_as_float(f[k & 1][j + 1]));
             if constexpr (MEAN) f32x2_unpack(f32x2_add(f32x2_add(f32x2_pack(acc_mean[c], acc_mean[c + 1]), g2), f2), acc_mean[c], acc_mean[c + 1]);
             if constexpr (SQUARE) {
               float& s0 = RUNS ? acc_run[RUNS ? c : 0] : acc_stat[c];
@@ -241,7 +207,44 @@ short_stats_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             if constexpr (SIGN && !COUNT)
               f32x2_unpack(f32x2_add(f32x2_add(f32x2_pack(acc_stat[c], acc_stat[c + 1]), sign_half2(g2)), sign_half2(f2)), acc_stat[c], acc_stat[c + 1]);
           }
+        };
+        // Reads that are in flight cross no join of branches that defines their registers: what the compiler might move there would be read before it
+        // has arrived.
+        if (!read_ahead) {
+          if (!mbar_wait_warp(done_bar(s), ph, abort_flag, p.dev_status, SHORT_WAIT_ACC)) { ok = false; break; }
+          tc_fence_after();
+          tmem_ld_issue(taddr, g[0]);
+          tmem_ld_issue(taddr + SHORT_NT, f[0]);
+          tmem_ld_wait_for(g[0], f[0]);
         }
+        bool next_done = false;
+#pragma unroll
+        for (int k = 0; k < STEPS; ++k) {
+          if (k > 0) tmem_ld_wait_for(g[k & 1], f[k & 1]);
+          if (k + 1 < STEPS) {
+            tmem_ld_issue(taddr + (k + 1) * W, g[(k + 1) & 1]);
+            tmem_ld_issue(taddr + SHORT_NT + (k + 1) * W, f[(k + 1) & 1]);
+            // whether the next unit is there already is asked a step before the answer is needed
+            if (k + 2 == STEPS && b + SHORT_G < t.b_end) next_done = mbar_test_wait(done_bar(next_s), next_ph);
+          }
+          if (!pair_of) {
+#pragma unroll
+            for (int j = 0; j < W; ++j) f[k & 1][j] = 0u;
+          }
+          if (k + 1 < STEPS) {
+            fold(k);
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        mbar_arrive_cluster_if(lane == 0, leader_go + 8u * free_s);        // this accumulator unit may be filled again
+        read_ahead = __all_sync(0xffffffffu, next_done);
+        if (read_ahead) tc_fence_after();
+        const uint32_t ahead = lane_base + (uint32_t)((buf ^ 1) * SHORT_G * SHORT_NT);
+        tmem_ld_issue_if(read_ahead, ahead, g[0]);
+        tmem_ld_issue_if(read_ahead, ahead + SHORT_NT, f[0]);
+        fold(STEPS - 1);
+        tmem_ld_wait_for(g[0], f[0]);
         if constexpr (RUNS) {
           if (((b - t.b_begin + SHORT_G) & (p.sum_run - 1)) == 0 || b + SHORT_G >= t.b_end) {
 #pragma unroll

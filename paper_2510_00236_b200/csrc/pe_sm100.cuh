@@ -332,6 +332,23 @@ __device__ __forceinline__ void tmem_ld_wait_for(uint32_t (&r)[16], uint32_t (&q
 __device__ __forceinline__ void tmem_ld_issue(uint32_t taddr, uint32_t (&r)[32]) { tmem_ld_32x32b_x32_issue(taddr, r); }
 __device__ __forceinline__ void tmem_ld_issue(uint32_t taddr, uint32_t (&r)[16]) { tmem_ld_32x32b_x16_issue(taddr, r); }
 
+// The same, or nothing, by a predicate that holds for the whole warp or for no lane: without a branch, so that no join lies between the read and
+// the wait that names its registers (what the compiler might move there would be read before it has arrived).
+__device__ __forceinline__ void tmem_ld_issue_if(bool all, uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %17, 0;\n\t@p tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t}"
+      : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+      : "r"(taddr), "r"((uint32_t)all)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld_issue_if(bool all, uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %9, 0;\n\t@p tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t}"
+      : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
+      : "r"(taddr), "r"((uint32_t)all)
+      : "memory");
+}
+
 // 32 lanes x 16 consecutive columns, and the wait, in one statement.
 __device__ __forceinline__ void tmem_ld_32x32b_x16_wait(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
