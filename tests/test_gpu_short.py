@@ -11,9 +11,11 @@ DEV = "cuda:0"
 
 
 # one and two MMA steps, odd batches (a last unit of one example), one example, partial 128- and 32-column pieces, tiles on both sides of the
-# number of pairs, batches split so finely that a slice holds one example, widths that go by way of padded copies (rows of 4 k and of odd length; the sliced tiles of a last wave among them)
+# number of pairs, batches split so finely that a slice holds one example, widths that go by way of padded copies (rows of 4 k and of odd length),
+# whole tiles of many examples beside sliced ones, with and without copies
 @pytest.mark.parametrize("B,T,d_in,d_out", [(1, 1, 8, 8), (5, 16, 136, 264), (4, 17, 128, 256), (33, 32, 200, 520), (2, 31, 264, 40), (9, 2, 96, 76 * 256),
-                                            (3, 32, 1032, 21 * 256 + 8), (200, 3, 64, 72), (70, 9, 612, 1037), (64, 32, 333, 520), (49, 2, 1123, 5035)])
+                                            (3, 32, 1032, 21 * 256 + 8), (200, 3, 64, 72), (70, 9, 612, 1037), (64, 32, 333, 520), (49, 2, 1123, 5035),
+                                            (90, 20, 1544, 2824)])
 @pytest.mark.parametrize("zeros", [False, True])
 def test_short_sequences_against_fp64(B, T, d_in, d_out, zeros):
     g = torch.Generator(device=DEV).manual_seed(B * T)
@@ -89,3 +91,39 @@ def test_precision_of_sums_over_many_examples(outputs, B, T, d_in, d_out, p):
     if mean is not None:
         assert (mean[rows].double() - m).norm() <= 1.25 * u * math.sqrt((p + B / p) / 6) * m.norm()
     assert (square[rows].double() - q).norm() <= 1.25 * u * math.sqrt(p * p / (18 * B) + B / p / 18 + T / 6) * q.norm()
+
+
+# an infinity or a NaN of one example reaches its own column of the sums and nothing else: not the other example of its unit of two, the missing one of a
+# last unit, the tokens past the sequence's end
+@pytest.mark.parametrize("T", [2, 17, 32])
+@pytest.mark.parametrize("bad", [0, 1, 4])
+def test_infinities_and_nan_stay_in_their_columns(T, bad):
+    B, d_in, d_out = 5, 136, 264
+    g = torch.Generator(device=DEV).manual_seed(T)
+    X = torch.randn((B, T, d_in), generator=g, device=DEV).bfloat16()
+    dY = (torch.rand((B, T, d_out), generator=g, device=DEV) + 0.5).bfloat16()
+    dY[:, :, ::3] *= -1
+    X[bad, T - 1, 7], X[bad, 0, 70], X[bad, 0, 130] = float("inf"), float("-inf"), float("nan")
+    new = lambda: torch.empty((d_out, d_in), device=DEV)       # noqa: E731
+    mean, square, sign, mean1, square1, square2, mean3, sign3, sign4 = (new() for _ in range(9))
+    pe.pe_linear_stats_all(X, dY, mean, square, sign)
+    pe.pe_linear_stats(X, dY, "square", mean1, square1)
+    pe.pe_linear_stats(X, dY, "square", None, square2)
+    pe.pe_linear_stats(X, dY, "sign", mean3, sign3)
+    pe.pe_linear_stats(X, dY, "sign", None, sign4)
+    assert pe.pe_get_async_status(DEV) == (0, 0)
+    G = torch.einsum("bto,bti->boi", dY.double(), X.double())
+    mag = torch.einsum("bto,bti->boi", dY.double().abs(), X.double().abs().nan_to_num(0, 0, 0))
+    finite = torch.ones(d_in, dtype=torch.bool, device=DEV)
+    finite[[7, 70, 130]] = False
+    eps = (T + B) * 2.0 ** -23
+    for got in (mean, mean1, mean3):
+        assert torch.all((got.double() - G.sum(0))[:, finite].abs() <= (eps * mag.sum(0))[:, finite])
+        assert torch.equal(got[:, [7, 70]].double(), G.sum(0)[:, [7, 70]]) and torch.isnan(got[:, 130]).all()
+    for got in (square, square1, square2):
+        assert torch.all((got.double() - (G * G).sum(0))[:, finite].abs() <= (3 * eps * (mag * mag).sum(0))[:, finite])
+        assert torch.isinf(got[:, [7, 70]]).all() and torch.isnan(got[:, 130]).all()
+    number = torch.arange(d_in, device=DEV) != 130               # (the sign of a NaN is not specified)
+    unsure = (G.abs() <= eps * mag).sum(0)
+    for got in (sign, sign3, sign4):
+        assert torch.all((got.double() - G.sign().sum(0))[:, number].abs() <= 2 * unsure[:, number])
