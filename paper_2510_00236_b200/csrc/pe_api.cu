@@ -314,9 +314,9 @@ static pe_status_t launch_dependent(Kernel kernel, dim3 grid, int threads, int s
   if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess) { cudaGetLastError(); return PE_ERR_CUDA; }
   return check_launch();
 }
-// Zeroes up to three [d_out, d_in] outputs with a kernel that lets its successor start when everything older has completed: the successor
-// may run its main loop beside it.  A programmatic dependent itself: 25 layers with MicroAdam 1597 -> 1576 us against ordinary launches, 1024 x 32 x 1024^2,
-// both outputs, 113 -> 110, 64 x 32 x 256 x 4096 18.6 -> 16.2.  early: the successor starts at once and has to wait for it before anything else (what came
+// Zeroes up to three [d_out, d_in] outputs with a kernel that lets its successor start when everything older has completed: the successor's
+// blocks follow on each SM as the zeroing block leaves it.  A programmatic dependent itself: against ordinary launches 1024 x 32 x 1024^2, both outputs,
+// 113 -> 110, 64 x 32 x 256 x 4096 18.6 -> 16.2 us (25 layers with MicroAdam 1597 -> 1576, which is within the runs' spread).  early: the successor starts at once and has to wait for it before anything else (what came
 // before may still be running), worth it where there is little to zero: the norms of 64 x 256 x 512 x 2048 36.1 -> 32.6 us.
 // Shared memory that these kernels do not use, so that an SM takes one block: as dependents they would else crowd the SMs that become free first, and
 // zero 8 MB from there (64 x 256 x 512 x 2048, three statistics, calls one after the other, 47.2 us against 43.4; 45.2 as ordinary launches).

@@ -7,12 +7,14 @@
 //  - One barrier pair per stage.  go: the operands' bytes and the 16 arrivals of the epilogue warps that free the accumulator unit (on the barrier of
 //    the stage that will be contracted into it), so that the issuer waits once per unit; done: one commit, which the epilogue and the producers
 //    wait for.  Separate barriers for stages and accumulators cost the issuer 680 of 901 cycles per unit.
-//  - The epilogue asks for the next unit's barrier a read ahead, without blocking, and issues that unit's first reads before its last
-//    arithmetic; it arrives by a predicated instruction (a branch around it costs about 80 cycles).  Releasing and looking ahead took 300 cycles a unit.
+//  - The epilogue asks for the next unit's barrier a read ahead, without blocking, and issues that unit's first reads, by a predicate, before its
+//    last arithmetic; it arrives by a predicated instruction (a branch around it costs about 80 cycles).  Releasing and looking ahead took 300 cycles a unit.
 //  - Results leave through a panel of shared memory of their own (TMA stores, or adds for a slice of the batch), so that the operand ring is
 //    filled for the next tile meanwhile.  Adds from registers, lanes transposed, took 7 us per tile and two sums.
-// 1024 x 32 tokens x 1024^2: both outputs 135 -> 110 us (clock cycles a unit: 901 -> 750), sign 166 -> 155, square 98 -> 92, three statistics
-// 275 -> 244; 128 x 32 x 4096^2: 219 -> 196, 304 -> 270, 178 -> 160, 472 -> 429; 512 x 2 x 1024^2: 72 -> 58, 92 -> 81, .. , 142 -> 127.
+// 1024 x 32 tokens x 1024^2: both outputs 135 -> 110 us (clock cycles a unit: 901 -> 750), sign 166 -> 155, three statistics
+// 275 -> 244; 128 x 32 x 4096^2: 219 -> 196, 304 -> 270, 472 -> 429; 512 x 2 x 1024^2: 72 -> 58, 92 -> 81, 142 -> 127.  The
+// square alone gains where tiles or tokens are few (512 x 8 x 4096 x 2048 407 -> 368, 64 x 32 x 4096^2 105 -> 99, 40 drawn layers 14 %, geometric mean); large layers of 32 tokens are
+// equal or up to 4 % slower than on the 256 x 256 tile, at a quarter of its rounding error (800 x 32 x 1024 x 4096 279 -> 287 us, 4.2e-7 -> 7.9e-8).
 // (before: stages and accumulators of tc_stats_kernel with two examples each).  What is left above the arithmetic is the two units' round trip
 // from release to the next unit's reads, about 780 cycles at T = 32.  Measured and dropped: signs counted from the sign bits by byte
 // permutes and 16-bit adds with zeros looked for by three-way minima (three statistics 244 -> 228 us where G_b holds no zeros, but every zero
