@@ -1468,7 +1468,10 @@ static bool unfold_tile(const ConvGeom& g, int sm_count, UnfoldTile* t) {
       if ((long long)chan * kk < (1 << 14) && cols < (1 << 16) && smem(chan, (int)cols) <= UNFOLD_SMEM_BYTES) {
         // one output row: the kernel's rows alone.  (An extra column where pairs have to start at an even one, and a whole pair at the end: less than
         // the 4 bytes per feature counted above.)
-        const int even = ((int)cols + 2) & ~1;
+        int even = ((int)cols + 2) & ~1;
+        // Rows an odd number of words apart, where there is room: threads side by side gather from rows two or three apart (12 images of 64 x 76 x 76, 3 x 3: 40
+        // words 93 us, 39 before pairs were loaded 85, 41 60; 32 of 3 x 56 x 56, 7 x 7, 44.5 -> 38.2).
+        if (even % 4 == 0 && (long long)chan * g.Kh * (even + 2) * 2 <= UNFOLD_SMEM_BYTES) even += 2;
         *t = {w, 1, chan, even, g.Kh, g.dh, 1, chan * g.Kh * even * 2};
         // Several output rows share their input rows, as long as about four blocks are left to an SM: fewer blocks hide less of each other's
         // latency (8 images of 64 x 28 x 28, 3 x 3, one row to a block 32 us, eight 39 before the loads were batched).
